@@ -730,46 +730,23 @@ static EncodeTiledFn encode_fn() {
     return fn;
 }
 
-struct MapKey {
-    const void* ptr;
-    int K, rows, box_rows, depth;   // depth 0: 2-D map; depth >= 1: 3-D map whose box holds `depth` chunks
-    bool operator==(const MapKey& o) const {
-        return ptr == o.ptr && K == o.K && rows == o.rows && box_rows == o.box_rows && depth == o.depth;
-    }
-};
-struct MapEntry {
-    MapKey key;
-    CUtensorMap map;
-};
-
 // Tensor map of a [rows, K] row-major bf16 matrix, 128-byte swizzled, out-of-range elements read as zero.
 //   depth == 0: 2-D (K, rows), box = 64 elements (128 bytes) x box_rows.
 //   depth >= 1: 3-D view (64, rows, K/64) with strides (K*2, 128) bytes, box = 64 x box_rows x depth, so a
 //               single copy lands `depth` consecutive k-chunks as `depth` consecutive [box_rows][128 B]
 //               tiles.  Needs K % 64 == 0 (a ragged last chunk would run into the next row).
-// Encoded maps are cached by (pointer, shape).
+// Encoded for every call: 0.05 us on the host, where a cache of 256 maps (searched under a lock; fewer than the layers of
+// a model need, so every lookup of a decoding stack missed) cost more than that.
 static int get_tensor_map(const void* ptr, int K, int rows, int box_rows, int depth, CUtensorMap* out) {
-    static std::mutex mu;
-    static std::vector<MapEntry> cache;
-    static size_t next_evict = 0;
-    const MapKey key{ptr, K, rows, box_rows, depth};
-    std::lock_guard<std::mutex> lock(mu);
-    for (const MapEntry& e : cache)
-        if (e.key == key) {
-            *out = e.map;
-            return METEORA_OK;
-        }
     EncodeTiledFn fn = encode_fn();
     if (!fn) return METEORA_ERR_CUDA;
-    MapEntry e;
-    e.key = key;
     CUresult r;
     if (depth == 0) {
         const cuuint64_t gdim[2] = {(cuuint64_t)K, (cuuint64_t)rows};
         const cuuint64_t gstride[1] = {(cuuint64_t)K * 2};
         const cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)box_rows};
         const cuuint32_t estride[2] = {1, 1};
-        r = fn(&e.map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), gdim, gstride, box, estride,
+        r = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), gdim, gstride, box, estride,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     } else {
@@ -777,19 +754,11 @@ static int get_tensor_map(const void* ptr, int K, int rows, int box_rows, int de
         const cuuint64_t gstride[2] = {(cuuint64_t)K * 2, (cuuint64_t)kBK * 2};
         const cuuint32_t box[3] = {(cuuint32_t)kBK, (cuuint32_t)box_rows, (cuuint32_t)depth};
         const cuuint32_t estride[3] = {1, 1, 1};
-        r = fn(&e.map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), gdim, gstride, box, estride,
+        r = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), gdim, gstride, box, estride,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     }
-    if (r != CUDA_SUCCESS) return METEORA_ERR_CUDA;
-    if (cache.size() < 256) {
-        cache.push_back(e);
-    } else {
-        cache[next_evict] = e;
-        next_evict = (next_evict + 1) % cache.size();
-    }
-    *out = e.map;
-    return METEORA_OK;
+    return r == CUDA_SUCCESS ? METEORA_OK : METEORA_ERR_CUDA;
 }
 
 // Tensor map of y[T, d_out] (bf16, row-major) for storing a tile of 128 outputs x box_tokens tokens from
