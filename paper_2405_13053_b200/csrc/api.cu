@@ -40,6 +40,7 @@ Workspace carve_workspace(const meteora_shape_t& s_in, void* base) {
     const size_t bn = (T + 15) / 16 * 16;
     const size_t part_tiles = s.T <= 256 ? row_tiles + 148 : 0;
     ws.part_g = (float*)take(part_tiles * bn * 128 * sizeof(float));
+    ws.simt_part = s.T > 0 && !tc_path_supported(s) ? (float*)take(simt_part_floats(s_in) * sizeof(float)) : nullptr;
     ws.x_dev = take(T * s.d_in * es);
     ws.y_dev = take(T * s.d_out * es);
     const bool pad = rank_pad_applies(s_in);
@@ -144,9 +145,7 @@ static int forward_device(const void* x, const void* W0, const void* A, const vo
         if (timed) cudaEventRecord(pf.ev[2 * pf.used++ + 1], st);
         return rc;
     }
-    if ((rc = launch_gate_topk(x, Wg, s, ws.topk_idx, ws.topk_w, nullptr, st)) != METEORA_OK) return rc;
-    if ((rc = launch_shrink_tokens(x, A, ws.topk_idx, ws.topk_w, s, ws.uw, st)) != METEORA_OK) return rc;
-    return launch_gemm_simt(x, W0, B, ws.topk_idx, ws.uw, s, y, st);
+    return launch_forward_simt(x, W0, A, B, Wg, s, ws, y, st);
 }
 
 // Workspace of a group call: the modules' own workspaces one after the other (module 0's header serves the

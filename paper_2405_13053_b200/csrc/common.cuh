@@ -28,6 +28,7 @@ struct Workspace {
     int32_t* tile_ctr;  // fused decode: one counter per 128-row tile of d_out (inside the header)
     void* A_pad;        // bf16 layers whose rank is no multiple of 8: A and B zero-padded to the next multiple,
     void* B_pad;        //           [N,r8,d_in] and [N,d_out,r8], rewritten by every call (nullptr otherwise)
+    float* simt_part;   // plain path only: [slice][T][stacked rows] partial products of W0, A and Wg (nullptr otherwise)
     void* x_dev;        // [T,d_in]  staging for the host-buffer entry point
     void* y_dev;        // [T,d_out]
     size_t bytes;       // total
@@ -70,13 +71,12 @@ int launch_route(const int32_t* topk_idx, int T, int k, int N, int32_t* counts, 
 // lora.cu
 int launch_shrink_segments(const void* x, const void* A, const int32_t* offsets, const int32_t* perm,
                            const meteora_shape_t& s, float* u, cudaStream_t st);
-int launch_shrink_tokens(const void* x, const void* A, const int32_t* topk_idx, const float* topk_w,
-                         const meteora_shape_t& s, float* uw, cudaStream_t st);
 int launch_expand(const void* B, const int32_t* topk_idx, const float* topk_w, const float* u,
                   const meteora_shape_t& s, float* delta, cudaStream_t st);
 // gemm_simt.cu
-int launch_gemm_simt(const void* x, const void* W0, const void* B, const int32_t* topk_idx, const float* uw,
-                     const meteora_shape_t& s, void* y, cudaStream_t st);
+size_t simt_part_floats(const meteora_shape_t& s);   // scratch of the plain path: sizes Workspace::simt_part
+int launch_forward_simt(const void* x, const void* W0, const void* A, const void* B, const void* Wg, const meteora_shape_t& s,
+                        const Workspace& ws, void* y, cudaStream_t st);
 // wgemm_tcgen05.cu
 bool tc_path_supported(const meteora_shape_t& s);
 int tc_stacked_pitch(const meteora_shape_t& s, int* col_logits);  // row pitch (floats) of u_all

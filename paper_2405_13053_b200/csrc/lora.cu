@@ -1,10 +1,7 @@
 // Low-rank shrink (x A_i) and expand ((x A_i) B_i, weighted and summed over the picks) of Eq. 2
-// on CUDA cores.  The shrink has two forms:
-//   - adapter by adapter over the grouped slots (Sec. 3.3 grouping from meteora_route): a CTA
-//     takes up to kSegSlots slots of ONE adapter, stages that adapter's A_i in shared memory
-//     chunk by chunk and reuses it for all its slots;
-//   - slot by slot in token order (one warp per (token, pick)), used by the plain forward path.
-// The expand is token-major and sums the k picks in pick order, so it needs no atomics.
+// on CUDA cores.  The shrink goes adapter by adapter over the grouped slots (Sec. 3.3 grouping from meteora_route): a CTA
+// takes up to kSegSlots slots of ONE adapter, stages that adapter's A_i in shared memory chunk by chunk and reuses it
+// for all its slots.  The expand is token-major and sums the k picks in pick order, so it needs no atomics.
 #include "common.cuh"
 
 namespace meteora {
@@ -139,24 +136,6 @@ k_shrink_segments(const TI* __restrict__ x, const TI* __restrict__ A, const int3
     }
 }
 
-// One warp per slot (t, j): uw[t,j,:] = w[t,j] * A[idx[t,j]] x[t].
-template <typename TI>
-__global__ void __launch_bounds__(256)
-k_shrink_tokens(const TI* __restrict__ x, const TI* __restrict__ A, const int32_t* __restrict__ topk_idx,
-                const float* __restrict__ topk_w, int S, int d_in, int N, int r, int k, float* __restrict__ uw) {
-    const int lane = threadIdx.x & 31;
-    const int s = blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (s >= S) return;
-    const int e = min(max(topk_idx[s], 0), N - 1);
-    const float w = topk_w[s];
-    const bool vec = (d_in % 8) == 0;
-    const TI* xt = x + (size_t)(s / k) * d_in;
-    for (int p = 0; p < r; ++p) {
-        const float v = warp_dot(xt, A + ((size_t)e * r + p) * d_in, d_in, lane, vec);
-        if (lane == 0) uw[(size_t)s * r + p] = w * v;
-    }
-}
-
 // delta[t,o] = sum_j w[t,j] * sum_p B[idx[t,j], o, p] * u[t*k + j, p].   One thread per output row o,
 // kExpTokens tokens per CTA so that the B rows of an adapter picked by several of them stay in L1.
 constexpr int kExpTokens = 8;
@@ -213,20 +192,6 @@ int launch_shrink_segments(const void* x, const void* A, const int32_t* offsets,
     else
         k_shrink_segments<float><<<blocks, kSegWarps * 32, 0, st>>>((const float*)x, (const float*)A, offsets, perm,
                                                                     s.d_in, s.N, s.r, s.k, u);
-    return last_launch_status();
-}
-
-int launch_shrink_tokens(const void* x, const void* A, const int32_t* topk_idx, const float* topk_w,
-                         const meteora_shape_t& s, float* uw, cudaStream_t st) {
-    if (s.T == 0) return METEORA_OK;
-    const int S = s.T * s.k;
-    const int blocks = (S + 7) / 8;
-    if (s.dtype == METEORA_BF16)
-        k_shrink_tokens<__nv_bfloat16><<<blocks, 256, 0, st>>>((const __nv_bfloat16*)x, (const __nv_bfloat16*)A,
-                                                                topk_idx, topk_w, S, s.d_in, s.N, s.r, s.k, uw);
-    else
-        k_shrink_tokens<float><<<blocks, 256, 0, st>>>((const float*)x, (const float*)A, topk_idx, topk_w, S, s.d_in,
-                                                        s.N, s.r, s.k, uw);
     return last_launch_status();
 }
 
