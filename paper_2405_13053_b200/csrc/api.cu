@@ -136,10 +136,14 @@ static int forward_device(const void* x, const void* W0, const void* A, const vo
     }
     if (tc_path_supported(s)) {
         const bool pdl = tuning().pdl != 0;
-        if ((rc = launch_stacked_shrink_tc(x, A, Wg, s, ws, st)) != METEORA_OK) return rc;
-        if ((rc = launch_select_from_stacked(ws.u_all, ws.ld_u, ws.col_logits, tc_stacked_zsplits(s), s, ws.topk_idx,
-                                             ws.topk_w, ws.uw, pdl, st)) != METEORA_OK)
-            return rc;
+        if (token_forward_supported(s)) {
+            if ((rc = launch_token_forward(x, A, Wg, s, ws, st)) != METEORA_OK) return rc;
+        } else {
+            if ((rc = launch_stacked_shrink_tc(x, A, Wg, s, ws, st)) != METEORA_OK) return rc;
+            if ((rc = launch_select_from_stacked(ws.u_all, ws.ld_u, ws.col_logits, tc_stacked_zsplits(s), s, ws.topk_idx,
+                                                 ws.topk_w, ws.uw, pdl, st)) != METEORA_OK)
+                return rc;
+        }
         if (timed) cudaEventRecord(pf.ev[2 * pf.used], st);
         rc = launch_base_lora_tc(x, W0, B, s, ws, y, pdl && !timed, st);
         if (timed) cudaEventRecord(pf.ev[2 * pf.used++ + 1], st);
@@ -199,6 +203,7 @@ int meteora_gate_topk(const void* x, const void* Wg, const meteora_shape_t* shap
     if (shape->T == 0) return METEORA_OK;
     if (!x || !Wg || !topk_idx || !topk_w) return METEORA_ERR_INVALID_ARG;
     if (!aligned16(x) || !aligned16(Wg)) return METEORA_ERR_MISALIGNED;
+    if (token_gate_supported(*shape)) return launch_token_gate(x, Wg, *shape, topk_idx, topk_w, logits, (cudaStream_t)stream);
     return launch_gate_topk(x, Wg, *shape, topk_idx, topk_w, logits, (cudaStream_t)stream);
 }
 
@@ -225,7 +230,7 @@ int meteora_lora_delta(const void* x, const void* A, const void* B, const int32_
     const Workspace ws = carve_workspace(*shape, workspace);
     if (workspace_bytes < ws.bytes) return METEORA_ERR_WORKSPACE_TOO_SMALL;
     cudaStream_t st = (cudaStream_t)stream;
-    if ((rc = launch_shrink_segments(x, A, offsets, perm, *shape, ws.uw, st)) != METEORA_OK) return rc;
+    if ((rc = launch_shrink(x, A, topk_idx, offsets, perm, *shape, ws.uw, st)) != METEORA_OK) return rc;
     return launch_expand(B, topk_idx, topk_w, ws.uw, *shape, delta, st);
 }
 
@@ -308,7 +313,8 @@ size_t meteora_gate_backward_workspace_bytes(const meteora_shape_t* shape) {
     const size_t S = (size_t)shape->T * shape->k, r = (size_t)shape->r;
     return kHeaderBytes + 2 * align_up(S * 4, 256) + 2 * align_up(gate_backward_shrink_floats(*shape) * 4, 256) +
            2 * align_up(((size_t)shape->N + 1) * 4, 256) +
-           align_up((size_t)shape->N * shape->d_out * r * elem_size(shape->dtype), 256);
+           align_up((size_t)shape->N * shape->d_out * r * elem_size(shape->dtype), 256) +
+           align_up(gate_backward_part_floats(*shape) * 4, 256);
 }
 
 // B != nullptr: transposed into the workspace first; else Bt_ready holds the transposed adapters.
@@ -338,11 +344,10 @@ static int gate_backward_impl(const void* x, const void* A, const void* B, const
     int32_t* counts = (int32_t*)take(((size_t)shape->N + 1) * 4);
     int32_t* offsets = (int32_t*)take(((size_t)shape->N + 1) * 4);
     void* Bt = take((size_t)shape->N * shape->d_out * r * elem_size(shape->dtype));
+    float* part = (float*)take(gate_backward_part_floats(*shape) * 4);
     cudaStream_t st = (cudaStream_t)stream;
-    // the header's first words take the error flags of the tensor-core kernels
-    if (cudaMemsetAsync(workspace, 0, 256, st) != cudaSuccess) return METEORA_ERR_CUDA;
     return launch_gate_backward(x, A, B, dy, topk_idx, topk_w, *shape, B ? Bt : const_cast<void*>(Bt_ready), u, z, dl,
-                                S > 0 ? dlogit : nullptr, counts, offsets, perm, (int32_t*)workspace, dWg, st);
+                                S > 0 ? dlogit : nullptr, counts, offsets, perm, (int32_t*)workspace, part, dWg, st);
 }
 
 int meteora_gate_backward(const void* x, const void* A, const void* B, const void* dy, const int32_t* topk_idx,

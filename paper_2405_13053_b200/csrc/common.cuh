@@ -62,13 +62,16 @@ int launch_select_from_stacked(const float* u_all, int ld_u, int col_logits, int
 int launch_gate_backward(const void* x, const void* A, const void* B, const void* dy, const int32_t* topk_idx,
                          const float* topk_w, const meteora_shape_t& s, void* Bt, float* u, float* z, float* dlogit,
                          float* dlogit_out, int32_t* counts, int32_t* offsets, int32_t* perm, int32_t* status,
-                         float* dWg, cudaStream_t st);
+                         float* part, float* dWg, cudaStream_t st);
 int launch_transpose_b(const void* B, const meteora_shape_t& s, void* Bt, cudaStream_t st);
 bool gate_backward_dense(const meteora_shape_t& s);            // both shrinks as dense products on the tensor cores
+size_t gate_backward_part_floats(const meteora_shape_t& s);    // scratch of the split reduction over tokens
 size_t gate_backward_shrink_floats(const meteora_shape_t& s);  // floats of each of the two shrink outputs
 int launch_route(const int32_t* topk_idx, int T, int k, int N, int32_t* counts, int32_t* offsets, int32_t* perm,
                  cudaStream_t st);
 // lora.cu
+int launch_shrink(const void* x, const void* A, const int32_t* topk_idx, const int32_t* offsets, const int32_t* perm,
+                  const meteora_shape_t& s, float* u, cudaStream_t st);
 int launch_shrink_segments(const void* x, const void* A, const int32_t* offsets, const int32_t* perm,
                            const meteora_shape_t& s, float* u, cudaStream_t st);
 int launch_expand(const void* B, const int32_t* topk_idx, const float* topk_w, const float* u,
@@ -90,6 +93,21 @@ int launch_stacked_shrink_tc(const void* x, const void* A, const void* Wg, const
                              const Workspace& ws, cudaStream_t st);
 int launch_base_lora_tc(const void* x, const void* W0, const void* B, const meteora_shape_t& s, const Workspace& ws,
                         void* y, bool pdl, cudaStream_t st);
+
+// token tiles (wgemm_tcgen05.cu + token_tile.cuh): gate, selection, shrink of the picks, gate gradient
+bool token_gate_supported(const meteora_shape_t& s);
+int launch_token_gate(const void* x, const void* Wg, const meteora_shape_t& s, int32_t* topk_idx, float* topk_w, float* logits,
+                      cudaStream_t st);
+bool token_forward_supported(const meteora_shape_t& s);
+int launch_token_forward(const void* x, const void* A, const void* Wg, const meteora_shape_t& s, const Workspace& ws, cudaStream_t st);
+bool token_shrink_supported(const meteora_shape_t& s);
+int launch_token_shrink(const void* x, const void* A, const int32_t* topk_idx, const meteora_shape_t& s, float* u, int32_t* status,
+                        bool beside, cudaStream_t st);
+// dWg as a tensor-core product (wgemm_tcgen05.cu + gate_dwg.cuh)
+bool gate_dwg_tc_supported(const meteora_shape_t& s);
+int gate_dwg_shares(const meteora_shape_t& s);
+int launch_gate_dwg_tc(const void* x, const int32_t* topk_idx, const float* topk_w, const float* u, const float* z, const meteora_shape_t& s,
+                       int32_t* status, float* part, float* dlogit, float* dWg, cudaStream_t st);
 
 // fused decode kernel (wgemm_tcgen05.cu + decode_fused.cuh)
 bool decode_fused_supported(const meteora_shape_t& s);
@@ -176,6 +194,23 @@ __device__ __forceinline__ void load8(const float* p, float (&v)[8]) {
     const float4 b = *reinterpret_cast<const float4*>(p + 4);
     v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
     v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+}
+
+// Two fp32 FMAs as one instruction (each rounded like fmaf).
+__device__ __forceinline__ void fma2(unsigned long long& acc, unsigned long long a, unsigned long long b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ unsigned long long twice(float v) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
+    return r;
+}
+
+// Two packed bf16 as two fp32, the lower half first.
+__device__ __forceinline__ unsigned long long bf16x2_to_f32x2(uint32_t v) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(v << 16), "r"(v & 0xFFFF0000u));
+    return r;
 }
 
 __device__ __forceinline__ float warp_sum(float v) {

@@ -221,15 +221,38 @@ constexpr size_t kScanSlots = 2048;
 int launch_gate_backward(const void* x, const void* A, const void* B, const void* dy, const int32_t* topk_idx,
                          const float* topk_w, const meteora_shape_t& s, void* Bt, float* u, float* z, float* dlogit,
                          float* dlogit_out, int32_t* counts, int32_t* offsets, int32_t* perm, int32_t* status,
-                         float* dWg, cudaStream_t st) {
+                         float* part, float* dWg, cudaStream_t st) {
     int rc;
+    if (s.T == 0 && cudaMemsetAsync(status, 0, 256, st) != cudaSuccess) return METEORA_ERR_CUDA;
     if (s.T == 0) return cuda_status(cudaMemsetAsync(dWg, 0, (size_t)s.N * s.d_in * sizeof(float), st));
+    const float inv_tau = 1.0f / s.temperature;
+    meteora_shape_t sb = s;
+    sb.d_in = s.d_out;                                           // the contraction of B_e^T dy runs over d_out
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((s.T + 7) / 8);
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = tuning().pdl ? 1 : 0;
+    const float* uc = u;
+    const float* zc = z;
+    if (token_shrink_supported(s) && token_shrink_supported(sb) && gate_dwg_tc_supported(s)) {
+        // u and z per slot from token tiles, side by side (the second launch does not read the first one's results), then
+        // the Jacobian with dWg as a tensor-core product: 3 - 4 launches, each resident under the one ahead
+        if (B && (rc = launch_transpose_b(B, s, Bt, st)) != METEORA_OK) return rc;
+        if ((rc = launch_token_shrink(x, A, topk_idx, s, u, status, false, st)) != METEORA_OK) return rc;
+        if ((rc = launch_token_shrink(dy, Bt, topk_idx, sb, z, status, true, st)) != METEORA_OK) return rc;
+        return launch_gate_dwg_tc(x, topk_idx, topk_w, u, z, s, status, part, dlogit_out, dWg, st);
+    }
+    // the header's first words take the error flags of the tensor-core kernels
+    if (cudaMemsetAsync(status, 0, 256, st) != cudaSuccess) return METEORA_ERR_CUDA;
     const bool dense = gate_backward_dense(s);
     const bool scan = dense && (size_t)s.T * s.k <= kScanSlots;   // the grouped shrink kernel needs the buckets
     if (!scan && (rc = launch_route(topk_idx, s.T, s.k, s.N, counts, offsets, perm, st)) != METEORA_OK) return rc;
     if (B && (rc = launch_transpose_b(B, s, Bt, st)) != METEORA_OK) return rc;
-    meteora_shape_t sb = s;
-    sb.d_in = s.d_out;                                           // the contraction of B_e^T dy runs over d_out
     int ld = 0, zs_u = 1, zs_z = 1;
     if (dense && stacked_dual_supported(s)) {
         // u = [A_0; ..; A_{N-1}] x and z = [B_0^T; ..; B_{N-1}^T] dy as one launch: z's columns follow u's
@@ -259,20 +282,10 @@ int launch_gate_backward(const void* x, const void* A, const void* B, const void
     }
     // The last two kernels are launched programmatically dependent: resident while their predecessor still runs,
     // they wait for it (griddepcontrol.wait) before their first read.
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.blockDim = dim3(256);
-    cfg.stream = st;
-    cfg.attrs = attr;
-    cfg.numAttrs = tuning().pdl ? 1 : 0;
-    cfg.gridDim = dim3((s.T + 7) / 8);
-    const float inv_tau = 1.0f / s.temperature;
     const int dense_i = dense ? 1 : 0;
     const size_t zstride = (size_t)s.T * ld;
-    const float* uc = u;
-    const float* zc = z;
+    uc = u;
+    zc = z;
     if ((rc = cuda_status(cudaLaunchKernelEx(&cfg, k_gate_dlogit, uc, zc, topk_idx, topk_w, s.T, s.N, s.k, s.r, inv_tau,
                                              dense_i, ld, zs_u, zs_z, zstride, dlogit, dlogit_out))) != METEORA_OK)
         return rc;
@@ -302,6 +315,12 @@ size_t gate_backward_shrink_floats(const meteora_shape_t& s) {
     const size_t slots = (size_t)s.T * s.k * s.r;
     if (!gate_backward_dense(s)) return slots;
     return std::max(slots, (size_t)s.T * tc_stacked_pitch(s, nullptr) * stacked_zsplits_bound(s.T));
+}
+
+size_t gate_backward_part_floats(const meteora_shape_t& s) {
+    if (s.T == 0 || !gate_dwg_tc_supported(s)) return 0;
+    const int shares = gate_dwg_shares(s);
+    return shares > 1 ? (size_t)shares * s.N * s.d_in : 0;
 }
 
 }  // namespace meteora

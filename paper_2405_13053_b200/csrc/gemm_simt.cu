@@ -48,16 +48,6 @@ __device__ __forceinline__ float4 load_quad(const __nv_bfloat16* row, int d, int
     return v;
 }
 
-// Two fp32 FMAs as one instruction (each rounded like fmaf).
-__device__ __forceinline__ void fma2(unsigned long long& acc, unsigned long long a, unsigned long long b) {
-    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
-}
-__device__ __forceinline__ unsigned long long twice(float v) {
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
-    return r;
-}
-
 struct SimtParams {
     int T, d_in, d_out, a_rows, N, ldp;   // stacked rows: d_out of W0, a_rows = N * r of A, N of Wg; ldp = row pitch of a copy
     size_t zstride;                       // floats between the copies

@@ -20,6 +20,7 @@
 
 #include <stdio.h>
 
+#include <atomic>
 #include <mutex>
 #include <vector>
 
@@ -708,6 +709,8 @@ k_wgemm(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__ CUtens
 #include "wgemm_pair.cuh"
 #include "decode_stream.cuh"
 #include "decode_cluster.cuh"
+#include "token_tile.cuh"
+#include "gate_dwg.cuh"
 
 namespace meteora {
 
@@ -2155,6 +2158,265 @@ int launch_decode_cluster(const void* x, const void* W0, const void* A, const vo
     return cuda_status(err);
 }
 
+// ------------------------------------------------------------------------------------------------
+// Token tiles (token_tile.cuh): gate, selection, shrink of the picks, gate gradient
+// ------------------------------------------------------------------------------------------------
+struct TokenPlan {
+    bool ok;
+    int S, stages, stage_bytes, tmem_cols, pitch, rounds, cols[2], gate_box, a_box, a_copies;
+    int groups, a_group;   // clusters per tile, each with its own adapters (SHRINK), and adapters per cluster
+    size_t smem;
+    long long cost;
+};
+constexpr size_t kTokenSmem = 226 * 1024;
+
+typedef void (*TokenKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const TokenTileParams);
+static TokenKernel token_kernel(int S) {
+    switch (S) {
+        case 1: return k_token_tile<1>;
+        case 2: return k_token_tile<2>;
+        case 3: return k_token_tile<3>;
+        case 4: return k_token_tile<4>;
+        case 5: return k_token_tile<5>;
+        case 6: return k_token_tile<6>;
+        case 7: return k_token_tile<7>;
+        case 8: return k_token_tile<8>;
+        default: return k_token_tile<16>;
+    }
+}
+
+// How many clusters of S token-tile CTAs the device holds at once (0: the device cannot say, or none).
+static int token_cluster_capacity(int S) {
+    static std::atomic<int> cache[64][kTokMaxSplit + 1];         // 0: not asked yet, else capacity + 1
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    int have = cache[dev][S].load(std::memory_order_relaxed);
+    if (have == 0) {
+        int n = 0;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(S * 148);
+        cfg.blockDim = dim3(kThreads);
+        cfg.dynamicSmemBytes = kTokenSmem;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = S;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        const TokenKernel f = token_kernel(S);
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
+            (S > 8 && cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
+            cudaOccupancyMaxActiveClusters(&n, f, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;                                            // (asked again next time: no device, or not ready yet)
+        }
+        have = n + 1;
+        cache[dev][S].store(have, std::memory_order_relaxed);
+    }
+    return have - 1;
+}
+
+static TokenPlan make_token_plan_with(const meteora_shape_t& s, int mode, int groups) {
+    TokenPlan tp = {};
+    tp.groups = groups;
+    tp.a_group = (s.N + groups - 1) / groups;
+    const int a_rows = mode == TOKEN_GATE ? 0 : tp.a_group * s.r;
+    if (a_rows > 0 && s.r % 8 != 0) return tp;
+    tp.gate_box = mode <= TOKEN_FORWARD ? (s.N + 7) / 8 * 8 : 0;
+    tp.a_copies = a_rows == 0 ? 0 : a_rows <= 256 ? 1 : 2;       // (a copy's box has 256 rows at the most)
+    if (tp.a_copies > 0) tp.a_box = (a_rows / tp.a_copies + 7) / 8 * 8;
+    const int total = (tp.gate_box + tp.a_copies * tp.a_box + 15) / 16 * 16;
+    // Two rounds of columns (80 KB per k-step, two stages) are slower than the stacked kernels and their selection: 27 against
+    // 20 us at 5120, rank 16, 1531 tokens.  For the shrink alone the alternative is the gather on CUDA cores.
+    if (tp.a_box > 256 || total > (mode == TOKEN_SHRINK ? 2 : 1) * kTokCols) return tp;
+    tp.cols[0] = std::min(total, kTokCols);
+    tp.cols[1] = total - tp.cols[0];
+    tp.rounds = tp.cols[1] > 0 ? 2 : 1;
+    tp.pitch = tp.cols[0] + 4;
+    const int cols = tp.rounds == 2 ? kTokCols + tp.cols[1] : tp.cols[0];
+    tp.tmem_cols = 32;
+    while (tp.tmem_cols < cols) tp.tmem_cols *= 2;
+    tp.stage_bytes = kTokXBytes + total * 128;
+    const int ks = (s.d_in + kBK - 1) / kBK;
+    // CTAs per tile: the split with the least intake per SM, counting a wave's set-up and exchanges as 240 KB (2.5 us)
+    const int tiles = (s.T + kTokTile - 1) / kTokTile;
+    for (int S = 1; S <= kTokMaxSplit && S <= ks; S += S == 8 ? 8 : 1) {
+        const int cap = token_cluster_capacity(S);
+        if (cap <= 0 || (groups > 1 && 2 * tiles * groups > cap)) continue;
+        const long long cost = (long long)((tiles * groups + cap - 1) / cap) * ((long long)((ks + S - 1) / S) * tp.stage_bytes + 240 * 1024);
+        if (tp.cost == 0 || cost < tp.cost) {
+            tp.cost = cost;
+            tp.S = S;
+        }
+    }
+    if (tp.cost == 0) return tp;
+    const int iters = (ks + tp.S - 1) / tp.S;
+    tp.stages = (int)std::min<size_t>((kTokenSmem - 2048) / tp.stage_bytes, (size_t)std::min(16, std::max(iters, 2)));
+    // the accumulators' copy and, behind it, the owned tokens' summed logits
+    const size_t own = (size_t)((kTokTile + tp.S - 1) / tp.S) * 4 * (s.N | 1);
+    tp.smem = 2048 + std::max((size_t)tp.stages * tp.stage_bytes, (size_t)kTokTile * tp.pitch * 4 + own);
+    tp.ok = tp.stages >= 2 && tp.smem <= kTokenSmem;
+    return tp;
+}
+
+// Few tiles leave SMs idle, and an SM takes in 100 GB/s at the most: the shrink's adapters are then dealt to two or four
+// clusters per tile (16 KB of tokens + 28 KB of rows per k-step with one, 16 + 7 KB with four), as long as two such
+// launches fit side by side.
+static TokenPlan make_token_plan(const meteora_shape_t& s, int mode) {
+    TokenPlan best = {};
+    if (s.dtype != METEORA_BF16 || s.d_in % 8 != 0 || s.T <= 0 || tuning().force_simt) return best;
+    for (int groups = 1; groups <= (mode == TOKEN_SHRINK ? 4 : 1); groups *= 2) {
+        const TokenPlan tp = make_token_plan_with(s, mode, groups);
+        if (tp.ok && (!best.ok || tp.cost < best.cost)) best = tp;
+    }
+    return best;
+}
+
+// Clusters of S CTAs of kThreads, launched programmatically dependent.
+static void cluster_launch(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&attr)[2], int ctas, int S, size_t smem, cudaStream_t st) {
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = S;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = tuning().pdl ? 2 : 1;
+}
+
+static int launch_token_tile(const TokenPlan& tp, int mode, const meteora_shape_t& s, const void* x, const void* Wg, const void* A,
+                             TokenTileParams p, cudaStream_t st) {
+    CUtensorMap mX, mG, mA;
+    int rc;
+    if ((rc = get_tensor_map(x, s.d_in, s.T, kTokTile, 0, &mX)) != METEORA_OK) return rc;
+    mG = mA = mX;                                                // maps that the mode does not read
+    if (tp.gate_box > 0 && (rc = get_tensor_map(Wg, s.d_in, s.N, tp.gate_box, 0, &mG)) != METEORA_OK) return rc;
+    if (tp.a_copies > 0 && (rc = get_tensor_map(A, s.d_in, s.N * s.r, tp.a_box, 0, &mA)) != METEORA_OK) return rc;
+    p.T = s.T;
+    p.mode = mode;
+    p.N = s.N;
+    p.r = s.r;
+    p.k = s.k;
+    p.ksteps = (s.d_in + kBK - 1) / kBK;
+    p.gate_box = tp.gate_box;
+    p.a_box = tp.a_box;
+    p.a_copies = tp.a_copies;
+    p.a_group = tp.a_group;
+    p.stages = tp.stages;
+    p.stage_bytes = tp.stage_bytes;
+    p.tmem_cols = tp.tmem_cols;
+    p.pitch = tp.pitch;
+    p.rounds = tp.rounds;
+    p.cols[0] = tp.cols[0];
+    p.cols[1] = tp.cols[1];
+    p.inv_tau = 1.0f / s.temperature;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
+    cluster_launch(cfg, attr, (s.T + kTokTile - 1) / kTokTile * tp.S, tp.S, tp.smem, st);
+    cfg.gridDim.y = tp.groups;
+    return cuda_status(cudaLaunchKernelEx(&cfg, token_kernel(tp.S), mX, mG, mA, p));
+}
+
+bool token_gate_supported(const meteora_shape_t& s) { return make_token_plan(s, TOKEN_GATE).ok; }
+
+int launch_token_gate(const void* x, const void* Wg, const meteora_shape_t& s, int32_t* topk_idx, float* topk_w, float* logits,
+                      cudaStream_t st) {
+    TokenTileParams p = {};
+    p.topk_idx = topk_idx;
+    p.topk_w = topk_w;
+    p.logits = logits;
+    return launch_token_tile(make_token_plan(s, TOKEN_GATE), TOKEN_GATE, s, x, Wg, nullptr, p, st);
+}
+
+bool token_forward_supported(const meteora_shape_t& s) { return make_token_plan(s, TOKEN_FORWARD).ok; }
+
+int launch_token_forward(const void* x, const void* A, const void* Wg, const meteora_shape_t& s, const Workspace& ws, cudaStream_t st) {
+    TokenTileParams p = {};
+    p.topk_idx = ws.topk_idx;
+    p.topk_w = ws.topk_w;
+    p.u = ws.uw;
+    p.status = ws.status;
+    return launch_token_tile(make_token_plan(s, TOKEN_FORWARD), TOKEN_FORWARD, s, x, Wg, A, p, st);
+}
+
+bool token_shrink_supported(const meteora_shape_t& s) { return make_token_plan(s, TOKEN_SHRINK).ok; }
+
+// status (optional) is cleared first; `beside`: launched right behind another shrink whose results it does not read.
+int launch_token_shrink(const void* x, const void* A, const int32_t* topk_idx, const meteora_shape_t& s, float* u, int32_t* status,
+                        bool beside, cudaStream_t st) {
+    TokenTileParams p = {};
+    p.topk_idx = const_cast<int32_t*>(topk_idx);
+    p.u = u;
+    p.status = status;
+    p.clear_status = status && !beside ? 1 : 0;
+    p.late_wait = beside && tuning().pdl ? 1 : 0;
+    return launch_token_tile(make_token_plan(s, TOKEN_SHRINK), TOKEN_SHRINK, s, x, nullptr, A, p, st);
+}
+
+// dWg on the tensor cores (gate_dwg.cuh): dlogit in three bf16 parts, so up to 42 adapters.
+bool gate_dwg_tc_supported(const meteora_shape_t& s) {
+    return s.dtype == METEORA_BF16 && s.d_in % 8 == 0 && s.N <= kDwgMaxN && s.T > 0 && !tuning().force_simt;
+}
+
+// Shares of the tokens: until the column tiles fill the SMs, one block of 64 tokens each at the least.
+int gate_dwg_shares(const meteora_shape_t& s) {
+    const int tiles = (s.d_in + kDwgCols - 1) / kDwgCols, blocks = (s.T + kDwgTok - 1) / kDwgTok;
+    return std::max(1, std::min(std::min(kDwgMaxShares, blocks), 148 / tiles));
+}
+
+// part: gate_dwg_shares(s) * N * d_in floats of scratch (not used where there is one share).
+int launch_gate_dwg_tc(const void* x, const int32_t* topk_idx, const float* topk_w, const float* u, const float* z, const meteora_shape_t& s,
+                       int32_t* status, float* part, float* dlogit, float* dWg, cudaStream_t st) {
+    CUtensorMap mX;
+    int rc;
+    if ((rc = get_tensor_map(x, s.d_in, s.T, kDwgTok, 0, &mX)) != METEORA_OK) return rc;
+    constexpr size_t smem = 1024 + (size_t)kDwgStages * (kDwgXBytes + kDwgLBytes) + 256 + 2 * kDwgSlots * 4;
+    static std::atomic<bool> attr_set[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return METEORA_ERR_CUDA;
+    if (dev < 0 || dev >= 64) return METEORA_ERR_UNSUPPORTED_SHAPE;
+    if (!attr_set[dev].load(std::memory_order_relaxed)) {
+        if (cudaFuncSetAttribute(k_gate_dwg_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return METEORA_ERR_CUDA;
+        attr_set[dev].store(true, std::memory_order_relaxed);
+    }
+    const int shares = gate_dwg_shares(s);
+    GateDwgParams p = {};
+    p.T = s.T;
+    p.N = s.N;
+    p.k = s.k;
+    p.d_in = s.d_in;
+    p.topk_idx = topk_idx;
+    p.topk_w = topk_w;
+    p.u = u;
+    p.z = z;
+    p.r = s.r;
+    p.inv_tau = 1.0f / s.temperature;
+    p.dlogit = dlogit;
+    p.out = shares > 1 ? part : dWg;
+    p.status = status;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((s.d_in + kDwgCols - 1) / kDwgCols, shares);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = tuning().pdl ? 1 : 0;
+    if ((rc = cuda_status(cudaLaunchKernelEx(&cfg, k_gate_dwg_tc, mX, p))) != METEORA_OK || shares == 1) return rc;
+    const size_t n = (size_t)s.N * s.d_in;
+    cfg.gridDim = dim3((unsigned)((n + 255) / 256));
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = 0;
+    return cuda_status(cudaLaunchKernelEx(&cfg, k_gate_dwg_sum, (const float*)part, shares, n, dWg));
+}
+
 // Human-readable launch plan of meteora_linear_forward for this shape (for logs and benchmark records).
 int describe_plan(const meteora_shape_t& s, char* buf, size_t n) {
     if (!tc_path_supported(s)) return snprintf(buf, n, "path=simt");
@@ -2179,19 +2441,21 @@ int describe_plan(const meteora_shape_t& s, char* buf, size_t n) {
                         fp.n_main, fp.row_tiles, (double)fp.row_tiles * fp.upt / fp.n_main, fp.n_aux, fp.aux_slices,
                         fp.main.BN, fp.main.stages, fp.main.kc, fp.main.smem, max_resident_ctas(fp.main.smem));
     const int row_tiles = (s.d_out + kBM - 1) / kBM;
+    const TokenPlan tp = make_token_plan(s, TOKEN_FORWARD);   // routing in one launch of token tiles, else in two
+    const int routing = tp.ok ? 1 : 2;
     const PairPlan pp = make_pair_plan(s);
     if (pp.ok)
         return snprintf(buf, n,
-                        "path=chain(not fused: reason %d) launches=%d base=pairs_of_ctas pairs=%d tile=256x256 stages=%d "
+                        "path=chain(not fused: reason %d) launches=%d token_tile_cluster=%d base=pairs_of_ctas pairs=%d tile=256x256 stages=%d "
                         "smem=%zu expand=mma tail_pairs_as_small_tiles=%d",
-                        fp.why, pair_tail_carve(s) > 0 ? 4 : 3,
+                        fp.why, routing + (pair_tail_carve(s) > 0 ? 2 : 1), tp.S,
                         (row_tiles + 1) / 2 * ((s.T + kPairTokens - 1) / kPairTokens) - pair_tail_carve(s), pp.stages,
                         pp.smem, pair_tail_carve(s));
     const Plan pl = make_plan(row_tiles, s.T, s.d_in, true, s.N, s.r, s.k);
     return snprintf(buf, n,
-                    "path=chain(not fused: reason %d) launches=3 base_ctas=%d cluster=%d tile_tokens=%d stages=%d kc=%d "
+                    "path=chain(not fused: reason %d) launches=%d token_tile_cluster=%d base_ctas=%d cluster=%d tile_tokens=%d stages=%d kc=%d "
                     "smem=%zu expand=%s",
-                    fp.why, row_tiles * pl.splits * pl.n_tiles, pl.splits, pl.BN, pl.stages, pl.kc, pl.smem,
+                    fp.why, routing + 1, tp.S, row_tiles * pl.splits * pl.n_tiles, pl.splits, pl.BN, pl.stages, pl.kc, pl.smem,
                     pl.lora_mma ? "mma" : "simt");
 }
 
