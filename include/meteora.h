@@ -324,6 +324,8 @@ int meteora_describe_plan(const meteora_shape_t* shape, char* buf, size_t buf_by
  *                    tiles through distributed shared memory, the stacked shrink is spread over all CTAs):
  *                    default 0 = never (measured slower than the streamed kernel except for the largest layers),
  *                    other = wherever the device can hold all clusters at once
+ *   "persist"        prefill base product on persistent pairs of SMs: default 1 = planner's choice, 0 = never, 2 = wherever the
+ *                    shape allows ("pair" 2 and a set "tail_carve" take the kernel with one tile per pair)
  *   "group_pairs"    > 0 = row pairs per scheduling group of the prefill kernel on pairs of SMs (0 = planner's choice)
  *   "tail_carve"     prefill on pairs of SMs: 0 = the planner carves the tiles of a nearly empty last wave out of the
  *                    pair launch (they follow as a launch of small tiles), -1 = never, n > 0 = the last token tile of n row pairs

@@ -33,6 +33,8 @@ Workspace carve_workspace(const meteora_shape_t& s_in, void* base) {
     ws.topk_idx = (int32_t*)take(T * s.k * sizeof(int32_t));
     ws.topk_w = (float*)take(T * s.k * sizeof(float));
     ws.uw = (float*)take(T * s.k * s.r * sizeof(float));
+    ws.ld_us = persist_us_pitch(s);
+    ws.us = ws.ld_us > 0 ? take(T * ws.ld_us * 2) : nullptr;
     ws.u_all = (float*)take(T * ws.ld_u * sizeof(float) * (size_t)stacked_zsplits_bound(s.T));   // one copy per slice of the contraction axis
     // decode kernel scratch: one partial tile of 128 x BN fp32 per (main CTA, row tile it touches), in slot
     // row tile + main CTA: fewer than row tiles + 148 slots
@@ -136,12 +138,13 @@ static int forward_device(const void* x, const void* W0, const void* A, const vo
     }
     if (tc_path_supported(s)) {
         const bool pdl = tuning().pdl != 0;
+        void* us = persist_supported(s) ? ws.us : nullptr;
         if (token_forward_supported(s)) {
-            if ((rc = launch_token_forward(x, A, Wg, s, ws, st)) != METEORA_OK) return rc;
+            if ((rc = launch_token_forward(x, A, Wg, s, ws, us, st)) != METEORA_OK) return rc;
         } else {
             if ((rc = launch_stacked_shrink_tc(x, A, Wg, s, ws, st)) != METEORA_OK) return rc;
             if ((rc = launch_select_from_stacked(ws.u_all, ws.ld_u, ws.col_logits, tc_stacked_zsplits(s), s, ws.topk_idx,
-                                                 ws.topk_w, ws.uw, pdl, st)) != METEORA_OK)
+                                                 ws.topk_w, ws.uw, us, ws.ld_us, pdl, st)) != METEORA_OK)
                 return rc;
         }
         if (timed) cudaEventRecord(pf.ev[2 * pf.used], st);
@@ -526,6 +529,7 @@ int meteora_set_tuning(const char* name, int value) {
     else if (!strcmp(name, "cluster_decode")) t.cluster_decode = value;
     else if (!strcmp(name, "aux_plain")) t.aux_plain = value;
     else if (!strcmp(name, "tail_carve")) t.tail_carve = value;
+    else if (!strcmp(name, "persist")) t.persist = value;
     else if (!strcmp(name, "wait_limit_us")) return set_wait_limit_us(value);
     else if (!strcmp(name, "coop")) t.coop = value;
     else if (!strcmp(name, "no_hold")) t.no_hold = value;

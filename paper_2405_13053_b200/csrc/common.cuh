@@ -20,6 +20,8 @@ struct Workspace {
     int32_t* topk_idx;  // [T,k]
     float* topk_w;      // [T,k]
     float* uw;          // [T,k,r]   w_j * (A_{i_j} x): the shrunk, gate-weighted activations
+    void* us;           // [T,ld_us] bf16: masked, gate-weighted shrink, the token operand of the expand on persistent pairs
+    int ld_us;          //           (0: not laid out for this shape)
     float* u_all;       // [Z][T,ld_u]  stacked shrink: every adapter's A_i x, then the gate logits; Z partial
                         //           copies (slices of the contraction axis) that the selection kernel adds up
     int ld_u;           // row pitch of u_all in floats
@@ -57,7 +59,7 @@ inline size_t elem_size(meteora_dtype_t t) { return t == METEORA_BF16 ? 2 : 4; }
 int launch_gate_topk(const void* x, const void* Wg, const meteora_shape_t& s, int32_t* topk_idx, float* topk_w,
                      float* logits, cudaStream_t st);
 int launch_select_from_stacked(const float* u_all, int ld_u, int col_logits, int zsplits, const meteora_shape_t& s,
-                               int32_t* topk_idx, float* topk_w, float* uw, bool pdl, cudaStream_t st);
+                               int32_t* topk_idx, float* topk_w, float* uw, void* us, int ld_us, bool pdl, cudaStream_t st);
 // route.cu
 int launch_gate_backward(const void* x, const void* A, const void* B, const void* dy, const int32_t* topk_idx,
                          const float* topk_w, const meteora_shape_t& s, void* Bt, float* u, float* z, float* dlogit,
@@ -82,6 +84,8 @@ int launch_forward_simt(const void* x, const void* W0, const void* A, const void
                         const Workspace& ws, void* y, cudaStream_t st);
 // wgemm_tcgen05.cu
 bool tc_path_supported(const meteora_shape_t& s);
+int persist_us_pitch(const meteora_shape_t& s);                   // columns of Workspace::us, 0 where no path reads it
+bool persist_supported(const meteora_shape_t& s);                 // base product on persistent pairs, which reads us
 int tc_stacked_pitch(const meteora_shape_t& s, int* col_logits);  // row pitch (floats) of u_all
 int stacked_zsplits_bound(int T);                                  // upper bound of those copies, sizes the workspace
 bool stacked_dual_supported(const meteora_shape_t& s);            // both shrinks of the gate gradient in one launch?
@@ -99,7 +103,8 @@ bool token_gate_supported(const meteora_shape_t& s);
 int launch_token_gate(const void* x, const void* Wg, const meteora_shape_t& s, int32_t* topk_idx, float* topk_w, float* logits,
                       cudaStream_t st);
 bool token_forward_supported(const meteora_shape_t& s);
-int launch_token_forward(const void* x, const void* A, const void* Wg, const meteora_shape_t& s, const Workspace& ws, cudaStream_t st);
+int launch_token_forward(const void* x, const void* A, const void* Wg, const meteora_shape_t& s, const Workspace& ws, void* us,
+                         cudaStream_t st);
 bool token_shrink_supported(const meteora_shape_t& s);
 int launch_token_shrink(const void* x, const void* A, const int32_t* topk_idx, const meteora_shape_t& s, float* u, int32_t* status,
                         bool beside, cudaStream_t st);
@@ -164,6 +169,7 @@ struct Tuning {
     int no_hold = 0;         // decode kernel, head start of the aux CTAs: 0 planner's choice, 1 none, 64 counter wait, other = nanoseconds
     int hold_after = 0;      // decode kernel: ring stages of W0 the main CTAs request before the aux CTAs' head start (0: planner, -1: none)
     int narrow_select = 0;   // decode kernel's selection: 0 by batch size, 1 always two narrow round trips, -1 always one wide one
+    int persist = 1;         // prefill on persistent pairs of SMs: 0 never, 1 planner, 2 wherever the shape allows
     int tail_carve = 0;      // prefill on pairs of SMs: 0 = the planner carves a nearly empty last wave out, -1 = never, n = n row pairs
     int aux_plain = 1;       // streamed kernel: the aux CTAs' partial tiles leave as plain stores (0: staged, one bulk copy)
     int cluster_decode = 0;  // decode batches on clusters that exchange through distributed shared memory (0: never)

@@ -38,6 +38,8 @@ struct TokenTileParams {
     float* topk_w;             // (not read by SHRINK)
     float* logits;             // GATE: optional out
     float* u;                  // out: [slot][r], FORWARD weighted by w
+    __nv_bfloat16* us;         // FORWARD, optional out: the same values as [T][ld_us] with zeros elsewhere
+    int ld_us;
     int32_t* status;           // error flag of expired waits (may be null)
     int clear_status;          // CTA 0 zeroes the status words first
     int late_wait;             // nothing here depends on the kernel ahead: only leave after it
@@ -75,6 +77,10 @@ __device__ __forceinline__ void token_round(const TokenTileParams& p, uint32_t p
     const uint32_t pitch4 = (uint32_t)p.pitch * 4u;
     if (p.mode <= TOKEN_FORWARD && round == 0) {
         const int ld = p.N | 1;
+        if (p.us) {
+            uint4* rows = reinterpret_cast<uint4*>(p.us + (size_t)t0 * p.ld_us);
+            for (int i = etid; i < own * (p.ld_us / 8); i += kEpiThreads) rows[i] = make_uint4(0u, 0u, 0u, 0u);
+        }
 #pragma unroll 2
         for (int i = etid; i < own * p.N; i += kEpiThreads) {
             const int tt = i / p.N, c = i - tt * p.N;
@@ -110,7 +116,9 @@ __device__ __forceinline__ void token_round(const TokenTileParams& p, uint32_t p
         const int e = min(max(p.topk_idx[g], 0), p.N - 1) - e0, col = p.gate_box + e * p.r + q;
         if (e >= 0 && e < p.a_group && col >= c_lo && col < c_hi) {
             const float v = cluster_sum<S>(base, (uint32_t)(own0 + slot / p.k) * pitch4 + 4u * (col - c_lo));
-            p.u[(size_t)t0 * n + i] = p.mode == TOKEN_FORWARD ? p.topk_w[g] * v : v;
+            const float out = p.mode == TOKEN_FORWARD ? p.topk_w[g] * v : v;
+            p.u[(size_t)t0 * n + i] = out;
+            if (p.us) p.us[(size_t)(t0 + slot / p.k) * p.ld_us + (e0 + e) * p.r + q] = __float2bfloat16_rn(out);
         }
     }
 }

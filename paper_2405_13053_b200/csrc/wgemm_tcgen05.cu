@@ -710,6 +710,7 @@ k_wgemm(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__ CUtens
 #include "decode_stream.cuh"
 #include "decode_cluster.cuh"
 #include "token_tile.cuh"
+#include "wgemm_persist.cuh"
 #include "gate_dwg.cuh"
 
 namespace meteora {
@@ -777,6 +778,30 @@ static int get_store_map(const void* y, int d_out, int T, int box_tokens, CUtens
                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? METEORA_OK : METEORA_ERR_CUDA;
+}
+
+// Tensor map of the adapters' B[N, d_out, r] (bf16) whose box holds, for 128 output rows, 8 blocks of 8 rank entries as
+// un-swizzled K-major core matrices: [block][row][16 bytes].  Rank 8: a block's rows are contiguous, so 8 rows (128 bytes) are
+// the inner axis; larger ranks: (8 entries, rows, r / 8, N), 16 bytes at a time.  Needs d_out % 8 == 0, r / 8 in {1, 2, 4, 8}.
+static int get_adapter_map(const void* B, int N, int d_out, int r, CUtensorMap* out) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return METEORA_ERR_CUDA;
+    CUresult rc;
+    const cuuint32_t estride[4] = {1, 1, 1, 1};
+    if (r == 8) {
+        const cuuint64_t gdim[3] = {64, (cuuint64_t)d_out / 8, (cuuint64_t)N};
+        const cuuint64_t gstride[2] = {128, (cuuint64_t)d_out * 16};
+        const cuuint32_t box[3] = {64, 16, 8};
+        rc = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(B), gdim, gstride, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    } else {
+        const cuuint64_t gdim[4] = {8, (cuuint64_t)d_out, (cuuint64_t)r / 8, (cuuint64_t)N};
+        const cuuint64_t gstride[3] = {(cuuint64_t)r * 2, 16, (cuuint64_t)d_out * r * 2};
+        const cuuint32_t box[4] = {8, (cuuint32_t)kBM, (cuuint32_t)r / 8, 64 / (cuuint32_t)r};
+        rc = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(B), gdim, gstride, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    }
+    return rc == CUDA_SUCCESS ? METEORA_OK : METEORA_ERR_CUDA;
 }
 
 static int sm_count() {
@@ -1354,8 +1379,113 @@ static int pair_tail_carve(const meteora_shape_t& s) {
     return carve;
 }
 
+// ------------------------------------------------------------------------------------------------
+// Persistent pairs (wgemm_persist.cuh)
+// ------------------------------------------------------------------------------------------------
+struct PersistPlan {
+    bool ok;
+    int BN, CT, stages, stage_bytes, pairs, tok_tiles, tiles;
+    size_t smem;
+};
+
+// Columns of the masked token operand: the expand takes N r columns in k-steps of 64.  Other ranks than 8, 16, 32, 64 (a k-step
+// is whole adapters or a whole part of one) and more than 2048 columns stay with the kernel that stages them in rounds.
+int persist_us_pitch(const meteora_shape_t& s) {
+    const int cols = (s.N * s.r + kBK - 1) / kBK * kBK, cpa = s.r / 8;
+    if (s.dtype != METEORA_BF16 || s.T <= 256 || s.d_in % 8 != 0 || s.d_out % 8 != 0 || s.r % 8 != 0 || cols > 2048) return 0;
+    return cpa == 1 || cpa == 2 || cpa == 4 || cpa == 8 ? cols : 0;
+}
+
+// Pairs the device holds at once (0: it cannot say).
+static int persist_pairs() {
+    static std::atomic<int> cache[64];                           // 0: not asked yet, else pairs + 1
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    int have = cache[dev].load(std::memory_order_relaxed);
+    if (have == 0) {
+        int n = 0;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(2 * kPersistMaxPairs);
+        cfg.blockDim = dim3(kThreads);
+        cfg.dynamicSmemBytes = 227 * 1024;
+        if (cudaFuncSetAttribute(k_wgemm_persist, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&n, k_wgemm_persist, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
+        have = std::min(n, kPersistMaxPairs) + 1;
+        cache[dev].store(have, std::memory_order_relaxed);
+    }
+    return have - 1;
+}
+
+static PersistPlan make_persist_plan(const meteora_shape_t& s) {
+    PersistPlan pp = {};
+    const Tuning& tn = tuning();
+    if (!tn.persist || tn.pair != 1 || tn.tail_carve != 0 || tn.simt_expand || tn.no_tma_store || tn.tile_tokens || tn.splits > 1) return pp;
+    if (persist_us_pitch(s) == 0 || !tc_path_supported(s)) return pp;
+    const int pairs = persist_pairs();
+    if (pairs < 1) return pp;
+    // tokens per tile: 256-token tiles, narrower ones (whole 32s) where that spreads a ragged token count over as many tiles
+    pp.tok_tiles = (s.T + kPairTokens - 1) / kPairTokens;
+    pp.BN = ((s.T + pp.tok_tiles - 1) / pp.tok_tiles + 31) / 32 * 32;
+    pp.CT = pp.BN % 64 == 0 ? 64 : 32;
+    pp.tiles = ((s.d_out + kBM - 1) / kBM + 1) / 2 * pp.tok_tiles;
+    if (tn.persist == 1 && pp.tiles * 4 < sm_count()) return pp;
+    pp.pairs = std::min(pairs, pp.tiles);
+    pp.stage_bytes = kWTileBytes + pp.BN / 2 * 128;
+    const size_t fixed = 1024 + (size_t)kPersistStageBufs * kPersistStoreBytes + 512;
+    pp.stages = (int)std::min<size_t>((227 * 1024 - fixed) / pp.stage_bytes, 12);
+    pp.smem = fixed + (size_t)pp.stages * pp.stage_bytes;
+    pp.ok = pp.stages >= 2;
+    return pp;
+}
+
+bool persist_supported(const meteora_shape_t& s) { return make_persist_plan(s).ok; }
+
+static int launch_base_persist(const void* x, const void* W0, const void* B, const meteora_shape_t& s, const Workspace& ws, void* y,
+                               const PersistPlan& pp, bool pdl, cudaStream_t st) {
+    CUtensorMap mW, mX, mB, mU, mY;
+    int rc;
+    if ((rc = get_tensor_map(W0, s.d_in, s.d_out, kBM, 0, &mW)) != METEORA_OK) return rc;
+    if ((rc = get_tensor_map(x, s.d_in, s.T, pp.BN / 2, 0, &mX)) != METEORA_OK) return rc;
+    if ((rc = get_tensor_map(ws.us, ws.ld_us, s.T, pp.BN / 2, 0, &mU)) != METEORA_OK) return rc;
+    if ((rc = get_store_map(y, s.d_out, s.T, pp.CT, &mY)) != METEORA_OK) return rc;
+    if ((rc = get_adapter_map(B, s.N, s.d_out, s.r, &mB)) != METEORA_OK) return rc;
+    PersistParams p = {};
+    p.T = s.T;
+    p.BN = pp.BN;
+    p.CT = pp.CT;
+    p.ksteps = (s.d_in + kBK - 1) / kBK;
+    p.iters = p.ksteps + ws.ld_us / kBK;
+    p.cpa = s.r / 8;
+    p.nblk = s.N * p.cpa;
+    p.stages = pp.stages;
+    p.stage_bytes = pp.stage_bytes;
+    p.row_tiles = (s.d_out + kBM - 1) / kBM;
+    p.row_pairs = (p.row_tiles + 1) / 2;
+    p.tok_tiles = pp.tok_tiles;
+    p.group_pairs = std::min(tuning().group_pairs > 0 ? tuning().group_pairs : std::max(1, (pp.pairs / pp.tok_tiles + 1) / 2), p.row_pairs);
+    p.tiles = pp.tiles;
+    p.status = ws.status;
+    p.pdl_wait = pdl ? 1 : 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * pp.pairs);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = pp.smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cuda_status(cudaLaunchKernelEx(&cfg, k_wgemm_persist, mW, mX, mB, mU, mY, p));
+}
+
 int launch_base_lora_tc(const void* x, const void* W0, const void* B, const meteora_shape_t& s, const Workspace& ws,
                         void* y, bool pdl, cudaStream_t st) {
+    const PersistPlan ps = make_persist_plan(s);
+    if (ps.ok) return launch_base_persist(x, W0, B, s, ws, y, ps, pdl, st);
     const PairPlan pp = make_pair_plan(s);
     if (pp.ok) {
         const int row_tiles = (s.d_out + kBM - 1) / kBM, row_pairs = (row_tiles + 1) / 2;
@@ -2335,11 +2465,14 @@ int launch_token_gate(const void* x, const void* Wg, const meteora_shape_t& s, i
 
 bool token_forward_supported(const meteora_shape_t& s) { return make_token_plan(s, TOKEN_FORWARD).ok; }
 
-int launch_token_forward(const void* x, const void* A, const void* Wg, const meteora_shape_t& s, const Workspace& ws, cudaStream_t st) {
+int launch_token_forward(const void* x, const void* A, const void* Wg, const meteora_shape_t& s, const Workspace& ws, void* us,
+                         cudaStream_t st) {
     TokenTileParams p = {};
     p.topk_idx = ws.topk_idx;
     p.topk_w = ws.topk_w;
     p.u = ws.uw;
+    p.us = (__nv_bfloat16*)us;
+    p.ld_us = ws.ld_us;
     p.status = ws.status;
     return launch_token_tile(make_token_plan(s, TOKEN_FORWARD), TOKEN_FORWARD, s, x, Wg, A, p, st);
 }
@@ -2443,6 +2576,12 @@ int describe_plan(const meteora_shape_t& s, char* buf, size_t n) {
     const int row_tiles = (s.d_out + kBM - 1) / kBM;
     const TokenPlan tp = make_token_plan(s, TOKEN_FORWARD);   // routing in one launch of token tiles, else in two
     const int routing = tp.ok ? 1 : 2;
+    const PersistPlan ps = make_persist_plan(s);
+    if (ps.ok)
+        return snprintf(buf, n,
+                        "path=chain(not fused: reason %d) launches=%d token_tile_cluster=%d base=pairs_of_ctas persistent_pairs=%d "
+                        "tiles=%d tile=256x%d stages=%d smem=%zu expand=mma",
+                        fp.why, routing + 1, tp.S, ps.pairs, ps.tiles, ps.BN, ps.stages, ps.smem);
     const PairPlan pp = make_pair_plan(s);
     if (pp.ok)
         return snprintf(buf, n,

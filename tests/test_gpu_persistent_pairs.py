@@ -1,0 +1,44 @@
+"""The prefill base product on persistent pairs of SMs at the edges of its tiles, against the CPU oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2405_13053_b200 import binding as mb
+from paper_2405_13053_b200 import workloads
+from .gpu_util import bf16_bound_ok, check_selection, rel_l2, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+# Tile widths 160 / 192 / 224 / 256 (257, 380, 1300, 1281 tokens), a last token tile with few tokens, odd numbers of row tiles and
+# a ragged last one, axes of 5 k-steps and of no whole number, several adapters per block of expand columns (ranks 16 - 64), an
+# odd number of blocks (33), fewer tiles than pairs, less and more than two rounds, whole rounds.
+@pytest.mark.parametrize("T,d_in,d_out,N,r,k", [
+    (257, 4096, 200, 28, 8, 2), (380, 2048, 384, 28, 8, 2), (512, 8192, 1024, 28, 8, 2), (700, 520, 2184, 28, 16, 2),
+    (1281, 520, 2184, 28, 8, 2), (1300, 1024, 4096, 33, 8, 4), (1201, 1536, 5120, 5, 32, 2), (2560, 512, 2048, 28, 64, 2),
+    (5000, 320, 2560, 28, 16, 2), (2400, 256, 1024, 100, 8, 2), (300, 320, 9472, 28, 8, 1), (1024, 640, 9472, 28, 8, 2),
+])
+def test_persistent_pairs_match_oracle(T, d_in, d_out, N, r, k):
+    w = workloads.make_workload("persist", T=T, d_in=d_in, d_out=d_out, N=N, r=r, k=k, dtype="bf16", seed=90 + T, b_std=0.3)
+    t = to_dev(w, "x", "W0", "A", "B", "Wg")
+    mb.meteora_set_tuning("persist", 2)
+    try:
+        shape = mb.make_shape(T, d_in, d_out, N, r, k, torch.bfloat16)
+        assert "persistent_pairs" in mb.meteora_describe_plan(shape)
+        ws = mb.alloc_workspace(shape)
+        y, idx, _ = mb.meteora_linear_forward(*t, k, workspace=ws, return_routing=True)
+        y, idx = y.float().cpu().numpy(), idx.cpu().numpy()
+        assert mb.meteora_workspace_status(ws) == 0
+        for _ in range(3):                               # sums in the same order, whatever the workspace holds
+            again = mb.meteora_linear_forward(*t, k, workspace=ws)
+        np.testing.assert_array_equal(y, again.float().cpu().numpy())
+        assert mb.meteora_workspace_status(ws) == 0
+    finally:
+        mb.meteora_set_tuning("persist", 1)
+    o_idx, _, o_logits = oracle.gate_topk(w["x"], w["Wg"], k)
+    check_selection(idx, o_idx, o_logits, k)
+    sel = np.unique(np.concatenate([np.arange(0, T, 61), np.arange(159, T, 160), np.arange(255, T, 256), [T - 1]]))
+    ref = oracle.linear_forward_routed(w["x"][sel], w["W0"], w["A"], w["B"], w["Wg"], idx[sel])
+    assert rel_l2(y[sel], ref) <= 5e-3
+    assert bf16_bound_ok(y[sel], ref) <= 0.0
