@@ -146,7 +146,8 @@ int meteora_lora_delta_static(const void* x, const void* A, const void* B, const
  * paths with A and B zero-padded to the next multiple of 8 inside the workspace (rewritten by every call).  Every other shape
  * runs on a plain CUDA-core path with the same results up to rounding order.  The workspace header
  * must have been zeroed once (meteora_workspace_init) before its first use; the kernels leave it
- * ready for the next call.  meteora_describe_plan tells which path a shape takes.
+ * ready for the next call.  Prefill batches of rank 8, 16, 32 or 64 run the base product on persistent pairs of SMs; where
+ * [Wg; A] has at most 512 rows gate, selection and shrink are part of the same launch.  meteora_describe_plan tells which path a shape takes.
  */
 int meteora_linear_forward(const void* x, const void* W0, const void* A, const void* B, const void* Wg,
                            const meteora_shape_t* shape, void* y, void* workspace, size_t workspace_bytes,
@@ -160,7 +161,8 @@ int meteora_linear_forward(const void* x, const void* W0, const void* A, const v
  * array; T, d_in, N, r, k, dtype, temperature come from `shape` (its d_out is ignored).  Results per module are
  * those of meteora_linear_forward up to the rounding order of fp32 sums.  Decode batches (T <= 256, rank a
  * multiple of 8, bf16, all modules together at most about 120 row tiles of 128) run as ONE kernel launch for the whole group;
- * anything else runs module by module.  workspace: meteora_group_workspace_bytes(shape, d_out, n_modules) bytes of
+ * prefill batches of modules whose [Wg; A] has at most 512 rows run as ONE launch as well (persistent pairs of SMs, from about
+ * 10 K outputs x 1 K tokens on); anything else runs module by module.  workspace: meteora_group_workspace_bytes(shape, d_out, n_modules) bytes of
  * device memory, its first 4 KB zeroed once (meteora_workspace_init); meteora_workspace_status reads the group's
  * status word.  meteora_group_workspace_routing returns where module `module` left its routing;
  * meteora_group_plan returns 1 if the group runs as one launch, 0 if module by module, or an error code.
@@ -325,7 +327,7 @@ int meteora_describe_plan(const meteora_shape_t* shape, char* buf, size_t buf_by
  *                    default 0 = never (measured slower than the streamed kernel except for the largest layers),
  *                    other = wherever the device can hold all clusters at once
  *   "persist"        prefill base product on persistent pairs of SMs: default 1 = planner's choice, 0 = never, 2 = wherever the
- *                    shape allows ("pair" 2 and a set "tail_carve" take the kernel with one tile per pair)
+ *                    shape allows, 3 = without gate and selection in the same launch ("pair" 2 and a set "tail_carve" take the kernel with one tile per pair)
  *   "group_pairs"    > 0 = row pairs per scheduling group of the prefill kernel on pairs of SMs (0 = planner's choice)
  *   "tail_carve"     prefill on pairs of SMs: 0 = the planner carves the tiles of a nearly empty last wave out of the
  *                    pair launch (they follow as a launch of small tiles), -1 = never, n > 0 = the last token tile of n row pairs

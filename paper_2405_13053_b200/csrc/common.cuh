@@ -127,6 +127,10 @@ struct GroupModule {
     int d_out;
     Workspace ws;       // topk_idx, topk_w, uw, u_all, ld_u, col_logits of this module
 };
+// Prefill: the whole layer of such modules on persistent pairs of SMs, one launch (wgemm_persist.cuh)
+bool persist_forward_supported(const meteora_shape_t& s, const int* d_outs, int n_modules);
+int launch_persist_forward(const void* x, const GroupModule* mods, int n_modules, const meteora_shape_t& s, int32_t* status,
+                           int32_t* flags, cudaStream_t st);
 bool decode_group_supported(const meteora_shape_t& s, const int* d_outs, int n_modules);
 int launch_decode_group(const void* x, const GroupModule* mods, int n_modules, const meteora_shape_t& s,
                         int32_t* status, float* part_g, int32_t* tile_ctr, cudaStream_t st);
@@ -169,7 +173,7 @@ struct Tuning {
     int no_hold = 0;         // decode kernel, head start of the aux CTAs: 0 planner's choice, 1 none, 64 counter wait, other = nanoseconds
     int hold_after = 0;      // decode kernel: ring stages of W0 the main CTAs request before the aux CTAs' head start (0: planner, -1: none)
     int narrow_select = 0;   // decode kernel's selection: 0 by batch size, 1 always two narrow round trips, -1 always one wide one
-    int persist = 1;         // prefill on persistent pairs of SMs: 0 never, 1 planner, 2 wherever the shape allows
+    int persist = 1;         // prefill on persistent pairs of SMs: 0 never, 1 planner, 2 wherever the shape allows, 3 without the routing
     int tail_carve = 0;      // prefill on pairs of SMs: 0 = the planner carves a nearly empty last wave out, -1 = never, n = n row pairs
     int aux_plain = 1;       // streamed kernel: the aux CTAs' partial tiles leave as plain stores (0: staged, one bulk copy)
     int cluster_decode = 0;  // decode batches on clusters that exchange through distributed shared memory (0: never)

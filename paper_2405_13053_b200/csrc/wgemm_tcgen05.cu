@@ -767,12 +767,12 @@ static int get_tensor_map(const void* ptr, int K, int rows, int box_rows, int de
 
 // Tensor map of y[T, d_out] (bf16, row-major) for storing a tile of 128 outputs x box_tokens tokens from
 // shared memory laid out [token][128 outputs]; not swizzled.  Needs d_out % 8 == 0 (16-byte row pitch).
-static int get_store_map(const void* y, int d_out, int T, int box_tokens, CUtensorMap* out) {
+static int get_store_map(const void* y, int d_out, int T, int box_tokens, CUtensorMap* out, int box_cols = kBM) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return METEORA_ERR_CUDA;
     const cuuint64_t gdim[2] = {(cuuint64_t)d_out, (cuuint64_t)T};
     const cuuint64_t gstride[1] = {(cuuint64_t)d_out * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)kBM, (cuuint32_t)box_tokens};
+    const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_tokens};
     const cuuint32_t estride[2] = {1, 1};
     const CUresult r = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(y), gdim, gstride, box, estride,
                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
@@ -1385,6 +1385,7 @@ static int pair_tail_carve(const meteora_shape_t& s) {
 struct PersistPlan {
     bool ok;
     int BN, CT, stages, stage_bytes, pairs, tok_tiles, tiles;
+    int stacked_pairs, gate_rows, us_cols;                       // stacked_pairs 0: the routing comes from kernels of its own
     size_t smem;
 };
 
@@ -1419,19 +1420,41 @@ static int persist_pairs() {
     return have - 1;
 }
 
-static PersistPlan make_persist_plan(const meteora_shape_t& s) {
+// One module, or a group of modules that share x; with_routing: gate, selection and shrink as the walk's first tiles.
+static PersistPlan make_persist_plan(const meteora_shape_t& s, const int* d_outs, int G, bool with_routing) {
     PersistPlan pp = {};
     const Tuning& tn = tuning();
     if (!tn.persist || tn.pair != 1 || tn.tail_carve != 0 || tn.simt_expand || tn.no_tma_store || tn.tile_tokens || tn.splits > 1) return pp;
-    if (persist_us_pitch(s) == 0 || !tc_path_supported(s)) return pp;
+    if (!tc_path_supported(s)) return pp;
     const int pairs = persist_pairs();
     if (pairs < 1) return pp;
     // tokens per tile: 256-token tiles, narrower ones (whole 32s) where that spreads a ragged token count over as many tiles
     pp.tok_tiles = (s.T + kPairTokens - 1) / kPairTokens;
     pp.BN = ((s.T + pp.tok_tiles - 1) / pp.tok_tiles + 31) / 32 * 32;
     pp.CT = pp.BN % 64 == 0 ? 64 : 32;
-    pp.tiles = ((s.d_out + kBM - 1) / kBM + 1) / 2 * pp.tok_tiles;
-    if (tn.persist == 1 && pp.tiles * 4 < sm_count()) return pp;
+    for (int m = 0; m < G; ++m) {
+        meteora_shape_t sm = s;
+        sm.d_out = d_outs[m];
+        if (persist_us_pitch(sm) == 0) return pp;
+        pp.tiles += ((d_outs[m] + kBM - 1) / kBM + 1) / 2 * pp.tok_tiles;
+    }
+    if (tn.persist != 2 && pp.tiles * 4 < sm_count()) return pp;
+    if (with_routing) {
+        // [Wg; A] in 128-row tiles: Wg padded to whole 32 rows (a warp's TMEM lanes), then A, padded to whole MMAs of the expand
+        pp.gate_rows = (s.N + 31) / 32 * 32;
+        pp.us_cols = (s.N * s.r + 15) / 16 * 16;
+        pp.stacked_pairs = (pp.gate_rows + pp.us_cols + 2 * kBM - 1) / (2 * kBM);
+        if (pp.stacked_pairs > 2 || s.N > kPersistMaxN || 2 * G * pp.tok_tiles > kMaxFusedRowTiles ||
+            G * pp.stacked_pairs * pp.tok_tiles > pairs)             // (a stacked tile is a pair's first)
+            return pp;
+        if (tn.persist == 3) return pp;
+        // one round of tiles that the stacked ones would make two (4096 -> 1024 at 4096 tokens: 55.9 us, 52.4 with the routing ahead)
+        const int with = pp.tiles + G * pp.stacked_pairs * pp.tok_tiles;
+        if (tn.persist != 2 && pp.tiles <= pairs && with > pairs) return pp;
+        pp.tiles = with;
+    } else if (G > 1) {
+        return pp;
+    }
     pp.pairs = std::min(pairs, pp.tiles);
     pp.stage_bytes = kWTileBytes + pp.BN / 2 * 128;
     const size_t fixed = 1024 + (size_t)kPersistStageBufs * kPersistStoreBytes + 512;
@@ -1441,51 +1464,115 @@ static PersistPlan make_persist_plan(const meteora_shape_t& s) {
     return pp;
 }
 
-bool persist_supported(const meteora_shape_t& s) { return make_persist_plan(s).ok; }
+bool persist_supported(const meteora_shape_t& s) { return make_persist_plan(s, &s.d_out, 1, false).ok; }
+bool persist_forward_supported(const meteora_shape_t& s, const int* d_outs, int G) { return make_persist_plan(s, d_outs, G, true).ok; }
 
-static int launch_base_persist(const void* x, const void* W0, const void* B, const meteora_shape_t& s, const Workspace& ws, void* y,
-                               const PersistPlan& pp, bool pdl, cudaStream_t st) {
-    CUtensorMap mW, mX, mB, mU, mY;
-    int rc;
-    if ((rc = get_tensor_map(W0, s.d_in, s.d_out, kBM, 0, &mW)) != METEORA_OK) return rc;
-    if ((rc = get_tensor_map(x, s.d_in, s.T, pp.BN / 2, 0, &mX)) != METEORA_OK) return rc;
-    if ((rc = get_tensor_map(ws.us, ws.ld_us, s.T, pp.BN / 2, 0, &mU)) != METEORA_OK) return rc;
-    if ((rc = get_store_map(y, s.d_out, s.T, pp.CT, &mY)) != METEORA_OK) return rc;
-    if ((rc = get_adapter_map(B, s.N, s.d_out, s.r, &mB)) != METEORA_OK) return rc;
+static int launch_persist(const PersistPlan& pp, const void* x, const GroupModule* mods, int G, const meteora_shape_t& s, int32_t* status,
+                          int32_t* flags, bool pdl, cudaStream_t st) {
+    PersistMaps maps;
     PersistParams p = {};
+    int rc;
+    if ((rc = get_tensor_map(x, s.d_in, s.T, pp.BN / 2, 0, &maps.X)) != METEORA_OK) return rc;
+    int tile0 = G * pp.stacked_pairs * pp.tok_tiles;
+    for (int m = 0; m < kMaxGroupModules; ++m) {
+        const GroupModule& gm = mods[m < G ? m : 0];             // unused slots repeat module 0's (valid) maps
+        if ((rc = get_tensor_map(gm.W0, s.d_in, gm.d_out, kBM, 0, &maps.W0[m])) != METEORA_OK) return rc;
+        if ((rc = get_adapter_map(gm.B, s.N, gm.d_out, s.r, &maps.B[m])) != METEORA_OK) return rc;
+        if ((rc = get_tensor_map(gm.ws.us, gm.ws.ld_us, s.T, pp.BN / 2, 0, &maps.U[m])) != METEORA_OK) return rc;
+        if ((rc = get_store_map(gm.y, gm.d_out, s.T, pp.CT, &maps.Y[m])) != METEORA_OK) return rc;
+        if ((rc = get_store_map(gm.ws.us, gm.ws.ld_us, s.T, 32, &maps.S[m], 32)) != METEORA_OK) return rc;
+        maps.A[m] = maps.A0[m] = maps.G[m] = maps.X;
+        if (pp.stacked_pairs > 0) {
+            if ((rc = get_tensor_map(gm.A, s.d_in, s.N * s.r, kBM, 0, &maps.A[m])) != METEORA_OK) return rc;
+            if ((rc = get_tensor_map(gm.A, s.d_in, s.N * s.r, kBM - pp.gate_rows, 0, &maps.A0[m])) != METEORA_OK) return rc;
+            if ((rc = get_tensor_map(gm.Wg, s.d_in, s.N, pp.gate_rows, 0, &maps.G[m])) != METEORA_OK) return rc;
+        }
+        PersistModule& mo = p.mod[m];
+        mo.row_tiles = (gm.d_out + kBM - 1) / kBM;
+        mo.row_pairs = (mo.row_tiles + 1) / 2;
+        mo.group_pairs = std::min(tuning().group_pairs > 0 ? tuning().group_pairs : std::max(1, (pp.pairs / pp.tok_tiles + 1) / 2), mo.row_pairs);
+        mo.tile0 = m < G ? tile0 : 0x7FFFFFFF;
+        mo.us = (__nv_bfloat16*)gm.ws.us;
+        mo.topk_idx = gm.ws.topk_idx;
+        mo.topk_w = gm.ws.topk_w;
+        tile0 += mo.row_pairs * pp.tok_tiles;
+    }
     p.T = s.T;
     p.BN = pp.BN;
     p.CT = pp.CT;
     p.ksteps = (s.d_in + kBK - 1) / kBK;
-    p.iters = p.ksteps + ws.ld_us / kBK;
+    p.esteps = mods[0].ws.ld_us / kBK;
+    p.N = s.N;
+    p.r = s.r;
+    p.k = s.k;
     p.cpa = s.r / 8;
     p.nblk = s.N * p.cpa;
     p.stages = pp.stages;
     p.stage_bytes = pp.stage_bytes;
-    p.row_tiles = (s.d_out + kBM - 1) / kBM;
-    p.row_pairs = (p.row_tiles + 1) / 2;
+    p.n_mod = G;
     p.tok_tiles = pp.tok_tiles;
-    p.group_pairs = std::min(tuning().group_pairs > 0 ? tuning().group_pairs : std::max(1, (pp.pairs / pp.tok_tiles + 1) / 2), p.row_pairs);
     p.tiles = pp.tiles;
-    p.status = ws.status;
-    p.pdl_wait = pdl ? 1 : 0;
+    p.stacked_pairs = pp.stacked_pairs;
+    p.gate_rows = pp.gate_rows;
+    p.us_cols = pp.us_cols;
+    p.ld_us = mods[0].ws.ld_us;
+    p.inv_tau = 1.0f / s.temperature;
+    p.flags = flags;
+    p.leave_ctr = status + 20;
+    p.status = status;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * pp.pairs);
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = pp.smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2];
+    int na = 0;
+    if (pp.stacked_pairs > 0) {                                  // the pairs wait for one another: all must be resident
+        attr[na].id = cudaLaunchAttributeCooperative;
+        attr[na].val.cooperative = 1;
+        ++na;
+    }
+    static std::atomic<bool> pdl_accepted{true};
+    const bool want_pdl = pdl && (pp.stacked_pairs == 0 || pdl_accepted.load(std::memory_order_relaxed));
+    if (want_pdl) {
+        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[na].val.programmaticStreamSerializationAllowed = 1;
+        ++na;
+    }
     cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
-    return cuda_status(cudaLaunchKernelEx(&cfg, k_wgemm_persist, mW, mX, mB, mU, mY, p));
+    cfg.numAttrs = na;
+    p.pdl = want_pdl ? 1 : 0;
+    cudaError_t err = cudaLaunchKernelEx(&cfg, k_wgemm_persist, maps, p);
+    if (pp.stacked_pairs > 0 && launch_config_refused(err) && want_pdl) {   // the two attributes together: try without the second
+        cudaGetLastError();
+        pdl_accepted.store(false, std::memory_order_relaxed);
+        tuning().pdl_decode_refused += 1;
+        cfg.numAttrs = na - 1;
+        p.pdl = 0;
+        err = cudaLaunchKernelEx(&cfg, k_wgemm_persist, maps, p);
+    }
+    if (pp.stacked_pairs > 0 && launch_config_refused(err)) {    // the caller may take the routing kernels instead
+        cudaGetLastError();
+        return kLaunchRefused;
+    }
+    return cuda_status(err);
+}
+
+// The whole layer of one module or of a group of modules that share x, one launch.
+int launch_persist_forward(const void* x, const GroupModule* mods, int G, const meteora_shape_t& s, int32_t* status, int32_t* flags,
+                           cudaStream_t st) {
+    int d_outs[kMaxGroupModules] = {};
+    for (int m = 0; m < G; ++m) d_outs[m] = mods[m].d_out;
+    return launch_persist(make_persist_plan(s, d_outs, G, true), x, mods, G, s, status, flags, tuning().pdl != 0, st);
 }
 
 int launch_base_lora_tc(const void* x, const void* W0, const void* B, const meteora_shape_t& s, const Workspace& ws,
                         void* y, bool pdl, cudaStream_t st) {
-    const PersistPlan ps = make_persist_plan(s);
-    if (ps.ok) return launch_base_persist(x, W0, B, s, ws, y, ps, pdl, st);
+    const PersistPlan ps = make_persist_plan(s, &s.d_out, 1, false);
+    if (ps.ok) {
+        const GroupModule gm = {W0, nullptr, B, nullptr, y, s.d_out, ws};
+        return launch_persist(ps, x, &gm, 1, s, ws.status, ws.tile_ctr, pdl, st);
+    }
     const PairPlan pp = make_pair_plan(s);
     if (pp.ok) {
         const int row_tiles = (s.d_out + kBM - 1) / kBM, row_pairs = (row_tiles + 1) / 2;
@@ -2576,7 +2663,13 @@ int describe_plan(const meteora_shape_t& s, char* buf, size_t n) {
     const int row_tiles = (s.d_out + kBM - 1) / kBM;
     const TokenPlan tp = make_token_plan(s, TOKEN_FORWARD);   // routing in one launch of token tiles, else in two
     const int routing = tp.ok ? 1 : 2;
-    const PersistPlan ps = make_persist_plan(s);
+    const PersistPlan whole = make_persist_plan(s, &s.d_out, 1, true);
+    if (whole.ok)
+        return snprintf(buf, n,
+                        "path=persistent_prefill launches=1 base=pairs_of_ctas persistent_pairs=%d tiles=%d stacked_tiles=%d tile=256x%d "
+                        "stages=%d smem=%zu expand=mma",
+                        whole.pairs, whole.tiles, whole.stacked_pairs * whole.tok_tiles, whole.BN, whole.stages, whole.smem);
+    const PersistPlan ps = make_persist_plan(s, &s.d_out, 1, false);
     if (ps.ok)
         return snprintf(buf, n,
                         "path=chain(not fused: reason %d) launches=%d token_tile_cluster=%d base=pairs_of_ctas persistent_pairs=%d "

@@ -14,18 +14,23 @@ pytestmark = pytest.mark.gpu
 # Tile widths 160 / 192 / 224 / 256 (257, 380, 1300, 1281 tokens), a last token tile with few tokens, odd numbers of row tiles and
 # a ragged last one, axes of 5 k-steps and of no whole number, several adapters per block of expand columns (ranks 16 - 64), an
 # odd number of blocks (33), fewer tiles than pairs, less and more than two rounds, whole rounds.
-@pytest.mark.parametrize("T,d_in,d_out,N,r,k", [
+# With the routing in the walk (persist 2) and from kernels of its own (3: from 37 pair tiles on); 56 adapters: two pairs of
+# stacked tiles, two logits per lane; 40 of rank 8: Wg in a tile of its own.
+@pytest.mark.parametrize("persist,T,d_in,d_out,N,r,k", [(p, *c) for p in (2, 3) for c in [
     (257, 4096, 200, 28, 8, 2), (380, 2048, 384, 28, 8, 2), (512, 8192, 1024, 28, 8, 2), (700, 520, 2184, 28, 16, 2),
     (1281, 520, 2184, 28, 8, 2), (1300, 1024, 4096, 33, 8, 4), (1201, 1536, 5120, 5, 32, 2), (2560, 512, 2048, 28, 64, 2),
     (5000, 320, 2560, 28, 16, 2), (2400, 256, 1024, 100, 8, 2), (300, 320, 9472, 28, 8, 1), (1024, 640, 9472, 28, 8, 2),
-])
-def test_persistent_pairs_match_oracle(T, d_in, d_out, N, r, k):
+    (600, 256, 3200, 56, 8, 2), (900, 512, 3200, 32, 8, 8),
+] if p == 2 or (c[0] + 255) // 256 * ((c[2] + 255) // 256) > 37])
+def test_persistent_pairs_match_oracle(persist, T, d_in, d_out, N, r, k):
     w = workloads.make_workload("persist", T=T, d_in=d_in, d_out=d_out, N=N, r=r, k=k, dtype="bf16", seed=90 + T, b_std=0.3)
     t = to_dev(w, "x", "W0", "A", "B", "Wg")
-    mb.meteora_set_tuning("persist", 2)
+    mb.meteora_set_tuning("persist", persist)
     try:
         shape = mb.make_shape(T, d_in, d_out, N, r, k, torch.bfloat16)
-        assert "persistent_pairs" in mb.meteora_describe_plan(shape)
+        plan = mb.meteora_describe_plan(shape)
+        whole = persist == 2 and N * (r + 1) <= 512 and N <= 64
+        assert ("path=persistent_prefill" if whole else "path=chain") in plan and "persistent_pairs" in plan, plan
         ws = mb.alloc_workspace(shape)
         y, idx, _ = mb.meteora_linear_forward(*t, k, workspace=ws, return_routing=True)
         y, idx = y.float().cpu().numpy(), idx.cpu().numpy()
@@ -42,3 +47,25 @@ def test_persistent_pairs_match_oracle(T, d_in, d_out, N, r, k):
     ref = oracle.linear_forward_routed(w["x"][sel], w["W0"], w["A"], w["B"], w["Wg"], idx[sel])
     assert rel_l2(y[sel], ref) <= 5e-3
     assert bf16_bound_ok(y[sel], ref) <= 0.0
+
+
+@pytest.mark.parametrize("T,d_in,d_outs", [(2100, 512, (2048, 512, 520)), (700, 1024, (4096, 4096)), (1500, 320, (256, 3000, 128, 2048))])
+def test_a_prefill_group_is_one_walk(T, d_in, d_outs):
+    ws_list = [workloads.make_workload("walk", T=T, d_in=d_in, d_out=d, dtype="bf16", seed=70, b_std=0.3) for d in d_outs]
+    for m, w in enumerate(ws_list):                      # one x, weights of their own
+        other = workloads.make_workload("walk", T=1, d_in=d_in, d_out=d_outs[m], dtype="bf16", seed=71 + m, b_std=0.3)
+        w.tensors.update({n: other[n] for n in ("W0", "A", "B", "Wg")})
+    x = to_dev(ws_list[0], "x")[0]
+    dev = [to_dev(w, "W0", "A", "B", "Wg") for w in ws_list]
+    assert mb.meteora_group_plan(T, d_in, list(d_outs), 28, 8, 2, torch.bfloat16) == 1
+    W0s, As, Bs, Wgs = (list(t) for t in zip(*dev))
+    ys, routing = mb.meteora_linear_forward_group(x, W0s, As, Bs, Wgs, 2, return_routing=True)
+    ys2 = mb.meteora_linear_forward_group(x, W0s, As, Bs, Wgs, 2)
+    sel = np.unique(np.concatenate([np.arange(0, T, 97), np.arange(255, T, 256), [T - 1]]))
+    for w, y, y2, (idx, _) in zip(ws_list, ys, ys2, routing):
+        assert torch.equal(y, y2)
+        idx = idx.cpu().numpy()
+        o_idx, _, o_logits = oracle.gate_topk(w["x"], w["Wg"], 2)
+        check_selection(idx, o_idx, o_logits, 2)
+        ref = oracle.linear_forward_routed(w["x"][sel], w["W0"], w["A"], w["B"], w["Wg"], idx[sel])
+        assert rel_l2(y.float().cpu().numpy()[sel], ref) <= 5e-3
