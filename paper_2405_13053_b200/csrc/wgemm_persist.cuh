@@ -176,8 +176,8 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
     const uint32_t bar_accf = bar_base + 2 * p.stages * 8, bar_acce = bar_accf + 16, bar_pick = bar_accf + 32;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem_raw + (bar_base - raw) + (2 * p.stages + 6) * 8);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t rank = cluster_rank();
+    const int warp = warp_id(), lane = threadIdx.x & 31;
+    const uint32_t rank = __shfl_sync(0xFFFFFFFFu, cluster_rank(), 0);
     const bool leader = rank == 0;
     const int pair0 = (int)blockIdx.x >> 1, npairs = (int)gridDim.x >> 1;
     // where the tile before gets its expand: late, so that the selection is ready for the first tiles, and early enough for
@@ -211,7 +211,7 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer (both CTAs)
-        if (lane == 0) {
+        {
             int s = 0, round = 0;                                 // ring slot, how often the ring has been filled
             bool waited = !p.pdl;
             // with stacked tiles x comes from the kernel ahead; else the kernel ahead is this call's routing, which read x
@@ -219,12 +219,11 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                 asm volatile("griddepcontrol.wait;" ::: "memory");
                 waited = true;
             }
-            auto slot = [&](uint32_t& full_leader, uint32_t& dst) {   // the next free stage
+            auto slot = [&](uint32_t& full, uint32_t& full_leader, uint32_t& dst) {   // the next free stage
                 if (round > 0 && !mbar_wait(bar_base + (p.stages + s) * 8, (round & 1) ^ 1)) return false;
-                const uint32_t full = bar_base + s * 8;
+                full = bar_base + s * 8;
                 full_leader = map_to_cta(full, 0);
                 dst = ring + s * p.stage_bytes;
-                if (leader) mbar_expect_tx(full, 2 * (uint32_t)p.stage_bytes);
                 if (++s == p.stages) {
                     s = 0;
                     ++round;
@@ -240,15 +239,19 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                     waited = true;
                 }
                 const int row0 = (t.row_pair * 2 + (int)rank) * kBM, tokh = t.tok_tile * p.BN + (int)rank * (p.BN / 2);
-                uint32_t full, dst;
+                uint32_t own, full, dst;
                 for (int i = 0; i < p.esteps; ++i) {
-                    if (!slot(full, dst)) return false;
+                    if (!slot(own, full, dst)) return false;
                     const int q0 = i * 8;                         // first of the 8 blocks
-                    if (p.cpa == 1)
-                        tma_load_3d_grp(dst, &maps.B[t.mod], 0, row0 / 8, q0, full);
-                    else
-                        tma_load_4d_grp(dst, &maps.B[t.mod], 0, row0, q0 % p.cpa, q0 / p.cpa, full);
-                    tma_load_2d_pair(dst + kWTileBytes, &maps.U[t.mod], q0 * 8, tokh, full);
+                    if (elect_one()) {
+                        if (leader) mbar_expect_tx(own, 2 * (uint32_t)p.stage_bytes);
+                        if (p.cpa == 1)
+                            tma_load_3d_grp(dst, &maps.B[t.mod], 0, row0 / 8, q0, full);
+                        else
+                            tma_load_4d_grp(dst, &maps.B[t.mod], 0, row0, q0 % p.cpa, q0 / p.cpa, full);
+                        tma_load_2d_pair(dst + kWTileBytes, &maps.U[t.mod], q0 * 8, tokh, full);
+                    }
+                    __syncwarp();
                 }
                 return true;
             };
@@ -263,26 +266,30 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                 const CUtensorMap* mW = !t.stacked ? &maps.W0[t.mod] : gate ? &maps.A0[t.mod] : &maps.A[t.mod];
                 const int w_row = !t.stacked ? row_tile * kBM : gate ? 0 : row_tile * kBM - p.gate_rows;
                 const uint32_t w_off = gate ? (uint32_t)p.gate_rows * 128u : 0u;
-                uint32_t full, dst;
+                uint32_t own, full, dst;
                 for (int i = 0; i < p.ksteps && ok; ++i) {
                     if (i == mid && pending) ok = expand(before);
-                    if (!ok || !(ok = slot(full, dst))) break;
-                    tma_load_2d_pair(dst + w_off, mW, i * kBK, w_row, full);
-                    if (gate) tma_load_2d_pair(dst, &maps.G[t.mod], i * kBK, 0, full);
-                    tma_load_2d_pair(dst + kWTileBytes, &maps.X, i * kBK, tokh, full);
+                    if (!ok || !(ok = slot(own, full, dst))) break;
+                    if (elect_one()) {
+                        if (leader) mbar_expect_tx(own, 2 * (uint32_t)p.stage_bytes);
+                        tma_load_2d_pair(dst + w_off, mW, i * kBK, w_row, full);
+                        if (gate) tma_load_2d_pair(dst, &maps.G[t.mod], i * kBK, 0, full);
+                        tma_load_2d_pair(dst + kWTileBytes, &maps.X, i * kBK, tokh, full);
+                    }
+                    __syncwarp();
                 }
                 pending = !t.stacked;
                 before = t;
             }
             if (ok && pending) ok = expand(before);
-            if (!ok) {
+            if (!ok && lane == 0) {
                 atomicExch(p.status, 1);
                 atomicExch(p.status + 1, 5100);
             }
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer (leader only)
-        if (lane == 0 && leader) {
+        if (leader) {
             const uint32_t idesc = instr_desc_bf16_pair_n(p.BN);
             bool ok = true, pending = false;
             int s = 0, phase = 0, n = 0;
@@ -293,7 +300,6 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                 return true;
             };
             auto release = [&]() {
-                umma_commit_pair(bar_base + (p.stages + s) * 8);
                 if (++s == p.stages) {
                     s = 0;
                     phase ^= 1;
@@ -305,12 +311,17 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                     if (!next(wa)) return false;
                     const uint64_t db = smem_desc_sw128(wa + kWTileBytes);
                     const int nm = min(4, (p.nblk - i * 8 + 1) / 2);   // two blocks per MMA: 8-row x 16-byte core matrices, 2 KB per block
-                    for (int kk = 0; kk < nm; ++kk)
-                        umma_bf16_pair(tmem_base + b * kPairTokens, smem_desc_plain(wa + kk * 2 * kBM * 16, kBM * 16, 128),
-                                       db + (uint64_t)(kk * 2), idesc, 1);
+                    if (elect_one()) {
+                        for (int kk = 0; kk < nm; ++kk)
+                            umma_bf16_pair(tmem_base + b * kPairTokens, smem_desc_plain(wa + kk * 2 * kBM * 16, kBM * 16, 128),
+                                           db + (uint64_t)(kk * 2), idesc, 1);
+                        umma_commit_pair(bar_base + (p.stages + s) * 8);
+                    }
+                    __syncwarp();
                     release();
                 }
-                umma_commit_pair(bar_accf + b * 8);
+                if (elect_one()) umma_commit_pair(bar_accf + b * 8);
+                __syncwarp();
                 return true;
             };
             for (int lin = pair0; lin < p.tiles && ok; lin += npairs, ++n) {
@@ -326,17 +337,22 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                     if (i == mid && pending && !(ok = expand(b ^ 1))) break;
                     if (!(ok = next(wa))) break;
                     const uint64_t da = smem_desc_sw128(wa), db = smem_desc_sw128(wa + kWTileBytes);
+                    if (elect_one()) {
 #pragma unroll
-                    for (int kk = 0; kk < kBK / kUmmaK; ++kk)
-                        umma_bf16_pair(acc, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc, (i | kk) != 0);
+                        for (int kk = 0; kk < kBK / kUmmaK; ++kk)
+                            umma_bf16_pair(acc, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc, (i | kk) != 0);
+                        umma_commit_pair(bar_base + (p.stages + s) * 8);
+                    }
+                    __syncwarp();
                     release();
                 }
                 if (!ok) break;
                 pending = lin >= p.mod[0].tile0;
-                if (!pending) umma_commit_pair(bar_accf + b * 8);
+                if (!pending && elect_one()) umma_commit_pair(bar_accf + b * 8);
+                __syncwarp();
             }
             if (ok && pending) ok = expand((n & 1) ^ 1);
-            if (!ok) {
+            if (!ok && lane == 0) {
                 atomicExch(p.status, 1);
                 atomicExch(p.status + 2, 5200);
             }

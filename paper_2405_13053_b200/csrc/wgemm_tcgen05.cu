@@ -103,6 +103,22 @@ struct WGemmParams {
 // ------------------------------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// True in one lane of the (converged) warp.  The threads that issue TMA copies and MMAs take their operands from uniform registers:
+// a warp that stays together and elects the lane for each instruction computes them there, while a loop entered by one
+// lane moves every descriptor and coordinate over one by one (450 - 530 cycles per k-step for two copies, four MMAs and
+// a commit, on both sides of the ring: more than the k-step's data or its MMAs take).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xFFFFFFFF;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok));
+    return ok != 0;
+}
+// The warp's number, as a value the compiler knows to be the same in all its lanes.
+__device__ __forceinline__ int warp_id() { return __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0); }
+
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
@@ -1393,7 +1409,7 @@ struct PersistPlan {
 // is whole adapters or a whole part of one) and more than 2048 columns stay with the kernel that stages them in rounds.
 int persist_us_pitch(const meteora_shape_t& s) {
     const int cols = (s.N * s.r + kBK - 1) / kBK * kBK, cpa = s.r / 8;
-    if (s.dtype != METEORA_BF16 || s.T <= 256 || s.d_in % 8 != 0 || s.d_out % 8 != 0 || s.r % 8 != 0 || cols > 2048) return 0;
+    if (s.dtype != METEORA_BF16 || s.T <= 32 || s.d_in % 8 != 0 || s.d_out % 8 != 0 || s.r % 8 != 0 || cols > 2048) return 0;
     return cpa == 1 || cpa == 2 || cpa == 4 || cpa == 8 ? cols : 0;
 }
 
@@ -1438,7 +1454,7 @@ static PersistPlan make_persist_plan(const meteora_shape_t& s, const int* d_outs
         if (persist_us_pitch(sm) == 0) return pp;
         pp.tiles += ((d_outs[m] + kBM - 1) / kBM + 1) / 2 * pp.tok_tiles;
     }
-    if (tn.persist != 2 && pp.tiles * 4 < sm_count()) return pp;
+    if (tn.persist < 2 && pp.tiles * 4 < sm_count()) return pp;
     if (with_routing) {
         // [Wg; A] in 128-row tiles: Wg padded to whole 32 rows (a warp's TMEM lanes), then A, padded to whole MMAs of the expand
         pp.gate_rows = (s.N + 31) / 32 * 32;
