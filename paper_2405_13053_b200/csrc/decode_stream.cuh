@@ -237,7 +237,7 @@ k_decode_stream(const __grid_constant__ CUtensorMap tmW0, const __grid_constant_
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(ring_ptr + ring_bytes + (2 * d.bar_slots + 4) * 8);
     uint8_t* slab_ptr = ring_ptr + ring_bytes + d.slab_off;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_id(), lane = threadIdx.x & 31;
     const bool is_aux = (int)blockIdx.x < d.n_aux;
     const int n_active = d.aux_tiles * d.aux_slices;
 
@@ -290,7 +290,7 @@ k_decode_stream(const __grid_constant__ CUtensorMap tmW0, const __grid_constant_
         const int ks1 = active ? (d.ksteps * (slice + 1)) / d.aux_slices : 0;
         const int niter = ks1 - ks0;
         if (warp == 0) {
-            if (lane == 0 && active) {
+            if (active) {
                 // A's last tile has its own map (its box stops at A's last row when Wg follows in the same tile)
                 const CUtensorMap* mA = tile >= d.a_tiles ? nullptr : tile == d.a_tiles - 1 ? &tmAt : &tmA;
                 const CUtensorMap* mG = tile == d.gate_tile ? &tmG : nullptr;
@@ -299,51 +299,70 @@ k_decode_stream(const __grid_constant__ CUtensorMap tmW0, const __grid_constant_
                 // weights first: they do not depend on the kernel ahead
                 for (int i = 0; i < pre; ++i) {
                     const uint32_t full = bar_base + i * 8, dst = ring + i * aux_stage_bytes;
-                    mbar_expect_tx_only(full, kWTileBytes);
-                    if (mA) tma_load_3d(dst, mA, 0, tile * kBM, ks0 + i, full);
-                    if (mG) tma_load_3d(dst + g_off, mG, 0, 0, ks0 + i, full);
+                    if (elect_one()) {
+                        mbar_expect_tx_only(full, kWTileBytes);
+                        if (mA) tma_load_3d(dst, mA, 0, tile * kBM, ks0 + i, full);
+                        if (mG) tma_load_3d(dst + g_off, mG, 0, 0, ks0 + i, full);
+                    }
+                    __syncwarp();
                 }
                 for (int i = pre; i < min(niter, pre + d.pf_aux); ++i) {
-                    if (mA) tma_prefetch_l2_3d(mA, 0, tile * kBM, ks0 + i);
-                    if (mG) tma_prefetch_l2_3d(mG, 0, 0, ks0 + i);
+                    if (elect_one()) {
+                        if (mA) tma_prefetch_l2_3d(mA, 0, tile * kBM, ks0 + i);
+                        if (mG) tma_prefetch_l2_3d(mG, 0, 0, ks0 + i);
+                    }
+                    __syncwarp();
                 }
                 if (d.pdl) asm volatile("griddepcontrol.wait;" ::: "memory");
                 STREAM_STAMP(1);
                 for (int i = 0; i < pre; ++i) {
                     const uint32_t full = bar_base + i * 8, dst = ring + i * aux_stage_bytes;
-                    mbar_expect_tx(full, aux_x_bytes);
-                    tma_load_3d(dst + kWTileBytes, &tmX1, 0, 0, ks0 + i, full);
+                    if (elect_one()) {
+                        mbar_expect_tx(full, aux_x_bytes);
+                        tma_load_3d(dst + kWTileBytes, &tmX1, 0, 0, ks0 + i, full);
+                    }
+                    __syncwarp();
                 }
                 bool ok = true;
                 for (int i = pre; i < niter; ++i) {
                     const int s = i % d.aux_stages, round = i / d.aux_stages;
-                    ok = mbar_wait(bar_base + (d.bar_slots + s) * 8, (round & 1) ^ 1);
+                    ok = mbar_wait_warp(bar_base + (d.bar_slots + s) * 8, (round & 1) ^ 1);
                     if (!ok) break;
                     const uint32_t full = bar_base + s * 8, dst = ring + s * aux_stage_bytes;
-                    mbar_expect_tx(full, aux_stage_bytes);
-                    if (mA) tma_load_3d(dst, mA, 0, tile * kBM, ks0 + i, full);
-                    if (mG) tma_load_3d(dst + g_off, mG, 0, 0, ks0 + i, full);
-                    tma_load_3d(dst + kWTileBytes, &tmX1, 0, 0, ks0 + i, full);
+                    if (elect_one()) {
+                        mbar_expect_tx(full, aux_stage_bytes);
+                        if (mA) tma_load_3d(dst, mA, 0, tile * kBM, ks0 + i, full);
+                        if (mG) tma_load_3d(dst + g_off, mG, 0, 0, ks0 + i, full);
+                        tma_load_3d(dst + kWTileBytes, &tmX1, 0, 0, ks0 + i, full);
+                    }
+                    __syncwarp();
                 }
-                if (!ok) stream_flag_error(d, 1, 400);
+                if (!ok && lane == 0) stream_flag_error(d, 1, 400);
             }
         } else if (warp == 1) {
-            if (lane == 0 && active) {
+            if (active) {
                 bool ok = true;
                 for (int i = 0; i < niter; ++i) {
                     const int s = i % d.aux_stages, round = i / d.aux_stages;
-                    ok = mbar_wait(bar_base + s * 8, round & 1);
+                    ok = mbar_wait_warp(bar_base + s * 8, round & 1);
                     if (!ok) break;
                     tc_fence_after();
                     const uint32_t wa = ring + s * aux_stage_bytes, xa = wa + kWTileBytes;
                     const uint64_t da = smem_desc_sw128(wa), db = smem_desc_sw128(xa);
+                    if (elect_one()) {
 #pragma unroll
-                    for (int kk = 0; kk < kBK / kUmmaK; ++kk)
-                        umma_bf16(tmem_base, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc, (i | kk) != 0);
-                    umma_commit(bar_base + (d.bar_slots + s) * 8);
+                        for (int kk = 0; kk < kBK / kUmmaK; ++kk)
+                            umma_bf16(tmem_base, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc, (i | kk) != 0);
+                        umma_commit(bar_base + (d.bar_slots + s) * 8);
+                        if (i == niter - 1) umma_commit(bar_acc);
+                    }
+                    __syncwarp();
                 }
-                umma_commit(bar_acc);
-                if (!ok) stream_flag_error(d, 2, 500);
+                if (niter == 0 || !ok) {                             // (a failed wait: whatever was issued)
+                    if (elect_one()) umma_commit(bar_acc);
+                    __syncwarp();
+                }
+                if (!ok && lane == 0) stream_flag_error(d, 2, 500);
                 STREAM_STAMP(2);
             }
         } else if (active) {
@@ -481,7 +500,7 @@ k_decode_stream(const __grid_constant__ CUtensorMap tmW0, const __grid_constant_
         const uint32_t idx_off = delta_off + blk_bytes, uw_off = idx_off + ((idx_bytes + 127u) & ~127u);
         int* s_done = reinterpret_cast<int*>(tmem_slot) + 1;          // warps 0 and 1: who is last counts the CTA out
         if (warp == 0) {
-            if (lane == 0) {
+            {
                 const uint32_t w_bytes = d.kc * kWTileBytes, xs_bytes = d.kc * x_tile_bytes;
                 const uint32_t both = kPair ? 2u : 1u;               // the leader's barrier expects both CTAs' bytes
                 const int tok0 = kPair ? (int)rank * (d.BN / 2) : 0;  // own half of the token tile
@@ -499,34 +518,48 @@ k_decode_stream(const __grid_constant__ CUtensorMap tmW0, const __grid_constant_
                     else tma_load_3d(dst, &tmX, 0, tok0, it * d.kc, bar);
                 };
                 for (int i = 0; i < pre; ++i) {
-                    if (leader) mbar_expect_tx_only(bar_base + i * 8, both * w_bytes);
-                    load_w(ring + i * stage_bytes, it0 + i, full_bar(i));
+                    if (elect_one()) {
+                        if (leader) mbar_expect_tx_only(bar_base + i * 8, both * w_bytes);
+                        load_w(ring + i * stage_bytes, it0 + i, full_bar(i));
+                    }
+                    __syncwarp();
                 }
-                for (int i = pre; i < min(n_it, pre + d.pf_main); ++i) tma_prefetch_l2_3d(&tmW0, 0, row0, (it0 + i) * d.kc);
+                for (int i = pre; i < min(n_it, pre + d.pf_main); ++i) {
+                    if (elect_one()) tma_prefetch_l2_3d(&tmW0, 0, row0, (it0 + i) * d.kc);
+                    __syncwarp();
+                }
                 if (d.pdl) asm volatile("griddepcontrol.wait;" ::: "memory");
                 STREAM_STAMP(1);
                 for (int i = 0; i < pre; ++i) {
-                    if (leader) mbar_expect_tx(bar_base + i * 8, both * xs_bytes);
-                    load_x(ring + i * stage_bytes + w_bytes, it0 + i, full_bar(i));
+                    if (elect_one()) {
+                        if (leader) mbar_expect_tx(bar_base + i * 8, both * xs_bytes);
+                        load_x(ring + i * stage_bytes + w_bytes, it0 + i, full_bar(i));
+                    }
+                    __syncwarp();
                 }
                 bool ok = true;
                 int st = pre == d.stages ? 0 : pre, round = pre == d.stages ? 1 : 0;
                 for (int i = pre; i < n_it; ++i) {
-                    ok = mbar_wait(bar_base + (d.bar_slots + st) * 8, (round & 1) ^ 1);
+                    ok = mbar_wait_warp(bar_base + (d.bar_slots + st) * 8, (round & 1) ^ 1);
                     if (!ok) break;
                     const uint32_t dst = ring + st * stage_bytes;
-                    if (leader) mbar_expect_tx(bar_base + st * 8, both * stage_bytes);
-                    load_w(dst, it0 + i, full_bar(st));
-                    load_x(dst + w_bytes, it0 + i, full_bar(st));
+                    if (elect_one()) {
+                        if (leader) mbar_expect_tx(bar_base + st * 8, both * stage_bytes);
+                        load_w(dst, it0 + i, full_bar(st));
+                        load_x(dst + w_bytes, it0 + i, full_bar(st));
+                    }
+                    __syncwarp();
                     if (++st == d.stages) {
                         st = 0;
                         ++round;
                     }
                 }
-                if (!ok) stream_flag_error(d, 1, 100);
+                if (!ok && lane == 0) stream_flag_error(d, 1, 100);
+            }
+            if (lane == 0) {
                 STREAM_STAMP(2);
                 // The routing into the landing area, as soon as the ring is idle and the aux CTAs have published it.
-                ok = mbar_wait(bar_acc, 0);
+                bool ok = mbar_wait(bar_acc, 0);
                 if (ok) ok = wait_counter_slow(d.ctr + 1, n_active, 200);
                 if (!ok) stream_flag_error(d, 4, 800);
                 STREAM_STAMP(7);
@@ -537,7 +570,7 @@ k_decode_stream(const __grid_constant__ CUtensorMap tmW0, const __grid_constant_
                 mbar_wait(bar_route, 0);    // own copies have landed before the CTA may leave (the epilogue may have given up)
             }
         } else if (warp == 1) {
-            if (lane == 0) {
+            {
                 bool ok = true;
                 if (leader) {                                        // of a pair, the leader alone issues the MMAs
                     const uint32_t idesc_main =
@@ -545,38 +578,46 @@ k_decode_stream(const __grid_constant__ CUtensorMap tmW0, const __grid_constant_
                               : idesc;
                     int st = 0, round = 0;
                     for (int i = 0; i < n_it; ++i) {
-                        ok = mbar_wait(bar_base + st * 8, round & 1);
+                        ok = mbar_wait_warp(bar_base + st * 8, round & 1);
                         if (!ok) break;
                         tc_fence_after();
                         const uint32_t wa = ring + st * stage_bytes, xa = wa + d.kc * kWTileBytes;
-                        for (int c = 0; c < d.kc; ++c) {
-                            const uint64_t da = smem_desc_sw128(wa + c * kWTileBytes);
-                            const uint64_t db = smem_desc_sw128(xa + c * x_tile_bytes);
+                        if (elect_one()) {
+                            for (int c = 0; c < d.kc; ++c) {
+                                const uint64_t da = smem_desc_sw128(wa + c * kWTileBytes);
+                                const uint64_t db = smem_desc_sw128(xa + c * x_tile_bytes);
 #pragma unroll
-                            for (int kk = 0; kk < kBK / kUmmaK; ++kk) {
-                                if (kPair)
-                                    umma_bf16_pair(tmem_base, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc_main,
-                                                   (i | c | kk) != 0);
-                                else
-                                    umma_bf16(tmem_base, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc_main,
-                                              (i | c | kk) != 0);
+                                for (int kk = 0; kk < kBK / kUmmaK; ++kk) {
+                                    if (kPair)
+                                        umma_bf16_pair(tmem_base, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc_main,
+                                                       (i | c | kk) != 0);
+                                    else
+                                        umma_bf16(tmem_base, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc_main,
+                                                  (i | c | kk) != 0);
+                                }
                             }
+                            if (kPair) umma_commit_pair(bar_base + (d.bar_slots + st) * 8);   // both rings may refill the stage
+                            else umma_commit(bar_base + (d.bar_slots + st) * 8);
                         }
-                        if (kPair) umma_commit_pair(bar_base + (d.bar_slots + st) * 8);   // both rings may refill the stage
-                        else umma_commit(bar_base + (d.bar_slots + st) * 8);
+                        __syncwarp();
                         if (++st == d.stages) {
                             st = 0;
                             ++round;
                         }
                     }
-                    if (kPair) umma_commit_pair(bar_acc);            // accumulators complete in both CTAs
-                    else umma_commit(bar_acc);
-                    if (!ok) stream_flag_error(d, 2, 200);
+                    if (elect_one()) {
+                        if (kPair) umma_commit_pair(bar_acc);        // accumulators complete in both CTAs
+                        else umma_commit(bar_acc);
+                    }
+                    __syncwarp();
+                    if (!ok && lane == 0) stream_flag_error(d, 2, 200);
                 }
+            }
+            if (lane == 0) {
                 STREAM_STAMP(3);
                 // The other CTAs' partials of this CTA's row slice into the landing area, once the ring is idle and
                 // all S CTAs of the tile have delivered (this CTA's own delivery included).
-                ok = mbar_wait(bar_deliv, 0);                      // not before this CTA's own partial is out
+                bool ok = mbar_wait(bar_deliv, 0);                      // not before this CTA's own partial is out
                 if (d.pdl) asm volatile("griddepcontrol.wait;" ::: "memory");
                 if (ok && S > 1 && live) ok = wait_counter_slow(d.tile_ctr + tile, S, 100);
                 if (!ok) stream_flag_error(d, 4, 900);

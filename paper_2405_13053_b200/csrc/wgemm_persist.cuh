@@ -220,7 +220,7 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                 waited = true;
             }
             auto slot = [&](uint32_t& full, uint32_t& full_leader, uint32_t& dst) {   // the next free stage
-                if (round > 0 && !mbar_wait(bar_base + (p.stages + s) * 8, (round & 1) ^ 1)) return false;
+                if (round > 0 && !mbar_wait_warp(bar_base + (p.stages + s) * 8, (round & 1) ^ 1)) return false;
                 full = bar_base + s * 8;
                 full_leader = map_to_cta(full, 0);
                 dst = ring + s * p.stage_bytes;
@@ -232,7 +232,8 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
             };
             auto expand = [&](const PersistTile& t) {
                 if (p.stacked_pairs > 0) {                        // the selection of these tokens
-                    if (!wait_counter_slow(p.flags + (t.mod * p.tok_tiles + t.tok_tile) * 2 + 1, 4 * p.stacked_pairs, 100)) return false;
+                    const bool there = lane != 0 || wait_counter_slow(p.flags + (t.mod * p.tok_tiles + t.tok_tile) * 2 + 1, 4 * p.stacked_pairs, 100);
+                    if (!__all_sync(0xFFFFFFFFu, there)) return false;
                     asm volatile("fence.proxy.async;" ::: "memory");
                 } else if (!waited) {
                     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -294,7 +295,7 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
             bool ok = true, pending = false;
             int s = 0, phase = 0, n = 0;
             auto next = [&](uint32_t& wa) {                       // the next filled stage
-                if (!mbar_wait(bar_base + s * 8, phase)) return false;
+                if (!mbar_wait_warp(bar_base + s * 8, phase)) return false;
                 tc_fence_after();
                 wa = ring + s * p.stage_bytes;
                 return true;
@@ -328,7 +329,7 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                 const int b = n & 1;
                 const uint32_t acc = tmem_base + b * kPairTokens;
                 if (n >= 2) {                                     // the epilogue of tile n - 2 has read this accumulator
-                    ok = mbar_wait_cluster(bar_acce + b * 8, ((n >> 1) & 1) ^ 1);
+                    ok = __all_sync(0xFFFFFFFFu, mbar_wait_cluster(bar_acce + b * 8, ((n >> 1) & 1) ^ 1));
                     if (!ok) break;
                     tc_fence_after();
                 }

@@ -145,6 +145,15 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
         if ((spin & 0x3FF) == 0 && clock64() - t0 > limit) return false;
     }
 }
+// The same by a whole (converged) warp, which learns one answer.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity) {
+    if (__all_sync(0xFFFFFFFFu, mbar_try(bar, parity))) return true;
+    const long long t0 = clock64(), limit = g_wait_limit_cycles;
+    for (uint32_t spin = 1;; ++spin) {
+        if (__all_sync(0xFFFFFFFFu, mbar_try(bar, parity))) return true;
+        if ((spin & 0x3FF) == 0 && __any_sync(0xFFFFFFFFu, clock64() - t0 > limit)) return false;
+    }
+}
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm, int c0, int c1, uint32_t bar) {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
