@@ -371,7 +371,7 @@ struct RingGeom {
     int stages, kc, maps3d;
 };
 
-// Producer side of a main loop (one thread).  `first_batch_done`, if not null, is bumped once the loads
+// Producer side of a main loop (a whole warp: the lanes stay together and one is elected per instruction).  `first_batch_done`, if not null, is bumped once the loads
 // that fit into the ring without waiting have been issued.
 // A second weight map `tmW2` (or the only one, when tmW is null) lands `w2_off` bytes into the weight tile: the
 // rows of Wg behind the last rows of A.
@@ -379,49 +379,55 @@ __device__ __forceinline__ bool fused_producer(const RingGeom& g, const CUtensor
                                                int row0, int ks0, int niter, int32_t* first_batch_done,
                                                const CUtensorMap* tmW2 = nullptr, uint32_t w2_off = 0) {
     bool ok = true;
-    for (int i = 0; i < niter; ++i) {
-        const int s = i % g.stages, round = i / g.stages;
+    for (int i = 0, s = 0, round = 0; i < niter; ++i) {
         if (i == g.stages && first_batch_done) {
-            atomicAdd(first_batch_done, 1);
+            if ((threadIdx.x & 31) == 0) atomicAdd(first_batch_done, 1);
             first_batch_done = nullptr;
         }
-        if (round > 0) ok = mbar_wait(g.bar_base + (g.stages + s) * 8, (round & 1) ^ 1);
+        if (round > 0) ok = mbar_wait_warp(g.bar_base + (g.stages + s) * 8, (round & 1) ^ 1);
         if (!ok) break;
         const uint32_t full = g.bar_base + s * 8;
         const uint32_t dst = g.ring + s * g.stage_bytes;
         const int kstep = ks0 + i * g.kc;
-        mbar_expect_tx(full, g.stage_bytes);
-        if (g.maps3d) {
-            if (tmW) tma_load_3d(dst, tmW, 0, row0, kstep, full);
-            if (tmW2) tma_load_3d(dst + w2_off, tmW2, 0, 0, kstep, full);
-            tma_load_3d(dst + g.kc * kWTileBytes, tmXp, 0, 0, kstep, full);
-        } else {
-            if (tmW) tma_load_2d(dst, tmW, kstep * kBK, row0, full);
-            if (tmW2) tma_load_2d(dst + w2_off, tmW2, kstep * kBK, 0, full);
-            tma_load_2d(dst + kWTileBytes, tmXp, kstep * kBK, 0, full);
+        if (elect_one()) {
+            mbar_expect_tx(full, g.stage_bytes);
+            if (g.maps3d) {
+                if (tmW) tma_load_3d(dst, tmW, 0, row0, kstep, full);
+                if (tmW2) tma_load_3d(dst + w2_off, tmW2, 0, 0, kstep, full);
+                tma_load_3d(dst + g.kc * kWTileBytes, tmXp, 0, 0, kstep, full);
+            } else {
+                if (tmW) tma_load_2d(dst, tmW, kstep * kBK, row0, full);
+                if (tmW2) tma_load_2d(dst + w2_off, tmW2, kstep * kBK, 0, full);
+                tma_load_2d(dst + kWTileBytes, tmXp, kstep * kBK, 0, full);
+            }
         }
+        __syncwarp();
+        if (++s == g.stages) s = 0, ++round;
     }
-    if (first_batch_done) atomicAdd(first_batch_done, 1);
+    if (first_batch_done && (threadIdx.x & 31) == 0) atomicAdd(first_batch_done, 1);
     return ok;
 }
 
-// MMA side of a main loop (one thread); does not commit the accumulator barrier.
+// MMA side of a main loop (a whole warp); does not commit the accumulator barrier.
 __device__ __forceinline__ bool fused_mma(const RingGeom& g, uint32_t tmem_base, uint32_t idesc, int niter) {
     bool ok = true;
-    for (int i = 0; i < niter; ++i) {
-        const int s = i % g.stages, round = i / g.stages;
-        ok = mbar_wait(g.bar_base + s * 8, round & 1);
+    for (int i = 0, s = 0, round = 0; i < niter; ++i) {
+        ok = mbar_wait_warp(g.bar_base + s * 8, round & 1);
         if (!ok) break;
         tc_fence_after();
         const uint32_t wa = g.ring + s * g.stage_bytes, xa = wa + g.kc * kWTileBytes;
-        for (int c = 0; c < g.kc; ++c) {
-            const uint64_t da = smem_desc_sw128(wa + c * kWTileBytes);
-            const uint64_t db = smem_desc_sw128(xa + c * g.x_tile_bytes);
+        if (elect_one()) {
+            for (int c = 0; c < g.kc; ++c) {
+                const uint64_t da = smem_desc_sw128(wa + c * kWTileBytes);
+                const uint64_t db = smem_desc_sw128(xa + c * g.x_tile_bytes);
 #pragma unroll
-            for (int kk = 0; kk < kBK / kUmmaK; ++kk)
-                umma_bf16(tmem_base, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc, (i | c | kk) != 0);
+                for (int kk = 0; kk < kBK / kUmmaK; ++kk)
+                    umma_bf16(tmem_base, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc, (i | c | kk) != 0);
+            }
+            umma_commit(g.bar_base + (g.stages + s) * 8);
         }
-        umma_commit(g.bar_base + (g.stages + s) * 8);
+        __syncwarp();
+        if (++s == g.stages) s = 0, ++round;
     }
     return ok;
 }
@@ -455,7 +461,7 @@ k_decode_fused(const __grid_constant__ DecodeMaps maps, const __grid_constant__ 
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(ring_ptr + ring_bytes + nbar * 8);
     uint8_t* epi = ring_ptr + ring_bytes + p.epi_off;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_id(), lane = threadIdx.x & 31;
     const bool is_aux = (int)blockIdx.x < d.n_aux;
     const int main_id = (int)blockIdx.x - d.n_aux;
     const int n_active = d.n_mod * d.aux_tiles * d.aux_slices;
@@ -514,24 +520,25 @@ k_decode_fused(const __grid_constant__ DecodeMaps maps, const __grid_constant__ 
         const RingGeom geom = {ring, bar_base, x_tile_bytes, kWTileBytes + x_tile_bytes, d.aux_stages, 1, p.maps3d};
         const uint32_t bar_acc = bar_base + 2 * d.aux_stages * 8;
         if (warp == 0) {
-            if (lane == 0 && active) {
+            if (active) {
                 // A's last tile has its own map (its box stops at A's last row when Wg follows in the same tile)
                 const CUtensorMap* mA = tile >= d.a_tiles ? nullptr : tile == d.a_tiles - 1 ? &maps.At[am] : &maps.A[am];
                 const CUtensorMap* mG = tile == d.gate_tile ? &maps.G[am] : nullptr;
-                if (tr_aux) FUSED_STAMP(p, 48, 6);
-                if (!fused_producer(geom, mA, &tmX1, tile * kBM, ks0, niter, d.ctr + 3, mG, (uint32_t)d.gate_row0 * 128u))
+                if (tr_aux && lane == 0) FUSED_STAMP(p, 48, 6);
+                if (!fused_producer(geom, mA, &tmX1, tile * kBM, ks0, niter, d.ctr + 3, mG, (uint32_t)d.gate_row0 * 128u) && lane == 0)
                     flag_error(p, 1, 400);
-                if (tr_aux) FUSED_STAMP(p, 48, 7);
+                if (tr_aux && lane == 0) FUSED_STAMP(p, 48, 7);
             }
         } else if (warp == 1) {
-            if (lane == 0 && active) {
+            if (active) {
 #ifdef METEORA_TRACE
                 if (niter > 0) mbar_wait(bar_base, 0);                          // first stage landed
-                FUSED_STAMP(p, 48, 8);
+                if (lane == 0) FUSED_STAMP(p, 48, 8);
 #endif
-                if (!fused_mma(geom, tmem_base, idesc, niter)) flag_error(p, 2, 500);
-                umma_commit(bar_acc);
-                if (tr_aux) FUSED_STAMP(p, 48, 1);
+                if (!fused_mma(geom, tmem_base, idesc, niter) && lane == 0) flag_error(p, 2, 500);
+                if (elect_one()) umma_commit(bar_acc);
+                __syncwarp();
+                if (tr_aux && lane == 0) FUSED_STAMP(p, 48, 1);
             }
         } else if (active) {
             bool acc_ok = mbar_wait(bar_acc, 0);
@@ -603,19 +610,19 @@ k_decode_fused(const __grid_constant__ DecodeMaps maps, const __grid_constant__ 
         const uint32_t bar_acc = bar_base + 2 * p.stages * 8;                        // [0 .. kMaxSeg): one per segment
         const size_t part_stride = (size_t)p.BN * kBM;                               // floats per partial tile
         if (warp == 0) {
-            if (lane == 0) {
+            {
                 // let the stacked shrink get its loads into the memory queues first
                 bool ok = true;
                 unsigned long long t0 = 0;
                 if (d.hold > 1) asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
-                if (tr_main) FUSED_STAMP(p, 32, 1);
+                if (tr_main && lane == 0) FUSED_STAMP(p, 32, 1);
                 int cur_tile = -1, row0 = 0;
                 const CUtensorMap* tmW0 = &maps.W0[0];
                 int tile = tile_a, kpos = u0 - tile_a * upt, st = 0, round = 0;
                 for (int it = 0; it < n_it && ok; ++it) {
                     if (it == d.hold_after) {                    // the first hold_after stages go out at once
                         if (d.hold == 1) {
-                            ok = wait_counter(d.ctr + 3, n_active);
+                            ok = __all_sync(0xFFFFFFFFu, lane != 0 || wait_counter(d.ctr + 3, n_active));
                             if (!ok) break;
                         } else if (d.hold > 1) {                 // a fixed head start for the aux CTAs, in nanoseconds
                             unsigned long long t1;
@@ -624,9 +631,10 @@ k_decode_fused(const __grid_constant__ DecodeMaps maps, const __grid_constant__ 
                                 __nanosleep(64);
                                 asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
                             } while (t1 - t0 < (unsigned long long)d.hold && ++spins < 4096);
+                            __syncwarp();
                         }
                     }
-                    if (round > 0) ok = mbar_wait(bar_base + (geom.stages + st) * 8, (round & 1) ^ 1);
+                    if (round > 0) ok = mbar_wait_warp(bar_base + (geom.stages + st) * 8, (round & 1) ^ 1);
                     if (!ok) break;
                     const uint32_t full = bar_base + st * 8, dst = ring + st * stage_bytes;
                     const int kstep = kpos * p.kc;
@@ -636,14 +644,17 @@ k_decode_fused(const __grid_constant__ DecodeMaps maps, const __grid_constant__ 
                         tmW0 = &maps.W0[wm];
                         row0 = (tile - d.mod[wm].tile0) * kBM;
                     }
-                    mbar_expect_tx(full, stage_bytes);
-                    if (p.maps3d) {
-                        tma_load_3d(dst, tmW0, 0, row0, kstep, full);
-                        tma_load_3d(dst + p.kc * kWTileBytes, &tmX, 0, 0, kstep, full);
-                    } else {
-                        tma_load_2d(dst, tmW0, kstep * kBK, row0, full);
-                        tma_load_2d(dst + kWTileBytes, &tmX, kstep * kBK, 0, full);
+                    if (elect_one()) {
+                        mbar_expect_tx(full, stage_bytes);
+                        if (p.maps3d) {
+                            tma_load_3d(dst, tmW0, 0, row0, kstep, full);
+                            tma_load_3d(dst + p.kc * kWTileBytes, &tmX, 0, 0, kstep, full);
+                        } else {
+                            tma_load_2d(dst, tmW0, kstep * kBK, row0, full);
+                            tma_load_2d(dst + kWTileBytes, &tmX, kstep * kBK, 0, full);
+                        }
                     }
+                    __syncwarp();
                     if (++kpos == upt) {
                         kpos = 0;
                         ++tile;
@@ -653,9 +664,11 @@ k_decode_fused(const __grid_constant__ DecodeMaps maps, const __grid_constant__ 
                         ++round;
                     }
                 }
-                if (!ok) flag_error(p, 1, 100);
-                if (!wait_counter(d.ctr + 1, n_active)) flag_error(p, 4, 800);              // routing published
-                if (tr_main) FUSED_STAMP(p, 32, 4);
+                if (lane == 0) {
+                    if (!ok) flag_error(p, 1, 100);
+                    if (!wait_counter(d.ctr + 1, n_active)) flag_error(p, 4, 800);          // routing published
+                    if (tr_main) FUSED_STAMP(p, 32, 4);
+                }
             }
             __syncwarp();
             // The routing into shared memory for the epilogue warps, once per tile this CTA finishes rows of (two
@@ -709,30 +722,32 @@ k_decode_fused(const __grid_constant__ DecodeMaps maps, const __grid_constant__ 
                 }
             }
         } else if (warp == 1) {
-            if (lane == 0) {
+            {
                 bool ok = true;
                 int committed = 0;                                                  // segments announced so far
                 int sg = 0, kpos = u0 - tile_a * upt, st = 0, round = 0;            // no divisions in this loop: it paces the tensor cores
                 for (int it = 0; it < n_it; ++it) {
-                    ok = mbar_wait(bar_base + st * 8, round & 1);
+                    ok = mbar_wait_warp(bar_base + st * 8, round & 1);
                     if (!ok) break;
                     tc_fence_after();
                     const bool fresh = it == 0 || kpos == 0;                        // first MMA of a segment overwrites
                     const uint32_t acc = tmem_base + (uint32_t)(sg * p.BN);
                     const uint32_t wa = ring + st * stage_bytes, xa = wa + p.kc * kWTileBytes;
-                    for (int c = 0; c < p.kc; ++c) {
-                        const uint64_t da = smem_desc_sw128(wa + c * kWTileBytes);
-                        const uint64_t db = smem_desc_sw128(xa + c * x_tile_bytes);
-#pragma unroll
-                        for (int kk = 0; kk < kBK / kUmmaK; ++kk)
-                            umma_bf16(acc, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc, !fresh || (c | kk) != 0);
-                    }
-                    umma_commit(bar_base + (geom.stages + st) * 8);
                     ++kpos;
-                    if (it + 1 == n_it || kpos == upt) {                            // the segment is complete
-                        umma_commit(bar_acc + 8 * sg);
-                        committed = sg + 1;
+                    const bool complete = it + 1 == n_it || kpos == upt;            // the segment is
+                    if (elect_one()) {
+                        for (int c = 0; c < p.kc; ++c) {
+                            const uint64_t da = smem_desc_sw128(wa + c * kWTileBytes);
+                            const uint64_t db = smem_desc_sw128(xa + c * x_tile_bytes);
+#pragma unroll
+                            for (int kk = 0; kk < kBK / kUmmaK; ++kk)
+                                umma_bf16(acc, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc, !fresh || (c | kk) != 0);
+                        }
+                        umma_commit(bar_base + (geom.stages + st) * 8);
+                        if (complete) umma_commit(bar_acc + 8 * sg);
                     }
+                    __syncwarp();
+                    if (complete) committed = sg + 1;
                     if (kpos == upt) {
                         kpos = 0;
                         ++sg;
@@ -742,9 +757,12 @@ k_decode_fused(const __grid_constant__ DecodeMaps maps, const __grid_constant__ 
                         ++round;
                     }
                 }
-                if (tr_main) FUSED_STAMP(p, 32, 2);
-                for (int sg = committed; sg < nseg; ++sg) umma_commit(bar_acc + 8 * sg);   // only after a failed wait
-                if (!ok) flag_error(p, 2, 200);
+                if (lane == 0 && tr_main) FUSED_STAMP(p, 32, 2);
+                for (int sg = committed; sg < nseg; ++sg) {                          // only after a failed wait
+                    if (elect_one()) umma_commit(bar_acc + 8 * sg);
+                    __syncwarp();
+                }
+                if (!ok && lane == 0) flag_error(p, 2, 200);
             }
         } else {
             // Which rows of which tile this CTA finishes: tile `t` is shared by the CTAs owner(first unit) ..

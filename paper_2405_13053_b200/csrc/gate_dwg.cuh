@@ -49,7 +49,7 @@ k_gate_dwg_tc(const __grid_constant__ CUtensorMap tmX, const GateDwgParams p) {
     const uint32_t bar_acc = bar_free + kDwgStages * 8;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(ring_ptr + kDwgStages * kStage + (3 * kDwgStages + 1) * 8);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_id(), lane = threadIdx.x & 31;
     const int col0 = blockIdx.x * kDwgCols;
     const int blocks = (p.T + kDwgTok - 1) / kDwgTok;
     const int b0 = (int)((long long)blocks * blockIdx.y / gridDim.y), nb = (int)((long long)blocks * (blockIdx.y + 1) / gridDim.y) - b0;
@@ -75,47 +75,54 @@ k_gate_dwg_tc(const __grid_constant__ CUtensorMap tmX, const GateDwgParams p) {
 
     bool acc_ok = true;
     if (warp == 0) {
-        if (lane == 0) {
+        {
             bool ok = true;
-            for (int i = 0; i < nb && ok; ++i) {
+            for (int i = 0; i < nb; ++i) {
                 const int s = i % kDwgStages, round = i / kDwgStages;
-                if (round > 0) ok = mbar_wait(bar_free + s * 8, (round & 1) ^ 1);
+                if (round > 0) ok = mbar_wait_warp(bar_free + s * 8, (round & 1) ^ 1);
                 if (!ok) break;
-                mbar_expect_tx(bar_x + s * 8, kDwgXBytes);
+                if (elect_one()) {
+                    mbar_expect_tx(bar_x + s * 8, kDwgXBytes);
 #pragma unroll
-                for (int c = 0; c < kDwgCols / 64; ++c)              // (columns beyond d_in and tokens beyond T read as zero)
-                    tma_load_2d(ring + s * kStage + c * (kDwgTok * 128), &tmX, col0 + c * 64, (b0 + i) * kDwgTok, bar_x + s * 8);
+                    for (int c = 0; c < kDwgCols / 64; ++c)              // (columns beyond d_in and tokens beyond T read as zero)
+                        tma_load_2d(ring + s * kStage + c * (kDwgTok * 128), &tmX, col0 + c * 64, (b0 + i) * kDwgTok, bar_x + s * 8);
+                }
+                __syncwarp();
             }
-            if (!ok) {
+            if (!ok && lane == 0) {
                 atomicExch(p.status, 1);
                 atomicExch(p.status + 1, 4100);
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        {
             // A = L (K-major), B = x (MN-major: instruction descriptor bit 16), N = 64 columns
             const uint32_t idesc = instr_desc_bf16(64) | (1u << 16);
             bool ok = true;
             for (int i = 0; i < nb; ++i) {
                 const int s = i % kDwgStages, round = i / kDwgStages;
-                ok = mbar_wait(bar_x + s * 8, round & 1) && mbar_wait(bar_l + s * 8, round & 1);
+                ok = mbar_wait_warp(bar_x + s * 8, round & 1) && mbar_wait_warp(bar_l + s * 8, round & 1);
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t xa = ring + s * kStage, la = xa + kDwgXBytes;
                 const uint64_t da = smem_desc_sw128(la);
+                if (elect_one()) {
 #pragma unroll
-                for (int kk = 0; kk < kDwgTok / kUmmaK; ++kk)
+                    for (int kk = 0; kk < kDwgTok / kUmmaK; ++kk)
 #pragma unroll
-                    for (int c = 0; c < kDwgCols / 64; ++c) {
-                        // 16 tokens = two groups of 8 rows of 128 bytes, 1024 bytes apart
-                        const uint64_t db = (smem_desc_sw128(xa + c * (kDwgTok * 128) + kk * 2048) & ~((uint64_t)0x3FFF << 16)) |
-                                            ((uint64_t)(1024 >> 4) << 16);
-                        umma_bf16(tmem_base + c * 64, da + (uint64_t)(kk * 2), db, idesc, (i | kk) != 0);
-                    }
-                umma_commit(bar_free + s * 8);
+                        for (int c = 0; c < kDwgCols / 64; ++c) {
+                            // 16 tokens = two groups of 8 rows of 128 bytes, 1024 bytes apart
+                            const uint64_t db = (smem_desc_sw128(xa + c * (kDwgTok * 128) + kk * 2048) & ~((uint64_t)0x3FFF << 16)) |
+                                                ((uint64_t)(1024 >> 4) << 16);
+                            umma_bf16(tmem_base + c * 64, da + (uint64_t)(kk * 2), db, idesc, (i | kk) != 0);
+                        }
+                    umma_commit(bar_free + s * 8);
+                }
+                __syncwarp();
             }
-            umma_commit(bar_acc);
-            if (!ok) {
+            if (elect_one()) umma_commit(bar_acc);
+            __syncwarp();
+            if (!ok && lane == 0) {
                 atomicExch(p.status, 1);
                 atomicExch(p.status + 2, 4200);
             }

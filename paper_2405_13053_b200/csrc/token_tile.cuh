@@ -136,8 +136,8 @@ k_token_tile(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CU
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem_raw + (ring - raw) + (2 * p.stages + 1) * 8);
     const uint32_t data = ring + 1024u;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int rank = (int)cluster_rank();
+    const int warp = warp_id(), lane = threadIdx.x & 31;
+    const int rank = __shfl_sync(0xFFFFFFFFu, (int)cluster_rank(), 0);
     const int tok0 = (blockIdx.x / S) * kTokTile;
     const int a_row0 = (int)blockIdx.y * p.a_group * p.r;
     const int k0 = p.ksteps * rank / S, niter = p.ksteps * (rank + 1) / S - k0;
@@ -165,46 +165,53 @@ k_token_tile(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CU
         if (!p.late_wait) asm volatile("griddepcontrol.wait;" ::: "memory");
         if (lane == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         if (p.clear_status && blockIdx.x == 0) p.status[lane] = p.status[lane + 32] = 0;
-        if (lane == 0) {
+        {
             bool ok = true;
-            for (int i = 0; i < niter && ok; ++i) {
-                const int s = i % p.stages, round = i / p.stages;
-                if (round > 0) ok = mbar_wait(bar_base + (p.stages + s) * 8, (round & 1) ^ 1);
+            for (int i = 0, s = 0, round = 0; i < niter; ++i) {
+                if (round > 0) ok = mbar_wait_warp(bar_base + (p.stages + s) * 8, (round & 1) ^ 1);
                 if (!ok) break;
                 const uint32_t full = bar_base + s * 8, dst = data + s * p.stage_bytes;
                 const int c0 = (k0 + i) * kBK;
-                mbar_expect_tx(full, kTokXBytes + (uint32_t)(p.gate_box + p.a_copies * p.a_box) * 128u);
-                tma_load_2d(dst, &tmX, c0, tok0, full);
-                if (p.gate_box) tma_load_2d(dst + kTokXBytes, &tmG, c0, 0, full);
-                for (int q = 0; q < p.a_copies; ++q)
-                    tma_load_2d(dst + kTokXBytes + (uint32_t)(p.gate_box + q * p.a_box) * 128u, &tmA, c0, a_row0 + q * p.a_box, full);
+                if (elect_one()) {
+                    mbar_expect_tx(full, kTokXBytes + (uint32_t)(p.gate_box + p.a_copies * p.a_box) * 128u);
+                    tma_load_2d(dst, &tmX, c0, tok0, full);
+                    if (p.gate_box) tma_load_2d(dst + kTokXBytes, &tmG, c0, 0, full);
+                    for (int q = 0; q < p.a_copies; ++q)
+                        tma_load_2d(dst + kTokXBytes + (uint32_t)(p.gate_box + q * p.a_box) * 128u, &tmA, c0, a_row0 + q * p.a_box, full);
+                }
+                __syncwarp();
+                if (++s == p.stages) s = 0, ++round;
             }
-            if (!ok && p.status) {
+            if (!ok && lane == 0 && p.status) {
                 atomicExch(p.status, 1);
                 atomicExch(p.status + 1, 3100);
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        {
             bool ok = true;
-            for (int i = 0; i < niter; ++i) {
-                const int s = i % p.stages, round = i / p.stages;
-                ok = mbar_wait(bar_base + s * 8, round & 1);
+            for (int i = 0, s = 0, round = 0; i < niter; ++i) {
+                ok = mbar_wait_warp(bar_base + s * 8, round & 1);
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t xa = data + s * p.stage_bytes, wa = xa + kTokXBytes;
                 const uint64_t da = smem_desc_sw128(xa);
-                for (int tile = 0; tile < p.rounds; ++tile) {
-                    const uint64_t db = smem_desc_sw128(wa + (uint32_t)tile * kTokCols * 128u);
-                    const uint32_t idesc = instr_desc_bf16(p.cols[tile]);
+                if (elect_one()) {
+                    for (int tile = 0; tile < p.rounds; ++tile) {
+                        const uint64_t db = smem_desc_sw128(wa + (uint32_t)tile * kTokCols * 128u);
+                        const uint32_t idesc = instr_desc_bf16(p.cols[tile]);
 #pragma unroll
-                    for (int kk = 0; kk < kBK / kUmmaK; ++kk)
-                        umma_bf16(tmem_base + tile * kTokCols, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc, (i | kk) != 0);
+                        for (int kk = 0; kk < kBK / kUmmaK; ++kk)
+                            umma_bf16(tmem_base + tile * kTokCols, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc, (i | kk) != 0);
+                    }
+                    umma_commit(bar_base + (p.stages + s) * 8);
                 }
-                umma_commit(bar_base + (p.stages + s) * 8);
+                __syncwarp();
+                if (++s == p.stages) s = 0, ++round;
             }
-            umma_commit(bar_acc);
-            if (!ok && p.status) {
+            if (elect_one()) umma_commit(bar_acc);
+            __syncwarp();
+            if (!ok && lane == 0 && p.status) {
                 atomicExch(p.status, 1);
                 atomicExch(p.status + 2, 3200);
             }

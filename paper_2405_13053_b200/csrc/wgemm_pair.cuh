@@ -117,8 +117,8 @@ k_wgemm_pair(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CU
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(ring_ptr + ring_bytes + (2 * p.stages + 3) * 8);
     uint8_t* epi = ring_ptr + ring_bytes + p.epi_off;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t rank = cluster_rank();
+    const int warp = warp_id(), lane = threadIdx.x & 31;
+    const uint32_t rank = __shfl_sync(0xFFFFFFFFu, cluster_rank(), 0);
     const bool leader = rank == 0;
     // Which tile this pair takes.  Pairs are dispatched in the order of p = blockIdx.y * (gridDim.x / 2) + blockIdx.x / 2;
     // taken row-major (all row pairs of one token tile, then the next token tile) every token tile streams the whole of
@@ -166,61 +166,72 @@ k_wgemm_pair(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CU
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer (both CTAs)
-        if (lane == 0) {
+        {
             bool ok = true;
             int issued = 0;
-            for (int i = 0; i < niter; ++i) {
-                const int s = i % p.stages, round = i / p.stages;
-                if (round > 0) ok = mbar_wait(bar_base + (p.stages + s) * 8, (round & 1) ^ 1);
+            for (int i = 0, s = 0, round = 0; i < niter; ++i) {
+                if (round > 0) ok = mbar_wait_warp(bar_base + (p.stages + s) * 8, (round & 1) ^ 1);
                 if (!ok) break;
                 const uint32_t full = bar_base + s * 8;
                 const uint32_t full_leader = map_to_cta(full, 0);
                 const uint32_t dst = ring + s * kStageBytes;
-                if (leader) mbar_expect_tx(full, 2 * kStageBytes);
-                tma_load_2d_pair(dst, &tmW, i * kBK, tile_m * kBM, full_leader);
-                tma_load_2d_pair(dst + kWTileBytes, &tmX, i * kBK, tokh, full_leader);
+                if (elect_one()) {
+                    if (leader) mbar_expect_tx(full, 2 * kStageBytes);
+                    tma_load_2d_pair(dst, &tmW, i * kBK, tile_m * kBM, full_leader);
+                    tma_load_2d_pair(dst + kWTileBytes, &tmX, i * kBK, tokh, full_leader);
+                }
+                __syncwarp();
                 issued = i + 1;
+                if (++s == p.stages) s = 0, ++round;
             }
-            if (!ok) {
+            if (!ok && lane == 0) {
                 atomicExch(p.status, 1);
                 atomicExch(p.status + 1, 1100 + issued);
             }
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer (leader only)
-        if (lane == 0 && leader) {
+        if (leader) {
             const uint32_t idesc = instr_desc_bf16_pair();
             bool ok = true;
-            for (int i = 0; i < niter; ++i) {
-                const int s = i % p.stages, round = i / p.stages;
-                ok = mbar_wait(bar_base + s * 8, round & 1);
+            for (int i = 0, s = 0, round = 0; i < niter; ++i) {
+                ok = mbar_wait_warp(bar_base + s * 8, round & 1);
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t wa = ring + s * kStageBytes, xa = wa + kWTileBytes;
                 const uint64_t da = smem_desc_sw128(wa), db = smem_desc_sw128(xa);
+                if (elect_one()) {
 #pragma unroll
-                for (int kk = 0; kk < kBK / kUmmaK; ++kk)
-                    umma_bf16_pair(tmem_base, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc, (i | kk) != 0);
-                umma_commit_pair(bar_base + (p.stages + s) * 8);  // both rings may refill this stage
+                    for (int kk = 0; kk < kBK / kUmmaK; ++kk)
+                        umma_bf16_pair(tmem_base, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc, (i | kk) != 0);
+                    umma_commit_pair(bar_base + (p.stages + s) * 8);   // both rings may refill this stage
+                }
+                __syncwarp();
+                if (++s == p.stages) s = 0, ++round;
             }
-            umma_commit_pair(bar_main);                            // both rings are idle
+            if (elect_one()) umma_commit_pair(bar_main);           // both rings are idle
+            __syncwarp();
             // LoRA expand as a K extension of the same accumulation, round by round: rb/2 MMAs of K = 16 (two
             // blocks of 8 expand columns) over un-swizzled core matrices, 2 KB per block and operand
             const int rounds = (p.nblk + p.rb - 1) / p.rb;
             for (int rho = 0; rho < rounds && ok; ++rho) {
-                ok = mbar_wait_cluster(bar_us, rho & 1);           // both CTAs have staged this round's operands
+                ok = __all_sync(0xFFFFFFFFu, mbar_wait_cluster(bar_us, rho & 1));   // both CTAs have staged this round's operands
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t slab_a = smem_u32(epi + p.slab_off), us_a = ring;
                 const uint32_t ka = kBM * 16, kb = kPairHalf * 16;   // bytes from one block to the next
                 const int nb = min(p.rb, (p.nblk - rho * p.rb + 1) / 2 * 2);
-                for (int m = 0; m < nb / 2; ++m)
-                    umma_bf16_pair(tmem_base, smem_desc_plain(slab_a + 2 * m * ka, ka, 128),
-                                   smem_desc_plain(us_a + 2 * m * kb, kb, 128), idesc, (niter | rho | m) != 0);
-                if (rho + 1 < rounds) umma_commit_pair(bar_main);  // staging buffers free for the next round
+                if (elect_one()) {
+                    for (int m = 0; m < nb / 2; ++m)
+                        umma_bf16_pair(tmem_base, smem_desc_plain(slab_a + 2 * m * ka, ka, 128),
+                                       smem_desc_plain(us_a + 2 * m * kb, kb, 128), idesc, (niter | rho | m) != 0);
+                    if (rho + 1 < rounds) umma_commit_pair(bar_main);  // staging buffers free for the next round
+                }
+                __syncwarp();
             }
-            umma_commit_pair(bar_acc);                             // accumulators complete in both CTAs
-            if (!ok) {
+            if (elect_one()) umma_commit_pair(bar_acc);             // accumulators complete in both CTAs
+            __syncwarp();
+            if (!ok && lane == 0) {
                 atomicExch(p.status, 1);
                 atomicExch(p.status + 2, 1200);
             }
@@ -371,8 +382,8 @@ k_stacked_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const uint32_t bar_acc = bar_base + 2 * p.stages * 8;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(ring_ptr + ring_bytes + (2 * p.stages + 1) * 8);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t rank = cluster_rank();
+    const int warp = warp_id(), lane = threadIdx.x & 31;
+    const uint32_t rank = __shfl_sync(0xFFFFFFFFu, cluster_rank(), 0);
     const bool leader = rank == 0;
     const int tile = (blockIdx.x >> 1) * 2 + (int)rank;           // own 128 rows of the stacked matrix
     const int tok0 = blockIdx.y * kPairTokens;
@@ -404,7 +415,7 @@ k_stacked_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(tmem_slot);
 
     if (warp == 0) {
-        if (lane == 0) {
+        {
             // Own tile of the stacked matrix: rows of A (the last A tile through the map whose box stops at A's
             // last row when Wg follows in the same tile), rows of Wg, or nothing but zero fill (a tile past
             // the end reads A out of range).  Every stage is 16 KB of weights + 16 KB of tokens whatever the tile.
@@ -413,43 +424,50 @@ k_stacked_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             const CUtensorMap* mA = merged_tail ? &tmAt : &tmA;
             bool ok = true;
             int issued = 0;
-            for (int i = 0; i < niter; ++i) {
-                const int s = i % p.stages, round = i / p.stages;
-                if (round > 0) ok = mbar_wait(bar_base + (p.stages + s) * 8, (round & 1) ^ 1);
+            for (int i = 0, s = 0, round = 0; i < niter; ++i) {
+                if (round > 0) ok = mbar_wait_warp(bar_base + (p.stages + s) * 8, (round & 1) ^ 1);
                 if (!ok) break;
                 const uint32_t full = bar_base + s * 8;
                 const uint32_t full_leader = map_to_cta(full, 0);
                 const uint32_t dst = ring + s * kStageBytes;
                 const int c0 = (ks0 + i) * kBK;
-                if (leader) mbar_expect_tx(full, 2 * kStageBytes);
-                if (has_a) tma_load_2d_pair(dst, mA, c0, tile * kBM, full_leader);
-                if (tile == p.gate_tile) tma_load_2d_pair(dst + (uint32_t)p.gate_row0 * 128u, &tmG, c0, 0, full_leader);
-                tma_load_2d_pair(dst + kWTileBytes, &tmX, c0, tokh, full_leader);
+                if (elect_one()) {
+                    if (leader) mbar_expect_tx(full, 2 * kStageBytes);
+                    if (has_a) tma_load_2d_pair(dst, mA, c0, tile * kBM, full_leader);
+                    if (tile == p.gate_tile) tma_load_2d_pair(dst + (uint32_t)p.gate_row0 * 128u, &tmG, c0, 0, full_leader);
+                    tma_load_2d_pair(dst + kWTileBytes, &tmX, c0, tokh, full_leader);
+                }
+                __syncwarp();
                 issued = i + 1;
+                if (++s == p.stages) s = 0, ++round;
             }
-            if (!ok) {
+            if (!ok && lane == 0) {
                 atomicExch(p.status, 1);
                 atomicExch(p.status + 1, 2100 + issued);
             }
         }
     } else if (warp == 1) {
-        if (lane == 0 && leader) {
+        if (leader) {
             const uint32_t idesc = instr_desc_bf16_pair();
             bool ok = true;
-            for (int i = 0; i < niter; ++i) {
-                const int s = i % p.stages, round = i / p.stages;
-                ok = mbar_wait(bar_base + s * 8, round & 1);
+            for (int i = 0, s = 0, round = 0; i < niter; ++i) {
+                ok = mbar_wait_warp(bar_base + s * 8, round & 1);
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t wa = ring + s * kStageBytes, xa = wa + kWTileBytes;
                 const uint64_t da = smem_desc_sw128(wa), db = smem_desc_sw128(xa);
+                if (elect_one()) {
 #pragma unroll
-                for (int kk = 0; kk < kBK / kUmmaK; ++kk)
-                    umma_bf16_pair(tmem_base, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc, (i | kk) != 0);
-                umma_commit_pair(bar_base + (p.stages + s) * 8);
+                    for (int kk = 0; kk < kBK / kUmmaK; ++kk)
+                        umma_bf16_pair(tmem_base, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc, (i | kk) != 0);
+                    umma_commit_pair(bar_base + (p.stages + s) * 8);
+                }
+                __syncwarp();
+                if (++s == p.stages) s = 0, ++round;
             }
-            umma_commit_pair(bar_acc);
-            if (!ok) {
+            if (elect_one()) umma_commit_pair(bar_acc);
+            __syncwarp();
+            if (!ok && lane == 0) {
                 atomicExch(p.status, 1);
                 atomicExch(p.status + 2, 2200);
             }

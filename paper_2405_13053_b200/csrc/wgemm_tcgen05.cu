@@ -498,9 +498,9 @@ k_wgemm(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__ CUtens
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(ring_ptr + ring_bytes + (2 * p.stages + 3) * 8);
     uint8_t* epi = ring_ptr + ring_bytes + p.epi_off;             // staging of the LoRA operands
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_id(), lane = threadIdx.x & 31;
     const int S = p.splits;
-    const int split = (int)cluster_rank();
+    const int split = __shfl_sync(0xFFFFFFFFu, (int)cluster_rank(), 0);
     const int tile_m = p.row_tile0 + blockIdx.x / S;
     const int tok0 = p.tok_base + blockIdx.y * p.BN;
     const int ntok = min(p.BN, p.T - tok0);
@@ -541,72 +541,83 @@ k_wgemm(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__ CUtens
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
-        if (lane == 0) {
+        {
             const bool second = tile_m >= p.split_tile;
             const CUtensorMap* tmW = second ? &tmW1 : &tmW0;
             const CUtensorMap* tmT = second_x ? &tmY : &tmX;
             const int row0 = (second ? tile_m - p.split_tile : tile_m) * kBM;
             int issued = 0;
             bool ok = true;
-            for (int i = 0; i < niter; ++i) {
-                const int s = i % p.stages, round = i / p.stages;
-                if (round > 0) ok = mbar_wait(bar_base + (p.stages + s) * 8, (round & 1) ^ 1);
+            for (int i = 0, s = 0, round = 0; i < niter; ++i) {
+                if (round > 0) ok = mbar_wait_warp(bar_base + (p.stages + s) * 8, (round & 1) ^ 1);
                 if (!ok) break;
                 const uint32_t full = bar_base + s * 8;
                 const uint32_t dst = ring + s * stage_bytes;
                 const int kstep = ks0 + i * p.kc;
-                mbar_expect_tx(full, stage_bytes);
-                if (p.maps3d) {      // one instruction per operand brings kc consecutive 64-element chunks
-                    tma_load_3d(dst, tmW, 0, row0, kstep, full);
-                    tma_load_3d(dst + p.kc * kWTileBytes, tmT, 0, tok0, kstep, full);
-                } else {
-                    tma_load_2d(dst, tmW, kstep * kBK, row0, full);
-                    tma_load_2d(dst + kWTileBytes, tmT, kstep * kBK, tok0, full);
+                if (elect_one()) {
+                    mbar_expect_tx(full, stage_bytes);
+                    if (p.maps3d) {      // one instruction per operand brings kc consecutive 64-element chunks
+                        tma_load_3d(dst, tmW, 0, row0, kstep, full);
+                        tma_load_3d(dst + p.kc * kWTileBytes, tmT, 0, tok0, kstep, full);
+                    } else {
+                        tma_load_2d(dst, tmW, kstep * kBK, row0, full);
+                        tma_load_2d(dst + kWTileBytes, tmT, kstep * kBK, tok0, full);
+                    }
                 }
+                __syncwarp();
                 issued = i + 1;
+                if (++s == p.stages) s = 0, ++round;
             }
-            if (!ok) {
+            if (!ok && lane == 0) {
                 atomicExch(p.status, 1);
                 atomicExch(p.status + 1, 100 + issued);
             }
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        {
             const uint32_t idesc = instr_desc_bf16(p.BN);
             bool ok = true;
-            for (int i = 0; i < niter; ++i) {
-                const int s = i % p.stages, round = i / p.stages;
-                ok = mbar_wait(bar_base + s * 8, round & 1);
+            for (int i = 0, s = 0, round = 0; i < niter; ++i) {
+                ok = mbar_wait_warp(bar_base + s * 8, round & 1);
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t wa = ring + s * stage_bytes, xa = wa + p.kc * kWTileBytes;
-                for (int c = 0; c < p.kc; ++c) {
-                    const uint64_t da = smem_desc_sw128(wa + c * kWTileBytes);
-                    const uint64_t db = smem_desc_sw128(xa + c * x_tile_bytes);
+                if (elect_one()) {
+                    for (int c = 0; c < p.kc; ++c) {
+                        const uint64_t da = smem_desc_sw128(wa + c * kWTileBytes);
+                        const uint64_t db = smem_desc_sw128(xa + c * x_tile_bytes);
 #pragma unroll
-                    for (int kk = 0; kk < kBK / kUmmaK; ++kk)
-                        umma_bf16(tmem_base, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc, (i | c | kk) != 0);
+                        for (int kk = 0; kk < kBK / kUmmaK; ++kk)
+                            umma_bf16(tmem_base, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc, (i | c | kk) != 0);
+                    }
+                    umma_commit(bar_base + (p.stages + s) * 8);   // stage reusable once these MMAs have read it
                 }
-                umma_commit(bar_base + (p.stages + s) * 8);   // stage reusable once these MMAs have read it
+                __syncwarp();
+                if (++s == p.stages) s = 0, ++round;
             }
             if (p.lora_mma && ok) {
                 // LoRA expand as a K extension of the same accumulation: na/2 MMAs of K = 16 (two adapters)
-                umma_commit(bar_main);
-                ok = mbar_wait(bar_us, 0);
+                if (elect_one()) umma_commit(bar_main);
+                __syncwarp();
+                ok = mbar_wait_warp(bar_us, 0);
                 if (ok) {
                     tc_fence_after();
                     const uint32_t slab_a = smem_u32(epi + p.slab_off);
                     const uint32_t us_a = p.us_in_ring ? ring : smem_u32(epi + p.us_off);
                     const uint32_t ka = kBM * 16, kb = p.BN * 16;      // bytes from one adapter to the next
-                    for (int m = 0; m < p.na / 2; ++m)
-                        umma_bf16(tmem_base, smem_desc_plain(slab_a + 2 * m * ka, ka, 128),
-                                  smem_desc_plain(us_a + 2 * m * kb, kb, 128), idesc, (niter | m) != 0);
+                    if (elect_one()) {
+                        for (int m = 0; m < p.na / 2; ++m)
+                            umma_bf16(tmem_base, smem_desc_plain(slab_a + 2 * m * ka, ka, 128),
+                                      smem_desc_plain(us_a + 2 * m * kb, kb, 128), idesc, (niter | m) != 0);
+                    }
+                    __syncwarp();
                 }
             }
-            umma_commit(bar_acc);                              // accumulators complete
-            METEORA_STAMP(p, 1);                                // all MMAs issued
-            if (!ok) {
+            if (elect_one()) umma_commit(bar_acc);             // accumulators complete
+            __syncwarp();
+            if (lane == 0) METEORA_STAMP(p, 1);                 // all MMAs issued
+            if (!ok && lane == 0) {
                 atomicExch(p.status, 1);
                 atomicExch(p.status + 2, 200);
             }
@@ -1463,7 +1474,7 @@ static PersistPlan make_persist_plan(const meteora_shape_t& s, const int* d_outs
         if (persist_us_pitch(sm) == 0) return pp;
         pp.tiles += ((d_outs[m] + kBM - 1) / kBM + 1) / 2 * pp.tok_tiles;
     }
-    if (tn.persist < 2 && pp.tiles * 4 < sm_count()) return pp;
+    if (tn.persist < 2 && (pp.tiles * 4 < sm_count() || (s.T <= 128 && s.d_in < 1024))) return pp;
     if (with_routing) {
         // [Wg; A] in 128-row tiles: Wg padded to whole 32 rows (a warp's TMEM lanes), then A, padded to whole MMAs of the expand
         pp.gate_rows = (s.N + 31) / 32 * 32;
