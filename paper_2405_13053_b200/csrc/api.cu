@@ -121,9 +121,10 @@ static int forward_device(const void* x, const void* W0, const void* A, const vo
         }
         tuning().fused_refused += 1;   // the cluster launch was refused: the streamed kernel takes the call
     }
-    if (decode_stream_supported(s)) {
+    const GroupModule gm = {W0, A, B, Wg, y, s.d_out, ws};
+    if (decode_stream_supported(s, &s.d_out, 1)) {
         if (timed) cudaEventRecord(pf.ev[2 * pf.used], st);
-        rc = launch_decode_stream(x, W0, A, B, Wg, s, ws, y, st);
+        rc = launch_decode_stream(x, &gm, 1, s, ws.status, ws.part_g, ws.tile_ctr, st);
         if (timed) cudaEventRecord(pf.ev[2 * pf.used++ + 1], st);
         return rc;
     }
@@ -137,7 +138,6 @@ static int forward_device(const void* x, const void* W0, const void* A, const vo
         tuning().fused_refused += 1;   // the cooperative launch was refused (not all CTAs can be resident): use the chain
     }
     if (persist_forward_supported(s, &s.d_out, 1)) {
-        const GroupModule gm = {W0, A, B, Wg, y, s.d_out, ws};
         if (timed) cudaEventRecord(pf.ev[2 * pf.used], st);
         rc = launch_persist_forward(x, &gm, 1, s, ws.status, ws.tile_ctr, st);
         if (rc != kLaunchRefused) {
@@ -270,7 +270,7 @@ size_t meteora_group_workspace_bytes(const meteora_shape_t* shape, const int* d_
 int meteora_group_plan(const meteora_shape_t* shape, const int* d_out, int n_modules) {
     const int rc = check_group(shape, d_out, n_modules);
     if (rc != METEORA_OK) return rc;
-    return n_modules > 1 && (decode_group_supported(*shape, d_out, n_modules) || persist_forward_supported(*shape, d_out, n_modules)) ? 1 : 0;
+    return n_modules > 1 && (decode_stream_supported(*shape, d_out, n_modules) || decode_group_supported(*shape, d_out, n_modules) || persist_forward_supported(*shape, d_out, n_modules)) ? 1 : 0;
 }
 
 int meteora_group_workspace_routing(const meteora_shape_t* shape, const int* d_out, int n_modules, int module,
@@ -306,16 +306,16 @@ int meteora_linear_forward_group(const void* x, const void* const* W0, const voi
         gw.mod[m].status = gw.mod[0].status;
         gw.mod[m].tile_ctr = gw.mod[0].tile_ctr;
     }
+    GroupModule gm[kMaxGroupModules];
+    for (int m = 0; m < n_modules; ++m) gm[m] = GroupModule{W0[m], A[m], B[m], Wg[m], y[m], d_out[m], gw.mod[m]};
+    if (n_modules > 1 && decode_stream_supported(*shape, d_out, n_modules))
+        return launch_decode_stream(x, gm, n_modules, *shape, gw.mod[0].status, gw.part_g, gw.mod[0].tile_ctr, st);
     if (n_modules > 1 && decode_group_supported(*shape, d_out, n_modules)) {
-        GroupModule gm[kMaxGroupModules];
-        for (int m = 0; m < n_modules; ++m) gm[m] = GroupModule{W0[m], A[m], B[m], Wg[m], y[m], d_out[m], gw.mod[m]};
         rc = launch_decode_group(x, gm, n_modules, *shape, gw.mod[0].status, gw.part_g, gw.mod[0].tile_ctr, st);
         if (rc != kLaunchRefused) return rc;
         tuning().fused_refused += 1;   // the cooperative launch was refused: one call per module instead
     }
     if (n_modules > 1 && persist_forward_supported(*shape, d_out, n_modules)) {
-        GroupModule gm[kMaxGroupModules];
-        for (int m = 0; m < n_modules; ++m) gm[m] = GroupModule{W0[m], A[m], B[m], Wg[m], y[m], d_out[m], gw.mod[m]};
         rc = launch_persist_forward(x, gm, n_modules, *shape, gw.mod[0].status, gw.mod[0].tile_ctr, st);
         if (rc != kLaunchRefused) return rc;
         tuning().fused_refused += 1;

@@ -127,6 +127,10 @@ struct GroupModule {
     int d_out;
     Workspace ws;       // topk_idx, topk_w, uw, u_all, ld_u, col_logits of this module
 };
+// Decode batch, weights streamed (decode_stream.cuh): one module or several that share x; part_g and tile_ctr serve all row tiles
+bool decode_stream_supported(const meteora_shape_t& s, const int* d_outs, int n_modules);
+int launch_decode_stream(const void* x, const GroupModule* mods, int n_modules, const meteora_shape_t& s, int32_t* status,
+                         float* part_g, int32_t* tile_ctr, cudaStream_t st);
 // Prefill: the whole layer of such modules on persistent pairs of SMs, one launch (wgemm_persist.cuh)
 bool persist_forward_supported(const meteora_shape_t& s, const int* d_outs, int n_modules);
 int launch_persist_forward(const void* x, const GroupModule* mods, int n_modules, const meteora_shape_t& s, int32_t* status,
@@ -142,9 +146,6 @@ int launch_decode_fused(const void* x, const void* W0, const void* A, const void
 bool decode_cluster_supported(const meteora_shape_t& s);
 int launch_decode_cluster(const void* x, const void* W0, const void* A, const void* B, const void* Wg,
                           const meteora_shape_t& s, const Workspace& ws, void* y, cudaStream_t st);
-bool decode_stream_supported(const meteora_shape_t& s);
-int launch_decode_stream(const void* x, const void* W0, const void* A, const void* B, const void* Wg,
-                         const meteora_shape_t& s, const Workspace& ws, void* y, cudaStream_t st);
 
 struct Tuning {
     int splits = 0;

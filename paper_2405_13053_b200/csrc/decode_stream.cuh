@@ -1,4 +1,5 @@
-// Whole MeteoRA linear forward (Eq. 2 with Eq. 3) for a decode batch of up to 128 tokens as ONE kernel launch
+// Whole MeteoRA linear forward (Eq. 2 with Eq. 3) for a decode batch of up to 256 tokens as ONE kernel launch,
+// of one module or of several that share x (q/k/v, gate/up),
 // whose CTAs are small enough that TWO launches fit on the SMs at the same time, so that under programmatic
 // dependent launch the next call's CTAs are resident while this call still runs.
 // Included by wgemm_tcgen05.cu after decode_fused.cuh, whose device helpers it shares.
@@ -21,6 +22,9 @@
 //     of the slice from the staged B rows and the routing (fetched the same way by the idle producer thread);
 //     then partials in CTA order + expand, one rounding to bf16, store.  The epilogue threads never poll a
 //     counter: warp 0 waits for the routing, warp 1 for the tile.
+// A group of modules is the same split over all modules' row tiles and stacked tiles: the modules' loads, barriers and tails
+// overlap instead of following one another (4096 -> 4096 + 1024 + 1024, measured per call at 1 / 64 / 128 / 192 tokens: 15.8 / 16.8 /
+// 21.2 / 26.6 us; module by module 29.1 / 33.8 / 38.8 / 45.8, on ranges of units across CTAs 20.3 / 23.8 / 29.1 / 37.3).
 // Every wait is bounded; on expiry the status word is set and the CTA drains.  The workspace counters are
 // re-armed by the last CTA to stop reading them.
 #pragma once
@@ -32,7 +36,9 @@ struct StreamParams {
     int stages, kc;            // main ring: stages of kc k-steps, [kc W tiles][kc x tiles]
     int aux_stages;            // aux ring: one k-step per stage
     int tmem_cols;
-    int N, r, k, d_out;
+    int N, r, k;
+    int n_mod;                 // modules that read the same x; their row tiles are numbered one after the other
+    DecodeModule mod[kMaxGroup];   // (u_part: [aux_slices][aux_tiles][T][128])
     int row_tiles, S, n_main;  // S main CTAs per 128-row tile of W0
     int n_aux, aux_tiles, aux_slices, a_tiles, gate_tile, gate_row0;
     int pf_main, pf_aux;       // stages beyond the ring whose weights are prefetched into L2 before the wait
@@ -40,12 +46,6 @@ struct StreamParams {
     int ring_bytes;            // ring of both kinds of CTA; later the landing area of the last step
     int bar_slots;             // ring slots the barrier area is laid out for
     float inv_tau;
-    const __nv_bfloat16* B;
-    __nv_bfloat16* y;
-    int32_t* topk_idx;
-    float* topk_w;
-    float* uw;
-    float* u_part;             // [aux_slices][aux_tiles][T][128] partial stacked shrink
     float* part_g;             // [row tile * S + j][BN * 128] partial accumulator tiles, cut into S row slices
     int32_t* ctr;              // [0] aux partials in, [1] routing published, [2] CTAs counted out
     int32_t* tile_ctr;         // [row tiles] partials delivered
@@ -216,9 +216,8 @@ __device__ __forceinline__ void row_slice(int j, int S, int& q0, int& nq) {
 // leader alone issues MMAs and releases stages by commits that arrive in both CTAs.  Aux CTAs work alone as before.
 template <bool kPair>
 __global__ void __launch_bounds__(kThreads, 2)
-k_decode_stream(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__ CUtensorMap tmA,
-                const __grid_constant__ CUtensorMap tmAt, const __grid_constant__ CUtensorMap tmG,
-                const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmX1,
+k_decode_stream(const __grid_constant__ DecodeMaps maps, const __grid_constant__ CUtensorMap tmX,
+                const __grid_constant__ CUtensorMap tmX1,
                 const StreamParams d) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
@@ -239,7 +238,7 @@ k_decode_stream(const __grid_constant__ CUtensorMap tmW0, const __grid_constant_
 
     const int warp = warp_id(), lane = threadIdx.x & 31;
     const bool is_aux = (int)blockIdx.x < d.n_aux;
-    const int n_active = d.aux_tiles * d.aux_slices;
+    const int per_mod = d.aux_tiles * d.aux_slices, n_active = d.n_mod * per_mod;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < 2 * d.bar_slots + 4; ++s) mbar_init(bar_base + s * 8, 1);
@@ -285,15 +284,18 @@ k_decode_stream(const __grid_constant__ CUtensorMap tmW0, const __grid_constant_
         // ================================================================== aux CTA
         const int aux_id = blockIdx.x;
         const bool active = aux_id < n_active;
-        const int tile = aux_id % d.aux_tiles, slice = aux_id / d.aux_tiles;
+        // (one module after the other; the tokens of a module are selected by its own CTAs)
+        const int am = active ? aux_id / per_mod : 0, local = aux_id - am * per_mod;
+        const DecodeModule& mo = d.mod[am];
+        const int tile = local % d.aux_tiles, slice = local / d.aux_tiles;
         const int ks0 = active ? (d.ksteps * slice) / d.aux_slices : 0;
         const int ks1 = active ? (d.ksteps * (slice + 1)) / d.aux_slices : 0;
         const int niter = ks1 - ks0;
         if (warp == 0) {
             if (active) {
                 // A's last tile has its own map (its box stops at A's last row when Wg follows in the same tile)
-                const CUtensorMap* mA = tile >= d.a_tiles ? nullptr : tile == d.a_tiles - 1 ? &tmAt : &tmA;
-                const CUtensorMap* mG = tile == d.gate_tile ? &tmG : nullptr;
+                const CUtensorMap* mA = tile >= d.a_tiles ? nullptr : tile == d.a_tiles - 1 ? &maps.At[am] : &maps.A[am];
+                const CUtensorMap* mG = tile == d.gate_tile ? &maps.G[am] : nullptr;
                 const uint32_t g_off = (uint32_t)d.gate_row0 * 128u;
                 const int pre = min(niter, d.aux_stages);
                 // weights first: they do not depend on the kernel ahead
@@ -376,7 +378,7 @@ k_decode_stream(const __grid_constant__ CUtensorMap tmW0, const __grid_constant_
                 // straight from registers: lane = row, a warp writes 128 contiguous bytes per token (the scratch holds
                 // BN token rows per tile, so nothing is predicated)
                 if (d.pdl) asm volatile("griddepcontrol.wait;" ::: "memory");
-                float* dst = d.u_part + (((size_t)slice * d.aux_tiles + tile) * d.T) * kBM + trow;
+                float* dst = mo.u_part + (((size_t)slice * d.aux_tiles + tile) * d.T) * kBM + trow;
                 for (int c0 = c_begin; c0 < c_end; c0 += 16) {
                     float v[16];
                     if (acc_ok && niter > 0) {
@@ -406,7 +408,7 @@ k_decode_stream(const __grid_constant__ CUtensorMap tmW0, const __grid_constant_
         if (active) {
             if (d.pdl) asm volatile("griddepcontrol.wait;" ::: "memory");     // every thread below touches the scratch
             if (threadIdx.x == 0) {
-                float* dst = d.u_part + (((size_t)slice * d.aux_tiles + tile) * d.T) * kBM;
+                float* dst = mo.u_part + (((size_t)slice * d.aux_tiles + tile) * d.T) * kBM;
                 if (!d.aux_plain) bulk_store_block(dst, ring, (uint32_t)d.T * kBM * 4u);
                 __threadfence();
                 atomicAdd(d.ctr + 0, 1);
@@ -416,15 +418,15 @@ k_decode_stream(const __grid_constant__ CUtensorMap tmW0, const __grid_constant_
             }
             // This CTA's share of the tokens: their rows of every partial tile into the idle ring (one bulk copy per
             // tile and slice, a token range is contiguous there), then a warp per token selects from shared memory.
-            const int t0 = d.T * aux_id / n_active, t1 = d.T * (aux_id + 1) / n_active, ntl = t1 - t0;
-            const uint32_t rows_bytes = (uint32_t)(n_active * ntl * kBM * 4);
+            const int t0 = d.T * local / per_mod, t1 = d.T * (local + 1) / per_mod, ntl = t1 - t0;
+            const uint32_t rows_bytes = (uint32_t)(per_mod * ntl * kBM * 4);
             __syncthreads();                                         // thread 0 has seen all partials; its staged tile has left the ring
             if (ntl > 0) {
                 // one copy per (slice, tile), each issued by a thread of its own (twenty issued by one thread took over a microsecond)
                 if (threadIdx.x == 0) mbar_expect_tx(bar_land, rows_bytes);
-                if ((int)threadIdx.x < n_active)
+                if ((int)threadIdx.x < per_mod)
                     bulk_load_block(ring + (uint32_t)((int)threadIdx.x * ntl * kBM * 4),
-                                    d.u_part + ((size_t)threadIdx.x * d.T + t0) * kBM, (uint32_t)(ntl * kBM * 4), bar_land);
+                                    mo.u_part + ((size_t)threadIdx.x * d.T + t0) * kBM, (uint32_t)(ntl * kBM * 4), bar_land);
                 bool ok = mbar_wait(bar_land, 0);
                 if (!ok && lane == 0) stream_flag_error(d, 4, 750);
                 ok = __all_sync(0xFFFFFFFFu, ok);                   // the selection is warp-collective
@@ -455,7 +457,7 @@ k_decode_stream(const __grid_constant__ CUtensorMap tmW0, const __grid_constant_
                 const int nwarps = kThreads / 32;
                 for (int tl = warp; tl < ntl && ok; tl += nwarps)
                     select_token_row(reinterpret_cast<const float*>(rows4 + tl * per_tok), d.gate_tile, d.gate_row0, t0 + tl, d.N,
-                                     d.r, d.k, d.inv_tau, lane, d.topk_idx, d.topk_w, d.uw);
+                                     d.r, d.k, d.inv_tau, lane, mo.topk_idx, mo.topk_w, mo.uw);
                 if (threadIdx.x == 0) STREAM_STAMP(7);
             }
             __syncthreads();
@@ -485,7 +487,10 @@ k_decode_stream(const __grid_constant__ CUtensorMap tmW0, const __grid_constant_
         const int nst = d.ksteps / d.kc;                             // stages of the whole contraction axis
         const int it0 = nst * j / S, it1 = nst * (j + 1) / S;
         const int n_it = it1 - it0;
-        const int row0 = tile * kBM;
+        const int wm = module_of_tile(d.mod, d.n_mod, tile);
+        const DecodeModule& mo = d.mod[wm];
+        const CUtensorMap* tmW0 = &maps.W0[wm];
+        const int row0 = (tile - mo.tile0) * kBM;
         int q0, nq;
         row_slice(j, S, q0, nq);
         const int cpa = d.r >> 3;
@@ -510,8 +515,8 @@ k_decode_stream(const __grid_constant__ CUtensorMap tmW0, const __grid_constant_
                     return kPair ? map_to_cta(local, 0) : local;
                 };
                 auto load_w = [&](uint32_t dst, int it, uint32_t bar) {
-                    if (kPair) tma_load_3d_pair(dst, &tmW0, 0, row0, it * d.kc, bar);
-                    else tma_load_3d(dst, &tmW0, 0, row0, it * d.kc, bar);
+                    if (kPair) tma_load_3d_pair(dst, tmW0, 0, row0, it * d.kc, bar);
+                    else tma_load_3d(dst, tmW0, 0, row0, it * d.kc, bar);
                 };
                 auto load_x = [&](uint32_t dst, int it, uint32_t bar) {
                     if (kPair) tma_load_3d_pair(dst, &tmX, 0, tok0, it * d.kc, bar);
@@ -525,7 +530,7 @@ k_decode_stream(const __grid_constant__ CUtensorMap tmW0, const __grid_constant_
                     __syncwarp();
                 }
                 for (int i = pre; i < min(n_it, pre + d.pf_main); ++i) {
-                    if (elect_one()) tma_prefetch_l2_3d(&tmW0, 0, row0, (it0 + i) * d.kc);
+                    if (elect_one()) tma_prefetch_l2_3d(tmW0, 0, row0, (it0 + i) * d.kc);
                     __syncwarp();
                 }
                 if (d.pdl) asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -564,8 +569,8 @@ k_decode_stream(const __grid_constant__ CUtensorMap tmW0, const __grid_constant_
                 if (!ok) stream_flag_error(d, 4, 800);
                 STREAM_STAMP(7);
                 mbar_expect_tx(bar_route, idx_bytes + uw_bytes);
-                bulk_load_block(ring + idx_off, d.topk_idx, idx_bytes, bar_route);
-                bulk_load_block(ring + uw_off, d.uw, uw_bytes, bar_route);
+                bulk_load_block(ring + idx_off, mo.topk_idx, idx_bytes, bar_route);
+                bulk_load_block(ring + uw_off, mo.uw, uw_bytes, bar_route);
                 if (atomicAdd_block(s_done, 1) == 1) stream_count_out(d);   // the CTA reads no workspace counter any more
                 mbar_wait(bar_route, 0);    // own copies have landed before the CTA may leave (the epilogue may have given up)
             }
@@ -634,7 +639,7 @@ k_decode_stream(const __grid_constant__ CUtensorMap tmW0, const __grid_constant_
             }
         } else {
             // B rows of this CTA's row slice for every adapter: weights, staged before the wait
-            if (live) stage_slab_rows(d.B, d.d_out, d.N, cpa, slab, row0 + 4 * q0, 4 * nq, etid);
+            if (live) stage_slab_rows(mo.B, mo.d_out, d.N, cpa, slab, row0 + 4 * q0, 4 * nq, etid);
             // Where this thread's accumulator row goes (worked out before the accumulator is ready): the accumulator
             // is cut into the S row slices, each stored [token][rows of the slice] so that the CTA that finishes a
             // slice fetches it as one contiguous block: the own slice straight into the landing area, the others to scratch.
@@ -751,8 +756,8 @@ k_decode_stream(const __grid_constant__ CUtensorMap tmW0, const __grid_constant_
                 acc.z += dl.z;
                 acc.w += dl.w;
                 const int o = row0 + (q0 + ql) * 4;
-                __nv_bfloat16* dst = d.y + (size_t)t * d.d_out + o;
-                if ((d.d_out & 3) == 0 && o + 3 < d.d_out) {
+                __nv_bfloat16* dst = mo.y + (size_t)t * mo.d_out + o;
+                if ((mo.d_out & 3) == 0 && o + 3 < mo.d_out) {
                     const __nv_bfloat162 lo = __floats2bfloat162_rn(acc.x, acc.y), hi = __floats2bfloat162_rn(acc.z, acc.w);
                     uint2 pk;
                     pk.x = *reinterpret_cast<const uint32_t*>(&lo);
@@ -762,7 +767,7 @@ k_decode_stream(const __grid_constant__ CUtensorMap tmW0, const __grid_constant_
                     const float f[4] = {acc.x, acc.y, acc.z, acc.w};
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
-                        if (o + i < d.d_out) dst[i] = __float2bfloat16_rn(f[i]);
+                        if (o + i < mo.d_out) dst[i] = __float2bfloat16_rn(f[i]);
                 }
             }
             if (etid == 0) STREAM_STAMP(10);

@@ -103,8 +103,11 @@ meteora_shape_t make_shape(int64_t T, int64_t d_in, int64_t d_out, int64_t N, in
 }
 
 at::Tensor zeroed(size_t bytes, const at::Tensor& like, const char* where) {
+    // (the header alone needs zeros: clearing all of it took 2 to 30 us of a decode call made without a workspace)
     if (bytes == 0) check(METEORA_ERR_INVALID_ARG, where);
-    return at::zeros({(int64_t)bytes}, at::TensorOptions().dtype(at::kByte).device(like.device()));
+    at::Tensor ws = empty({(int64_t)bytes}, at::kByte, like);
+    check(meteora_workspace_init(ws.data_ptr(), stream()), where);
+    return ws;
 }
 
 // A [T, k] tensor over 4-byte values inside `workspace`: shares its storage and version counter, as a view does.

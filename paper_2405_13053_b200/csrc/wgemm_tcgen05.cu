@@ -1429,7 +1429,7 @@ struct PersistPlan {
 // is whole adapters or a whole part of one) and more than 2048 columns stay with the kernel that stages them in rounds.
 int persist_us_pitch(const meteora_shape_t& s) {
     const int cols = (s.N * s.r + kBK - 1) / kBK * kBK, cpa = s.r / 8;
-    if (s.dtype != METEORA_BF16 || s.T <= 32 || s.d_in % 8 != 0 || s.d_out % 8 != 0 || s.r % 8 != 0 || cols > 2048) return 0;
+    if (s.dtype != METEORA_BF16 || s.T < 1 || s.d_in % 8 != 0 || s.d_out % 8 != 0 || s.r % 8 != 0 || cols > 2048) return 0;
     return cpa == 1 || cpa == 2 || cpa == 4 || cpa == 8 ? cols : 0;
 }
 
@@ -1969,15 +1969,49 @@ struct StreamPlan {
 constexpr int kStreamBarSlots = 16;
 constexpr size_t kTwoPerSmBytes = 113 * 1024;    // dynamic shared memory with which two CTAs share an SM
 
-static StreamPlan make_stream_plan_with(const meteora_shape_t& s, int aux_budget_forced) {
+// Whether the current device confirms that a CTA with all of an SM's shared memory is resident on each SM (without a device: no).
+// Asked above 128 tokens, where every CTA of the streamed kernel takes an SM for itself.
+static bool stream_resident() {
+    static std::atomic<int> cache[64];                           // 0: not asked yet, 1 no, 2 yes
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+        cudaGetLastError();
+        return false;
+    }
+    int have = cache[dev].load(std::memory_order_relaxed);
+    if (have == 0) {
+        int n = 0;
+        if (cudaFuncSetAttribute(k_decode_stream<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_decode_stream<false>, kThreads, 226 * 1024) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        have = n >= 1 ? 2 : 1;
+        cache[dev].store(have, std::memory_order_relaxed);
+    }
+    return have == 2;
+}
+
+static StreamPlan make_stream_plan_with(const meteora_shape_t& s, const int* d_outs, int G, int aux_budget_forced) {
     const Tuning& tn = tuning();
     StreamPlan sp = {};
     sp.why = 1;
     if (!tn.fused || !tn.stream || tn.simt_expand) return sp;
-    if (!tc_path_supported(s) || s.T > 128 || s.r % 8 != 0 || s.d_in % kBK != 0 || s.d_out <= 0) return sp;
+    if (!tc_path_supported(s) || s.T > 256 || s.r % 8 != 0 || s.d_in % kBK != 0) return sp;
     const int sms = std::min(sm_count(), 148);                   // the workspace holds partial tiles for 148 CTAs
     const int ksteps = s.d_in / kBK;
-    sp.row_tiles = (s.d_out + kBM - 1) / kBM;
+    size_t w0_bytes = 0;
+    for (int m = 0; m < G; ++m) {
+        meteora_shape_t sm = s;
+        sm.d_out = d_outs[m];
+        if (d_outs[m] <= 0 || !tc_path_supported(sm)) return sp;
+        sp.row_tiles += (d_outs[m] + kBM - 1) / kBM;
+        w0_bytes += (size_t)d_outs[m] * s.d_in * 2;
+    }
+    // Above 128 tokens the ring holds three to five stages and the landing area most of the shared memory, yet layers are faster
+    // here than on ranges of units, which keep those of up to 2 MB of W0 (us at 129 / 200 / 256 tokens: 4096 -> 4096 17.1 / 19.5 / 21.9 against 20.0 / 22.9 /
+    // 26.8, 2048 -> 2048 12.9 / 14.6 / 16.6 against 15.1 / 17.0 / 21.6, 14336 -> 4096 30.5 / 33.4 / 38.2 against 36.8 / 40.8 / 43.4).
+    if (s.T > 128 && ((w0_bytes <= ((size_t)2 << 20) && tn.stream < 2) || !stream_resident())) return sp;
     if (sp.row_tiles > kMaxFusedRowTiles) return sp;
     // stacked shrink: tiles of [A; Wg] (Wg behind A's last rows when the tile has room), slices of the contraction axis
     sp.a_tiles = (s.N * s.r + kBM - 1) / kBM;
@@ -1987,13 +2021,14 @@ static StreamPlan make_stream_plan_with(const meteora_shape_t& s, int aux_budget
     sp.gate_tile = sp.aux_tiles - 1;
     sp.gate_row0 = merged ? tail_rows : 0;
     sp.why = 2;
-    int aux_budget = std::max(20, 4 * sp.aux_tiles);
-    if (aux_budget_forced > 0) aux_budget = std::max(aux_budget_forced, sp.aux_tiles);
-    if (tn.aux_ctas > 0) aux_budget = std::max(tn.aux_ctas, sp.aux_tiles);
+    const int stacked = G * sp.aux_tiles;                        // tiles of all modules' stacked matrices
+    int aux_budget = std::max(20, 4 * stacked);
+    if (aux_budget_forced > 0) aux_budget = std::max(aux_budget_forced, stacked);
+    if (tn.aux_ctas > 0) aux_budget = std::max(tn.aux_ctas, stacked);
     aux_budget = std::min(aux_budget, sms - 8);
-    sp.aux_slices = std::min(std::min(aux_budget / sp.aux_tiles, ksteps), 16);
+    sp.aux_slices = std::min(std::min(aux_budget / stacked, ksteps), 16);
     if (sp.aux_slices < 1) return sp;
-    sp.n_aux = sp.aux_tiles * sp.aux_slices;
+    sp.n_aux = stacked * sp.aux_slices;
     sp.kc = 1;
     if (tn.kc > 0 && tn.kc <= 4 && ksteps % tn.kc == 0) sp.kc = tn.kc;
     const int nst = ksteps / sp.kc;
@@ -2002,7 +2037,7 @@ static StreamPlan make_stream_plan_with(const meteora_shape_t& s, int aux_budget
     // stage.  Measured at 4096 -> 4096: the main loop ends no earlier (8.6 against 8.3 us after the call ahead at 128
     // tokens, 8.4 against 8.0 at 64) and a call takes 18.1 against 16.9 us and 15.4 against 14.6: the loop waits for W0's
     // lines, not for the token tile, and the pair adds two cluster barriers.  Kept as a knob, off by default.
-    sp.pair = tn.pair_decode == 0 ? 0 : (s.T >= (tn.pair_decode >= 2 ? 17 : 64) ? 1 : 0);
+    sp.pair = tn.pair_decode == 0 || G > 1 ? 0 : (s.T >= (tn.pair_decode >= 2 ? 17 : 64) ? 1 : 0);
     const int tiles_padded = sp.pair ? (sp.row_tiles + 1) / 2 * 2 : sp.row_tiles;
     if (sp.pair) sp.n_aux = (sp.n_aux + 1) / 2 * 2;              // whole clusters of two
     int S = std::min(8, (sms - sp.n_aux) / tiles_padded);
@@ -2016,9 +2051,9 @@ static StreamPlan make_stream_plan_with(const meteora_shape_t& s, int aux_budget
     if (tn.aux_ctas == 0) {
         const int spare = sms - sp.n_main - sp.n_aux;
         const int full = std::min(ksteps, 16);
-        if (sp.aux_slices < full && sp.aux_slices + spare / sp.aux_tiles >= full) {
+        if (sp.aux_slices < full && sp.aux_slices + spare / stacked >= full) {
             sp.aux_slices = full;
-            sp.n_aux = sp.aux_tiles * sp.aux_slices;
+            sp.n_aux = stacked * sp.aux_slices;
             if (sp.pair) sp.n_aux = (sp.n_aux + 1) / 2 * 2;
         }
     }
@@ -2041,7 +2076,8 @@ static StreamPlan make_stream_plan_with(const meteora_shape_t& s, int aux_budget
     const size_t landing = parts + align_up(align_up((size_t)ntok * s.k * 4, 16), 128) + (size_t)ntok * s.k * s.r * 4;
     // an aux CTA stages its accumulator tile there, later its tokens' rows of every partial tile of the stacked shrink
     // (and the summed rows of those tokens behind them)
-    const size_t aux_rows = (size_t)(sp.n_aux + sp.aux_tiles) * ((s.T + sp.n_aux - 1) / sp.n_aux) * kBM * 4;
+    const int per_mod = sp.aux_tiles * sp.aux_slices;
+    const size_t aux_rows = (size_t)(per_mod + sp.aux_tiles) * ((s.T + per_mod - 1) / per_mod) * kBM * 4;
     const size_t ring_need = std::max(std::max(landing, (size_t)sp.BN * kBM * 4), aux_rows);
     const int n_it_max = (nst + S - 1) / S;
     const int nks_aux = (ksteps + sp.aux_slices - 1) / sp.aux_slices;
@@ -2053,7 +2089,6 @@ static StreamPlan make_stream_plan_with(const meteora_shape_t& s, int aux_budget
     // 4096 -> 1024 (8 MB) 10.3 / 10.3 at 1, 12.1 / 11.8 at 64; 4096 -> 14336 (117 MB) 30.3 / 26.7 at 1, 31.2 / 31.5 at 64;
     // 5120 -> 13824 (142 MB) 36.5 / 31.8 at 1.  So: two per SM for 16 - 56 MB of W0 and up to 32 tokens, else one.
     // (Knob stream: 2 or 4 always one per SM, 3 always two where they fit.)
-    const size_t w0_bytes = (size_t)s.d_out * s.d_in * 2;
     // (later, at 4096 -> 4096: 12.9 / 13.3 at 48 tokens, 13.4 / 13.5 at 64, 14.4 / 14.3 at 80; at 5120 -> 5120 16.8 / 16.6 at 48
     // and 18.6 / 16.8 at 64: up to 64 tokens for the layers up to 40 MB.)
     const int two_tokens = w0_bytes <= ((size_t)40 << 20) ? 64 : 32;
@@ -2100,28 +2135,42 @@ static StreamPlan make_stream_plan_with(const meteora_shape_t& s, int aux_budget
 // rows, and the B rows of all adapters for them do not fit beside the ring.  One aux CTA per stacked tile leaves more
 // main CTAs with fewer rows each (measured at 4096 -> 4096, 32 tokens, rank 64: 34.4 us against 41.6 on the three-launch
 // chain; an expand that reads the picked adapters' rows from L2 instead of staging them took 68 - 78 us).
-static StreamPlan make_stream_plan(const meteora_shape_t& s) {
-    StreamPlan sp = make_stream_plan_with(s, 0);
-    if (!sp.ok && sp.why == 5 && tuning().aux_ctas == 0) sp = make_stream_plan_with(s, 20);
+static StreamPlan make_stream_plan(const meteora_shape_t& s, const int* d_outs, int G) {
+    StreamPlan sp = make_stream_plan_with(s, d_outs, G, 0);
+    if (!sp.ok && sp.why == 5 && tuning().aux_ctas == 0) sp = make_stream_plan_with(s, d_outs, G, 20);
     return sp;
 }
 
-bool decode_stream_supported(const meteora_shape_t& s) { return make_stream_plan(s).ok; }
+bool decode_stream_supported(const meteora_shape_t& s, const int* d_outs, int G) { return make_stream_plan(s, d_outs, G).ok; }
 
-int launch_decode_stream(const void* x, const void* W0, const void* A, const void* B, const void* Wg,
-                         const meteora_shape_t& s, const Workspace& ws, void* y, cudaStream_t st) {
-    const StreamPlan sp = make_stream_plan(s);
+int launch_decode_stream(const void* x, const GroupModule* mods, int G, const meteora_shape_t& s, int32_t* status, float* part_g,
+                         int32_t* tile_ctr, cudaStream_t st) {
+    int d_outs[kMaxGroup] = {};
+    if (G < 1 || G > kMaxGroup) return METEORA_ERR_UNSUPPORTED_SHAPE;
+    for (int m = 0; m < G; ++m) d_outs[m] = mods[m].d_out;
+    const StreamPlan sp = make_stream_plan(s, d_outs, G);
     if (!sp.ok) return METEORA_ERR_UNSUPPORTED_SHAPE;
-    CUtensorMap mW, mA, mAt, mG, mX, mX1;
-    int rc;
+    DecodeMaps maps;
+    CUtensorMap mX, mX1;
+    StreamParams d = {};
+    int rc, tile0 = 0;
     const int tail_box = sp.gate_row0 > 0 ? sp.gate_row0 : kBM, gate_box = kBM - sp.gate_row0;
-    if ((rc = get_tensor_map(W0, s.d_in, s.d_out, kBM, sp.kc, &mW)) != METEORA_OK) return rc;
-    if ((rc = get_tensor_map(A, s.d_in, s.N * s.r, kBM, 1, &mA)) != METEORA_OK) return rc;
-    if ((rc = get_tensor_map(A, s.d_in, s.N * s.r, tail_box, 1, &mAt)) != METEORA_OK) return rc;
-    if ((rc = get_tensor_map(Wg, s.d_in, s.N, gate_box, 1, &mG)) != METEORA_OK) return rc;
+    for (int m = 0; m < kMaxGroup; ++m) {
+        if (m >= G) {                                            // unused slots repeat module 0's (valid) maps
+            maps.W0[m] = maps.W0[0], maps.A[m] = maps.A[0], maps.At[m] = maps.At[0], maps.G[m] = maps.G[0];
+            continue;
+        }
+        const GroupModule& gm = mods[m];
+        if ((rc = get_tensor_map(gm.W0, s.d_in, gm.d_out, kBM, sp.kc, &maps.W0[m])) != METEORA_OK) return rc;
+        if ((rc = get_tensor_map(gm.A, s.d_in, s.N * s.r, kBM, 1, &maps.A[m])) != METEORA_OK) return rc;
+        if ((rc = get_tensor_map(gm.A, s.d_in, s.N * s.r, tail_box, 1, &maps.At[m])) != METEORA_OK) return rc;
+        if ((rc = get_tensor_map(gm.Wg, s.d_in, s.N, gate_box, 1, &maps.G[m])) != METEORA_OK) return rc;
+        d.mod[m] = DecodeModule{(const __nv_bfloat16*)gm.B, (__nv_bfloat16*)gm.y, gm.d_out, tile0, gm.ws.topk_idx, gm.ws.topk_w,
+                                gm.ws.uw, gm.ws.u_all};
+        tile0 += (gm.d_out + kBM - 1) / kBM;
+    }
     if ((rc = get_tensor_map(x, s.d_in, s.T, sp.pair ? sp.BN / 2 : sp.BN, sp.kc, &mX)) != METEORA_OK) return rc;
     if ((rc = get_tensor_map(x, s.d_in, s.T, sp.BN, 1, &mX1)) != METEORA_OK) return rc;
-    StreamParams d = {};
     d.T = s.T;
     d.BN = sp.BN;
     d.ksteps = s.d_in / kBK;
@@ -2132,7 +2181,7 @@ int launch_decode_stream(const void* x, const void* W0, const void* A, const voi
     d.N = s.N;
     d.r = s.r;
     d.k = s.k;
-    d.d_out = s.d_out;
+    d.n_mod = G;
     d.row_tiles = sp.row_tiles;
     d.S = sp.S;
     d.n_main = sp.n_main;
@@ -2148,16 +2197,10 @@ int launch_decode_stream(const void* x, const void* W0, const void* A, const voi
     d.ring_bytes = sp.ring_bytes;
     d.bar_slots = kStreamBarSlots;
     d.inv_tau = 1.0f / s.temperature;
-    d.B = (const __nv_bfloat16*)B;
-    d.y = (__nv_bfloat16*)y;
-    d.topk_idx = ws.topk_idx;
-    d.topk_w = ws.topk_w;
-    d.uw = ws.uw;
-    d.u_part = ws.u_all;
-    d.part_g = ws.part_g;
-    d.ctr = ws.status + 16;
-    d.tile_ctr = ws.tile_ctr;
-    d.status = ws.status;
+    d.part_g = part_g;
+    d.ctr = status + 16;
+    d.tile_ctr = tile_ctr;
+    d.status = status;
     // Knob bulk_deliver = 1: the partial tiles leave through shared memory and one bulk copy per row slice (where all
     // slices have the same size) instead of plain stores.  Measured at 4096 -> 4096: the same 2.2 - 2.6 us from the
     // accumulator to the counter at 128 tokens either way, 0.3 us slower at one token; off by default.
@@ -2208,8 +2251,8 @@ int launch_decode_stream(const void* x, const void* W0, const void* A, const voi
     static int trace_calls = 0;
     d.trace_call = trace_calls++;
 #endif
-    if (sp.pair) return cuda_status(cudaLaunchKernelEx(&cfg, k_decode_stream<true>, mW, mA, mAt, mG, mX, mX1, d));
-    return cuda_status(cudaLaunchKernelEx(&cfg, k_decode_stream<false>, mW, mA, mAt, mG, mX, mX1, d));
+    if (sp.pair) return cuda_status(cudaLaunchKernelEx(&cfg, k_decode_stream<true>, maps, mX, mX1, d));
+    return cuda_status(cudaLaunchKernelEx(&cfg, k_decode_stream<false>, maps, mX, mX1, d));
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -2682,7 +2725,7 @@ int describe_plan(const meteora_shape_t& s, char* buf, size_t n) {
                         "path=cluster_decode launches=1 ctas=%d row_tiles=%d cluster=%d stacked_tiles=%d stacked_slices=%d "
                         "tile_tokens=%d stages=%d smem=%zu",
                         cp.n_cta, cp.row_tiles, cp.S, cp.aux_tiles, cp.SL, cp.BN, cp.stages, cp.smem);
-    const StreamPlan sp = make_stream_plan(s);
+    const StreamPlan sp = make_stream_plan(s, &s.d_out, 1);
     if (sp.ok)
         return snprintf(buf, n,
                         "path=stream_decode launches=1 main_ctas=%d row_tiles=%d ctas_per_tile=%d aux_ctas=%d aux_slices=%d "

@@ -1,0 +1,27 @@
+"""Decode batches on the streamed kernel where its tiling has edges: several modules in one launch (each with its own aux
+CTAs and row tiles, a last row tile that is not full, more CTAs than tokens), and batches of 129 to 256 tokens, against the CPU oracle."""
+import pytest
+import torch
+
+from paper_2405_13053_b200 import binding as mb
+from .test_gpu_group import check_group, make_group
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("T,d_in,d_outs,k", [(1, 512, (384, 128, 128), 2),        # fewer tokens than aux CTAs
+                                             (3, 2048, (1032, 264), 4),           # ragged last row tiles
+                                             (64, 1024, (512, 512, 512, 512), 1),
+                                             (65, 1024, (136, 2048), 2),
+                                             (128, 512, (1536, 256, 256), 2),
+                                             (129, 2048, (1024, 256), 2),         # one token above 128
+                                             (256, 2048, (1024, 264), 2),
+                                             (129, 2048, (1032,), 4),
+                                             (200, 2048, (2048,), 2),
+                                             (256, 1088, (1288,), 1)])
+def test_streamed_batches(T, d_in, d_outs, k):
+    if len(d_outs) > 1:
+        assert mb.meteora_group_plan(T, d_in, list(d_outs), 28, 8, k, torch.bfloat16) == 1
+    else:
+        assert "path=stream_decode" in mb.meteora_describe_plan(mb.make_shape(T, d_in, d_outs[0], 28, 8, k, torch.bfloat16))
+    check_group(make_group(T, d_in, d_outs, seed=9100 + T, k=k), 1e-2)
