@@ -122,13 +122,14 @@ static int forward_device(const void* x, const void* W0, const void* A, const vo
         tuning().fused_refused += 1;   // the cluster launch was refused: the streamed kernel takes the call
     }
     const GroupModule gm = {W0, A, B, Wg, y, s.d_out, ws};
-    if (decode_stream_supported(s, &s.d_out, 1)) {
+    const bool on_pairs = decode_on_pairs(s, &s.d_out, 1);
+    if (!on_pairs && decode_stream_supported(s, &s.d_out, 1)) {
         if (timed) cudaEventRecord(pf.ev[2 * pf.used], st);
         rc = launch_decode_stream(x, &gm, 1, s, ws.status, ws.part_g, ws.tile_ctr, st);
         if (timed) cudaEventRecord(pf.ev[2 * pf.used++ + 1], st);
         return rc;
     }
-    if (decode_fused_supported(s)) {
+    if (!on_pairs && decode_fused_supported(s)) {
         if (timed) cudaEventRecord(pf.ev[2 * pf.used], st);
         rc = launch_decode_fused(x, W0, A, B, Wg, s, ws, y, st);
         if (rc != kLaunchRefused) {
@@ -137,7 +138,7 @@ static int forward_device(const void* x, const void* W0, const void* A, const vo
         }
         tuning().fused_refused += 1;   // the cooperative launch was refused (not all CTAs can be resident): use the chain
     }
-    if (persist_forward_supported(s, &s.d_out, 1)) {
+    if (!on_pairs && persist_forward_supported(s, &s.d_out, 1)) {
         if (timed) cudaEventRecord(pf.ev[2 * pf.used], st);
         rc = launch_persist_forward(x, &gm, 1, s, ws.status, ws.tile_ctr, st);
         if (rc != kLaunchRefused) {
@@ -150,7 +151,7 @@ static int forward_device(const void* x, const void* W0, const void* A, const vo
         const bool pdl = tuning().pdl != 0;
         void* us = persist_supported(s) ? ws.us : nullptr;
         if (token_forward_supported(s)) {
-            if ((rc = launch_token_forward(x, A, Wg, s, ws, us, st)) != METEORA_OK) return rc;
+            if ((rc = launch_token_forward(x, A, Wg, s, ws, us, false, st)) != METEORA_OK) return rc;
         } else {
             if ((rc = launch_stacked_shrink_tc(x, A, Wg, s, ws, st)) != METEORA_OK) return rc;
             if ((rc = launch_select_from_stacked(ws.u_all, ws.ld_u, ws.col_logits, tc_stacked_zsplits(s), s, ws.topk_idx,
@@ -270,7 +271,7 @@ size_t meteora_group_workspace_bytes(const meteora_shape_t* shape, const int* d_
 int meteora_group_plan(const meteora_shape_t* shape, const int* d_out, int n_modules) {
     const int rc = check_group(shape, d_out, n_modules);
     if (rc != METEORA_OK) return rc;
-    return n_modules > 1 && (decode_stream_supported(*shape, d_out, n_modules) || decode_group_supported(*shape, d_out, n_modules) || persist_forward_supported(*shape, d_out, n_modules)) ? 1 : 0;
+    return n_modules > 1 && (decode_on_pairs(*shape, d_out, n_modules) || decode_stream_supported(*shape, d_out, n_modules) || decode_group_supported(*shape, d_out, n_modules) || persist_forward_supported(*shape, d_out, n_modules)) ? 1 : 0;
 }
 
 int meteora_group_workspace_routing(const meteora_shape_t* shape, const int* d_out, int n_modules, int module,
@@ -308,6 +309,11 @@ int meteora_linear_forward_group(const void* x, const void* const* W0, const voi
     }
     GroupModule gm[kMaxGroupModules];
     for (int m = 0; m < n_modules; ++m) gm[m] = GroupModule{W0[m], A[m], B[m], Wg[m], y[m], d_out[m], gw.mod[m]};
+    if (n_modules > 1 && decode_on_pairs(*shape, d_out, n_modules)) {
+        for (int m = 0; m < n_modules; ++m)                          // (the modules' launches do not depend on one another: beside)
+            if ((rc = launch_token_forward(x, A[m], Wg[m], *shape, gw.mod[m], gw.mod[m].us, m > 0, st)) != METEORA_OK) return rc;
+        return launch_persist_base(x, gm, n_modules, *shape, gw.mod[0].status, gw.mod[0].tile_ctr, st);
+    }
     if (n_modules > 1 && decode_stream_supported(*shape, d_out, n_modules))
         return launch_decode_stream(x, gm, n_modules, *shape, gw.mod[0].status, gw.part_g, gw.mod[0].tile_ctr, st);
     if (n_modules > 1 && decode_group_supported(*shape, d_out, n_modules)) {

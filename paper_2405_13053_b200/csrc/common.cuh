@@ -104,7 +104,7 @@ int launch_token_gate(const void* x, const void* Wg, const meteora_shape_t& s, i
                       cudaStream_t st);
 bool token_forward_supported(const meteora_shape_t& s);
 int launch_token_forward(const void* x, const void* A, const void* Wg, const meteora_shape_t& s, const Workspace& ws, void* us,
-                         cudaStream_t st);
+                         bool beside, cudaStream_t st);
 bool token_shrink_supported(const meteora_shape_t& s);
 int launch_token_shrink(const void* x, const void* A, const int32_t* topk_idx, const meteora_shape_t& s, float* u, int32_t* status,
                         bool beside, cudaStream_t st);
@@ -132,6 +132,9 @@ bool decode_stream_supported(const meteora_shape_t& s, const int* d_outs, int n_
 int launch_decode_stream(const void* x, const GroupModule* mods, int n_modules, const meteora_shape_t& s, int32_t* status,
                          float* part_g, int32_t* tile_ctr, cudaStream_t st);
 // Prefill: the whole layer of such modules on persistent pairs of SMs, one launch (wgemm_persist.cuh)
+bool decode_on_pairs(const meteora_shape_t& s, const int* d_outs, int n_modules);
+int launch_persist_base(const void* x, const GroupModule* mods, int n_modules, const meteora_shape_t& s, int32_t* status,
+                        int32_t* flags, cudaStream_t st);
 bool persist_forward_supported(const meteora_shape_t& s, const int* d_outs, int n_modules);
 int launch_persist_forward(const void* x, const GroupModule* mods, int n_modules, const meteora_shape_t& s, int32_t* status,
                            int32_t* flags, cudaStream_t st);

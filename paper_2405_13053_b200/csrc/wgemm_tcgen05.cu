@@ -1474,7 +1474,10 @@ static PersistPlan make_persist_plan(const meteora_shape_t& s, const int* d_outs
         if (persist_us_pitch(sm) == 0) return pp;
         pp.tiles += ((d_outs[m] + kBM - 1) / kBM + 1) / 2 * pp.tok_tiles;
     }
-    if (tn.persist < 2 && (pp.tiles * 4 < sm_count() || (s.T <= 128 && s.d_in < 1024))) return pp;
+    // Fewer tiles than a quarter of the SMs: split tiles of other kernels use more of the chip.  (One token tile behind a launch of
+    // token tiles: from 24 row pairs up, see decode_on_pairs.)  A short contraction leaves nothing to hide a tile's epilogue under.
+    const int least = !with_routing && s.T <= kPairTokens ? 24 : (sm_count() + 3) / 4;
+    if (tn.persist < 2 && (pp.tiles < least || (s.T <= 128 && s.d_in < 1024))) return pp;
     if (with_routing) {
         // [Wg; A] in 128-row tiles: Wg padded to whole 32 rows (a warp's TMEM lanes), then A, padded to whole MMAs of the expand
         pp.gate_rows = (s.N + 31) / 32 * 32;
@@ -1484,12 +1487,13 @@ static PersistPlan make_persist_plan(const meteora_shape_t& s, const int* d_outs
             G * pp.stacked_pairs * pp.tok_tiles > pairs)             // (a stacked tile is a pair's first)
             return pp;
         if (tn.persist == 3) return pp;
+        // a handful of tokens for gate / up: two streamed launches (4096 -> 2 x 11008 at 1 / 16 / 32 tokens 39.9 / 42.4 / 45.7 us, here
+        // 46.8 / 46.3 / 46.6; 4096 -> 2 x 14336 at 1 / 16 tokens 45.6 / 48.2 against 46.9 / 47.0)
+        if (tn.persist != 2 && G > 1 && s.T <= 12) return pp;
         // one round of tiles that the stacked ones would make two (4096 -> 1024 at 4096 tokens: 55.9 us, 52.4 with the routing ahead)
         const int with = pp.tiles + G * pp.stacked_pairs * pp.tok_tiles;
         if (tn.persist != 2 && pp.tiles <= pairs && with > pairs) return pp;
         pp.tiles = with;
-    } else if (G > 1) {
-        return pp;
     }
     pp.pairs = std::min(pairs, pp.tiles);
     pp.stage_bytes = kWTileBytes + pp.BN / 2 * 128;
@@ -1498,6 +1502,27 @@ static PersistPlan make_persist_plan(const meteora_shape_t& s, const int* d_outs
     pp.smem = fixed + (size_t)pp.stages * pp.stage_bytes;
     pp.ok = pp.stages >= 2;
     return pp;
+}
+
+// Decode batches whose base product goes to the persistent pairs behind a launch of token tiles (per module), ahead of the
+// one-launch decode kernels.  The streamed kernel gives each row tile of a
+// layer with more than 64 of them one CTA, which takes in W0 at half the rate of a pair and alone turns its accumulator into y; from
+// 48 tokens up that costs more than the extra launch.  Narrower layers gain only once a row tile's exchange among its CTAs outgrows the
+// launch.  Measured, us per call here and on the kernels otherwise taken:
+//   4096 -> 14336 (56 row pairs)  48 / 64 / 128 / 200 / 256 tokens  26.4 / 27.4 / 28.9 / 31.9 / 33.6 and 27.7 / 29.4 / 35.7 / 55.2 / 61.2
+//   5120 -> 13824 (54)            64 / 200 tokens  30.8 / 36.1 and 32.8 / 61.7;  2048 -> 9216 (36)  48 / 128 tokens  14.6 / 15.8 and 25.2 / 22.4
+//   4096 -> 8192 (32)             192 / 256 tokens 25.5 / 28.6 and 26.5 / 36.8;  8192 -> 8192  192 / 256 tokens  41.0 / 46.3 and 40.0 / 53.8
+//   4096 -> 6144 (24)             256 tokens 28.4 and 38.4;  4096 -> 22016 (86, two rounds)  16 / 32 / 128 tokens  45.9 / 46.2 / 48 and 46.9 / 64.4 / 89
+//   groups: 5120 -> 3 x 5120 (60) 96 / 128 / 256 tokens 40.1 / 40.5 / 47.4 and 38.7 / 41.9 / 69.4;  4096 -> 3 x 4096 (48)  128 / 256 tokens
+//   28.8 / 38.4 and 34.0 / 44.2;  4096 -> 2 x 11008 (86, two rounds)  128 / 160 / 256 tokens  49.0 / 49.8 / 56.5 and 48.8 / 55.2 / 62.3
+bool decode_on_pairs(const meteora_shape_t& s, const int* d_outs, int G) {
+    const Tuning& tn = tuning();
+    if (s.T > kPairTokens || s.d_in < 2048 || tn.persist != 1 || tn.fused != 1 || tn.stream != 1) return false;
+    if (!token_forward_supported(s)) return false;
+    const PersistPlan pp = make_persist_plan(s, d_outs, G, false);
+    if (!pp.ok) return false;
+    if (G > 1) return s.T >= (pp.tiles > pp.pairs ? 160 : pp.tiles > 32 ? 112 : 209);
+    return s.T >= (pp.tiles > pp.pairs ? 17 : pp.tiles > 32 ? 48 : pp.tiles > 28 ? 201 : 209);
 }
 
 bool persist_supported(const meteora_shape_t& s) { return make_persist_plan(s, &s.d_out, 1, false).ok; }
@@ -1600,6 +1625,14 @@ int launch_persist_forward(const void* x, const GroupModule* mods, int G, const 
     int d_outs[kMaxGroupModules] = {};
     for (int m = 0; m < G; ++m) d_outs[m] = mods[m].d_out;
     return launch_persist(make_persist_plan(s, d_outs, G, true), x, mods, G, s, status, flags, tuning().pdl != 0, st);
+}
+
+// The base products of modules whose routing and us are there: one launch.
+int launch_persist_base(const void* x, const GroupModule* mods, int G, const meteora_shape_t& s, int32_t* status, int32_t* flags,
+                        cudaStream_t st) {
+    int d_outs[kMaxGroupModules] = {};
+    for (int m = 0; m < G; ++m) d_outs[m] = mods[m].d_out;
+    return launch_persist(make_persist_plan(s, d_outs, G, false), x, mods, G, s, status, flags, tuning().pdl != 0, st);
 }
 
 int launch_base_lora_tc(const void* x, const void* W0, const void* B, const meteora_shape_t& s, const Workspace& ws,
@@ -2081,18 +2114,16 @@ static StreamPlan make_stream_plan_with(const meteora_shape_t& s, const int* d_o
     const size_t ring_need = std::max(std::max(landing, (size_t)sp.BN * kBM * 4), aux_rows);
     const int n_it_max = (nst + S - 1) / S;
     const int nks_aux = (ksteps + sp.aux_slices - 1) / sp.aux_slices;
-    // Two CTAs per SM (the next call's CTAs resident under this call) or one with twice the ring?  Two hide the set-up
-    // and load the first tiles under the call ahead, but the in-order ring stalls on its slowest line and five
-    // stages run at 3.3 - 4 TB/s where eleven reach HBM's rate: the longer the stream, the more the deeper ring counts.
-    // Measured per call, two / one per SM (us): 4096 -> 4096 (34 MB of W0) 12.2 / 13.1 at 1 token, 12.4 / 13.2 at 8,
-    // 14.3 / 13.8 at 64, 16.6 / 16.4 at 128; 5120 -> 5120 (52 MB) 15.3 / 15.9 at 1, 15.4 / 16.1 at 16, 19.1 / 17.1 at 64;
-    // 4096 -> 1024 (8 MB) 10.3 / 10.3 at 1, 12.1 / 11.8 at 64; 4096 -> 14336 (117 MB) 30.3 / 26.7 at 1, 31.2 / 31.5 at 64;
-    // 5120 -> 13824 (142 MB) 36.5 / 31.8 at 1.  So: two per SM for 16 - 56 MB of W0 and up to 32 tokens, else one.
-    // (Knob stream: 2 or 4 always one per SM, 3 always two where they fit.)
-    // (later, at 4096 -> 4096: 12.9 / 13.3 at 48 tokens, 13.4 / 13.5 at 64, 14.4 / 14.3 at 80; at 5120 -> 5120 16.8 / 16.6 at 48
-    // and 18.6 / 16.8 at 64: up to 64 tokens for the layers up to 40 MB.)
+    // Two CTAs per SM (the next call's CTAs resident under this call) or one with twice the ring?  Two hide the set-up and load the
+    // first tiles under the call ahead, but their rings hold two to five stages: that pays only where a CTA has few k-steps, of its
+    // row tile (three or more CTAs share one) as of the stacked matrix, and W0 is long enough for the next call to fill the gap.
+    // Measured per call, two / one per SM (us): 4096 -> 4096 (34 MB of W0, 4 CTAs per row tile) 11.5 / 11.8 at 1 token, 12.3 / 12.0 at
+    // 32, 13.5 / 12.9 at 64; 5120 -> 5120 (52 MB, 3 CTAs) 14.5 / 14.1 at 1, 15.7 / 14.9 at 32, 18.2 / 15.8 at 64; with one or two
+    // CTAs per row tile 4096 -> 6144 (50 MB) 15.5 / 13.4 at 1, 16.5 / 14.2 at 32; 2048 -> 9216 (38 MB) 14.6 / 11.2 at 1, 23.4 / 13.5
+    // at 32; 3072 -> 9216 (57 MB) 20.1 / 15.3, 32.0 / 17.3; with 13 k-steps of the stacked matrix per aux CTA 8192 -> 2048 (34 MB)
+    // 13.1 / 12.6, 14.2 / 13.0; 14336 -> 4096 (117 MB) 25.2 / 23.6 at 1.  (Knob stream: 2 or 4 always one, 3 always two where they fit.)
     const int two_tokens = w0_bytes <= ((size_t)40 << 20) ? 64 : 32;
-    const bool want_two = tn.stream == 3 || (tn.stream == 1 && s.T <= two_tokens && w0_bytes >= ((size_t)16 << 20) &&
+    const bool want_two = tn.stream == 3 || (tn.stream == 1 && S >= 3 && nks_aux <= 8 && s.T <= two_tokens && w0_bytes >= ((size_t)16 << 20) &&
                                              w0_bytes <= ((size_t)56 << 20));
     for (int per_sm = 2; per_sm >= 1; --per_sm) {
         if (per_sm == 2 && !want_two) continue;
@@ -2632,7 +2663,7 @@ int launch_token_gate(const void* x, const void* Wg, const meteora_shape_t& s, i
 bool token_forward_supported(const meteora_shape_t& s) { return make_token_plan(s, TOKEN_FORWARD).ok; }
 
 int launch_token_forward(const void* x, const void* A, const void* Wg, const meteora_shape_t& s, const Workspace& ws, void* us,
-                         cudaStream_t st) {
+                         bool beside, cudaStream_t st) {
     TokenTileParams p = {};
     p.topk_idx = ws.topk_idx;
     p.topk_w = ws.topk_w;
@@ -2640,6 +2671,7 @@ int launch_token_forward(const void* x, const void* A, const void* Wg, const met
     p.us = (__nv_bfloat16*)us;
     p.ld_us = ws.ld_us;
     p.status = ws.status;
+    p.late_wait = beside && tuning().pdl ? 1 : 0;
     return launch_token_tile(make_token_plan(s, TOKEN_FORWARD), TOKEN_FORWARD, s, x, Wg, A, p, st);
 }
 
@@ -2725,15 +2757,16 @@ int describe_plan(const meteora_shape_t& s, char* buf, size_t n) {
                         "path=cluster_decode launches=1 ctas=%d row_tiles=%d cluster=%d stacked_tiles=%d stacked_slices=%d "
                         "tile_tokens=%d stages=%d smem=%zu",
                         cp.n_cta, cp.row_tiles, cp.S, cp.aux_tiles, cp.SL, cp.BN, cp.stages, cp.smem);
+    const bool on_pairs = decode_on_pairs(s, &s.d_out, 1);
     const StreamPlan sp = make_stream_plan(s, &s.d_out, 1);
-    if (sp.ok)
+    if (sp.ok && !on_pairs)
         return snprintf(buf, n,
                         "path=stream_decode launches=1 main_ctas=%d row_tiles=%d ctas_per_tile=%d aux_ctas=%d aux_slices=%d "
                         "tile_tokens=%d stages=%d kc=%d smem=%zu ctas_per_sm=%d pairs=%d l2_prefetch_stages=%d",
                         sp.n_main, sp.row_tiles, sp.S, sp.n_aux, sp.aux_slices, sp.BN, sp.stages, sp.kc, sp.smem,
                         sp.ctas_per_sm, sp.pair, sp.pf_main);
     const FusedPlan fp = make_fused_plan(s);
-    if (fp.ok)
+    if (fp.ok && !on_pairs)
         return snprintf(buf, n,
                         "path=fused_decode launches=1 main_ctas=%d row_tiles=%d units_per_cta=%.1f aux_ctas=%d "
                         "aux_slices=%d tile_tokens=%d stages=%d kc=%d smem=%zu resident_ctas=%d",
@@ -2743,7 +2776,7 @@ int describe_plan(const meteora_shape_t& s, char* buf, size_t n) {
     const TokenPlan tp = make_token_plan(s, TOKEN_FORWARD);   // routing in one launch of token tiles, else in two
     const int routing = tp.ok ? 1 : 2;
     const PersistPlan whole = make_persist_plan(s, &s.d_out, 1, true);
-    if (whole.ok)
+    if (whole.ok && !on_pairs)
         return snprintf(buf, n,
                         "path=persistent_prefill launches=1 base=pairs_of_ctas persistent_pairs=%d tiles=%d stacked_tiles=%d tile=256x%d "
                         "stages=%d smem=%zu expand=mma",

@@ -4,6 +4,7 @@ import pytest
 import torch
 
 from paper_2405_13053_b200 import binding as mb
+from paper_2405_13053_b200 import workloads
 from .test_gpu_group import check_group, make_group
 
 pytestmark = pytest.mark.gpu
@@ -25,3 +26,20 @@ def test_streamed_batches(T, d_in, d_outs, k):
     else:
         assert "path=stream_decode" in mb.meteora_describe_plan(mb.make_shape(T, d_in, d_outs[0], 28, 8, k, torch.bfloat16))
     check_group(make_group(T, d_in, d_outs, seed=9100 + T, k=k), 1e-2)
+
+
+@pytest.mark.parametrize("T,d_in,d_outs,N,r", [(48, 2048, (9216,), 28, 8),           # the first batch that leaves the streamed kernel
+                                               (201, 2048, (7432,), 28, 8),          # ragged row pairs and tokens
+                                               (256, 2048, (6144,), 28, 8),
+                                               (96, 2120, (8456,), 12, 16),          # rank 16, a last k-step that is not full
+                                               (112, 2048, (4096, 4360), 28, 8),     # two modules' token tiles side by side
+                                               (256, 2048, (3072, 1544, 1544), 8, 8)])
+def test_wide_batches_behind_token_tiles(T, d_in, d_outs, N, r):
+    shape = mb.make_shape(T, d_in, d_outs[0], N, r, 2, torch.bfloat16)
+    if len(d_outs) == 1:
+        assert "launches=2" in mb.meteora_describe_plan(shape) and "persistent_pairs=" in mb.meteora_describe_plan(shape)
+        w = workloads.make_workload("wide", T=T, d_in=d_in, d_out=d_outs[0], N=N, r=r, k=2, dtype="bf16", x_kind="rms", seed=9300 + T, b_std=0.3)
+        check_group([w], 1e-2)
+    else:
+        assert mb.meteora_group_plan(T, d_in, list(d_outs), N, r, 2, torch.bfloat16) == 1
+        check_group(make_group(T, d_in, d_outs, seed=9300 + T, N=N), 1e-2)
