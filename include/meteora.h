@@ -312,7 +312,7 @@ int meteora_describe_plan(const meteora_shape_t* shape, char* buf, size_t buf_by
  *                    the kernel is launched without it (pdl_decode_refused in the plan string counts these).
  *   "pair"           default 1 = prefill base product on pairs of SMs (two-CTA MMA, 256 x 256 tiles)
  *                    where the pairs cover a quarter of the SMs; 0 = never; 2 = wherever the shape allows
- *   "stream"         decode batches up to 128 tokens on the streamed one-launch kernel: default 1 = planner's
+ *   "stream"         decode batches up to 256 tokens on the streamed one-launch kernel: default 1 = planner's
  *                    choice of one or two CTAs per SM, 0 = never (the cooperative kernel takes them), 2 = always one
  *                    CTA per SM with a deep ring, 3 = two per SM wherever they fit
  *   "pf"             L2 prefetch of the weights beyond the streamed kernel's ring: default 0 / -1 = none, n > 0 = cap in MB

@@ -14,13 +14,14 @@
 //     the B rows of the tile, both by TMA.  A tile's expand is issued near the end of the NEXT tile's main loop, by
 //     which time the selection is ready: nothing waits for the routing;
 //   - modules that share x (q/k/v, gate/up) are one walk: their tiles fill rounds of pairs together.
-// Where the stacked matrix has more than 512 rows or the batch more token tiles than pairs, the routing kernels ahead
-// write us and only the base product runs here (stacked_pairs = 0).
-// What bounds it: the tensor cores under the board's power limit (0.43 us per 64-element k-step and 256 x 256 tile, 1460
-// TFLOP/s over 74 pairs).  All pairs walk the contraction axis in step, so a line of W0 or x is fetched once for the pairs
+// Where the stacked matrix has more than 512 rows, the batch more token tiles than pairs, or all tokens fit one tile, the
+// routing kernels ahead write us and only the base product runs here (stacked_pairs = 0).
+// What bounds it: the tensor cores under the board's power limit (514 cycles per 64-element k-step and 256 x 256 tile, of
+// the 512 that its four MMAs take).  All pairs walk the contraction axis in step, so a line of W0 or x is fetched once for the pairs
 // that share it: dealing the last rounds as equal ranges of k-steps instead (partial tiles through L2) took 428 against 415 us
-// at 4096 -> 14336, 517 against 477 at 14336 -> 4096 (4096 tokens, sustained load).  Tiles narrower than 192 tokens gain
-// nothing more per k-step (0.37 us: an SM's intake).
+// at 4096 -> 14336, 517 against 477 at 14336 -> 4096 (4096 tokens, sustained load).  The issuing warps stay together and elect a
+// lane per k-step: a loop entered by one lane moved every operand to uniform registers by itself, 450 - 530 cycles per step
+// (4096 -> 4096 at 64 tokens 29.4 -> 18.7 us, 4096 -> 14336 at 2048 tokens 188 -> 178 us for the walk).
 //   warp 0 (both CTAs)  TMA producer; every copy signals the leader's full barrier, which expects both CTAs' bytes.
 //   warp 1 (leader)     MMA issue; stages are released and accumulators announced by commits that arrive in both CTAs.
 //   warps 2-9 (both)    epilogue: two groups of four warps take turns at chunks of CT tokens, each with a staging buffer of
