@@ -1474,9 +1474,13 @@ static PersistPlan make_persist_plan(const meteora_shape_t& s, const int* d_outs
         if (persist_us_pitch(sm) == 0) return pp;
         pp.tiles += ((d_outs[m] + kBM - 1) / kBM + 1) / 2 * pp.tok_tiles;
     }
-    // Fewer tiles than a quarter of the SMs: split tiles of other kernels use more of the chip.  (One token tile behind a launch of
-    // token tiles: from 24 row pairs up, see decode_on_pairs.)  A short contraction leaves nothing to hide a tile's epilogue under.
-    const int least = !with_routing && s.T <= kPairTokens ? 24 : (sm_count() + 3) / 4;
+    // Few tiles: split tiles of other kernels use more of the chip.  Behind routing kernels the walk pays from 20 tiles up where the
+    // contraction axis is not so long that the routing takes as long as the walk (us per call, walk / split tiles: 4096 -> 4096 at 257 / 512
+    // tokens, 32 tiles, 23.2 / 28.3 and 28.6 / 33.7; 4096 -> 2048 at 512 / 768 tokens, 16 and 24 tiles, 27.4 / 27.7 and 26.8 / 34.8;
+    // 4096 -> 1024 at 1280 tokens, 20 tiles, 27.3 and 33.0; 14336 -> 4096 at 512 tokens 73.4 and 69.1; rank 32, whose
+    // expand outweighs the tiles, from 8: 4096 -> 1024 at 512 tokens 43.6 and 66.7); one token tile: see
+    // decode_on_pairs.  A short contraction leaves nothing to hide a tile's epilogue under.
+    const int least = with_routing || s.d_in > 8192 ? (sm_count() + 3) / 4 : s.T <= kPairTokens ? 24 : s.N * s.r > 512 ? 8 : 20;
     if (tn.persist < 2 && (pp.tiles < least || (s.T <= 128 && s.d_in < 1024))) return pp;
     if (with_routing) {
         // [Wg; A] in 128-row tiles: Wg padded to whole 32 rows (a warp's TMEM lanes), then A, padded to whole MMAs of the expand
@@ -1490,6 +1494,11 @@ static PersistPlan make_persist_plan(const meteora_shape_t& s, const int* d_outs
         // a handful of tokens for gate / up: two streamed launches (4096 -> 2 x 11008 at 1 / 16 / 32 tokens 39.9 / 42.4 / 45.7 us, here
         // 46.8 / 46.3 / 46.6; 4096 -> 2 x 14336 at 1 / 16 tokens 45.6 / 48.2 against 46.9 / 47.0)
         if (tn.persist != 2 && G > 1 && s.T <= 12) return pp;
+        // one round of tiles, or little more, has nothing to cover the selection with (us with the routing ahead / inside: 5120 -> 5120
+        // at 257 / 512 / 768 tokens 27.5 / 33.3 / 41.9 and 40.2 / 46.8 / 47.6; 4096 -> 4096 at 768 / 1024 / 1280, 80 tiles, 36.0 / 38.1 / 48.2
+        // and 42.6 / 43.4 / 52.4; 5120 -> 5120 at 1280, 100 tiles, 60.2 and 59.1; 14336 -> 4096 at 1024 102.5 and 97.7; rank 16, whose
+        // routing ahead is two launches, at 512 tokens: 4096 -> 4096 46.1 and 53.0, 8192 -> 4096 81.3 and 68.4)
+        if (tn.persist != 2 && G == 1 && s.d_in <= (pp.stacked_pairs > 1 ? 4096 : 8192) && pp.tiles * 8 <= pairs * 9) return pp;
         // one round of tiles that the stacked ones would make two (4096 -> 1024 at 4096 tokens: 55.9 us, 52.4 with the routing ahead)
         const int with = pp.tiles + G * pp.stacked_pairs * pp.tok_tiles;
         if (tn.persist != 2 && pp.tiles <= pairs && with > pairs) return pp;

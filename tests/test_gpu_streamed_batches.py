@@ -43,3 +43,14 @@ def test_wide_batches_behind_token_tiles(T, d_in, d_outs, N, r):
     else:
         assert mb.meteora_group_plan(T, d_in, list(d_outs), N, r, 2, torch.bfloat16) == 1
         check_group(make_group(T, d_in, d_outs, seed=9300 + T, N=N), 1e-2)
+
+
+@pytest.mark.parametrize("T,d_in,d_out,N,r", [(257, 1024, 2560, 28, 8),       # two token tiles of 160, the second a short one
+                                              (700, 520, 1800, 28, 8),        # a last k-step and a last row pair that are not full
+                                              (1280, 512, 4096, 28, 8),       # a few tiles more than pairs
+                                              (300, 512, 1024, 28, 32)])      # 8 tiles, rank 32
+def test_short_prefill_walks_behind_its_routing(T, d_in, d_out, N, r):
+    plan = mb.meteora_describe_plan(mb.make_shape(T, d_in, d_out, N, r, 2, torch.bfloat16))
+    assert "path=chain" in plan and "persistent_pairs=" in plan, plan
+    check_group([workloads.make_workload("short", T=T, d_in=d_in, d_out=d_out, N=N, r=r, k=2, dtype="bf16", x_kind="rms",
+                                         seed=9500 + T, b_std=0.3)], 1e-2)
