@@ -192,7 +192,7 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(bar_accf + b * 8, 1);                       // one multicast commit
-            mbar_init(bar_acce + b * 8, 4);                       // (leader's) two epilogue groups of each CTA
+            mbar_init(bar_acce + b * 8, 4);                       // (leader's) two epilogue groups of each CTA, once per tile
             mbar_init(bar_pick + b * 8, 1);                       // the peer's group with the logits
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -536,6 +536,8 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                 }
                 continue;
             }
+            // a tile of one chunk (64 tokens at the most) is read by the first group alone: the other one owes its arrival all the same
+            if (grp >= chunks && elected) mbar_arrive_cluster(map_to_cta(bar_acce + b * 8, 0));
             for (int c = grp; c < chunks; c += 2) {
                 uint32_t v[4][16];
 #pragma unroll

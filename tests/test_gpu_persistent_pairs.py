@@ -7,6 +7,7 @@ import oracle
 from paper_2405_13053_b200 import binding as mb
 from paper_2405_13053_b200 import workloads
 from .gpu_util import bf16_bound_ok, check_selection, rel_l2, to_dev
+from .test_gpu_group import check_group, make_group
 
 pytestmark = pytest.mark.gpu
 
@@ -69,3 +70,20 @@ def test_a_prefill_group_is_one_walk(T, d_in, d_outs):
         check_selection(idx, o_idx, o_logits, 2)
         ref = oracle.linear_forward_routed(w["x"][sel], w["W0"], w["A"], w["B"], w["Wg"], idx[sel])
         assert rel_l2(y.float().cpu().numpy()[sel], ref) <= 5e-3
+
+
+# Three and four tiles per pair with tiles of at most 64 tokens, which are one chunk of the epilogue: only one of its two groups has
+# anything to read, and the accumulator's next tile waits for both.  Routing inside the walk (1 and 16 tokens, the groups) and ahead
+# of it (17 on); 65 tokens are the first with more chunks than one.
+@pytest.mark.parametrize("T,d_in,d_outs", [(1, 1024, (38664,)), (16, 2048, (38144,)), (17, 2048, (38664,)), (48, 2048, (38144,)),
+                                           (64, 2048, (38664,)), (65, 2048, (38144,)), (13, 1024, (28672, 28680)), (64, 1024, (28680, 28672))])
+def test_many_tiles_per_pair_of_one_chunk(T, d_in, d_outs):
+    ws = make_group(T, d_in, d_outs, seed=9700 + T, N=12)
+    if len(d_outs) == 1:
+        shape = mb.make_shape(T, d_in, d_outs[0], 12, 8, 2, torch.bfloat16)
+        assert "persistent_pairs=74 tiles=1" in mb.meteora_describe_plan(shape)
+        t = to_dev(ws[0], "x", "W0", "A", "B", "Wg")
+        workspace = mb.alloc_workspace(shape)
+        mb.meteora_linear_forward(*t, 2, workspace=workspace)
+        assert mb.meteora_workspace_status(workspace) == 0
+    check_group(ws, 1e-2)
