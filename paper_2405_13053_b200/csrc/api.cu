@@ -33,8 +33,9 @@ Workspace carve_workspace(const meteora_shape_t& s_in, void* base) {
     ws.topk_idx = (int32_t*)take(T * s.k * sizeof(int32_t));
     ws.topk_w = (float*)take(T * s.k * sizeof(float));
     ws.uw = (float*)take(T * s.k * s.r * sizeof(float));
-    ws.ld_us = persist_us_pitch(s);
-    ws.us = ws.ld_us > 0 ? take(T * ws.ld_us * 2) : nullptr;
+    ws.us_cols = persist_us_cols(s);
+    ws.us_parts = persist_us_parts(s);
+    ws.us = ws.us_cols > 0 ? take(T * ws.us_cols * ws.us_parts * 2) : nullptr;
     ws.u_all = (float*)take(T * ws.ld_u * sizeof(float) * (size_t)stacked_zsplits_bound(s.T));   // one copy per slice of the contraction axis
     // decode kernel scratch: one partial tile of 128 x BN fp32 per (main CTA, row tile it touches), in slot
     // row tile + main CTA: fewer than row tiles + 148 slots
@@ -155,7 +156,7 @@ static int forward_device(const void* x, const void* W0, const void* A, const vo
         } else {
             if ((rc = launch_stacked_shrink_tc(x, A, Wg, s, ws, st)) != METEORA_OK) return rc;
             if ((rc = launch_select_from_stacked(ws.u_all, ws.ld_u, ws.col_logits, tc_stacked_zsplits(s), s, ws.topk_idx,
-                                                 ws.topk_w, ws.uw, us, ws.ld_us, pdl, st)) != METEORA_OK)
+                                                 ws.topk_w, ws.uw, us, ws.us_cols, ws.us_parts, pdl, st)) != METEORA_OK)
                 return rc;
         }
         if (timed) cudaEventRecord(pf.ev[2 * pf.used], st);

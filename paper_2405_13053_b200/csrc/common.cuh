@@ -20,8 +20,9 @@ struct Workspace {
     int32_t* topk_idx;  // [T,k]
     float* topk_w;      // [T,k]
     float* uw;          // [T,k,r]   w_j * (A_{i_j} x): the shrunk, gate-weighted activations
-    void* us;           // [T,ld_us] bf16: masked, gate-weighted shrink, the token operand of the expand on persistent pairs
-    int ld_us;          //           (0: not laid out for this shape)
+    void* us;           // [T,us_parts,us_cols] bf16: masked, gate-weighted shrink, the token operand of the expand on persistent
+    int us_cols;        //           pairs (0: not laid out for this shape), rounded (one part) or as three parts that
+    int us_parts;       //           hold the 24 bits of uw between them (persist_us_parts)
     float* u_all;       // [Z][T,ld_u]  stacked shrink: every adapter's A_i x, then the gate logits; Z partial
                         //           copies (slices of the contraction axis) that the selection kernel adds up
     int ld_u;           // row pitch of u_all in floats
@@ -59,7 +60,7 @@ inline size_t elem_size(meteora_dtype_t t) { return t == METEORA_BF16 ? 2 : 4; }
 int launch_gate_topk(const void* x, const void* Wg, const meteora_shape_t& s, int32_t* topk_idx, float* topk_w,
                      float* logits, cudaStream_t st);
 int launch_select_from_stacked(const float* u_all, int ld_u, int col_logits, int zsplits, const meteora_shape_t& s,
-                               int32_t* topk_idx, float* topk_w, float* uw, void* us, int ld_us, bool pdl, cudaStream_t st);
+                               int32_t* topk_idx, float* topk_w, float* uw, void* us, int us_cols, int us_parts, bool pdl, cudaStream_t st);
 // route.cu
 int launch_gate_backward(const void* x, const void* A, const void* B, const void* dy, const int32_t* topk_idx,
                          const float* topk_w, const meteora_shape_t& s, void* Bt, float* u, float* z, float* dlogit,
@@ -84,7 +85,8 @@ int launch_forward_simt(const void* x, const void* W0, const void* A, const void
                         const Workspace& ws, void* y, cudaStream_t st);
 // wgemm_tcgen05.cu
 bool tc_path_supported(const meteora_shape_t& s);
-int persist_us_pitch(const meteora_shape_t& s);                   // columns of Workspace::us, 0 where no path reads it
+int persist_us_cols(const meteora_shape_t& s);                    // columns of a part of Workspace::us, 0 where no path reads it
+int persist_us_parts(const meteora_shape_t& s);                   // its parts: 1 (bf16) or 3 (as exact as fp32)
 bool persist_supported(const meteora_shape_t& s);                 // base product on persistent pairs, which reads us
 int tc_stacked_pitch(const meteora_shape_t& s, int* col_logits);  // row pitch (floats) of u_all
 int stacked_zsplits_bound(int T);                                  // upper bound of those copies, sizes the workspace
@@ -225,6 +227,27 @@ __device__ __forceinline__ unsigned long long bf16x2_to_f32x2(uint32_t v) {
     unsigned long long r;
     asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(v << 16), "r"(v & 0xFFFF0000u));
     return r;
+}
+
+// The first 8 bits of v as a bf16 (cut off, not rounded: no part of a finite v overflows); v becomes the rest.  Three calls
+// give parts whose sum is v.  Infinities and NaN stay whole in the first part.
+__device__ __forceinline__ __nv_bfloat16 take_bf16_part(float& v) {
+    const uint32_t bits = __float_as_uint(v);
+    if ((bits & 0x7F800000u) == 0x7F800000u) {
+        const __nv_bfloat16 whole = __float2bfloat16_rn(v);
+        v = 0.f;
+        return whole;
+    }
+    v -= __uint_as_float(bits & 0xFFFF0000u);
+    return __ushort_as_bfloat16((unsigned short)(bits >> 16));
+}
+// v at column c of a token's row of Workspace::us ([parts][cols]).
+__device__ __forceinline__ void store_us(__nv_bfloat16* row, int c, int cols, int parts, float v) {
+    if (parts == 1) {
+        row[c] = __float2bfloat16_rn(v);
+        return;
+    }
+    for (int i = 0; i < parts; ++i) row[(size_t)i * cols + c] = take_bf16_part(v);
 }
 
 __device__ __forceinline__ float warp_sum(float v) {

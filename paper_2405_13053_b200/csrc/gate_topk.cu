@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(kGateWarps * 32)
 k_select_from_stacked(const float* __restrict__ u_all, int ld_u, int col_logits, int zsplits, size_t zstride, int T,
                       int N, int r, int k,
                       float inv_tau, int32_t* topk_idx, float* __restrict__ topk_w,
-                      float* uw, __nv_bfloat16* us, int ld_us, int pdl) {
+                      float* uw, __nv_bfloat16* us, int us_cols, int us_parts, int pdl) {
     if (pdl) {
         // Let the dependent launch (the base product) start streaming weights now; wait for the
         // stacked shrink, which produced u_all, before reading it.
@@ -124,12 +124,12 @@ k_select_from_stacked(const float* __restrict__ u_all, int ld_u, int col_logits,
     if (t >= T) return;
     select_token<false>(u_all, ld_u, col_logits, zsplits, zstride, t, N, r, k, inv_tau, lane, topk_idx, topk_w, uw);
     if (us) {                                                    // the same values as the masked operand of the expand
-        uint4* row = reinterpret_cast<uint4*>(us + (size_t)t * ld_us);
-        for (int i = lane; i < ld_us / 8; i += 32) row[i] = make_uint4(0u, 0u, 0u, 0u);
+        __nv_bfloat16* row = us + (size_t)t * us_cols * us_parts;
+        for (int i = lane; i < us_cols * us_parts / 8; i += 32) reinterpret_cast<uint4*>(row)[i] = make_uint4(0u, 0u, 0u, 0u);
         __syncwarp();
         for (int c = lane; c < k * r; c += 32) {
             const int j = c / r;
-            us[(size_t)t * ld_us + topk_idx[(size_t)t * k + j] * r + c - j * r] = __float2bfloat16_rn(uw[(size_t)t * k * r + c]);
+            store_us(row, topk_idx[(size_t)t * k + j] * r + c - j * r, us_cols, us_parts, uw[(size_t)t * k * r + c]);
         }
     }
 }
@@ -172,7 +172,8 @@ int launch_gate_topk(const void* x, const void* Wg, const meteora_shape_t& s, in
 }
 
 int launch_select_from_stacked(const float* u_all, int ld_u, int col_logits, int zsplits, const meteora_shape_t& s,
-                               int32_t* topk_idx, float* topk_w, float* uw, void* us, int ld_us, bool pdl, cudaStream_t st) {
+                               int32_t* topk_idx, float* topk_w, float* uw, void* us, int us_cols, int us_parts, bool pdl,
+                               cudaStream_t st) {
     if (s.T == 0) return METEORA_OK;
     const int blocks = (s.T + kGateWarps - 1) / kGateWarps;
     cudaLaunchConfig_t cfg = {};
@@ -187,7 +188,7 @@ int launch_select_from_stacked(const float* u_all, int ld_u, int col_logits, int
     const float inv_tau = 1.0f / s.temperature;
     cudaError_t e = cudaLaunchKernelEx(&cfg, k_select_from_stacked, u_all, ld_u, col_logits, zsplits,
                                        (size_t)s.T * ld_u, s.T, s.N, s.r, s.k,
-                                       inv_tau, topk_idx, topk_w, uw, (__nv_bfloat16*)us, ld_us, pdl ? 1 : 0);
+                                       inv_tau, topk_idx, topk_w, uw, (__nv_bfloat16*)us, us_cols, us_parts, pdl ? 1 : 0);
     return cuda_status(e);
 }
 

@@ -38,8 +38,8 @@ struct TokenTileParams {
     float* topk_w;             // (not read by SHRINK)
     float* logits;             // GATE: optional out
     float* u;                  // out: [slot][r], FORWARD weighted by w
-    __nv_bfloat16* us;         // FORWARD, optional out: the same values as [T][ld_us] with zeros elsewhere
-    int ld_us;
+    __nv_bfloat16* us;         // FORWARD, optional out: the same values as [T][us_parts][us_cols] with zeros elsewhere
+    int us_cols, us_parts;
     int32_t* status;           // error flag of expired waits (may be null)
     int clear_status;          // CTA 0 zeroes the status words first
     int late_wait;             // nothing here depends on the kernel ahead: only leave after it
@@ -78,8 +78,9 @@ __device__ __forceinline__ void token_round(const TokenTileParams& p, uint32_t p
     if (p.mode <= TOKEN_FORWARD && round == 0) {
         const int ld = p.N | 1;
         if (p.us) {
-            uint4* rows = reinterpret_cast<uint4*>(p.us + (size_t)t0 * p.ld_us);
-            for (int i = etid; i < own * (p.ld_us / 8); i += kEpiThreads) rows[i] = make_uint4(0u, 0u, 0u, 0u);
+            const int ld_us = p.us_cols * p.us_parts;
+            uint4* rows = reinterpret_cast<uint4*>(p.us + (size_t)t0 * ld_us);
+            for (int i = etid; i < own * (ld_us / 8); i += kEpiThreads) rows[i] = make_uint4(0u, 0u, 0u, 0u);
         }
 #pragma unroll 2
         for (int i = etid; i < own * p.N; i += kEpiThreads) {
@@ -118,7 +119,8 @@ __device__ __forceinline__ void token_round(const TokenTileParams& p, uint32_t p
             const float v = cluster_sum<S>(base, (uint32_t)(own0 + slot / p.k) * pitch4 + 4u * (col - c_lo));
             const float out = p.mode == TOKEN_FORWARD ? p.topk_w[g] * v : v;
             p.u[(size_t)t0 * n + i] = out;
-            if (p.us) p.us[(size_t)(t0 + slot / p.k) * p.ld_us + (e0 + e) * p.r + q] = __float2bfloat16_rn(out);
+            if (p.us)
+                store_us(p.us + (size_t)(t0 + slot / p.k) * p.us_cols * p.us_parts, (e0 + e) * p.r + q, p.us_cols, p.us_parts, out);
         }
     }
 }

@@ -13,9 +13,15 @@
 //   - the LoRA expand is a few more k-steps of the same ring: the contraction goes on over the N r columns of us against
 //     the B rows of the tile, both by TMA.  A tile's expand is issued near the end of the NEXT tile's main loop, by
 //     which time the selection is ready: nothing waits for the routing;
+//   - where the kernels otherwise taken expand in fp32 (decode batches, few tiles of large ranks: persist_us_parts) us is
+//     three bf16 parts whose sum is w_j (A_e x_t)_q exactly: a k-step of the expand is then two stages, (B, part 0) and
+//     (part 1, part 2), so that B is read once; the routing kernels ahead write the parts.  Such a token's y depends on its
+//     own picks alone, also where an adapter that it did not pick holds an infinity or a NaN: 0 times those is NaN, and a
+//     NaN of such a row is computed again from the picks.  Measured against rounded parts: 4096 -> 2 x 14336 at 64 tokens
+//     49.9 -> 52.2 us, 5120 -> 13824 at 200 tokens 37.3 -> 39.4 (four stages more per tile);
 //   - modules that share x (q/k/v, gate/up) are one walk: their tiles fill rounds of pairs together.
-// Where the stacked matrix has more than 512 rows, the batch more token tiles than pairs, or all tokens fit one tile, the
-// routing kernels ahead write us and only the base product runs here (stacked_pairs = 0).
+// Where the stacked matrix has more than 512 rows, the batch more token tiles than pairs, one round of tiles would become two, or
+// us is three parts, the routing kernels ahead write us and only the base product runs here (stacked_pairs = 0).
 // What bounds it: the tensor cores under the board's power limit (514 cycles per 64-element k-step and 256 x 256 tile, of
 // the 512 that its four MMAs take).  All pairs walk the contraction axis in step, so a line of W0 or x is fetched once for the pairs
 // that share it: dealing the last rounds as equal ranges of k-steps instead (partial tiles through L2) took 428 against 415 us
@@ -46,9 +52,12 @@ struct PersistMaps {                                              // per module,
 struct PersistModule {
     int tile0;                    // its first tile
     int row_tiles, row_pairs, group_pairs;   // group_pairs: row pairs per scheduling group
-    __nv_bfloat16* us;            // [T][ld_us]
+    int parts;                    // of us
+    const __nv_bfloat16* us;      // [T][parts][64 esteps]
     int32_t* topk_idx;
     float* topk_w;
+    const __nv_bfloat16 *W0, *B;  // for the elements that are computed again
+    int d_out;
 };
 struct PersistParams {
     int T, BN, CT;                // tokens per tile, tokens per epilogue chunk (divides BN)
@@ -57,12 +66,14 @@ struct PersistParams {
     int stages, stage_bytes;
     int n_mod, tok_tiles, tiles;
     int stacked_pairs;            // pairs of 128-row tiles of [Wg; A] (0: us comes from the kernel ahead)
-    int gate_rows, us_cols, ld_us;   // Wg's rows padded to whole 32s; columns of us that are read
+    int gate_rows, us_cols;       // Wg's rows padded to whole 32s; columns of a part of us that are read
     float inv_tau;
     int32_t* flags;               // [module][token tile][2]: picks written, us written; zero between calls
     int32_t* leave_ctr;           // CTAs that are done with the flags
     int32_t* status;
     int pdl;
+    const __nv_bfloat16* x;
+    int d_in;
     PersistModule mod[kMaxGroupModules];
 };
 
@@ -161,6 +172,48 @@ __device__ __forceinline__ float persist_weight(const float* s, int tok, int j, 
     const float v = s[j * 64 + (tok ^ (j & 31))];
     return expf(((v > -CUDART_INF_F ? v : -CUDART_INF_F) + 0.f - first) * inv_tau) / sum;
 }
+// Whether 8 packed bf16 hold an infinity or a NaN.
+__device__ __forceinline__ bool any_nonfinite(const uint4& v) {
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    bool any = false;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) any |= (w[i] & 0x7F80u) == 0x7F80u || (w[i] & 0x7F800000u) == 0x7F800000u;
+    return any;
+}
+
+// A warp's 32 rows x `nt` tokens of a staged chunk of y ([token][128 rows]) in which some element is NaN: those of rows where some
+// adapter's B is not finite are computed again as W0 x + the picks' terms.  (A NaN of any other row is the row's own.)  Never
+// taken on finite weights; a row with such an entry costs a dot product per token.
+__device__ __noinline__ void persist_repair(const PersistParams& p, const PersistModule& mo, __nv_bfloat16* ystage, int tile_row0, int quad,
+                                            int tok0, int nt) {
+    const int lane = threadIdx.x & 31, row0 = tile_row0 + quad * 32, row = row0 + lane;
+    asm volatile("griddepcontrol.wait;" ::: "memory");               // (the producer has waited: this thread may read what it waited for)
+    bool odd = false;
+    if (row < mo.d_out)
+        for (int e = 0; e < p.N; ++e)
+            for (int c = 0; c < p.r; c += 8) odd |= any_nonfinite(*reinterpret_cast<const uint4*>(mo.B + ((size_t)e * mo.d_out + row) * p.r + c));
+    const int cols = 64 * p.esteps;
+    for (int i = 0; i < nt; ++i) {
+        unsigned todo = __ballot_sync(0xFFFFFFFFu, odd && __hisnan(ystage[i * kBM + quad * 32 + lane]));
+        const int t = tok0 + i;
+        while (todo) {
+            const int src = __ffs(todo) - 1;
+            todo &= todo - 1;
+            const float base = warp_dot(mo.W0 + (size_t)(row0 + src) * p.d_in, p.x + (size_t)t * p.d_in, p.d_in, lane, true);
+            float lora = 0.f;
+            for (int s = lane; s < p.k * p.r; s += 32) {
+                const int j = s / p.r, q = s - j * p.r, e = min(max(__ldcg(mo.topk_idx + (size_t)t * p.k + j), 0), p.N - 1);
+                const unsigned short* u = reinterpret_cast<const unsigned short*>(mo.us) + (size_t)t * 3 * cols + e * p.r + q;
+                const float rest = __uint_as_float((uint32_t)__ldcg(u + cols) << 16) + __uint_as_float((uint32_t)__ldcg(u + 2 * cols) << 16);
+                const float uw = __uint_as_float((uint32_t)__ldcg(u) << 16) + rest;
+                lora = fmaf(to_f32(mo.B[((size_t)e * mo.d_out + row0 + src) * p.r + q]), uw, lora);
+            }
+            lora = warp_sum(lora);
+            if (lane == src) ystage[i * kBM + quad * 32 + lane] = __float2bfloat16_rn(base + lora);
+        }
+    }
+}
+
 __device__ __forceinline__ void st_cluster_v2(uint32_t cluster_addr, int2 v) {
     asm volatile("st.shared::cluster.v2.b32 [%0], {%1, %2};" ::"r"(cluster_addr), "r"(v.x), "r"(v.y) : "memory");
 }
@@ -242,6 +295,7 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                 }
                 const int row0 = (t.row_pair * 2 + (int)rank) * kBM, tokh = t.tok_tile * p.BN + (int)rank * (p.BN / 2);
                 uint32_t own, full, dst;
+                const bool split = p.mod[t.mod].parts > 1;
                 for (int i = 0; i < p.esteps; ++i) {
                     if (!slot(own, full, dst)) return false;
                     const int q0 = i * 8;                         // first of the 8 blocks
@@ -252,6 +306,14 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                         else
                             tma_load_4d_grp(dst, &maps.B[t.mod], 0, row0, q0 % p.cpa, q0 / p.cpa, full);
                         tma_load_2d_pair(dst + kWTileBytes, &maps.U[t.mod], q0 * 8, tokh, full);
+                    }
+                    __syncwarp();
+                    if (!split) continue;
+                    if (!slot(own, full, dst)) return false;
+                    if (elect_one()) {                            // the other two parts: one where W0's rows would lie
+                        if (leader) mbar_expect_tx(own, 2 * (uint32_t)p.BN * 128u);
+                        tma_load_2d_pair(dst, &maps.U[t.mod], (p.esteps + i) * kBK, tokh, full);
+                        tma_load_2d_pair(dst + kWTileBytes, &maps.U[t.mod], (2 * p.esteps + i) * kBK, tokh, full);
                     }
                     __syncwarp();
                 }
@@ -307,17 +369,29 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                     phase ^= 1;
                 }
             };
+            int parts = 1;                                        // of the tile whose expand is pending
             auto expand = [&](int b) {
-                uint32_t wa;
+                uint32_t wa, ua;
                 for (int i = 0; i < p.esteps; ++i) {
                     if (!next(wa)) return false;
-                    const uint64_t db = smem_desc_sw128(wa + kWTileBytes);
+                    const int first = s;                          // stage with the B rows: released with the parts behind it
+                    uint64_t db[3] = {smem_desc_sw128(wa + kWTileBytes), 0, 0};
+                    if (parts > 1) {
+                        release();
+                        if (!next(ua)) return false;
+                        db[1] = smem_desc_sw128(ua);
+                        db[2] = smem_desc_sw128(ua + kWTileBytes);
+                    }
                     const int nm = min(4, (p.nblk - i * 8 + 1) / 2);   // two blocks per MMA: 8-row x 16-byte core matrices, 2 KB per block
                     if (elect_one()) {
-                        for (int kk = 0; kk < nm; ++kk)
-                            umma_bf16_pair(tmem_base + b * kPairTokens, smem_desc_plain(wa + kk * 2 * kBM * 16, kBM * 16, 128),
-                                           db + (uint64_t)(kk * 2), idesc, 1);
-                        umma_commit_pair(bar_base + (p.stages + s) * 8);
+#pragma unroll
+                        for (int h = 0; h < 3; ++h)
+                            if (h < parts)
+                                for (int kk = 0; kk < nm; ++kk)
+                                    umma_bf16_pair(tmem_base + b * kPairTokens, smem_desc_plain(wa + kk * 2 * kBM * 16, kBM * 16, 128),
+                                                   db[h] + (uint64_t)(kk * 2), idesc, 1);
+                        umma_commit_pair(bar_base + (p.stages + first) * 8);
+                        if (parts > 1) umma_commit_pair(bar_base + (p.stages + s) * 8);
                     }
                     __syncwarp();
                     release();
@@ -349,7 +423,9 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                     release();
                 }
                 if (!ok) break;
-                pending = lin >= p.mod[0].tile0;
+                const PersistTile t(p, lin);
+                pending = !t.stacked;
+                parts = p.mod[t.mod].parts;
                 if (!pending && elect_one()) umma_commit_pair(bar_accf + b * 8);
                 __syncwarp();
             }
@@ -486,7 +562,7 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                                 tmem_ld16_issue(taddr + (uint32_t)(c * p.CT + h + 16), v[1]);
                                 float w[32];
 #pragma unroll
-                                for (int i = 0; i < 32; ++i) w[i] = 0.f;
+                                for (int i = 0; i < 32; ++i) w[i] = -1.f;   // not picked (no weight is negative)
 #pragma unroll 1
                                 for (int j = 0; j < p.k; ++j)
 #pragma unroll
@@ -497,7 +573,7 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                                 tmem_ld_wait();
 #pragma unroll
                                 for (int i = 0; i < 32; ++i)
-                                    s_us[i * 32 + lane] = __float2bfloat16_rn(w[i] != 0.f ? w[i] * __uint_as_float(v[i >> 4][i & 15]) : 0.f);
+                                    s_us[i * 32 + lane] = __float2bfloat16_rn(w[i] < 0.f ? 0.f : w[i] * __uint_as_float(v[i >> 4][i & 15]));
                             } else {
 #pragma unroll
                                 for (int i = 0; i < 4; ++i) reinterpret_cast<uint4*>(s_us)[i * 32 + lane] = make_uint4(0u, 0u, 0u, 0u);
@@ -556,6 +632,16 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                         for (int i = 0; i < 16; ++i)
                             ystage[(16 * q + i) * kBM + row_in_tile] = __float2bfloat16_rn(__uint_as_float(v[q][i]));
                     }
+                if (mo.parts > 1) {
+                    bool nan = false;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (16 * q < p.CT) {
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) nan |= __uint_as_float(v[q][i]) != __uint_as_float(v[q][i]);
+                        }
+                    if (__any_sync(0xFFFFFFFFu, nan)) persist_repair(p, mo, ystage, tile_m * kBM, quad, tok0 + c * p.CT, min(p.CT, p.T - tok0 - c * p.CT));
+                }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> TMA read
                 asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
                 if (elected) {

@@ -1427,10 +1427,19 @@ struct PersistPlan {
 
 // Columns of the masked token operand: the expand takes N r columns in k-steps of 64.  Other ranks than 8, 16, 32, 64 (a k-step
 // is whole adapters or a whole part of one) and more than 2048 columns stay with the kernel that stages them in rounds.
-int persist_us_pitch(const meteora_shape_t& s) {
+int persist_us_cols(const meteora_shape_t& s) {
     const int cols = (s.N * s.r + kBK - 1) / kBK * kBK, cpa = s.r / 8;
     if (s.dtype != METEORA_BF16 || s.T < 1 || s.d_in % 8 != 0 || s.d_out % 8 != 0 || s.r % 8 != 0 || cols > 2048) return 0;
     return cpa == 1 || cpa == 2 || cpa == 4 || cpa == 8 ? cols : 0;
+}
+
+// Parts of that operand.  The kernels that the walk stands in for round uw to bf16 where their expand is MMAs too (the pair kernel, from
+// a quarter of the SMs in pair tiles on; rank 8 up to the adapters whose B rows fit beside a 256-token tile) and keep it in fp32
+// everywhere else; there the operand is three parts that add up to the fp32 value.
+int persist_us_parts(const meteora_shape_t& s) {
+    if (s.T <= kPairTokens) return 3;
+    const long long pairs = (long long)((s.d_out + 2 * kBM - 1) / (2 * kBM)) * ((s.T + kPairTokens - 1) / kPairTokens);
+    return pairs * 4 >= sm_count() || (s.r == 8 && s.N <= 80) ? 1 : 3;
 }
 
 // Pairs the device holds at once (0: it cannot say).
@@ -1471,7 +1480,7 @@ static PersistPlan make_persist_plan(const meteora_shape_t& s, const int* d_outs
     for (int m = 0; m < G; ++m) {
         meteora_shape_t sm = s;
         sm.d_out = d_outs[m];
-        if (persist_us_pitch(sm) == 0) return pp;
+        if (persist_us_cols(sm) == 0) return pp;
         pp.tiles += ((d_outs[m] + kBM - 1) / kBM + 1) / 2 * pp.tok_tiles;
     }
     // Few tiles: split tiles of other kernels use more of the chip.  Behind routing kernels the walk pays from 20 tiles up where the
@@ -1491,9 +1500,14 @@ static PersistPlan make_persist_plan(const meteora_shape_t& s, const int* d_outs
             G * pp.stacked_pairs * pp.tok_tiles > pairs)             // (a stacked tile is a pair's first)
             return pp;
         if (tn.persist == 3) return pp;
-        // a handful of tokens for gate / up: two streamed launches (4096 -> 2 x 11008 at 1 / 16 / 32 tokens 39.9 / 42.4 / 45.7 us, here
-        // 46.8 / 46.3 / 46.6; 4096 -> 2 x 14336 at 1 / 16 tokens 45.6 / 48.2 against 46.9 / 47.0)
-        if (tn.persist != 2 && G > 1 && s.T <= 12) return pp;
+        // the stacked tiles write us rounded to bf16: not where it is three parts (knob 2, a measurement: all the same).  The
+        // routing ahead costs such a batch nothing: 4096 -> 2 x 14336 at 64 / 128 tokens 54.4 / 56.3 us, with parts written from
+        // the stacked tiles 57.3 / 60.4 (their stores queue behind the next tile's loads).
+        for (int m = 0; m < G && tn.persist != 2; ++m) {
+            meteora_shape_t sm = s;
+            sm.d_out = d_outs[m];
+            if (persist_us_parts(sm) > 1) return pp;
+        }
         // one round of tiles, or little more, has nothing to cover the selection with (us with the routing ahead / inside: 5120 -> 5120
         // at 257 / 512 / 768 tokens 27.5 / 33.3 / 41.9 and 40.2 / 46.8 / 47.6; 4096 -> 4096 at 768 / 1024 / 1280, 80 tiles, 36.0 / 38.1 / 48.2
         // and 42.6 / 43.4 / 52.4; 5120 -> 5120 at 1280, 100 tiles, 60.2 and 59.1; 14336 -> 4096 at 1024 102.5 and 97.7; rank 16, whose
@@ -1516,22 +1530,25 @@ static PersistPlan make_persist_plan(const meteora_shape_t& s, const int* d_outs
 // Decode batches whose base product goes to the persistent pairs behind a launch of token tiles (per module), ahead of the
 // one-launch decode kernels.  The streamed kernel gives each row tile of a
 // layer with more than 64 of them one CTA, which takes in W0 at half the rate of a pair and alone turns its accumulator into y; from
-// 48 tokens up that costs more than the extra launch.  Narrower layers gain only once a row tile's exchange among its CTAs outgrows the
-// launch.  Measured, us per call here and on the kernels otherwise taken:
-//   4096 -> 14336 (56 row pairs)  48 / 64 / 128 / 200 / 256 tokens  26.4 / 27.4 / 28.9 / 31.9 / 33.6 and 27.7 / 29.4 / 35.7 / 55.2 / 61.2
-//   5120 -> 13824 (54)            64 / 200 tokens  30.8 / 36.1 and 32.8 / 61.7;  2048 -> 9216 (36)  48 / 128 tokens  14.6 / 15.8 and 25.2 / 22.4
-//   4096 -> 8192 (32)             192 / 256 tokens 25.5 / 28.6 and 26.5 / 36.8;  8192 -> 8192  192 / 256 tokens  41.0 / 46.3 and 40.0 / 53.8
-//   4096 -> 6144 (24)             256 tokens 28.4 and 38.4;  4096 -> 22016 (86, two rounds)  16 / 32 / 128 tokens  45.9 / 46.2 / 48 and 46.9 / 64.4 / 89
-//   groups: 5120 -> 3 x 5120 (60) 96 / 128 / 256 tokens 40.1 / 40.5 / 47.4 and 38.7 / 41.9 / 69.4;  4096 -> 3 x 4096 (48)  128 / 256 tokens
-//   28.8 / 38.4 and 34.0 / 44.2;  4096 -> 2 x 11008 (86, two rounds)  128 / 160 / 256 tokens  49.0 / 49.8 / 56.5 and 48.8 / 55.2 / 62.3
+// 48 - 64 tokens up that costs more than the extra launch.  Narrower layers gain only once a row tile's exchange among its CTAs
+// outgrows the launch, or the streamed kernel's landing area no longer fits.  Measured, us per call here and on the kernels otherwise
+// taken (pair tiles in parentheses):
+//   4096 -> 14336 (56)  48 / 64 / 80 tokens  29.6 / 30.1 / 30.8 and 28.7 / 30.2 / 32.0;  5120 -> 13824 (54)  64 / 80  32.7 / 34.5 and 33.5 / 35.3
+//   2048 -> 9216 (36)  48 / 64 / 96 tokens  16.4 / 16.5 / 17.4 and 14.6 / 15.9 / 18.8;  4096 -> 9216  160 tokens  27.5 and 40.3
+//   4096 -> 8192 (32)  201 / 224 / 240 / 256 tokens  30.0 / 30.5 / 31.4 / 31.7 and 27.2 / 28.2 / 36.4 / 37.2;  8192 -> 8192  224 / 256  46.8 / 50.1
+//   and 43.6 / 54.0;  2048 -> 7432 (30)  201 / 224 / 240  20.9 / 21.0 / 22.1 and 20.8 / 22.1 / 26.7;  4096 -> 6144 (24)  209 / 256  29.0 / 30.9 and
+//   25.9 / 30.8;  4096 -> 22016 (86, two rounds)  1 / 16 / 64 tokens  47.5 / 47.9 / 49.3 (no other kernel takes them in one launch)
+//   groups: 4096 -> 2 x 14336 (112, two rounds)  24 / 32 / 40 / 64 tokens  52.7 / 53.1 / 53.5 / 52.6 and 52.6 / 53.7 / 55.9 / 59.0;  4096 -> 2 x 11008 (86)
+//   32 / 48 / 64  50.8 / 50.1 / 50.7 and 46.2 / 50.6 / 51.9;  5120 -> 3 x 5120 (60)  112 / 128 / 144 tokens  43.8 / 43.9 / 45.7 and 41.8 / 43.1 / 46.8;
+//   4096 -> 3 x 4096 (48)  96 / 112 / 128  32.7 / 32.9 / 33.0 and 31.9 / 33.9 / 35.2;  4096 -> 4096 + 1024 + 1024 (24)  224 / 240  32.6 / 34.4 and 28.2 / 51.2
 bool decode_on_pairs(const meteora_shape_t& s, const int* d_outs, int G) {
     const Tuning& tn = tuning();
     if (s.T > kPairTokens || s.d_in < 2048 || tn.persist != 1 || tn.fused != 1 || tn.stream != 1) return false;
     if (!token_forward_supported(s)) return false;
     const PersistPlan pp = make_persist_plan(s, d_outs, G, false);
     if (!pp.ok) return false;
-    if (G > 1) return s.T >= (pp.tiles > pp.pairs ? 160 : pp.tiles > 32 ? 112 : 209);
-    return s.T >= (pp.tiles > pp.pairs ? 17 : pp.tiles > 32 ? 48 : pp.tiles > 28 ? 201 : 209);
+    if (G > 1) return s.T >= (pp.tiles > pp.pairs ? 40 : pp.tiles > 48 ? 129 : pp.tiles > 32 ? 112 : 225);
+    return s.T >= (pp.tiles > pp.pairs ? 17 : pp.tiles > 32 ? 48 : pp.tiles > 28 && s.d_in <= 2048 ? 201 : 225);
 }
 
 bool persist_supported(const meteora_shape_t& s) { return make_persist_plan(s, &s.d_out, 1, false).ok; }
@@ -1548,9 +1565,10 @@ static int launch_persist(const PersistPlan& pp, const void* x, const GroupModul
         const GroupModule& gm = mods[m < G ? m : 0];             // unused slots repeat module 0's (valid) maps
         if ((rc = get_tensor_map(gm.W0, s.d_in, gm.d_out, kBM, 0, &maps.W0[m])) != METEORA_OK) return rc;
         if ((rc = get_adapter_map(gm.B, s.N, gm.d_out, s.r, &maps.B[m])) != METEORA_OK) return rc;
-        if ((rc = get_tensor_map(gm.ws.us, gm.ws.ld_us, s.T, pp.BN / 2, 0, &maps.U[m])) != METEORA_OK) return rc;
+        const int parts = pp.stacked_pairs > 0 ? 1 : gm.ws.us_parts, ld_us = gm.ws.us_cols * parts;
+        if ((rc = get_tensor_map(gm.ws.us, ld_us, s.T, pp.BN / 2, 0, &maps.U[m])) != METEORA_OK) return rc;
         if ((rc = get_store_map(gm.y, gm.d_out, s.T, pp.CT, &maps.Y[m])) != METEORA_OK) return rc;
-        if ((rc = get_store_map(gm.ws.us, gm.ws.ld_us, s.T, 32, &maps.S[m], 32)) != METEORA_OK) return rc;
+        if ((rc = get_store_map(gm.ws.us, ld_us, s.T, 32, &maps.S[m], 32)) != METEORA_OK) return rc;
         maps.A[m] = maps.A0[m] = maps.G[m] = maps.X;
         if (pp.stacked_pairs > 0) {
             if ((rc = get_tensor_map(gm.A, s.d_in, s.N * s.r, kBM, 0, &maps.A[m])) != METEORA_OK) return rc;
@@ -1562,16 +1580,20 @@ static int launch_persist(const PersistPlan& pp, const void* x, const GroupModul
         mo.row_pairs = (mo.row_tiles + 1) / 2;
         mo.group_pairs = std::min(tuning().group_pairs > 0 ? tuning().group_pairs : std::max(1, (pp.pairs / pp.tok_tiles + 1) / 2), mo.row_pairs);
         mo.tile0 = m < G ? tile0 : 0x7FFFFFFF;
-        mo.us = (__nv_bfloat16*)gm.ws.us;
+        mo.parts = parts;
+        mo.us = (const __nv_bfloat16*)gm.ws.us;
         mo.topk_idx = gm.ws.topk_idx;
         mo.topk_w = gm.ws.topk_w;
+        mo.W0 = (const __nv_bfloat16*)gm.W0;
+        mo.B = (const __nv_bfloat16*)gm.B;
+        mo.d_out = gm.d_out;
         tile0 += mo.row_pairs * pp.tok_tiles;
     }
     p.T = s.T;
     p.BN = pp.BN;
     p.CT = pp.CT;
     p.ksteps = (s.d_in + kBK - 1) / kBK;
-    p.esteps = mods[0].ws.ld_us / kBK;
+    p.esteps = mods[0].ws.us_cols / kBK;
     p.N = s.N;
     p.r = s.r;
     p.k = s.k;
@@ -1585,11 +1607,12 @@ static int launch_persist(const PersistPlan& pp, const void* x, const GroupModul
     p.stacked_pairs = pp.stacked_pairs;
     p.gate_rows = pp.gate_rows;
     p.us_cols = pp.us_cols;
-    p.ld_us = mods[0].ws.ld_us;
     p.inv_tau = 1.0f / s.temperature;
     p.flags = flags;
     p.leave_ctr = status + 20;
     p.status = status;
+    p.x = (const __nv_bfloat16*)x;
+    p.d_in = s.d_in;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * pp.pairs);
     cfg.blockDim = dim3(kThreads);
@@ -2678,7 +2701,8 @@ int launch_token_forward(const void* x, const void* A, const void* Wg, const met
     p.topk_w = ws.topk_w;
     p.u = ws.uw;
     p.us = (__nv_bfloat16*)us;
-    p.ld_us = ws.ld_us;
+    p.us_cols = ws.us_cols;
+    p.us_parts = ws.us_parts;
     p.status = ws.status;
     p.late_wait = beside && tuning().pdl ? 1 : 0;
     return launch_token_tile(make_token_plan(s, TOKEN_FORWARD), TOKEN_FORWARD, s, x, Wg, A, p, st);
