@@ -127,8 +127,11 @@ static int forward_device(const void* x, const void* W0, const void* A, const vo
     if (!on_pairs && decode_stream_supported(s, &s.d_out, 1)) {
         if (timed) cudaEventRecord(pf.ev[2 * pf.used], st);
         rc = launch_decode_stream(x, &gm, 1, s, ws.status, ws.part_g, ws.tile_ctr, st);
-        if (timed) cudaEventRecord(pf.ev[2 * pf.used++ + 1], st);
-        return rc;
+        if (rc != kLaunchRefused) {
+            if (timed) cudaEventRecord(pf.ev[2 * pf.used++ + 1], st);
+            return rc;
+        }
+        tuning().fused_refused += 1;   // not all CTAs can be resident: the next kernel takes the call
     }
     if (!on_pairs && decode_fused_supported(s)) {
         if (timed) cudaEventRecord(pf.ev[2 * pf.used], st);
@@ -315,8 +318,11 @@ int meteora_linear_forward_group(const void* x, const void* const* W0, const voi
             if ((rc = launch_token_forward(x, A[m], Wg[m], *shape, gw.mod[m], gw.mod[m].us, m > 0, st)) != METEORA_OK) return rc;
         return launch_persist_base(x, gm, n_modules, *shape, gw.mod[0].status, gw.mod[0].tile_ctr, st);
     }
-    if (n_modules > 1 && decode_stream_supported(*shape, d_out, n_modules))
-        return launch_decode_stream(x, gm, n_modules, *shape, gw.mod[0].status, gw.part_g, gw.mod[0].tile_ctr, st);
+    if (n_modules > 1 && decode_stream_supported(*shape, d_out, n_modules)) {
+        rc = launch_decode_stream(x, gm, n_modules, *shape, gw.mod[0].status, gw.part_g, gw.mod[0].tile_ctr, st);
+        if (rc != kLaunchRefused) return rc;
+        tuning().fused_refused += 1;
+    }
     if (n_modules > 1 && decode_group_supported(*shape, d_out, n_modules)) {
         rc = launch_decode_group(x, gm, n_modules, *shape, gw.mod[0].status, gw.part_g, gw.mod[0].tile_ctr, st);
         if (rc != kLaunchRefused) return rc;

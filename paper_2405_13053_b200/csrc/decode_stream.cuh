@@ -10,7 +10,9 @@
 // therefore streams the next layer's weights while this layer exchanges partial tiles and stores y, and once
 // the call ahead has completed (griddepcontrol.wait) the CTA only adds the x tiles and runs from L2.
 //
-// Work split (no clusters, no co-residency requirement beyond "lower block indices are placed first"):
+// Work split (no clusters; all CTAs of a launch have to become resident, which a cooperative launch guarantees for groups and for
+// more than 128 tokens; one module of up to 128 tokens is launched without it and relies on the order of dispatch, so such calls
+// belong on one stream or on streams of equal priority):
 //   - aux CTAs (the lowest block indices): one 128-row tile of the stacked matrix [A_0..A_{N-1}; Wg] times one
 //     slice of the contraction axis each; the fp32 partial tile goes to scratch as one bulk copy; after a counter
 //     barrier among the aux CTAs a warp per token adds the slices in order, selects the top-k, applies the

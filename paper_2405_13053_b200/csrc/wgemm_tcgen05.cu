@@ -2292,8 +2292,7 @@ int launch_decode_stream(const void* x, const GroupModule* mods, int G, const me
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = sp.smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    const bool want_pdl = tuning().pdl_decode != 0;
+    cudaLaunchAttribute attr[3];
     int na = 0;
     if (sp.pair) {
         attr[na].id = cudaLaunchAttributeClusterDimension;
@@ -2302,6 +2301,18 @@ int launch_decode_stream(const void* x, const GroupModule* mods, int G, const me
         attr[na].val.clusterDim.z = 1;
         ++na;
     }
+    // The CTAs wait for one another: without the co-residency of a cooperative launch two such calls on two streams (of different
+    // priority, say) can hold a part of the SMs each.  It costs 1 - 2 us (4096 -> 4096 at 200 tokens 17.8 -> 19.3, with two modules of
+    // 1024 outputs at 64 tokens 16.4 -> 17.5: the next call's CTAs come when all SMs are free and not one by one), still
+    // ahead of the cooperative kernel for these shapes; one module of up to 128 tokens goes without, as it always has.
+    const bool coop = tuning().coop && (G > 1 || s.T > 128);
+    if (coop) {
+        attr[na].id = cudaLaunchAttributeCooperative;
+        attr[na].val.cooperative = 1;
+        ++na;
+    }
+    static std::atomic<bool> pdl_accepted{true};                 // together with a cooperative launch
+    const bool want_pdl = tuning().pdl_decode != 0 && (!coop || pdl_accepted.load(std::memory_order_relaxed));
     if (want_pdl) {
         attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[na].val.programmaticStreamSerializationAllowed = 1;
@@ -2314,8 +2325,23 @@ int launch_decode_stream(const void* x, const GroupModule* mods, int G, const me
     static int trace_calls = 0;
     d.trace_call = trace_calls++;
 #endif
-    if (sp.pair) return cuda_status(cudaLaunchKernelEx(&cfg, k_decode_stream<true>, maps, mX, mX1, d));
-    return cuda_status(cudaLaunchKernelEx(&cfg, k_decode_stream<false>, maps, mX, mX1, d));
+    auto launch = [&]() {
+        return sp.pair ? cudaLaunchKernelEx(&cfg, k_decode_stream<true>, maps, mX, mX1, d) : cudaLaunchKernelEx(&cfg, k_decode_stream<false>, maps, mX, mX1, d);
+    };
+    cudaError_t err = launch();
+    if (coop && want_pdl && launch_config_refused(err)) {        // the two attributes together: try without the second
+        cudaGetLastError();
+        pdl_accepted.store(false, std::memory_order_relaxed);
+        tuning().pdl_decode_refused += 1;
+        cfg.numAttrs = na - 1;
+        d.pdl = 0;
+        err = launch();
+    }
+    if (coop && launch_config_refused(err)) {                    // the caller may take another kernel instead
+        cudaGetLastError();
+        return kLaunchRefused;
+    }
+    return cuda_status(err);
 }
 
 // ------------------------------------------------------------------------------------------------
