@@ -40,6 +40,18 @@ void check(int status, const char* where) {
     throw PySet{};
 }
 
+// A call into the library with the GIL released, as ctypes makes it: a launch can block on a full queue and a copy of
+// pageable memory does, and other Python threads go on meanwhile.  Arguments are worked out before (under the GIL); the
+// caller's references keep their tensors.
+template <class Call>
+int released(Call&& call) {
+    struct Gil {
+        PyThreadState* state = PyEval_SaveThread();
+        ~Gil() { PyEval_RestoreThread(state); }
+    } gil;
+    return call();
+}
+
 const at::Tensor& tensor(PyObject* o, const char* name) {
     if (!THPVariable_Check(o)) fail(PyExc_TypeError, std::string(name) + " must be a torch.Tensor");
     return THPVariable_Unpack(o);
@@ -106,7 +118,8 @@ at::Tensor zeroed(size_t bytes, const at::Tensor& like, const char* where) {
     // (the header alone needs zeros: clearing all of it took 2 to 30 us of a decode call made without a workspace)
     if (bytes == 0) check(METEORA_ERR_INVALID_ARG, where);
     at::Tensor ws = empty({(int64_t)bytes}, at::kByte, like);
-    check(meteora_workspace_init(ws.data_ptr(), stream()), where);
+    void* const st = stream();
+    check(released([&] { return meteora_workspace_init(ws.data_ptr(), st); }), where);
     return ws;
 }
 
@@ -171,8 +184,10 @@ PyObject* gate_topk(PyObject* const* a) {
     void *px = dev(x, {T, d_in}, x.scalar_type(), "x"), *pg = dev(Wg, {N, d_in}, x.scalar_type(), "Wg");
     at::Tensor idx = empty({T, k}, at::kInt, x), w = empty({T, k}, at::kFloat, x), logits;
     if (want) logits = empty({T, N}, at::kFloat, x);
-    check(meteora_gate_topk(px, pg, &s, (int32_t*)idx.data_ptr(), (float*)w.data_ptr(), want ? (float*)logits.data_ptr() : nullptr, stream()),
-          "meteora_gate_topk");
+    int32_t* const pi = (int32_t*)idx.data_ptr();
+    float *const pw = (float*)w.data_ptr(), *const pl = want ? (float*)logits.data_ptr() : nullptr;
+    void* const st = stream();
+    check(released([&] { return meteora_gate_topk(px, pg, &s, pi, pw, pl, st); }), "meteora_gate_topk");
     return tuple(wrap(idx), wrap(w), want ? wrap(logits) : keep(Py_None));
 }
 
@@ -183,9 +198,9 @@ PyObject* route(PyObject* const* a) {
     const int64_t T = idx.size(0), k = idx.size(1), N = integer(a[1]);
     void* p = dev(idx, {T, k}, at::kInt, "topk_idx");
     at::Tensor counts = empty({N}, at::kInt, idx), offsets = empty({N + 1}, at::kInt, idx), perm = empty({T * k}, at::kInt, idx);
-    check(meteora_route((const int32_t*)p, (int)T, (int)k, (int)N, (int32_t*)counts.data_ptr(), (int32_t*)offsets.data_ptr(),
-                        (int32_t*)perm.data_ptr(), stream()),
-          "meteora_route");
+    int32_t *const pc = (int32_t*)counts.data_ptr(), *const po = (int32_t*)offsets.data_ptr(), *const pp = (int32_t*)perm.data_ptr();
+    void* const st = stream();
+    check(released([&] { return meteora_route((const int32_t*)p, (int)T, (int)k, (int)N, pc, po, pp, st); }), "meteora_route");
     return tuple(wrap(counts), wrap(offsets), wrap(perm));
 }
 
@@ -209,12 +224,14 @@ PyObject* lora_delta(PyObject* const* a) {
     const float* pw = (const float*)dev(a[4], {T, k}, at::kFloat, "topk_w");
     const int32_t* po = (const int32_t*)dev(a[5], {N + 1}, at::kInt, "offsets");
     const int32_t* pp = (const int32_t*)dev(a[6], {T * k}, at::kInt, "perm");
-    if (is_static)
-        check(meteora_lora_delta_static(px, pA, pB, pi, pw, po, pp, &s, (float*)dev(delta, {T, d_out}, at::kFloat, "delta"), stream()),
-              "meteora_lora_delta_static");
-    else
-        check(meteora_lora_delta(px, pA, pB, pi, pw, po, pp, &s, (float*)delta.data_ptr(), ws.data_ptr(), (size_t)ws.numel(), stream()),
-              "meteora_lora_delta");
+    float* const out = (float*)dev(delta, {T, d_out}, at::kFloat, "delta");
+    void *const pws = is_static ? nullptr : ws.data_ptr(), *const st = stream();
+    const size_t ws_bytes = is_static ? 0 : (size_t)ws.numel();
+    check(released([&] {
+              return is_static ? meteora_lora_delta_static(px, pA, pB, pi, pw, po, pp, &s, out, st)
+                               : meteora_lora_delta(px, pA, pB, pi, pw, po, pp, &s, out, pws, ws_bytes, st);
+          }),
+          is_static ? "meteora_lora_delta_static" : "meteora_lora_delta");
     return wrap(delta);
 }
 
@@ -231,10 +248,11 @@ PyObject* linear_forward(PyObject* const* a) {
     if (a[7] == Py_None) made_ws = zeroed(meteora_workspace_bytes(&s), x, "meteora_workspace_bytes");
     if (a[8] == Py_None) made_y = empty({T, d_out}, dt, x);
     const at::Tensor &ws = made_ws.defined() ? made_ws : tensor(a[7], "workspace"), &y = made_y.defined() ? made_y : tensor(a[8], "out");
-    check(meteora_linear_forward(dev(x, {T, d_in}, dt, "x"), dev(W0, {d_out, d_in}, dt, "W0"), dev(A, {N, r, d_in}, dt, "A"),
-                                 dev(a[3], {N, d_out, r}, dt, "B"), dev(a[4], {N, d_in}, dt, "Wg"), &s, dev(y, {T, d_out}, dt, "y"),
-                                 ws.data_ptr(), (size_t)ws.numel(), stream()),
-          "meteora_linear_forward");
+    const void *px = dev(x, {T, d_in}, dt, "x"), *pW = dev(W0, {d_out, d_in}, dt, "W0"), *pA = dev(A, {N, r, d_in}, dt, "A"),
+               *pB = dev(a[3], {N, d_out, r}, dt, "B"), *pG = dev(a[4], {N, d_in}, dt, "Wg");
+    void *const py = dev(y, {T, d_out}, dt, "y"), *const pws = ws.data_ptr(), *const st = stream();
+    const size_t ws_bytes = (size_t)ws.numel();
+    check(released([&] { return meteora_linear_forward(px, pW, pA, pB, pG, &s, py, pws, ws_bytes, st); }), "meteora_linear_forward");
     PyObject* y_obj = made_y.defined() ? wrap(y) : keep(a[8]);
     if (PyObject_IsTrue(a[9]) != 1) return y_obj;
     int32_t* p_idx = nullptr;
@@ -259,10 +277,11 @@ PyObject* linear_forward_host(PyObject* const* a) {
             fail(PyExc_ValueError, std::string(i ? "y_host" : "x_host") + " must be a contiguous host tensor of dtype " + c10::toString(dt));
     }
     if (y.dim() != 2 || y.size(0) != T || y.size(1) != d_out) fail(PyExc_ValueError, "y_host has the wrong shape");
-    check(meteora_linear_forward_host(x.data_ptr(), dev(W0, {d_out, d_in}, dt, "W0"), dev(A, {N, r, d_in}, dt, "A"),
-                                      dev(a[3], {N, d_out, r}, dt, "B"), dev(a[4], {N, d_in}, dt, "Wg"), &s, y.data_ptr(), ws.data_ptr(),
-                                      (size_t)ws.numel(), stream()),
-          "meteora_linear_forward_host");
+    const void *px = x.data_ptr(), *pW = dev(W0, {d_out, d_in}, dt, "W0"), *pA = dev(A, {N, r, d_in}, dt, "A"),
+               *pB = dev(a[3], {N, d_out, r}, dt, "B"), *pG = dev(a[4], {N, d_in}, dt, "Wg");
+    void *const py = y.data_ptr(), *const pws = ws.data_ptr(), *const st = stream();
+    const size_t ws_bytes = (size_t)ws.numel();
+    check(released([&] { return meteora_linear_forward_host(px, pW, pA, pB, pG, &s, py, pws, ws_bytes, st); }), "meteora_linear_forward_host");
     return keep(a[6]);
 }
 
@@ -284,10 +303,13 @@ PyObject* gate_backward(PyObject* const* a) {
     at::Tensor dWg = empty({N, d_in}, at::kFloat, x), dlogit = empty({T, k}, at::kFloat, x);
     const void* pB = bt ? dev(B, {N, r, d_out}, dt, "Bt") : dev(B, {N, d_out, r}, dt, "B");
     const auto fn = bt ? meteora_gate_backward_bt : meteora_gate_backward;
-    check(fn(dev(x, {T, d_in}, dt, "x"), dev(A, {N, r, d_in}, dt, "A"), pB, dev(a[3], {T, d_out}, dt, "dy"),
-             (const int32_t*)dev(idx, {T, k}, at::kInt, "topk_idx"), (const float*)dev(a[5], {T, k}, at::kFloat, "topk_w"), &s,
-             (float*)dlogit.data_ptr(), (float*)dWg.data_ptr(), ws.data_ptr(), (size_t)ws.numel(), stream()),
-          "meteora_gate_backward");
+    const void *px = dev(x, {T, d_in}, dt, "x"), *pA = dev(A, {N, r, d_in}, dt, "A"), *pdy = dev(a[3], {T, d_out}, dt, "dy");
+    const int32_t* pi = (const int32_t*)dev(idx, {T, k}, at::kInt, "topk_idx");
+    const float* pw = (const float*)dev(a[5], {T, k}, at::kFloat, "topk_w");
+    float *const pl = (float*)dlogit.data_ptr(), *const pd = (float*)dWg.data_ptr();
+    void *const pws = ws.data_ptr(), *const st = stream();
+    const size_t ws_bytes = (size_t)ws.numel();
+    check(released([&] { return fn(px, pA, pB, pdy, pi, pw, &s, pl, pd, pws, ws_bytes, st); }), "meteora_gate_backward");
     return tuple(wrap(dWg), wrap(dlogit));
 }
 
@@ -323,7 +345,8 @@ PyObject* linear_forward_group(PyObject* const* a) {
     const meteora_shape_t s = make_shape(T, d_in, d_out[0], N, r, k, code, temperature);
     at::Tensor ws = a[7] == Py_None ? zeroed(meteora_group_workspace_bytes(&s, d_out.data(), (int)G), x, "meteora_group_workspace_bytes")
                                     : tensor(a[7], "workspace");
-    std::vector<at::Tensor> ys(G);
+    std::vector<at::Tensor> ys(G), held;                             // (held: another thread may change the lists meanwhile)
+    held.reserve(4 * G);
     std::vector<const void*> ptr[4];
     for (auto& p : ptr) p.resize(G);
     std::vector<void*> py(G);
@@ -334,9 +357,15 @@ PyObject* linear_forward_group(PyObject* const* a) {
         ptr[1][m] = dev(item(1, m), {N, r, d_in}, dt, "A");
         ptr[2][m] = dev(item(2, m), {N, d_out[m], r}, dt, "B");
         ptr[3][m] = dev(item(3, m), {N, d_in}, dt, "Wg");
+        for (int i = 0; i < 4; ++i) held.push_back(item(i, m));
     }
-    check(meteora_linear_forward_group(dev(x, {T, d_in}, dt, "x"), ptr[0].data(), ptr[1].data(), ptr[2].data(), ptr[3].data(), d_out.data(),
-                                       (int)G, &s, py.data(), ws.data_ptr(), (size_t)ws.numel(), stream()),
+    const void* px = dev(x, {T, d_in}, dt, "x");
+    void *const pws = ws.data_ptr(), *const st = stream();
+    const size_t ws_bytes = (size_t)ws.numel();
+    check(released([&] {
+              return meteora_linear_forward_group(px, ptr[0].data(), ptr[1].data(), ptr[2].data(), ptr[3].data(), d_out.data(), (int)G, &s,
+                                                  py.data(), pws, ws_bytes, st);
+          }),
           "meteora_linear_forward_group");
     PyObject* out = PyList_New(G);
     if (!out) throw PySet{};
