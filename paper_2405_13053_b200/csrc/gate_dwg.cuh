@@ -9,7 +9,7 @@
 // it, and the parts are separate rows of the MMA's M axis: up to 42 adapters make 126 of its 128 rows, so the split
 // costs nothing.  x is read as it lies: columns contiguous, i.e. the MN-major form of the B operand.  A CTA takes 256
 // columns and a share of the tokens and writes its result; with more than one share a second kernel adds them in
-// order, so every run gives the same bits.
+// order, so every run gives the same bits.  Slots of one token that name the same adapter share an element of L: their sum.
 //
 // Bound by reading x once (16.8 MB at 2048 tokens x 4096) and the latency of building L and of the second launch.
 #pragma once
@@ -23,6 +23,7 @@ constexpr int kDwgStages = 4;
 constexpr int kDwgLBytes = kBM * kDwgTok * 2;       // L tile: 128 rows x 64 tokens of bf16, K-major, 128-byte swizzle
 constexpr int kDwgMaxN = kBM / 3;
 constexpr int kDwgSlots = 4096;                     // slots whose dlogit a CTA holds at a time (whole blocks of 64 tokens)
+constexpr uint32_t kDwgTaken = 0x7FE0ED0Eu;         // (a NaN that no sum gives) the token's adapter is with an earlier slot
 constexpr int kDwgMaxShares = 16;                   // shares of the tokens: bounds the scratch
 
 struct GateDwgParams {
@@ -135,33 +136,45 @@ k_gate_dwg_tc(const __grid_constant__ CUtensorMap tmX, const GateDwgParams p) {
         float* s_g = reinterpret_cast<float*>(ring_ptr + kDwgStages * kStage + 256);
         float* s_dl = s_g + kDwgSlots;
         const int chunk = kDwgSlots / (kDwgTok * p.k);               // blocks per pass over u and z (k <= 8: 8 at the least)
-        for (int i = 0; i < nb; ++i) {
-            if (i % chunk == 0) {
-                const size_t s0 = (size_t)(b0 + i) * kDwgTok * p.k;
-                const int slots = min(min(chunk, nb - i) * kDwgTok, p.T - (b0 + i) * kDwgTok) * p.k;
-                for (int q = etid; q < slots; q += kEpiThreads) {
-                    const float4 *up = reinterpret_cast<const float4*>(p.u + (s0 + q) * p.r), *zp = reinterpret_cast<const float4*>(p.z + (s0 + q) * p.r);
-                    float g = 0.f;
+        auto dlogits = [&](int i) {                                  // of the chunk whose first block is i, to s_dl
+            const size_t s0 = (size_t)(b0 + i) * kDwgTok * p.k;
+            const int slots = min(min(chunk, nb - i) * kDwgTok, p.T - (b0 + i) * kDwgTok) * p.k;
+            for (int q = etid; q < slots; q += kEpiThreads) {
+                const float4 *up = reinterpret_cast<const float4*>(p.u + (s0 + q) * p.r), *zp = reinterpret_cast<const float4*>(p.z + (s0 + q) * p.r);
+                float g = 0.f;
 #pragma unroll 2
-                    for (int c = 0; c < p.r / 4; ++c) {
-                        const float4 a = up[c], b = zp[c];
-                        g = fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, g))));
-                    }
-                    s_g[q] = g;
+                for (int c = 0; c < p.r / 4; ++c) {
+                    const float4 a = up[c], b = zp[c];
+                    g = fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, g))));
                 }
-                __syncwarp();
-                epi_barrier();
-                for (int q = etid; q < slots; q += kEpiThreads) {
-                    const int first = q / p.k * p.k;
-                    float mean = 0.f;
-                    for (int m = 0; m < p.k; ++m) mean = fmaf(p.topk_w[s0 + first + m], s_g[first + m], mean);
-                    const float v = p.topk_w[s0 + q] * (s_g[q] - mean) * p.inv_tau;
-                    s_dl[q] = v;
-                    if (p.dlogit && blockIdx.x == 0) p.dlogit[s0 + q] = v;
-                }
-                __syncwarp();
-                epi_barrier();
+                s_g[q] = g;
             }
+            __syncwarp();
+            epi_barrier();
+            for (int q = etid; q < slots; q += kEpiThreads) {
+                const int first = q / p.k * p.k, e = min(max(p.topk_idx[s0 + q], 0), p.N - 1);
+                uint32_t same = 0;                                   // picks of the token that name this slot's adapter
+                float mean = 0.f;
+                for (int m = 0; m < p.k; ++m) {
+                    mean = fmaf(p.topk_w[s0 + first + m], s_g[first + m], mean);
+                    if (min(max(p.topk_idx[s0 + first + m], 0), p.N - 1) == e) same |= 1u << m;
+                }
+                const float v = p.topk_w[s0 + q] * (s_g[q] - mean) * p.inv_tau;
+                if (p.dlogit && blockIdx.x == 0) p.dlogit[s0 + q] = v;
+                float sum = v;
+                if (same & (same - 1u)) {                            // more than one: the first has their sum
+                    sum = 0.f;
+                    for (int m = 0; m < p.k; ++m)
+                        if (same >> m & 1u) sum += p.topk_w[s0 + first + m] * (s_g[first + m] - mean) * p.inv_tau;
+                    if (same & ((1u << (q - first)) - 1u)) sum = __uint_as_float(kDwgTaken);
+                }
+                s_dl[q] = sum;
+            }
+            __syncwarp();
+            epi_barrier();
+        };
+        for (int i = 0; i < nb; ++i) {
+            if (i % chunk == 0) dlogits(i);
             const int s = i % kDwgStages, round = i / kDwgStages;
             if (round > 0) ok = ok && mbar_wait(bar_free + s * 8, (round & 1) ^ 1);
             uint8_t* L = ring_ptr + s * kStage + kDwgXBytes;
@@ -180,6 +193,7 @@ k_gate_dwg_tc(const __grid_constant__ CUtensorMap tmX, const GateDwgParams p) {
                 if (e_i[h] < 0) continue;
                 const int q = etid + h * kEpiThreads, tok = q / p.k;
                 float v = s_dl[(i % chunk) * kDwgTok * p.k + q];
+                if (__float_as_uint(v) == kDwgTaken) continue;
 #pragma unroll
                 for (int part = 0; part < 3; ++part) {
                     const __nv_bfloat16 b = __float2bfloat16_rn(v);

@@ -81,3 +81,35 @@ def test_gate_backward_argument_errors():
     assert lib.meteora_gate_backward_bt(p, p, p, p, p, p, ctypes.byref(shape), None, p, p, 64, None) == -4
     assert lib.meteora_transpose_adapters_b(None, ctypes.byref(shape), p, None) == -1
     assert lib.meteora_adapters_bt_bytes(ctypes.byref(shape)) == 8 * 64 * 8 * 2
+
+
+def _slot_sums(x, A, B, dy, idx, wts, temperature):
+    """dlogit and dWg in fp64, slot by slot; indices out of range count as the nearest adapter."""
+    e = idx.long().clamp(0, A.shape[0] - 1)
+    xd, dyd = x.double(), dy.double()
+    u = torch.einsum("td,nrd->tnr", xd, A.double())
+    z = torch.einsum("to,nor->tnr", dyd, B.double())
+    g = (u * z).sum(2).gather(1, e)
+    dlogit = wts.double() * (g - (wts.double() * g).sum(1, keepdim=True)) / temperature
+    dWg = torch.zeros(A.shape[0], x.shape[1], dtype=torch.double, device=x.device)
+    for j in range(idx.shape[1]):
+        dWg.index_add_(0, e[:, j], dlogit[:, j:j + 1] * xd)
+    return dlogit, dWg
+
+
+@pytest.mark.parametrize("T,N,k,r", [(5, 3, 3, 8), (70, 28, 3, 8), (300, 8, 8, 8), (700, 42, 4, 16), (200, 60, 3, 8)])
+def test_gate_backward_sums_repeated_picks(T, N, k, r):
+    # routing of the caller's own: adapters that a token names more than once (also after clamping) add up
+    g = torch.Generator(device="cuda").manual_seed(T)
+    rand = lambda *s: torch.randn(*s, device="cuda", generator=g)  # noqa: E731
+    d_in, d_out = 520, 264
+    x, dy = rand(T, d_in).bfloat16(), rand(T, d_out).bfloat16()
+    A, B = (rand(N, r, d_in) / d_in ** 0.5).bfloat16(), (0.3 * rand(N, d_out, r)).bfloat16()
+    low, high = (0, N) if N > 42 else (-2, N + 2)
+    idx = torch.randint(low, high, (T, k), device="cuda", generator=g, dtype=torch.int32)
+    idx[::3, 1] = idx[::3, 0]
+    wts = torch.softmax(rand(T, k), dim=1)
+    dWg, dlogit = mb.meteora_gate_backward(x, A, B, dy, idx, wts, 1.5)
+    o_dlogit, o_dWg = _slot_sums(x, A, B, dy, idx, wts, 1.5)
+    assert rel_l2(dlogit.cpu().numpy(), o_dlogit.cpu().numpy()) <= TOL["bf16"]
+    assert rel_l2(dWg.cpu().numpy(), o_dWg.cpu().numpy()) <= TOL["bf16"]
