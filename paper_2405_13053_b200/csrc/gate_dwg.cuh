@@ -10,6 +10,8 @@
 // costs nothing.  x is read as it lies: columns contiguous, i.e. the MN-major form of the B operand.  A CTA takes 256
 // columns and a share of the tokens and writes its result; with more than one share a second kernel adds them in
 // order, so every run gives the same bits.  Slots of one token that name the same adapter share an element of L: their sum.
+// The product multiplies the zeros of L too, and 0 times an infinity or a NaN in x is NaN: a column with a NaN is summed again
+// from the slots alone, so that such a token reaches the rows of its own picks only.
 //
 // Bound by reading x once (16.8 MB at 2048 tokens x 4096) and the latency of building L and of the second launch.
 #pragma once
@@ -34,6 +36,7 @@ struct GateDwgParams {
     const float* topk_w;
     const float* u;            // [slot][r]
     const float* z;
+    const __nv_bfloat16* x;    // (for the columns that are summed again)
     float* dlogit;             // optional out
     float* out;                // [share][N][d_in]
     int32_t* status;
@@ -42,6 +45,7 @@ struct GateDwgParams {
 __global__ void __launch_bounds__(kThreads)
 k_gate_dwg_tc(const __grid_constant__ CUtensorMap tmX, const GateDwgParams p) {
     extern __shared__ uint8_t smem_raw[];
+    __shared__ int s_odd;                               // 1: some result is NaN, 2: a wait has expired
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t ring = (raw + 1023u) & ~1023u;
     uint8_t* ring_ptr = smem_raw + (ring - raw);
@@ -62,6 +66,7 @@ k_gate_dwg_tc(const __grid_constant__ CUtensorMap tmX, const GateDwgParams p) {
             mbar_init(bar_free + s * 8, 1);
         }
         mbar_init(bar_acc, 1);
+        s_odd = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -231,13 +236,36 @@ k_gate_dwg_tc(const __grid_constant__ CUtensorMap tmX, const GateDwgParams p) {
 #pragma unroll
             for (int i = 0; i < 16; ++i) acc[(c0 + i) * pitch + row] = v[i];
         }
+        if (!acc_ok && lane == 0) atomicOr(&s_odd, 2);
         __syncwarp();
         epi_barrier();
+        float* a = acc + etid * pitch;
+        float* dst = p.out + (size_t)blockIdx.y * p.N * p.d_in + col0 + etid;
+        bool nan = false;
         if (col0 + etid < p.d_in) {
-            const float* a = acc + etid * pitch;
-            float* dst = p.out + (size_t)blockIdx.y * p.N * p.d_in + col0 + etid;
 #pragma unroll 4
-            for (int e = 0; e < p.N; ++e) dst[(size_t)e * p.d_in] = a[e] + (a[p.N + e] + a[2 * p.N + e]);
+            for (int e = 0; e < p.N; ++e) {
+                const float v = a[e] + (a[p.N + e] + a[2 * p.N + e]);
+                nan |= v != v;
+                dst[(size_t)e * p.d_in] = v;
+            }
+        }
+        if (nan) atomicOr(&s_odd, 1);
+        __syncwarp();
+        epi_barrier();
+        if (s_odd == 1) {                                            // (with an expired wait the NaNs stay)
+            for (int e = 0; e < p.N; ++e) a[e] = 0.f;                // this thread's column
+            for (int i = 0; i < nb; i += chunk) {
+                dlogits(i);
+                const int t0 = (b0 + i) * kDwgTok, slots = min(min(chunk, nb - i) * kDwgTok, p.T - t0) * p.k;
+                for (int q = 0; nan && q < slots; ++q) {
+                    const int e = min(max(p.topk_idx[(size_t)t0 * p.k + q], 0), p.N - 1);
+                    if (__float_as_uint(s_dl[q]) != kDwgTaken) a[e] = fmaf(s_dl[q], to_f32(p.x[(size_t)(t0 + q / p.k) * p.d_in + col0 + etid]), a[e]);
+                }
+                __syncwarp();
+                epi_barrier();                                       // s_dl is read before the next chunk's is written
+            }
+            for (int e = 0; nan && e < p.N; ++e) dst[(size_t)e * p.d_in] = a[e];
         }
     }
     __syncwarp();

@@ -2784,6 +2784,7 @@ int launch_gate_dwg_tc(const void* x, const int32_t* topk_idx, const float* topk
     p.topk_w = topk_w;
     p.u = u;
     p.z = z;
+    p.x = (const __nv_bfloat16*)x;
     p.r = s.r;
     p.inv_tau = 1.0f / s.temperature;
     p.dlogit = dlogit;

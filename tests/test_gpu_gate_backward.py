@@ -113,3 +113,22 @@ def test_gate_backward_sums_repeated_picks(T, N, k, r):
     o_dlogit, o_dWg = _slot_sums(x, A, B, dy, idx, wts, 1.5)
     assert rel_l2(dlogit.cpu().numpy(), o_dlogit.cpu().numpy()) <= TOL["bf16"]
     assert rel_l2(dWg.cpu().numpy(), o_dWg.cpu().numpy()) <= TOL["bf16"]
+
+
+@pytest.mark.parametrize("T", [40, 300, 2000])
+def test_gate_backward_keeps_a_non_finite_token_to_its_own_picks(T):
+    g = torch.Generator(device="cuda").manual_seed(T)
+    rand = lambda *s: torch.randn(*s, device="cuda", generator=g)  # noqa: E731
+    N, r, k, d_in, d_out = 28, 8, 2, 776, 256
+    x, dy = rand(T, d_in).bfloat16(), rand(T, d_out).bfloat16()
+    A, B = (rand(N, r, d_in) / d_in ** 0.5).bfloat16(), (0.3 * rand(N, d_out, r)).bfloat16()
+    idx = torch.stack([torch.randperm(N, device="cuda", generator=g)[:k] for _ in range(T)]).int()
+    wts = torch.softmax(rand(T, k), dim=1)
+    clean, _ = mb.meteora_gate_backward(x, A, B, dy, idx, wts)
+    x[T // 2, 3], x[T // 2, 700] = float("inf"), float("nan")
+    dWg, _ = mb.meteora_gate_backward(x, A, B, dy, idx, wts)
+    own = torch.zeros(N, dtype=torch.bool, device="cuda")
+    own[idx[T // 2].long()] = True
+    assert torch.isnan(dWg[own]).all()                    # its dlogit is NaN
+    # the others: the same fp32 sums, in another order where a column was summed again
+    assert rel_l2(dWg[~own].cpu().numpy(), clean[~own].cpu().numpy()) <= 1e-6
