@@ -13,6 +13,7 @@
 #include "select.cuh"
 
 #include <algorithm>
+#include <cmath>
 
 namespace meteora {
 
@@ -238,8 +239,11 @@ k_simt_finish(const TI* __restrict__ B, const SimtParams p, int zsplits, int r, 
 // per SM (2048 -> 2048, partial products at 1 / 512 tokens with one, two, three, four CTAs per SM: 17.6 / 12.5 / 11.2 / 10.5
 // and 142 / 120 / 114 / 114 us), each of two chunks at the least, and no more than 8 of a short axis: the second launch
 // adds them (512 -> 2000, 33 tokens: 11.4 us with 8, 13.0 with 13).
+// A large batch goes in blocks of tokens that share the scratch of one (a copy for all of 8192 tokens x 14336 outputs would be 478
+// MB): up to 128 MB and at least two waves of three CTAs per SM, the block whose last wave is fullest.  There is one slice then,
+// so the sums are the same.
 struct SimtPlan {
-    int bm, bn, z, ldp;
+    int bm, bn, z, ldp, tokens;                                     // tokens per block
 };
 static SimtPlan simt_plan(const meteora_shape_t& s) {
     SimtPlan sp;
@@ -251,42 +255,56 @@ static SimtPlan simt_plan(const meteora_shape_t& s) {
     const int cap = std::min(std::min(kSimtMaxSlices, chunks / 2), std::max(8, chunks / 8));
     sp.z = (int)std::max<long long>(1, std::min<long long>(cap, 444 / tiles(sp.bm, sp.bn)));
     sp.ldp = (int)align_up((size_t)rows, 4);
+    sp.tokens = s.T;
+    const long long row_tiles = (rows + sp.bm - 1) / sp.bm, least = (888 + row_tiles - 1) / row_tiles;
+    const long long most = std::max(least, ((long long)128 << 20) / (4LL * sp.ldp) / 64);   // tiles of 64 tokens
+    if (s.T > 64 * most) {
+        double fullest = 0.0;
+        for (long long n = least; n <= std::min(most, least + 64); ++n) {
+            const double waves = (double)(row_tiles * n) / 444, full = waves / std::ceil(waves);
+            if (full >= fullest) {
+                fullest = full;
+                sp.tokens = (int)(64 * n);
+            }
+        }
+    }
     return sp;
 }
 
 size_t simt_part_floats(const meteora_shape_t& s) {
     const SimtPlan sp = simt_plan(s);
-    return (size_t)sp.z * s.T * sp.ldp;
+    return (size_t)sp.z * sp.tokens * sp.ldp;
 }
 
+// Tokens [t0, t0 + n) of the batch.
 template <typename TI>
-static int launch_simt(const void* x, const void* W0, const void* A, const void* B, const void* Wg, const meteora_shape_t& s,
-                       const Workspace& ws, void* y, cudaStream_t st) {
-    const SimtPlan sp = simt_plan(s);
+static int launch_simt_block(const SimtPlan& sp, const TI* x, const TI* W0, const TI* A, const TI* B, const TI* Wg, const meteora_shape_t& s,
+                             const Workspace& ws, TI* y, int t0, int n, cudaStream_t st) {
     SimtParams p = {};
-    p.T = s.T;
+    p.T = n;
     p.d_in = s.d_in;
     p.d_out = s.d_out;
     p.a_rows = s.N * s.r;
     p.N = s.N;
     p.ldp = sp.ldp;
-    p.zstride = (size_t)s.T * sp.ldp;
+    p.zstride = (size_t)n * sp.ldp;
     p.part = ws.simt_part;
-    const dim3 grid((s.T + sp.bn - 1) / sp.bn, (s.d_out + p.a_rows + s.N + sp.bm - 1) / sp.bm, sp.z);
-    const TI *xp = (const TI*)x, *wp = (const TI*)W0, *ap = (const TI*)A, *gp = (const TI*)Wg;
+    x += (size_t)t0 * s.d_in;
+    const dim3 grid((n + sp.bn - 1) / sp.bn, (s.d_out + p.a_rows + s.N + sp.bm - 1) / sp.bm, sp.z);
+    // (no dependent launch: the block before has been finished when this one's products overwrite the scratch)
     if (sp.bn == 16)
-        k_simt_partial<TI, 64, 16, 4, 2><<<grid, 128, 0, st>>>(xp, wp, ap, gp, p);
+        k_simt_partial<TI, 64, 16, 4, 2><<<grid, 128, 0, st>>>(x, W0, A, Wg, p);
     else if (sp.bm == 64)
-        k_simt_partial<TI, 64, 64, 8, 4><<<grid, 128, 0, st>>>(xp, wp, ap, gp, p);
+        k_simt_partial<TI, 64, 64, 8, 4><<<grid, 128, 0, st>>>(x, W0, A, Wg, p);
     else
-        k_simt_partial<TI, 128, 64, 8, 8><<<grid, 128, 0, st>>>(xp, wp, ap, gp, p);
+        k_simt_partial<TI, 128, 64, 8, 8><<<grid, 128, 0, st>>>(x, W0, A, Wg, p);
     const int rc = last_launch_status();
     if (rc != METEORA_OK) return rc;
     cudaLaunchConfig_t cfg = {};
     // one token per CTA while that leaves at most four CTAs of 256 threads per SM, else four
     const int row_blocks = (s.d_out + 255) / 256;
-    const bool one = (long long)s.T * row_blocks <= 592;
-    cfg.gridDim = dim3(one ? s.T : (s.T + 3) / 4, row_blocks);
+    const bool one = (long long)n * row_blocks <= 592;
+    cfg.gridDim = dim3(one ? n : (n + 3) / 4, row_blocks);
     cfg.blockDim = dim3(256);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -294,8 +312,20 @@ static int launch_simt(const void* x, const void* W0, const void* A, const void*
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = tuning().pdl ? 1 : 0;
-    return cuda_status(cudaLaunchKernelEx(&cfg, one ? k_simt_finish<TI, 1> : k_simt_finish<TI, 4>, (const TI*)B, (const SimtParams)p, sp.z, s.r, s.k, 1.0f / s.temperature,
-                                          (TI*)y, ws.topk_idx, ws.topk_w));
+    return cuda_status(cudaLaunchKernelEx(&cfg, one ? k_simt_finish<TI, 1> : k_simt_finish<TI, 4>, B, (const SimtParams)p, sp.z, s.r, s.k,
+                                          1.0f / s.temperature, y + (size_t)t0 * s.d_out, ws.topk_idx + (size_t)t0 * s.k,
+                                          ws.topk_w + (size_t)t0 * s.k));
+}
+
+template <typename TI>
+static int launch_simt(const void* x, const void* W0, const void* A, const void* B, const void* Wg, const meteora_shape_t& s,
+                       const Workspace& ws, void* y, cudaStream_t st) {
+    const SimtPlan sp = simt_plan(s);
+    int rc = METEORA_OK;
+    for (int t0 = 0; t0 < s.T && rc == METEORA_OK; t0 += sp.tokens)
+        rc = launch_simt_block<TI>(sp, (const TI*)x, (const TI*)W0, (const TI*)A, (const TI*)B, (const TI*)Wg, s, ws, (TI*)y, t0,
+                                   std::min(sp.tokens, s.T - t0), st);
+    return rc;
 }
 
 int launch_forward_simt(const void* x, const void* W0, const void* A, const void* B, const void* Wg, const meteora_shape_t& s,

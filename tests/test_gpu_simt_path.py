@@ -22,6 +22,8 @@ pytestmark = pytest.mark.gpu
     (40, 1030, 100, 28, 64, 2, "f32"),        # the largest rank
     (33, 1027, 300, 28, 8, 2, "bf16"),        # bf16 rows of odd length
     (8, 2050, 130, 28, 5, 2, "bf16"),
+    (8300, 20, 4000, 4, 8, 2, "f32"),         # several blocks of tokens on the same scratch
+    (2300, 36, 30000, 4, 8, 1, "bf16"),
 ])
 def test_plain_path_matches_oracle(T, d_in, d_out, N, r, k, dtype):
     w = workloads.make_workload("simt", T=T, d_in=d_in, d_out=d_out, N=N, r=r, k=k, dtype=dtype, seed=40 + T, b_std=0.3)

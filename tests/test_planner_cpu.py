@@ -70,3 +70,12 @@ def test_shapes_the_tensor_cores_do_not_take():
     assert plan(32, 4096, 4096, dtype=torch.float32) == "path=simt" or "path=simt" in plan(32, 4096, 4096, dtype=torch.float32)
     assert "path=simt" in plan(33, 60, 50, N=6, r=4)            # d_in no multiple of 8
     assert "path=stream_decode" in plan(30, 512, 384, r=4)      # rank 4 on the tensor cores, padded to 8
+
+
+@pytest.mark.parametrize("T,d_in,d_out", [(8192, 4096, 14336), (65536, 1024, 8192), (200000, 2048, 250)])
+def test_scratch_of_the_plain_path_does_not_grow_with_the_batch(T, d_in, d_out):
+    """Beside the host entry point's staging, the routing and u_all (about 3 KB per token) the workspace holds the products
+    of one block of tokens, not of all."""
+    N, r = 28, 8
+    n = mb.meteora_workspace_bytes(mb.make_shape(T, d_in, d_out, N, r, 2, torch.float32))
+    assert n < T * (4 * (d_in + d_out) + 3072) + (160 << 20)
