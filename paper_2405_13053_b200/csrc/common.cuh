@@ -247,7 +247,9 @@ __device__ __forceinline__ void store_us(__nv_bfloat16* row, int c, int cols, in
         row[c] = __float2bfloat16_rn(v);
         return;
     }
-    for (int i = 0; i < parts; ++i) row[(size_t)i * cols + c] = take_bf16_part(v);
+    row[c] = take_bf16_part(v);                                      // (no loop: it would keep the callers' loads from overlapping)
+    row[c + cols] = take_bf16_part(v);
+    row[c + 2 * cols] = take_bf16_part(v);
 }
 
 __device__ __forceinline__ float warp_sum(float v) {
