@@ -224,9 +224,9 @@ def whole_job_value(modules, tokens, world, steps, ms_total):
 
 def prefill_line(mb, lib, tc_peak, tc_kind, hbm_peak):
     """One prefill figure for the default line (the headline workload is a decode batch and HBM-bound): config 2's
-    gate/up shape, 4096 -> 14336 with 2048 tokens from 4 clusters, the whole MeteoRA linear per call (three or four launches:
-    stacked shrink, selection, base product with the expand) against the sustained bf16 tensor peak, and the
-    base-product kernel alone from event pairs around its launches."""
+    gate/up shape, 4096 -> 14336 with 2048 tokens from 4 clusters, the whole MeteoRA linear per call (one launch of persistent
+    pairs of SMs) against the sustained bf16 tensor peak, and the kernel with the base product from event pairs around its
+    launches."""
     import ctypes
 
     import torch
@@ -444,11 +444,11 @@ def run_ours(args):
     # ---- dominant kernel.  Which kernels a call launches depends on the shape (meteora_describe_plan):
     #   single-launch decode kernel: one launch is the whole call, so its average duration over the timed region
     #     is the graph-replayed region itself divided by the launches (idle gaps between launches included);
-    #   three-launch chain: event pairs around the base-product launch of every call, in a second region of the
+    #   otherwise: event pairs around the base-product launch of every call, in a second region of the
     #     same launches issued behind a long blocker kernel so that the host is never the bottleneck.
     plan = mb.meteora_describe_plan(shape)
     single_launch = "path=fused_decode" in plan or "path=stream_decode" in plan
-    launches_per_call = 1 if single_launch else 3
+    launches_per_call = 1 if single_launch else int(plan.split("launches=")[1].split()[0]) if "launches=" in plan else 2
     if single_launch:
         kernel_name = ("k_decode_stream" if "path=stream_decode" in plan else "k_decode_fused") + \
             " (base product + stacked shrink + selection + LoRA expand, one launch per call)"
@@ -709,8 +709,7 @@ def run_layer_sweep():
                            "W0": vpa(*[m["W0"].data_ptr() for m in ms]), "A": vpa(*[m["A"].data_ptr() for m in ms]),
                            "B": vpa(*[m["B"].data_ptr() for m in ms]), "Wg": vpa(*[m["Wg"].data_ptr() for m in ms]),
                            "y": vpa(*[m["y"].data_ptr() for m in ms]),
-                           "ws": torch.zeros(n, dtype=torch.uint8, device="cuda"),
-                           "one_launch": lib.meteora_group_plan(ctypes.byref(ms[0]["shape"]), d_outs, G)})
+                           "ws": torch.zeros(n, dtype=torch.uint8, device="cuda")})
 
         def step_groups():
             for gq in groups:
@@ -754,9 +753,7 @@ def run_layer_sweep():
                               "frac_of_roofline": round(max(t_mem, t_tc) / us, 3),
                               "achieved": round(nbytes / us / 1e3, 1) if bound == "hbm" else round(flops / us / 1e6, 1),
                               "unit": "GB/s" if bound == "hbm" else "TFLOP/s",
-                              "launches": (sum(1 if gq["one_launch"] else 3 * gq["G"] if T > 256 else gq["G"]
-                                               for gq in groups) if step is step_groups
-                                           else len(mods) * (3 if T > 256 else 1)),
+                              "calls": len(groups) if step is step_groups else len(mods),
                               "l2": "436 MB of W0 per layer: no weight survives in the 126 MB L2 until its next visit"}),
                   flush=True)
         del mods, graph, groups
@@ -852,11 +849,8 @@ def run_layer():
 
 
 def run_standalone_sweep():
-    """The standalone entry points (gate + top-k, bucketing, LoRA term by per-adapter segments) at config 1 (T = 128) and
-    config 2 (4096 -> 14336, T = 2048), each against the HBM time of its algorithmic bytes, beside what the fused
-    forward spends on the same job with the stacked dense shrink [A; Wg] x on the tensor cores plus the selection
-    (time of a three-launch call minus its base-product launch).  This is the measured side of "per-adapter segments
-    or one stacked dense shrink" (Sec. 3.3's gather against Eq. 5's batched view)."""
+    """The standalone entry points (gate + top-k, bucketing, LoRA term) at config 1 (T = 128) and config 2 (4096 -> 14336,
+    T = 2048), each against the HBM time of its algorithmic bytes."""
     import torch
 
     from paper_2405_13053_b200 import binding as mb
@@ -886,7 +880,6 @@ def run_standalone_sweep():
     for cfg, d_in, d_out, T, x_kind in (("config1", 4096, 4096, 128, "rms"), ("config2", 4096, 14336, 2048, "clusters")):
         g = torch.Generator(device="cuda").manual_seed(9)
         x = torch.from_numpy(workloads.make_x(T, d_in, x_kind, 5, "bf16")).to(dt).cuda()
-        W0 = (0.02 * torch.randn(d_out, d_in, device="cuda", generator=g)).to(dt)
         A = ((torch.rand(N_ADAPTERS, RANK, d_in, device="cuda", generator=g) * 2 - 1) / d_in ** 0.5).to(dt)
         B = (0.01 * torch.randn(N_ADAPTERS, d_out, RANK, device="cuda", generator=g)).to(dt)
         Wg = (torch.randn(N_ADAPTERS, d_in, device="cuda", generator=g) / d_in ** 0.5).to(dt)
@@ -898,41 +891,20 @@ def run_standalone_sweep():
         touched = int((counts > 0).sum().item())
         rows = []
         us = timed_us(lambda: mb.meteora_gate_topk(x, Wg, TOPK))
-        rows.append(("meteora_gate_topk (k_gate_topk)", us, (T * d_in + N_ADAPTERS * d_in) * es + T * TOPK * 8))
+        rows.append(("meteora_gate_topk (token tiles)", us, (T * d_in + N_ADAPTERS * d_in) * es + T * TOPK * 8))
         us = timed_us(lambda: mb.meteora_route(idx, N_ADAPTERS))
         rows.append(("meteora_route (k_route)", us, T * TOPK * 8 + (2 * N_ADAPTERS + 1) * 4))
         us = timed_us(lambda: mb.meteora_lora_delta(x, A, B, idx, w, offsets, perm, workspace=ws))
-        rows.append(("meteora_lora_delta (k_shrink_segments + k_expand)", us,
+        rows.append(("meteora_lora_delta (shrink on token tiles + k_expand_slab)", us,
                      (T * d_in + touched * RANK * (d_in + d_out)) * es + T * d_out * 4 + 2 * T * TOPK * RANK * 4))
-        # the fused forward's side of the same job: three-launch chain, whole call minus its base-product launch
-        y = torch.empty(T, d_out, device="cuda", dtype=dt)
-        mb.meteora_set_tuning("fused", 0)
-        try:
-            call = lambda: mb.meteora_linear_forward(x, W0, A, B, Wg, TOPK, workspace=ws, out=y)
-            us_call = timed_us(call, 20)
-            call()
-            torch.cuda.synchronize()
-            mb.meteora_profile_begin(8)
-            for _ in range(8):
-                call()
-            ms, n = mb.meteora_profile_end()
-        finally:
-            mb.meteora_set_tuning("fused", 1)
-        us_base = ms * 1e3 / max(n, 1)
-        stacked_bytes = (T * d_in + (N_ADAPTERS * RANK + N_ADAPTERS) * d_in) * es + T * TOPK * (RANK + 2) * 4
-        rows.append(("stacked dense shrink [A; Wg] x on tcgen05 + selection (three-launch call minus its base product)",
-                     us_call - us_base, stacked_bytes))
-        seg_total = sum(r[1] for r in rows[:3])
+        seg_total = sum(r[1] for r in rows)
         for name, us, nbytes in rows:
             print(json.dumps({"op": "standalone", "config": cfg, "shape": f"{d_in}->{d_out}", "T": T, "kernel": name,
                               "us": round(us, 2), "algorithmic_bytes": int(nbytes), "bound": "hbm",
                               "roofline_us": round(nbytes / hbm / 1e3, 3),
                               "frac_of_roofline": round(nbytes / hbm / 1e3 / us, 4), "adapters_touched": touched}), flush=True)
-        print(json.dumps({"op": "segments_vs_stacked", "config": cfg, "shape": f"{d_in}->{d_out}", "T": T,
-                          "us_segments_path (gate_topk + route + shrink by segments + expand)": round(seg_total, 2),
-                          "us_stacked_path (stacked shrink + selection; the expand rides in the base product)":
-                              round(us_call - us_base, 2),
-                          "us_three_launch_call": round(us_call, 2), "us_base_product_launch": round(us_base, 2)}), flush=True)
+        print(json.dumps({"op": "standalone_total", "config": cfg, "shape": f"{d_in}->{d_out}", "T": T,
+                          "us_gate_topk_route_lora_delta": round(seg_total, 2)}), flush=True)
 
 
 def run_decode_loop():
@@ -966,7 +938,7 @@ def run_decode_loop():
     for T in (1, 16, 64):
         xs = {d: torch.from_numpy(workloads.make_x(T, d, "rms", 60 + i, "bf16")).to(dt).cuda()
               for i, d in enumerate(sorted({di for di, _ in workloads.CONFIG4_LINEARS.values()}))}
-        calls, nbytes, launches = [], 0.0, 0
+        calls, nbytes = [], 0.0
         for layer in weights:
             for names in (("q", "k", "v"), ("o",), ("gate", "up"), ("down",)):
                 d_in = workloads.CONFIG4_LINEARS[names[0]][0]
@@ -979,7 +951,6 @@ def run_decode_loop():
                               "W0": vpa([layer[n_]["W0"] for n_ in names]), "A": vpa([layer[n_]["A"] for n_ in names]),
                               "B": vpa([layer[n_]["B"] for n_ in names]), "Wg": vpa([layer[n_]["Wg"] for n_ in names]),
                               "y": vpa(ys), "ws": torch.zeros(n, dtype=torch.uint8, device="cuda")})
-                launches += 1 if lib.meteora_group_plan(ctypes.byref(shape), d_outs, len(names)) else len(names)
                 touched = min(N_ADAPTERS, T * TOPK)
                 for d_out in d_out_list:
                     nbytes += (d_in * d_out + N_ADAPTERS * d_in + touched * RANK * (d_in + d_out) + T * (d_in + d_out)) * es
@@ -1019,7 +990,7 @@ def run_decode_loop():
         ms = e0.elapsed_time(e1) / iters
         print(json.dumps({"op": "decode_step", "shape": "LLaMA3-8B stack: 32 layers x (q k v o gate up down), MeteoRA linears only",
                           "batch": T, "ms_per_generated_token": round(ms, 3), "tokens_per_s": round(T / ms * 1e3),
-                          "launches_per_step": launches, "bound": "hbm", "roofline_ms": round(nbytes / hbm / 1e6, 3),
+                          "calls_per_step": len(calls), "bound": "hbm", "roofline_ms": round(nbytes / hbm / 1e6, 3),
                           "frac_of_roofline": round(nbytes / hbm / 1e6 / ms, 3),
                           "modules": n_layers * len(workloads.CONFIG4_LINEARS)}), flush=True)
         del calls, graph
@@ -1040,7 +1011,6 @@ def run_gate_backward_sweep():
     for T in (1, 128, 2048, 8192):
         g = torch.Generator(device="cuda").manual_seed(13)
         x = torch.randn(T, d_in, device="cuda", generator=g).to(dt)
-        W0 = (0.02 * torch.randn(d_out, d_in, device="cuda", generator=g)).to(dt)
         A = ((torch.rand(N_ADAPTERS, RANK, d_in, device="cuda", generator=g) * 2 - 1) / d_in ** 0.5).to(dt)
         B = (0.01 * torch.randn(N_ADAPTERS, d_out, RANK, device="cuda", generator=g)).to(dt)
         Wg = (torch.randn(N_ADAPTERS, d_in, device="cuda", generator=g) / d_in ** 0.5).to(dt)
@@ -1088,9 +1058,8 @@ def run_gate_backward_sweep():
                           "tokens_per_s": round(T / us * 1e6), "bound": "hbm",
                           "roofline_us": round(nbytes / hbm / 1e3, 2),
                           "frac_of_roofline": round(nbytes / hbm / 1e3 / us, 3),
-                          "note": "B transposed beforehand (meteora_transpose_adapters_b); up to 256 tokens both stacked "
-                                  "shrinks as one launch and no bucketing, up to 1024 no bucketing; graph replay of 8 "
-                                  "stream-ordered calls"}),
+                          "note": "B transposed beforehand (meteora_transpose_adapters_b); both shrinks on token tiles, dWg as a "
+                                  "tensor-core product; graph replay of 8 stream-ordered calls"}),
               flush=True)
 
 

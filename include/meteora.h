@@ -139,15 +139,16 @@ int meteora_lora_delta_static(const void* x, const void* A, const void* B, const
  *   meteora_workspace_bytes(shape); calls that share a workspace must not overlap in time.
  * After the call the workspace holds the routing that was used (meteora_workspace_routing).
  * bf16 shapes with d_in % 8 == 0 and r % 8 == 0 run on the tensor-core paths (TMA + tcgen05):
- * decode batches (T <= 256, rank a multiple of 8 whose staged rows of B fit shared memory) as ONE cooperative
- * kernel launch in which the CTAs exchange partial results through the workspace, everything else as three launches
- * (stacked shrink [A; Wg] x, selection, base product with the LoRA expand; for prefill batches of
- * ranks that are multiples of 8 on pairs of SMs with two-CTA MMAs).  A bf16 layer whose rank is no multiple of 8 takes the same
+ * decode batches (T <= 256, rank a multiple of 8 whose staged rows of B fit shared memory) as ONE kernel launch in which the
+ * CTAs exchange partial results through the workspace (wide layers from 48 tokens as two launches, token tiles and persistent
+ * pairs of SMs), everything else as one to three launches (gate, selection and shrink; base product with the LoRA expand).
+ * The CTAs of a one-launch decode call wait for one another: batches of up to 128 tokens through one module are plain launches, to be kept on
+ * streams of equal priority; the others are cooperative.  A bf16 layer whose rank is no multiple of 8 takes the same
  * paths with A and B zero-padded to the next multiple of 8 inside the workspace (rewritten by every call).  Every other shape
  * runs on a plain CUDA-core path with the same results up to rounding order.  The workspace header
  * must have been zeroed once (meteora_workspace_init) before its first use; the kernels leave it
  * ready for the next call.  Prefill batches of rank 8, 16, 32 or 64 run the base product on persistent pairs of SMs; where
- * [Wg; A] has at most 512 rows gate, selection and shrink are part of the same launch.  meteora_describe_plan tells which path a shape takes.
+ * [Wg; A] has at most 512 rows gate, selection and shrink are part of the same launch from two rounds of tiles on.  meteora_describe_plan tells which path a shape takes.
  */
 int meteora_linear_forward(const void* x, const void* W0, const void* A, const void* B, const void* Wg,
                            const meteora_shape_t* shape, void* y, void* workspace, size_t workspace_bytes,
@@ -160,12 +161,14 @@ int meteora_linear_forward(const void* x, const void* W0, const void* A, const v
  * W0, A, B, Wg, y are HOST arrays of n_modules DEVICE pointers (1 <= n_modules <= METEORA_MAX_GROUP), d_out a host
  * array; T, d_in, N, r, k, dtype, temperature come from `shape` (its d_out is ignored).  Results per module are
  * those of meteora_linear_forward up to the rounding order of fp32 sums.  Decode batches (T <= 256, rank a
- * multiple of 8, bf16, all modules together at most about 120 row tiles of 128) run as ONE kernel launch for the whole group;
- * prefill batches of modules whose [Wg; A] has at most 512 rows run as ONE launch as well (persistent pairs of SMs, from about
- * 10 K outputs x 1 K tokens on); anything else runs module by module.  workspace: meteora_group_workspace_bytes(shape, d_out, n_modules) bytes of
+ * multiple of 8, bf16, all modules together at most about 120 row tiles of 128) run as ONE kernel launch for the whole group,
+ * wider ones (from 40 tokens) and large batches of them as a launch of token tiles per module and one walk of persistent pairs of SMs over all
+ * modules; prefill batches of modules whose [Wg; A] has at most 512 rows run as ONE launch as well (persistent pairs of SMs,
+ * from about 10 K outputs x 1 K tokens on); anything else runs module by module.  workspace: meteora_group_workspace_bytes(shape, d_out, n_modules) bytes of
  * device memory, its first 4 KB zeroed once (meteora_workspace_init); meteora_workspace_status reads the group's
  * status word.  meteora_group_workspace_routing returns where module `module` left its routing;
- * meteora_group_plan returns 1 if the group runs as one launch, 0 if module by module, or an error code.
+ * meteora_group_plan returns 1 if the modules run together (one launch, or one launch of token tiles per module and then one
+ * walk over all modules' tiles), 0 if module by module, or an error code.
  */
 #define METEORA_MAX_GROUP 4
 size_t meteora_group_workspace_bytes(const meteora_shape_t* shape, const int* d_out, int n_modules);

@@ -227,7 +227,8 @@ def meteora_gate_backward(x, A, B, dy, topk_idx, topk_w, temperature: float = 1.
 
 
 def meteora_group_plan(T, d_in, d_outs, N, r, k, dtype: torch.dtype) -> int:
-    """1 if meteora_linear_forward_group runs these modules as one kernel launch, 0 if module by module."""
+    """1 if meteora_linear_forward_group runs these modules together (one kernel launch, or one of token tiles per module and one walk
+    over all of them), 0 if module by module."""
     lib = load_library()
     shape = make_shape(T, d_in, d_outs[0], N, r, k, dtype)
     rc = lib.meteora_group_plan(ctypes.byref(shape), (ctypes.c_int * len(d_outs))(*d_outs), len(d_outs))
