@@ -4,11 +4,11 @@
 //                   cut into tiles and slices of the contraction axis; slice z writes its own fp32 copy of the result;
 //   k_simt_finish   adds the slices in order, selects and weighs (Eq. 3), expands (Eq. 2), rounds once and stores y.
 //
-// What bounds it: large problems the FMA pipe, small ones the chain of launches and load latencies, so a small problem
-// is cut along the contraction axis until its tiles fill the SMs.  Measured per call (graph replay; before: a gate
+// What bounds it: large problems instruction issue (12 warps per SM, packed FMAs), small ones the chain of launches and load
+// latencies, so a small problem is cut along the contraction axis until its tiles fill the SMs.  Measured per call (graph replay; before: a gate
 // kernel, a shrink kernel and a 64 x 64 GEMM with scalar loads and the whole axis per CTA): 256 -> 256, 4 adapters, 64
 // tokens 77 -> 7.9 us; 2048 -> 2048, 28 adapters: one token 258 -> 15.6 us, 512 tokens 495 -> 132 us (42 TFLOP/s of the
-// first launch, FMA-bound).
+// first launch, of 74 that the FMA pipes hold).
 #include "common.cuh"
 #include "select.cuh"
 
