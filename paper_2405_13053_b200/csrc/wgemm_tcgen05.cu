@@ -1048,7 +1048,7 @@ static int launch_wgemm(const CUtensorMap& m0, const CUtensorMap& m1, const CUte
                         WGemmParams& p,
                         int row_tiles, const Plan& pl, bool pdl_attr, cudaStream_t st) {
     if (pl.smem > 227 * 1024) return METEORA_ERR_UNSUPPORTED_SHAPE;
-    static int smem_set[64] = {};
+    static std::atomic<int> smem_set[64];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return METEORA_ERR_CUDA;
     if (dev < 0 || dev >= 64) return METEORA_ERR_UNSUPPORTED_SHAPE;
@@ -1136,7 +1136,7 @@ static int launch_stacked_shrink_pair(const void* x, const void* A, const void* 
     p.col_logits = ws.col_logits;
     p.status = ws.status;
     p.pdl_trigger = tuning().pdl ? 1 : 0;
-    static int smem_set[64] = {};
+    static std::atomic<int> smem_set[64];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return METEORA_ERR_CUDA;
     if (dev < 0 || dev >= 64) return METEORA_ERR_UNSUPPORTED_SHAPE;
@@ -1331,7 +1331,7 @@ static int launch_base_lora_pair(const void* x, const void* W0, const void* B, c
     p.skip_rp0 = skip_rp0;
     p.skip_tt0 = skip_tt0;
     p.pdl_trigger = skip_rp0 != 0x7FFFFFFF && tuning().pdl ? 1 : 0;
-    static int smem_set[64] = {};
+    static std::atomic<int> smem_set[64];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return METEORA_ERR_CUDA;
     if (dev < 0 || dev >= 64) return METEORA_ERR_UNSUPPORTED_SHAPE;
@@ -1982,7 +1982,7 @@ int launch_decode_group(const void* x, const GroupModule* mods, int G, const met
     }
     // Programmatic dependent launch on top (knob pdl_decode): the next launch is processed under this kernel's tail.
     // If the driver does not take the two attributes together, the kernel is launched without it from then on.
-    static bool pdl_accepted = true;
+    static std::atomic<bool> pdl_accepted{true};
     const bool want_pdl = tuning().pdl_decode != 0 && pdl_accepted;
     if (want_pdl) {
         attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -2272,7 +2272,7 @@ int launch_decode_stream(const void* x, const GroupModule* mods, int G, const me
     d.own_local = tuning().own_local && sp.S > 1 ? 1 : 0;
     if (d.bulk_deliver) d.own_local = 1;
     if (sp.S == 1) d.own_local = 1;                             // the tile is the CTA's alone: nothing goes through scratch
-    static bool attr_set[64] = {};
+    static std::atomic<bool> attr_set[64];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return METEORA_ERR_CUDA;
     if (dev < 0 || dev >= 64) return METEORA_ERR_UNSUPPORTED_SHAPE;
@@ -2358,10 +2358,10 @@ struct ClusterPlan {
 
 // How many clusters of `S` CTAs with `smem` bytes of dynamic shared memory the device holds at once (0: unknown).
 static int cluster_capacity(int S, size_t smem) {
-    static int cache[64][9][2] = {};                             // [device][S][smem above / below 113 KB]
+    static std::atomic<int> cache[64][9][2];                     // [device][S][smem above / below 113 KB]
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || S < 1 || S > 8) return 0;
-    int& slot = cache[dev][S][smem > kTwoPerSmBytes ? 0 : 1];
+    std::atomic<int>& slot = cache[dev][S][smem > kTwoPerSmBytes ? 0 : 1];
     if (slot != 0) return slot;
     if (cudaFuncSetAttribute(k_decode_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess)
         return 0;
@@ -2499,7 +2499,7 @@ int launch_decode_cluster(const void* x, const void* W0, const void* A, const vo
     d.u_part = ws.u_all;
     d.ctr = ws.status + 16;
     d.status = ws.status;
-    static bool attr_set[64] = {};
+    static std::atomic<bool> attr_set[64];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return METEORA_ERR_CUDA;
     if (dev < 0 || dev >= 64) return METEORA_ERR_UNSUPPORTED_SHAPE;
