@@ -247,7 +247,7 @@ __device__ __forceinline__ void store_us(__nv_bfloat16* row, int c, int cols, in
         row[c] = __float2bfloat16_rn(v);
         return;
     }
-    row[c] = take_bf16_part(v);                                      // (no loop: it would keep the callers' loads from overlapping)
+    row[c] = take_bf16_part(v);
     row[c + cols] = take_bf16_part(v);
     row[c + 2 * cols] = take_bf16_part(v);
 }

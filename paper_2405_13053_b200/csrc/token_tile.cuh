@@ -117,10 +117,17 @@ __device__ __forceinline__ void token_round(const TokenTileParams& p, uint32_t p
         const int e = min(max(p.topk_idx[g], 0), p.N - 1) - e0, col = p.gate_box + e * p.r + q;
         if (e >= 0 && e < p.a_group && col >= c_lo && col < c_hi) {
             const float v = cluster_sum<S>(base, (uint32_t)(own0 + slot / p.k) * pitch4 + 4u * (col - c_lo));
-            const float out = p.mode == TOKEN_FORWARD ? p.topk_w[g] * v : v;
-            p.u[(size_t)t0 * n + i] = out;
-            if (p.us)
-                store_us(p.us + (size_t)(t0 + slot / p.k) * p.us_cols * p.us_parts, (e0 + e) * p.r + q, p.us_cols, p.us_parts, out);
+            p.u[(size_t)t0 * n + i] = p.mode == TOKEN_FORWARD ? p.topk_w[g] * v : v;
+        }
+    }
+    // (a loop of its own, from what this thread has just written: in the loop above its stores hold back the next value's loads, and
+    // the kernel is short enough that the size of its code shows: 4096 -> 1024 at 512 tokens 18.2 -> 18.5 - 19.3 us for the call)
+    if (p.us) {
+#pragma unroll 1
+        for (int i = etid; i < own * n; i += kEpiThreads) {
+            const int slot = i / p.r;
+            store_us(p.us + (size_t)(t0 + slot / p.k) * p.us_cols * p.us_parts, p.topk_idx[(size_t)t0 * p.k + slot] * p.r + i - slot * p.r, p.us_cols,
+                     p.us_parts, p.u[(size_t)t0 * n + i]);
         }
     }
 }

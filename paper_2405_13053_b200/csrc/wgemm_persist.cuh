@@ -52,7 +52,6 @@ struct PersistMaps {                                              // per module,
 struct PersistModule {
     int tile0;                    // its first tile
     int row_tiles, row_pairs, group_pairs;   // group_pairs: row pairs per scheduling group
-    int parts;                    // of us
     const __nv_bfloat16* us;      // [T][parts][64 esteps]
     int32_t* topk_idx;
     float* topk_w;
@@ -67,6 +66,7 @@ struct PersistParams {
     int n_mod, tok_tiles, tiles;
     int stacked_pairs;            // pairs of 128-row tiles of [Wg; A] (0: us comes from the kernel ahead)
     int gate_rows, us_cols;       // Wg's rows padded to whole 32s; columns of a part of us that are read
+    int parts;                    // of us: 1 or 3
     float inv_tau;
     int32_t* flags;               // [module][token tile][2]: picks written, us written; zero between calls
     int32_t* leave_ctr;           // CTAs that are done with the flags
@@ -295,7 +295,6 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                 }
                 const int row0 = (t.row_pair * 2 + (int)rank) * kBM, tokh = t.tok_tile * p.BN + (int)rank * (p.BN / 2);
                 uint32_t own, full, dst;
-                const bool split = p.mod[t.mod].parts > 1;
                 for (int i = 0; i < p.esteps; ++i) {
                     if (!slot(own, full, dst)) return false;
                     const int q0 = i * 8;                         // first of the 8 blocks
@@ -308,7 +307,7 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                         tma_load_2d_pair(dst + kWTileBytes, &maps.U[t.mod], q0 * 8, tokh, full);
                     }
                     __syncwarp();
-                    if (!split) continue;
+                    if (p.parts == 1) continue;
                     if (!slot(own, full, dst)) return false;
                     if (elect_one()) {                            // the other two parts: one where W0's rows would lie
                         if (leader) mbar_expect_tx(own, 2 * (uint32_t)p.BN * 128u);
@@ -369,14 +368,13 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                     phase ^= 1;
                 }
             };
-            int parts = 1;                                        // of the tile whose expand is pending
             auto expand = [&](int b) {
                 uint32_t wa, ua;
                 for (int i = 0; i < p.esteps; ++i) {
                     if (!next(wa)) return false;
                     const int first = s;                          // stage with the B rows: released with the parts behind it
                     uint64_t db[3] = {smem_desc_sw128(wa + kWTileBytes), 0, 0};
-                    if (parts > 1) {
+                    if (p.parts > 1) {
                         release();
                         if (!next(ua)) return false;
                         db[1] = smem_desc_sw128(ua);
@@ -386,12 +384,12 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                     if (elect_one()) {
 #pragma unroll
                         for (int h = 0; h < 3; ++h)
-                            if (h < parts)
+                            if (h < p.parts)
                                 for (int kk = 0; kk < nm; ++kk)
                                     umma_bf16_pair(tmem_base + b * kPairTokens, smem_desc_plain(wa + kk * 2 * kBM * 16, kBM * 16, 128),
                                                    db[h] + (uint64_t)(kk * 2), idesc, 1);
                         umma_commit_pair(bar_base + (p.stages + first) * 8);
-                        if (parts > 1) umma_commit_pair(bar_base + (p.stages + s) * 8);
+                        if (p.parts > 1) umma_commit_pair(bar_base + (p.stages + s) * 8);
                     }
                     __syncwarp();
                     release();
@@ -423,9 +421,7 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                     release();
                 }
                 if (!ok) break;
-                const PersistTile t(p, lin);
-                pending = !t.stacked;
-                parts = p.mod[t.mod].parts;
+                pending = lin >= p.mod[0].tile0;
                 if (!pending && elect_one()) umma_commit_pair(bar_accf + b * 8);
                 __syncwarp();
             }
@@ -632,7 +628,7 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                         for (int i = 0; i < 16; ++i)
                             ystage[(16 * q + i) * kBM + row_in_tile] = __float2bfloat16_rn(__uint_as_float(v[q][i]));
                     }
-                if (mo.parts > 1) {
+                if (p.parts > 1) {
                     bool nan = false;
 #pragma unroll
                     for (int q = 0; q < 4; ++q)

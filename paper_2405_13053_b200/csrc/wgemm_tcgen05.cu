@@ -1561,11 +1561,13 @@ static int launch_persist(const PersistPlan& pp, const void* x, const GroupModul
     int rc;
     if ((rc = get_tensor_map(x, s.d_in, s.T, pp.BN / 2, 0, &maps.X)) != METEORA_OK) return rc;
     int tile0 = G * pp.stacked_pairs * pp.tok_tiles;
+    p.parts = pp.stacked_pairs > 0 ? 1 : mods[0].ws.us_parts;     // (base products of several modules: decode batches, 3 for all)
     for (int m = 0; m < kMaxGroupModules; ++m) {
         const GroupModule& gm = mods[m < G ? m : 0];             // unused slots repeat module 0's (valid) maps
         if ((rc = get_tensor_map(gm.W0, s.d_in, gm.d_out, kBM, 0, &maps.W0[m])) != METEORA_OK) return rc;
         if ((rc = get_adapter_map(gm.B, s.N, gm.d_out, s.r, &maps.B[m])) != METEORA_OK) return rc;
-        const int parts = pp.stacked_pairs > 0 ? 1 : gm.ws.us_parts, ld_us = gm.ws.us_cols * parts;
+        if (gm.ws.us_parts != mods[0].ws.us_parts && pp.stacked_pairs == 0) return METEORA_ERR_UNSUPPORTED_SHAPE;   // (not planned)
+        const int ld_us = gm.ws.us_cols * p.parts;
         if ((rc = get_tensor_map(gm.ws.us, ld_us, s.T, pp.BN / 2, 0, &maps.U[m])) != METEORA_OK) return rc;
         if ((rc = get_store_map(gm.y, gm.d_out, s.T, pp.CT, &maps.Y[m])) != METEORA_OK) return rc;
         if ((rc = get_store_map(gm.ws.us, ld_us, s.T, 32, &maps.S[m], 32)) != METEORA_OK) return rc;
@@ -1580,7 +1582,6 @@ static int launch_persist(const PersistPlan& pp, const void* x, const GroupModul
         mo.row_pairs = (mo.row_tiles + 1) / 2;
         mo.group_pairs = std::min(tuning().group_pairs > 0 ? tuning().group_pairs : std::max(1, (pp.pairs / pp.tok_tiles + 1) / 2), mo.row_pairs);
         mo.tile0 = m < G ? tile0 : 0x7FFFFFFF;
-        mo.parts = parts;
         mo.us = (const __nv_bfloat16*)gm.ws.us;
         mo.topk_idx = gm.ws.topk_idx;
         mo.topk_w = gm.ws.topk_w;
