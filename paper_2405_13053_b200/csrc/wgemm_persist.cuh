@@ -42,6 +42,7 @@ constexpr int kPersistStageBufs = 2;                              // one per epi
 constexpr int kPersistStoreBytes = 64 * kBM * 2;                  // a staging buffer: up to 64 tokens x 128 rows of bf16
 constexpr int kPersistMaxPairs = 74;
 constexpr int kPersistMaxN = 64;                                  // adapters the selection here takes
+constexpr int kPersistMaxStacked = 4;                             // pairs of stacked tiles per token tile
 
 struct PersistMaps {                                              // per module, then the shared tokens
     CUtensorMap W0[kMaxGroupModules], B[kMaxGroupModules], U[kMaxGroupModules], Y[kMaxGroupModules];
@@ -64,11 +65,11 @@ struct PersistParams {
     int N, r, k, nblk, cpa;       // N r / 8 blocks, r / 8 blocks per adapter
     int stages, stage_bytes;
     int n_mod, tok_tiles, tiles;
-    int stacked_pairs;            // pairs of 128-row tiles of [Wg; A] (0: us comes from the kernel ahead)
+    int stacked_pairs;            // pairs of 128-row tiles, [Wg; a share of A] each (0: us comes from the kernel ahead)
     int gate_rows, us_cols;       // Wg's rows padded to whole 32s; columns of a part of us that are read
     int parts;                    // of us: 1 or 3
     float inv_tau;
-    int32_t* flags;               // [module][token tile][2]: picks written, us written; zero between calls
+    int32_t* flags;               // [module][token tile]: warps whose part of us is written; zero between calls
     int32_t* leave_ctr;           // CTAs that are done with the flags
     int32_t* status;
     int pdl;
@@ -92,6 +93,12 @@ __device__ __forceinline__ void tma_load_4d_grp(uint32_t dst, const CUtensorMap*
 }
 __device__ __forceinline__ uint32_t instr_desc_bf16_pair_n(int bn) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
+}
+
+// First row of A in a stacked tile: each pair of tiles has Wg in front, the rest is A's rows in order.  (For the CTA with Wg the
+// number counts from the tile's first row: A begins gate_rows behind it.)
+__device__ __forceinline__ int persist_first_row(const PersistParams& p, int row_pair, int rank) {
+    return row_pair * (2 * kBM - p.gate_rows) + rank * kBM - p.gate_rows;
 }
 
 // Tile number -> module, kind and place.  Stacked tiles of all modules come first; then module by module, groups of row
@@ -122,56 +129,112 @@ struct PersistTile {
     }
 };
 
-// The token's k highest logits, descending, equal ones by ascending index, and their softmax (Eq. 3), by two adjacent lanes that
-// hold half of the logits each as keys in registers.  Logit j of the token in column `tok` lies at s[j * 64 + (tok ^ (j & 31))]:
-// neither the writers (a lane per logit) nor the readers meet in a bank.  NV: N padded to 32 or 64.  Returns the picks, a
-// byte each.  Bound by the latency of its chain of compares (a thread per token: 2.8 us for 64 tokens).
-template <int NV>
-__device__ __forceinline__ unsigned long long persist_topk(const float* s, int tok, int half, int N, int k, float inv_tau, float& first,
-                                                           float& sum) {
-    uint32_t key[NV / 2];                                         // order-preserving; 0: none or taken
+// ---- selection from the logits in shared memory: logit j of the token in slot `tok` of a span of SPAN slots lies at
+// s[j * SPAN + (tok ^ (j & 31))], where neither the writers (a lane per logit) nor the readers (a lane per token) meet in a bank.
+// A logit as it competes: NaN never wins, -0 is +0.
+__device__ __forceinline__ float persist_logit(const float* s, int at) { return fmaxf(s[at], -CUDART_INF_F) + 0.f; }
+__device__ __forceinline__ uint32_t persist_key(float v) {        // order-preserving, never 0
+    const int bits = __float_as_int(v);
+    return (uint32_t)(bits ^ ((bits >> 31) | (int)0x80000000));
+}
+
+// The KP largest of 32 distinct keys, descending, in key[0..KP): lists of KP are sorted and merged (bitonic), minima and maxima
+// only.  A tree of compares that carries the place along is three instructions per step and again two per key to strike out
+// each pick: 5200 cycles for k = 2 and 9000 for k = 4 under a main loop.
+template <int KP>
+__device__ __forceinline__ void persist_merge(uint32_t (&a)[KP]) {  // bitonic -> descending
 #pragma unroll
-    for (int i = 0; i < NV / 2; ++i) {
-        const int j = half * (NV / 2) + i;
-        float v = s[j * 64 + (tok ^ (j & 31))];
-        if (!(v > -CUDART_INF_F)) v = -CUDART_INF_F;              // NaN never wins
-        const uint32_t bits = __float_as_uint(v + 0.f);           // -0 becomes +0
-        key[i] = j >= N ? 0u : (bits & 0x80000000u) ? ~bits : (bits | 0x80000000u);
+    for (int d = KP / 2; d > 0; d /= 2)
+#pragma unroll
+        for (int i = 0; i < KP; ++i)
+            if ((i & d) == 0) {
+                const uint32_t hi = max(a[i], a[i + d]), lo = min(a[i], a[i + d]);
+                a[i] = hi;
+                a[i + d] = lo;
+            }
+}
+template <int KP>
+__device__ __forceinline__ void persist_largest(uint32_t (&key)[32], uint32_t (&best)[KP]) {
+#pragma unroll
+    for (int l = 0; l < 32; l += KP) {
+        uint32_t a[KP];
+#pragma unroll
+        for (int i = 0; i < KP; ++i) a[i] = key[l + i];
+#pragma unroll
+        for (int w = 2; w <= KP; w *= 2)                          // blocks of w, alternately descending and ascending
+#pragma unroll
+            for (int d = w / 2; d > 0; d /= 2)
+#pragma unroll
+                for (int i = 0; i < KP; ++i)
+                    if ((i & d) == 0) {
+                        const uint32_t hi = max(a[i], a[i + d]), lo = min(a[i], a[i + d]);
+                        const bool down = w == KP || (i & w) == 0;
+                        a[i] = down ? hi : lo;
+                        a[i + d] = down ? lo : hi;
+                    }
+        if (l == 0) {
+#pragma unroll
+            for (int i = 0; i < KP; ++i) best[i] = a[i];
+        } else {
+#pragma unroll
+            for (int i = 0; i < KP; ++i) best[i] = max(best[i], a[KP - 1 - i]);
+            persist_merge<KP>(best);
+        }
+    }
+}
+
+// The picks (a byte each) of one token by LPT adjacent lanes that take 32 logits each, from keys whose low bits are replaced by the
+// adapter (inverted: the lower one is the larger key).  `close`: two of the k + 1 largest differ in those bits alone.
+template <int LPT, int KP>
+__device__ __forceinline__ unsigned long long persist_picks(const float* s, int tok, int half, int N, int k, bool& close) {
+    constexpr int SPAN = 128 / LPT;
+    constexpr uint32_t low = 32 * LPT - 1;
+    uint32_t key[32], best[KP];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+        const int j = half * 32 + i;
+        const uint32_t full = persist_key(persist_logit(s, j * SPAN + (tok ^ i)));
+        key[i] = j < N ? (full & ~low) | (low - (uint32_t)j) : 0u;
+    }
+    persist_largest<KP>(key, best);
+    if (LPT == 2) {
+        uint32_t other[KP];
+#pragma unroll
+        for (int i = 0; i < KP; ++i) other[i] = __shfl_xor_sync(0xFFFFFFFFu, best[i], 1);
+#pragma unroll
+        for (int i = 0; i < KP; ++i) best[i] = max(best[i], other[KP - 1 - i]);
+        persist_merge<KP>(best);
     }
     unsigned long long picks = 0;
-    first = sum = 0.f;
-#pragma unroll 1
-    for (int n = 0; n < k; ++n) {
-        uint32_t best = key[0];
-        int at = 0;
 #pragma unroll
-        for (int i = 1; i < NV / 2; ++i)
-            if (key[i] > best) {
-                best = key[i];
-                at = i;
-            }
-        at += half * (NV / 2);
-        const uint32_t other = __shfl_xor_sync(0xFFFFFFFFu, best, 1);
-        const int other_at = __shfl_xor_sync(0xFFFFFFFFu, at, 1);
-        if (other > best || (other == best && half == 1)) {
-            best = other;
-            at = other_at;
+    for (int i = 0; i + 1 < KP; ++i)
+        if (i < k) {
+            picks |= (unsigned long long)(low - (best[i] & low)) << (8 * i);
+            close |= ((best[i] ^ best[i + 1]) & ~low) == 0;
         }
-#pragma unroll
-        for (int i = 0; i < NV / 2; ++i)
-            if (half * (NV / 2) + i == at) key[i] = 0u;
+    return picks;
+}
+// The same from whole keys, one compare after the other: ties (the lower adapter first), and k = 8.
+template <int LPT>
+__device__ __noinline__ unsigned long long persist_picks_exact(const float* s, int tok, int N, int k) {
+    unsigned long long picks = 0, taken = 0;
+    for (int n = 0; n < k; ++n) {
+        uint32_t best = 0;
+        int at = 0;
+#pragma unroll 1
+        for (int j = 0; j < N; ++j) {
+            const uint32_t key = (taken >> j) & 1 ? 0u : persist_key(persist_logit(s, j * (128 / LPT) + (tok ^ (j & 31))));
+            if (key > best) {
+                best = key;
+                at = j;
+            }
+        }
+        taken |= 1ull << at;
         picks |= (unsigned long long)at << (8 * n);
-        const float v = __uint_as_float((best & 0x80000000u) ? (best & 0x7FFFFFFFu) : ~best);
-        if (n == 0) first = v;
-        sum += expf((v - first) * inv_tau);
     }
     return picks;
 }
-// Weight of an adapter picked above.
-__device__ __forceinline__ float persist_weight(const float* s, int tok, int j, float inv_tau, float first, float sum) {
-    const float v = s[j * 64 + (tok ^ (j & 31))];
-    return expf(((v > -CUDART_INF_F ? v : -CUDART_INF_F) + 0.f - first) * inv_tau) / sum;
-}
+
 // Whether 8 packed bf16 hold an infinity or a NaN.
 __device__ __forceinline__ bool any_nonfinite(const uint4& v) {
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
@@ -216,6 +279,113 @@ __device__ __noinline__ void persist_repair(const PersistParams& p, const Persis
 
 __device__ __forceinline__ void st_cluster_v2(uint32_t cluster_addr, int2 v) {
     asm volatile("st.shared::cluster.v2.b32 [%0], {%1, %2};" ::"r"(cluster_addr), "r"(v.x), "r"(v.y) : "memory");
+}
+__device__ __forceinline__ void st_cluster_f32(uint32_t cluster_addr, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr), "f"(v) : "memory");
+}
+
+// 16 lanes x 32 columns of TMEM as accumulator fragments: register 4 b + 2 h + c of lane l holds row l / 4 + 8 h, column
+// 8 b + 2 (l % 4) + c.
+__device__ __forceinline__ void tmem_ld_frag_issue(uint32_t taddr, uint32_t (&v)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]),
+          "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+        : "r"(taddr));
+}
+// Four 8 x 8 blocks of such fragments (bf16, two columns per register), transposed: lane 8 i + j gives where column j of block i goes.
+__device__ __forceinline__ void stmatrix_x4_trans(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d)
+                 : "memory");
+}
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t*>(&v);
+}
+
+// Tokens of an epilogue group (chunks grp, grp + 2, ... of CT tokens) are its slots 0, 1, ...: the tile's column of a slot.
+__device__ __forceinline__ int persist_column(const PersistParams& p, int grp, int slot) {
+    const int c = slot / p.CT;
+    return (grp + 2 * c) * p.CT + slot - c * p.CT;
+}
+
+// What a group knows about its 128 slots, in the upper half of its staging buffer (both CTAs of the pair hold the same)
+struct PersistRouting {
+    unsigned long long picks[128];                                // adapters of a slot's token, a byte each; 0xFF: none, or no such token
+    float w[8][128];                                              // [pick][slot]
+    float4 spread[4][32];                                         // per warp: weights of 32 tokens for the warp's 4 x 8 columns (< 0: not picked)
+};
+static_assert(sizeof(PersistRouting) <= kPersistStoreBytes / 2, "routing must fit behind us");
+
+// Selection by the group of four warps whose accumulator has the logits in its first 32 LPT rows, for itself and the pair's peer.
+// The k largest logits, descending, equal ones by ascending adapter, and their softmax (Eq. 3).
+template <int LPT>
+__device__ __forceinline__ void persist_select(const PersistParams& p, float* s_lg, PersistRouting* rt, uint32_t peer_rt, uint32_t taddr,
+                                               int grp, int quad, int nslots, int tok0) {
+    constexpr int SPAN = 128 / LPT;
+    const int lane = threadIdx.x & 31, gtid = quad * 32 + lane, tok = gtid / LPT, half = gtid % LPT;
+    unsigned long long picks[LPT];
+    float w[LPT][8 / LPT];
+#pragma unroll
+    for (int sp = 0; sp < LPT; ++sp) {
+        const int slot0 = sp * SPAN;
+        if (sp > 0) asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
+        if (quad < LPT) {                                         // warp-uniform: lane = logit
+#pragma unroll 1
+            for (int q = 0; q < SPAN && slot0 + q < nslots; q += 32) {
+                const uint32_t col = (uint32_t)persist_column(p, grp, slot0 + q);
+                uint32_t v[2][16];
+                tmem_ld16_issue(taddr + col, v[0]);
+                tmem_ld16_issue(taddr + col + 16, v[1]);
+                tmem_ld_wait();
+#pragma unroll
+                for (int i = 0; i < 32; ++i) s_lg[gtid * SPAN + ((q + i) ^ lane)] = __uint_as_float(v[i >> 4][i & 15]);
+            }
+        }
+        asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
+        if (slot0 + tok < nslots) {                               // warp-uniform
+            bool close = p.k == 8;
+            unsigned long long got = 0;
+            if (p.k < 4) got = persist_picks<LPT, 4>(s_lg, tok, half, p.N, p.k, close);
+            else if (p.k < 8) got = persist_picks<LPT, 8>(s_lg, tok, half, p.N, p.k, close);
+            if (__any_sync(0xFFFFFFFFu, close)) got = persist_picks_exact<LPT>(s_lg, tok, p.N, p.k);
+            float first = 0.f, sum = 0.f;
+#pragma unroll 1
+            for (int j = 0; j < p.k; ++j) {
+                const int e = (int)(got >> (8 * j)) & 0xFF;
+                const float v = persist_logit(s_lg, e * SPAN + (tok ^ (e & 31)));
+                if (j == 0) first = v;
+                sum += expf((v - first) * p.inv_tau);
+            }
+#pragma unroll
+            for (int i = 0; i < 8 / LPT; ++i)
+                if (half + LPT * i < p.k) {
+                    const int e = (int)(got >> (8 * (half + LPT * i))) & 0xFF;
+                    w[sp][i] = expf((persist_logit(s_lg, e * SPAN + (tok ^ (e & 31))) - first) * p.inv_tau) / sum;
+                }
+            if (tok0 + persist_column(p, grp, slot0 + tok) >= p.T) got = ~0ull;
+            else if (p.k < 8) got |= ~0ull << (8 * p.k);
+            picks[sp] = got;
+        }
+    }
+    asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");   // all logits read: the routing takes their place
+#pragma unroll
+    for (int sp = 0; sp < LPT; ++sp) {
+        const int slot = sp * SPAN + tok;
+        if (slot >= nslots) continue;
+        if (half == 0) {
+            rt->picks[slot] = picks[sp];
+            st_cluster_v2(peer_rt + (uint32_t)(offsetof(PersistRouting, picks) + slot * 8), make_int2((int)(uint32_t)picks[sp], (int)(uint32_t)(picks[sp] >> 32)));
+        }
+#pragma unroll
+        for (int i = 0; i < 8 / LPT; ++i) {
+            const int j = half + LPT * i;
+            if (j >= p.k) continue;
+            rt->w[j][slot] = w[sp][i];
+            st_cluster_f32(peer_rt + (uint32_t)(offsetof(PersistRouting, w) + (j * 128 + slot) * 4), w[sp][i]);
+        }
+    }
+    asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
 }
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads)
@@ -286,7 +456,7 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
             };
             auto expand = [&](const PersistTile& t) {
                 if (p.stacked_pairs > 0) {                        // the selection of these tokens
-                    const bool there = lane != 0 || wait_counter_slow(p.flags + (t.mod * p.tok_tiles + t.tok_tile) * 2 + 1, 4 * p.stacked_pairs, 100);
+                    const bool there = lane != 0 || wait_counter_slow(p.flags + t.mod * p.tok_tiles + t.tok_tile, 16 * p.stacked_pairs, 100);
                     if (!__all_sync(0xFFFFFFFFu, there)) return false;
                     asm volatile("fence.proxy.async;" ::: "memory");
                 } else if (!waited) {
@@ -324,10 +494,10 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
             for (int lin = pair0; lin < p.tiles && ok; lin += npairs) {
                 const PersistTile t(p, lin);
                 const int row_tile = t.row_pair * 2 + (int)rank, tokh = t.tok_tile * p.BN + (int)rank * (p.BN / 2);
-                // own 128 rows of the stacked matrix: Wg and the first rows of A behind it, or 128 rows of A (zeros past the end)
-                const bool gate = t.stacked && row_tile == 0;
+                // own 128 rows of the stacked matrix: Wg and rows of A behind it, or 128 rows of A (zeros past the end)
+                const bool gate = t.stacked && leader;
                 const CUtensorMap* mW = !t.stacked ? &maps.W0[t.mod] : gate ? &maps.A0[t.mod] : &maps.A[t.mod];
-                const int w_row = !t.stacked ? row_tile * kBM : gate ? 0 : row_tile * kBM - p.gate_rows;
+                const int w_row = !t.stacked ? row_tile * kBM : persist_first_row(p, t.row_pair, (int)rank) + (gate ? p.gate_rows : 0);
                 const uint32_t w_off = gate ? (uint32_t)p.gate_rows * 128u : 0u;
                 uint32_t own, full, dst;
                 for (int i = 0; i < p.ksteps && ok; ++i) {
@@ -454,157 +624,106 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
             tc_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(b * kPairTokens);
             if (t.stacked) {
-                int32_t* flag = p.flags + (t.mod * p.tok_tiles + t.tok_tile) * 2;
-                float* s_lg = reinterpret_cast<float*>(ystage);
-                // [own chunk][pick][token]: adapter, weight.  One pair of stacked tiles: behind the logits (N <= 32), handed to the
-                // peer through distributed shared memory; two: through the routing arrays
-                const bool one = p.stacked_pairs == 1;
-                int2* s_pick = reinterpret_cast<int2*>(reinterpret_cast<uint8_t*>(ystage) + kPersistStoreBytes / 2);
-                const uint32_t peer_pick = map_to_cta(ysmem + kPersistStoreBytes / 2, rank ^ 1u);
-                const int gtid = quad * 32 + lane;                // thread of the group
-                if (tile_m == 0) {
-#pragma unroll 1
-                    for (int c = grp; c < chunks; c += 2) {
-                        if (quad * 32 < p.gate_rows) {            // warp-uniform: lane = logit
-#pragma unroll 1
-                            for (int q = 0; q < p.CT; q += 32) {
-                                uint32_t v[2][16];
-                                tmem_ld16_issue(taddr + (uint32_t)(c * p.CT + q), v[0]);
-                                tmem_ld16_issue(taddr + (uint32_t)(c * p.CT + q + 16), v[1]);
-                                tmem_ld_wait();
-#pragma unroll
-                                for (int i = 0; i < 32; ++i) s_lg[row_in_tile * 64 + ((q + i) ^ lane)] = __uint_as_float(v[i >> 4][i & 15]);
-                            }
-                        }
-                        asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
-                        const int col = gtid >> 1, half = gtid & 1, tk = tok0 + c * p.CT + col;   // two lanes per token
-                        if (col < p.CT) {                         // warp-uniform
-                            float first, sum;
-                            const unsigned long long picks = p.gate_rows <= 32
-                                                                 ? persist_topk<32>(s_lg, col, half, p.N, p.k, p.inv_tau, first, sum)
-                                                                 : persist_topk<64>(s_lg, col, half, p.N, p.k, p.inv_tau, first, sum);
-#pragma unroll 1
-                            for (int j = half; j < p.k; j += 2) {
-                                const int e = (int)(picks >> (8 * j)) & 0xFF;
-                                const float w = persist_weight(s_lg, col, e, p.inv_tau, first, sum);
-                                const int at = ((c >> 1) * p.k + j) * p.CT + col;
-                                const int2 pick = make_int2(tk < p.T ? e : -1, __float_as_int(w));
-                                if (one) {
-                                    s_pick[at] = pick;
-                                    st_cluster_v2(peer_pick + (uint32_t)at * 8u, pick);
-                                } else if (tk < p.T) {
-                                    mo.topk_idx[(size_t)tk * p.k + j] = e;
-                                    mo.topk_w[(size_t)tk * p.k + j] = w;
-                                }
-                            }
-                        }
-                        __syncwarp();
-                        asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
-                    }
-                    if (!one) {
-                        __threadfence();
-                        asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
-                    }
-                    if (elected) {
-                        if (one) mbar_arrive_cluster(map_to_cta(bar_pick + grp * 8, 1));
-                        else atomicAdd(flag, 1);
-                    }
-                }
+                int32_t* flag = p.flags + t.mod * p.tok_tiles + t.tok_tile;
+                // routing of the group's slots in the upper half of the staging buffer, us on its way out in the lower half
+                PersistRouting* rt = reinterpret_cast<PersistRouting*>(reinterpret_cast<uint8_t*>(ystage) + kPersistStoreBytes / 2);
+                const int nslots = grp < chunks ? (chunks - grp + 1) / 2 * p.CT : 0;
                 bool have = true;
-                if (one) {
-                    if (tile_m != 0) have = mbar_wait_cluster(bar_pick + grp * 8, 0);
+                if (rank == 0) {
+                    const uint32_t peer_rt = map_to_cta(ysmem + kPersistStoreBytes / 2, 1);
+                    if (p.gate_rows <= 32)
+                        persist_select<1>(p, reinterpret_cast<float*>(ystage), rt, peer_rt, taddr, grp, quad, nslots, tok0);
+                    else
+                        persist_select<2>(p, reinterpret_cast<float*>(ystage), rt, peer_rt, taddr, grp, quad, nslots, tok0);
+                    if (elected) mbar_arrive_cluster(map_to_cta(bar_pick + grp * 8, 1));
                 } else {
-                    if (elected) have = wait_counter(flag, 2);
-                    __syncwarp();
-                    asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
-                    __threadfence();
-#pragma unroll 1
-                    for (int c = grp; c < chunks; c += 2)
-#pragma unroll 1
-                        for (int i = gtid; i < p.CT * p.k; i += 128) {
-                            const int j = i / p.CT, tk = i - j * p.CT;
-                            const size_t src = (size_t)(tok0 + c * p.CT + tk) * p.k + j;
-                            s_pick[(c >> 1) * p.k * p.CT + i] =
-                                tok0 + c * p.CT + tk < p.T ? make_int2(__ldcg(mo.topk_idx + src), __float_as_int(__ldcg(mo.topk_w + src))) : make_int2(-1, 0);
-                        }
-                    __syncwarp();
-                    asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
+                    have = mbar_wait_cluster(bar_pick + grp * 8, 0);
                 }
                 if (!have && lane == 0) {
                     atomicExch(p.status, 1);
                     atomicExch(p.status + 4, 5400);
                 }
-                // a warp's 32 columns of us for 32 tokens at a time, in the lower half of the staging buffer
-                const int a0 = tile_m * kBM + quad * 32 - p.gate_rows, e = (a0 + lane) / p.r;
-                if (a0 >= 0 && a0 < p.us_cols) {
+                // the warp's 32 columns of us for 32 tokens at a time: a lane per token spreads its weights over the warp's adapters, a
+                // thread takes those of its fragments' 8 tokens, and the block leaves in four transposing stores.  As a lane per column
+                // (32 k broadcast loads with two compares each, 32 stores of 2 bytes) a block took 2.0 us for k = 2, 3.0 for k = 4
+                const int a0 = persist_first_row(p, t.row_pair, (int)rank) + quad * 32;
+                if ((rank == 1 || quad * 32 >= p.gate_rows) && a0 < p.us_cols) {
                     const uint32_t us_smem = ysmem + (uint32_t)quad * 2048u;
-                    __nv_bfloat16* s_us = ystage + quad * 1024;   // [token][32 columns]
+                    const int e0 = a0 / p.r, e1 = (a0 + 8) / p.r, e2 = (a0 + 16) / p.r, e3 = (a0 + 24) / p.r;
+                    // [token][32 columns], 64-byte swizzle
+                    const uint32_t st_addr = us_smem + (uint32_t)(lane & 7) * 64u + (uint32_t)(((lane >> 3) ^ ((lane >> 1) & 3)) * 16);
 #pragma unroll 1
-                    for (int c = grp; c < chunks; c += 2)
+                    for (int slot = 0; slot < nslots; slot += 32) {
+                        const int col = persist_column(p, grp, slot);
+                        const unsigned long long picks = rt->picks[slot + lane];
+                        float4 spread = make_float4(-1.f, -1.f, -1.f, -1.f);   // (no weight is negative)
+                        bool any = false;
 #pragma unroll 1
-                        for (int h = 0; h < p.CT; h += 32) {
-                            const int2* pk = s_pick + (c >> 1) * p.k * p.CT + h;
-                            bool any = false;
-                            for (int j = 0; j < p.k; ++j) {
-                                const int x = pk[j * p.CT + lane].x;
-                                any |= x >= 0 && x * p.r < a0 + 32 && (x + 1) * p.r > a0;
-                            }
-                            any = __any_sync(0xFFFFFFFFu, any);
-                            if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the store before
-                            __syncwarp();
-                            if (any) {
-                                uint32_t v[2][16];
-                                tmem_ld16_issue(taddr + (uint32_t)(c * p.CT + h), v[0]);
-                                tmem_ld16_issue(taddr + (uint32_t)(c * p.CT + h + 16), v[1]);
-                                float w[32];
-#pragma unroll
-                                for (int i = 0; i < 32; ++i) w[i] = -1.f;   // not picked (no weight is negative)
-#pragma unroll 1
-                                for (int j = 0; j < p.k; ++j)
-#pragma unroll
-                                    for (int i = 0; i < 32; ++i) {
-                                        const int2 pick = pk[j * p.CT + i];
-                                        w[i] = pick.x == e ? __int_as_float(pick.y) : w[i];
-                                    }
-                                tmem_ld_wait();
-#pragma unroll
-                                for (int i = 0; i < 32; ++i)
-                                    s_us[i * 32 + lane] = __float2bfloat16_rn(w[i] < 0.f ? 0.f : w[i] * __uint_as_float(v[i >> 4][i & 15]));
-                            } else {
-#pragma unroll
-                                for (int i = 0; i < 4; ++i) reinterpret_cast<uint4*>(s_us)[i * 32 + lane] = make_uint4(0u, 0u, 0u, 0u);
-                            }
-                            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> TMA read
-                            __syncwarp();
-                            if (lane == 0 && tok0 + c * p.CT + h < p.T) {
-                                asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
-                                             ::"l"((uint64_t)&maps.S[t.mod]), "r"(us_smem), "r"(a0), "r"(tok0 + c * p.CT + h)
-                                             : "memory");
-                                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-                            }
+                        for (int j = 0; j < p.k; ++j) {
+                            const int e = (int)(picks >> (8 * j)) & 0xFF;
+                            const float w = rt->w[j][slot + lane];
+                            if (e == e0) spread.x = w;
+                            if (e == e1) spread.y = w;
+                            if (e == e2) spread.z = w;
+                            if (e == e3) spread.w = w;
+                            any |= e >= e0 && e <= e3;
                         }
+                        any = __any_sync(0xFFFFFFFFu, any);
+                        uint32_t v[2][16];
+                        if (any) {
+                            tmem_ld_frag_issue(taddr + (uint32_t)col, v[0]);
+                            tmem_ld_frag_issue(taddr + (16u << 16) + (uint32_t)col, v[1]);
+                            rt->spread[quad][lane] = spread;
+                        }
+                        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the store before
+                        __syncwarp();
+                        if (any) {
+                            tmem_ld_wait();
+                            auto scaled = [&](float w, int g, int b, int c) {
+                                return w < 0.f ? 0.f : w * __uint_as_float(v[g >> 1][4 * b + 2 * (g & 1) + c]);
+                            };
+#pragma unroll
+                            for (int b = 0; b < 4; ++b) {
+                                const float4 w0 = rt->spread[quad][8 * b + 2 * (lane & 3)], w1 = rt->spread[quad][8 * b + 2 * (lane & 3) + 1];
+                                stmatrix_x4_trans(st_addr + b * 512, pack_bf16(scaled(w0.x, 0, b, 0), scaled(w1.x, 0, b, 1)),
+                                                  pack_bf16(scaled(w0.y, 1, b, 0), scaled(w1.y, 1, b, 1)),
+                                                  pack_bf16(scaled(w0.z, 2, b, 0), scaled(w1.z, 2, b, 1)),
+                                                  pack_bf16(scaled(w0.w, 3, b, 0), scaled(w1.w, 3, b, 1)));
+                            }
+                        } else {
+#pragma unroll
+                            for (int i = 0; i < 4; ++i)
+                                reinterpret_cast<uint4*>(ystage + quad * 1024)[i * 32 + lane] = make_uint4(0u, 0u, 0u, 0u);
+                        }
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> TMA read
+                        __syncwarp();
+                        if (lane == 0 && tok0 + col < p.T) {
+                            asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
+                                         ::"l"((uint64_t)&maps.S[t.mod]), "r"(us_smem), "r"(a0), "r"(tok0 + col)
+                                         : "memory");
+                            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                        }
+                    }
                     if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // written, not only read out
                 }
+                if (lane == 0) {                                  // a count per warp
+                    __threadfence();
+                    atomicAdd(flag, 1);
+                }
                 tc_fence_before();
-                __threadfence();
                 __syncwarp();
                 asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
-                if (elected) {
-                    mbar_arrive_cluster(map_to_cta(bar_acce + b * 8, 0));
-                    atomicAdd(flag + 1, 1);
-                }
-                if (one && tile_m == 0) {                         // the routing for the caller
+                if (elected) mbar_arrive_cluster(map_to_cta(bar_acce + b * 8, 0));
+                if (rank == 0 && t.row_pair == 0) {               // the routing for the caller
 #pragma unroll 1
-                    for (int c = grp; c < chunks; c += 2)
-#pragma unroll 1
-                        for (int i = gtid; i < p.CT * p.k; i += 128) {
-                            const int j = i / p.CT, tk = i - j * p.CT;
-                            const int2 pick = s_pick[(c >> 1) * p.k * p.CT + i];
-                            if (pick.x >= 0) {
-                                mo.topk_idx[(size_t)(tok0 + c * p.CT + tk) * p.k + j] = pick.x;
-                                mo.topk_w[(size_t)(tok0 + c * p.CT + tk) * p.k + j] = __int_as_float(pick.y);
-                            }
+                    for (int i = quad * 32 + lane; i < nslots * p.k; i += 128) {
+                        const int j = i / nslots, slot = i - j * nslots, e = (int)(rt->picks[slot] >> (8 * j)) & 0xFF;
+                        const size_t dst = (size_t)(tok0 + persist_column(p, grp, slot)) * p.k + j;
+                        if (e != 0xFF) {
+                            mo.topk_idx[dst] = e;
+                            mo.topk_w[dst] = rt->w[j][slot];
                         }
+                    }
                 }
                 continue;
             }
@@ -659,7 +778,7 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
     if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
     if (p.stacked_pairs > 0 && threadIdx.x == 0) {                // the last CTA to leave readies the flags for the next call
         if (atomicAdd(p.leave_ctr, 1) == (int)gridDim.x - 1) {
-            for (int i = 0; i < 2 * p.n_mod * p.tok_tiles; ++i) p.flags[i] = 0;
+            for (int i = 0; i < p.n_mod * p.tok_tiles; ++i) p.flags[i] = 0;
             *p.leave_ctr = 0;
         }
     }

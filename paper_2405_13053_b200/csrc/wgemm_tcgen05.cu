@@ -802,8 +802,9 @@ static int get_tensor_map(const void* ptr, int K, int rows, int box_rows, int de
 }
 
 // Tensor map of y[T, d_out] (bf16, row-major) for storing a tile of 128 outputs x box_tokens tokens from
-// shared memory laid out [token][128 outputs]; not swizzled.  Needs d_out % 8 == 0 (16-byte row pitch).
-static int get_store_map(const void* y, int d_out, int T, int box_tokens, CUtensorMap* out, int box_cols = kBM) {
+// shared memory laid out [token][box_cols outputs].  Needs d_out % 8 == 0 (16-byte row pitch).
+static int get_store_map(const void* y, int d_out, int T, int box_tokens, CUtensorMap* out, int box_cols = kBM,
+                         CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_NONE) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return METEORA_ERR_CUDA;
     const cuuint64_t gdim[2] = {(cuuint64_t)d_out, (cuuint64_t)T};
@@ -811,8 +812,7 @@ static int get_store_map(const void* y, int d_out, int T, int box_tokens, CUtens
     const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_tokens};
     const cuuint32_t estride[2] = {1, 1};
     const CUresult r = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(y), gdim, gstride, box, estride,
-                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? METEORA_OK : METEORA_ERR_CUDA;
 }
 
@@ -1492,11 +1492,11 @@ static PersistPlan make_persist_plan(const meteora_shape_t& s, const int* d_outs
     const int least = with_routing || s.d_in > 8192 ? (sm_count() + 3) / 4 : s.T <= kPairTokens ? 24 : s.N * s.r > 512 ? 8 : 20;
     if (tn.persist < 2 && (pp.tiles < least || (s.T <= 128 && s.d_in < 1024))) return pp;
     if (with_routing) {
-        // [Wg; A] in 128-row tiles: Wg padded to whole 32 rows (a warp's TMEM lanes), then A, padded to whole MMAs of the expand
+        // [Wg; a share of A] in pairs of 128-row tiles: Wg padded to whole 32 rows (a warp's TMEM lanes), A to whole MMAs of the expand
         pp.gate_rows = (s.N + 31) / 32 * 32;
         pp.us_cols = (s.N * s.r + 15) / 16 * 16;
-        pp.stacked_pairs = (pp.gate_rows + pp.us_cols + 2 * kBM - 1) / (2 * kBM);
-        if (pp.stacked_pairs > 2 || s.N > kPersistMaxN || 2 * G * pp.tok_tiles > kMaxFusedRowTiles ||
+        pp.stacked_pairs = (pp.us_cols + 2 * kBM - pp.gate_rows - 1) / (2 * kBM - pp.gate_rows);
+        if (pp.stacked_pairs > kPersistMaxStacked || s.N > kPersistMaxN || G * pp.tok_tiles > kMaxFusedRowTiles ||
             G * pp.stacked_pairs * pp.tok_tiles > pairs)             // (a stacked tile is a pair's first)
             return pp;
         if (tn.persist == 3) return pp;
@@ -1570,7 +1570,7 @@ static int launch_persist(const PersistPlan& pp, const void* x, const GroupModul
         const int ld_us = gm.ws.us_cols * p.parts;
         if ((rc = get_tensor_map(gm.ws.us, ld_us, s.T, pp.BN / 2, 0, &maps.U[m])) != METEORA_OK) return rc;
         if ((rc = get_store_map(gm.y, gm.d_out, s.T, pp.CT, &maps.Y[m])) != METEORA_OK) return rc;
-        if ((rc = get_store_map(gm.ws.us, ld_us, s.T, 32, &maps.S[m], 32)) != METEORA_OK) return rc;
+        if ((rc = get_store_map(gm.ws.us, ld_us, s.T, 32, &maps.S[m], 32, CU_TENSOR_MAP_SWIZZLE_64B)) != METEORA_OK) return rc;
         maps.A[m] = maps.A0[m] = maps.G[m] = maps.X;
         if (pp.stacked_pairs > 0) {
             if ((rc = get_tensor_map(gm.A, s.d_in, s.N * s.r, kBM, 0, &maps.A[m])) != METEORA_OK) return rc;

@@ -87,3 +87,41 @@ def test_many_tiles_per_pair_of_one_chunk(T, d_in, d_outs):
         mb.meteora_linear_forward(*t, 2, workspace=workspace)
         assert mb.meteora_workspace_status(workspace) == 0
     check_group(ws, 1e-2)
+
+
+# The selection inside the walk: the sorted lists of 4 and of 8 (k up to 3 and 7), whole keys (k = 8, equal logits), one and two lanes
+# per token, one to four pairs of stacked tiles (Wg in each), adapters of one 8-row block to 8; token counts of 5 to 8 chunks.
+@pytest.mark.parametrize("T,d_in,d_out,N,r,k", [
+    (300, 320, 9472, 28, 8, 1), (1250, 320, 2048, 28, 8, 3), (1250, 320, 2048, 28, 16, 4), (1250, 320, 2048, 9, 8, 7), (1250, 320, 2048, 8, 8, 8),
+    (1250, 320, 2048, 28, 32, 2), (1100, 512, 2048, 12, 64, 2), (1250, 320, 2048, 64, 8, 3), (1100, 320, 2048, 33, 16, 8), (1250, 320, 2048, 48, 8, 5),
+])
+def test_selection_in_the_walk(T, d_in, d_out, N, r, k):
+    w = workloads.make_workload("walk_pick", T=T, d_in=d_in, d_out=d_out, N=N, r=r, k=k, dtype="bf16", seed=190 + N + k, b_std=0.3)
+    w["Wg"][N - 1] = w["Wg"][1]                          # two adapters that always tie
+    w["x"][5] = 0.0                                      # a token whose logits all tie
+    t = to_dev(w, "x", "W0", "A", "B", "Wg")
+    mb.meteora_set_tuning("persist", 2)
+    try:
+        shape = mb.make_shape(T, d_in, d_out, N, r, k, torch.bfloat16)
+        assert "path=persistent_prefill" in mb.meteora_describe_plan(shape)
+        ws = mb.alloc_workspace(shape)
+        y, idx, weight = mb.meteora_linear_forward(*t, k, workspace=ws, return_routing=True)
+        again = mb.meteora_linear_forward(*t, k, workspace=ws)
+        assert mb.meteora_workspace_status(ws) == 0
+    finally:
+        mb.meteora_set_tuning("persist", 1)
+    assert torch.equal(y, again)
+    y, idx, weight = y.float().cpu().numpy(), idx.cpu().numpy(), weight.cpu().numpy()
+    o_idx, o_weight, o_logits = oracle.gate_topk(w["x"], w["Wg"], k)
+    check_selection(idx, o_idx, o_logits, k)
+    assert idx[5].tolist() == list(range(k))             # equal logits: the lower adapters, in order
+    last = idx == N - 1
+    tied = last.any(axis=1)
+    assert (idx == 1).any(axis=1)[tied].all()            # never the higher one alone, nor ahead of the lower one
+    assert (np.argmax(idx == 1, axis=1)[tied] < np.argmax(last, axis=1)[tied]).all()
+    same = (idx == o_idx).all(axis=1)
+    np.testing.assert_allclose(weight[same], o_weight[same], rtol=1e-4, atol=1e-5)
+    sel = np.unique(np.concatenate([np.arange(0, T, 61), np.arange(255, T, 256), [5, T - 1]]))
+    ref = oracle.linear_forward_routed(w["x"][sel], w["W0"], w["A"], w["B"], w["Wg"], idx[sel])
+    assert rel_l2(y[sel], ref) <= 5e-3
+    assert bf16_bound_ok(y[sel], ref) <= 0.0
