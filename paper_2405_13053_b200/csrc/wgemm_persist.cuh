@@ -6,10 +6,12 @@
 // does (each CTA loads its own 128 rows and its own half of the tokens; no load is multicast), but
 //   - the pairs stay and walk over the tiles: two accumulators in TMEM (256 columns each), so the MMAs of tile i + 1 run
 //     while the epilogue warps round, stage and store tile i;
-//   - the first tiles are those of the stacked matrix [Wg; A_0..A_{N-1}]: the CTA with Wg's rows selects from its accumulators
-//     (top-k, softmax: a thread per token), then every CTA writes its rows' share of us[t][e r + q] = bf16(w_j (A_e x_t)_q)
-//     where token t picked e, else 0, from its accumulators through shared memory and TMA (stores from
-//     registers queue behind the tiles' loads: 60 - 75 ns each, 15 us in all);
+//   - the first tiles are those of the stacked matrix: pairs of [Wg; a share of A_0..A_{N-1}].  The CTA with Wg's rows selects from
+//     its accumulators (top-k, softmax: a thread per token) and hands the routing to its peer, then both write their rows' share of
+//     us[t][e r + q] = bf16(w_j (A_e x_t)_q) where token t picked e, else 0, from their accumulators through shared memory
+//     and TMA (stores from registers queue behind the tiles' loads: 60 - 75 ns each, 15 us in all).  11 us from the last MMA to the
+//     flag at 256 tokens and k = 2, 12 at k = 4, under the next tile's main loop; with compares in a chain and a lane per column of us
+//     it was 20 and 29, and the other pairs waited for it;
 //   - the LoRA expand is a few more k-steps of the same ring: the contraction goes on over the N r columns of us against
 //     the B rows of the tile, both by TMA.  A tile's expand is issued near the end of the NEXT tile's main loop, by
 //     which time the selection is ready: nothing waits for the routing;
@@ -20,7 +22,7 @@
 //     NaN of such a row is computed again from the picks.  Measured against rounded parts: 4096 -> 2 x 14336 at 64 tokens
 //     49.9 -> 52.2 us, 5120 -> 13824 at 200 tokens 37.3 -> 39.4 (four stages more per tile);
 //   - modules that share x (q/k/v, gate/up) are one walk: their tiles fill rounds of pairs together.
-// Where the stacked matrix has more than 512 rows, the batch more token tiles than pairs, one round of tiles would become two, or
+// Where A has more rows than four pairs of stacked tiles take, the batch more stacked tiles than pairs, one round of tiles would become two, or
 // us is three parts, the routing kernels ahead write us and only the base product runs here (stacked_pairs = 0).
 // What bounds it: the tensor cores under the board's power limit (514 cycles per 64-element k-step and 256 x 256 tile, of
 // the 512 that its four MMAs take).  All pairs walk the contraction axis in step, so a line of W0 or x is fetched once for the pairs
@@ -78,17 +80,11 @@ struct PersistParams {
     PersistModule mod[kMaxGroupModules];
 };
 
-// 3-D and 4-D tile loads of a pair: the completion bytes go to a barrier that may live in the pair's other CTA.
+// 3-D tile load of a pair: the completion bytes go to a barrier that may live in the pair's other CTA.
 __device__ __forceinline__ void tma_load_3d_grp(uint32_t dst, const CUtensorMap* tm, int c0, int c1, int c2, uint32_t cluster_bar) {
     asm volatile(
         "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
         ::"r"(dst), "l"((uint64_t)tm), "r"(c0), "r"(c1), "r"(c2), "r"(cluster_bar)
-        : "memory");
-}
-__device__ __forceinline__ void tma_load_4d_grp(uint32_t dst, const CUtensorMap* tm, int c0, int c1, int c2, int c3, uint32_t cluster_bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
-        ::"r"(dst), "l"((uint64_t)tm), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(cluster_bar)
         : "memory");
 }
 __device__ __forceinline__ uint32_t instr_desc_bf16_pair_n(int bn) {
@@ -470,10 +466,7 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                     const int q0 = i * 8;                         // first of the 8 blocks
                     if (elect_one()) {
                         if (leader) mbar_expect_tx(own, 2 * (uint32_t)p.stage_bytes);
-                        if (p.cpa == 1)
-                            tma_load_3d_grp(dst, &maps.B[t.mod], 0, row0 / 8, q0, full);
-                        else
-                            tma_load_4d_grp(dst, &maps.B[t.mod], 0, row0, q0 % p.cpa, q0 / p.cpa, full);
+                        tma_load_3d_grp(dst, &maps.B[t.mod], 0, p.cpa == 1 ? row0 / 8 : row0, q0 / p.cpa, full);
                         tma_load_2d_pair(dst + kWTileBytes, &maps.U[t.mod], q0 * 8, tokh, full);
                     }
                     __syncwarp();
@@ -524,6 +517,9 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
         // ------------------------------------------------------------------ MMA issuer (leader only)
         if (leader) {
             const uint32_t idesc = instr_desc_bf16_pair_n(p.BN);
+            // B's rows in a stage: 16 columns (an MMA) of 128 rows every 4096 bytes, or 2 or 4 such side by side in rows of 64 or 128
+            const uint64_t b_desc = p.cpa == 1 ? smem_desc_plain(0, kBM * 16, 128) : smem_desc_rows(0, 16u * p.cpa);
+            const int b_side = p.cpa <= 2 ? 0 : p.cpa == 4 ? 1 : 2;   // log2 of the MMAs side by side
             bool ok = true, pending = false;
             int s = 0, phase = 0, n = 0;
             auto next = [&](uint32_t& wa) {                       // the next filled stage
@@ -556,7 +552,8 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                         for (int h = 0; h < 3; ++h)
                             if (h < p.parts)
                                 for (int kk = 0; kk < nm; ++kk)
-                                    umma_bf16_pair(tmem_base + b * kPairTokens, smem_desc_plain(wa + kk * 2 * kBM * 16, kBM * 16, 128),
+                                    umma_bf16_pair(tmem_base + b * kPairTokens,
+                                                   b_desc + ((wa + ((kk >> b_side) * (4096 << b_side)) + (kk & ((1 << b_side) - 1)) * 32) >> 4),
                                                    db[h] + (uint64_t)(kk * 2), idesc, 1);
                         umma_commit_pair(bar_base + (p.stages + first) * 8);
                         if (p.parts > 1) umma_commit_pair(bar_base + (p.stages + s) * 8);

@@ -229,6 +229,15 @@ __device__ __forceinline__ uint64_t smem_desc_plain(uint32_t addr, uint32_t kstr
     d |= (uint64_t)1 << 46;
     return d;
 }
+// The same of a K-major bf16 tile whose rows are 32, 64 or 128 bytes, swizzled over as many.
+__device__ __forceinline__ uint64_t smem_desc_rows(uint32_t addr, uint32_t row_bytes) {
+    uint64_t d = (uint64_t)((addr >> 4) & 0x3FFF);
+    d |= (uint64_t)1 << 16;
+    d |= (uint64_t)((8 * row_bytes) >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)(row_bytes == 32 ? 6 : row_bytes == 64 ? 4 : 2) << 61;
+    return d;
+}
 // Instruction descriptor: fp32 accumulate, bf16 x bf16, both operands K-major, M = 128, N = bn.
 __device__ __forceinline__ uint32_t instr_desc_bf16(int bn) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
@@ -816,27 +825,25 @@ static int get_store_map(const void* y, int d_out, int T, int box_tokens, CUtens
     return r == CUDA_SUCCESS ? METEORA_OK : METEORA_ERR_CUDA;
 }
 
-// Tensor map of the adapters' B[N, d_out, r] (bf16) whose box holds, for 128 output rows, 8 blocks of 8 rank entries as
-// un-swizzled K-major core matrices: [block][row][16 bytes].  Rank 8: a block's rows are contiguous, so 8 rows (128 bytes) are
-// the inner axis; larger ranks: (8 entries, rows, r / 8, N), 16 bytes at a time.  Needs d_out % 8 == 0, r / 8 in {1, 2, 4, 8}.
+// Tensor map of the adapters' B[N, d_out, r] (bf16) whose box holds, for 128 output rows, 64 rank entries as K-major MMA operands.
+// Rank 8: 8 adapters as un-swizzled core matrices, [adapter][row][16 bytes]; 8 rows (128 bytes) are contiguous and the inner
+// axis.  Larger ranks: 64 / r adapters, [adapter][row][2 r bytes], swizzled over those 32, 64 or 128 bytes.  (As core matrices they
+// came in pieces of 16 bytes, 1450 cycles for a box: 5120 -> 5120 at 1531 tokens, rank 16, 87.7 us then and 81.9 now; 4096 -> 4096 at 2048 tokens, rank 32, 104 and 91.)
+// Needs d_out % 8 == 0, r / 8 in {1, 2, 4, 8}.
 static int get_adapter_map(const void* B, int N, int d_out, int r, CUtensorMap* out) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return METEORA_ERR_CUDA;
-    CUresult rc;
-    const cuuint32_t estride[4] = {1, 1, 1, 1};
-    if (r == 8) {
-        const cuuint64_t gdim[3] = {64, (cuuint64_t)d_out / 8, (cuuint64_t)N};
-        const cuuint64_t gstride[2] = {128, (cuuint64_t)d_out * 16};
-        const cuuint32_t box[3] = {64, 16, 8};
-        rc = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(B), gdim, gstride, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    } else {
-        const cuuint64_t gdim[4] = {8, (cuuint64_t)d_out, (cuuint64_t)r / 8, (cuuint64_t)N};
-        const cuuint64_t gstride[3] = {(cuuint64_t)r * 2, 16, (cuuint64_t)d_out * r * 2};
-        const cuuint32_t box[4] = {8, (cuuint32_t)kBM, (cuuint32_t)r / 8, 64 / (cuuint32_t)r};
-        rc = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(B), gdim, gstride, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    }
+    const bool core = r == 8;
+    const cuuint32_t estride[3] = {1, 1, 1};
+    const cuuint64_t gdim[3] = {core ? 64 : (cuuint64_t)r, core ? (cuuint64_t)d_out / 8 : (cuuint64_t)d_out, (cuuint64_t)N};
+    const cuuint64_t gstride[2] = {core ? 128 : (cuuint64_t)r * 2, (cuuint64_t)d_out * r * 2};
+    const cuuint32_t box[3] = {core ? 64 : (cuuint32_t)r, core ? kBM / 8 : kBM, core ? 8 : 64 / (cuuint32_t)r};
+    const CUtensorMapSwizzle swizzle = core      ? CU_TENSOR_MAP_SWIZZLE_NONE
+                                       : r == 16 ? CU_TENSOR_MAP_SWIZZLE_32B
+                                       : r == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
+                                                 : CU_TENSOR_MAP_SWIZZLE_128B;
+    const CUresult rc = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(B), gdim, gstride, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                           swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return rc == CUDA_SUCCESS ? METEORA_OK : METEORA_ERR_CUDA;
 }
 

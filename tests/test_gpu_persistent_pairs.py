@@ -15,8 +15,8 @@ pytestmark = pytest.mark.gpu
 # Tile widths 160 / 192 / 224 / 256 (257, 380, 1300, 1281 tokens), a last token tile with few tokens, odd numbers of row tiles and
 # a ragged last one, axes of 5 k-steps and of no whole number, several adapters per block of expand columns (ranks 16 - 64), an
 # odd number of blocks (33), fewer tiles than pairs, less and more than two rounds, whole rounds.
-# With the routing in the walk (persist 2) and from kernels of its own (3: from 37 pair tiles on); 56 adapters: two pairs of
-# stacked tiles, two logits per lane; 40 of rank 8: Wg in a tile of its own.
+# With the routing in the walk (persist 2) and from kernels of its own (3: from 37 pair tiles on); 56 adapters: three pairs
+# of stacked tiles, two lanes per token.
 @pytest.mark.parametrize("persist,T,d_in,d_out,N,r,k", [(p, *c) for p in (2, 3) for c in [
     (257, 4096, 200, 28, 8, 2), (380, 2048, 384, 28, 8, 2), (512, 8192, 1024, 28, 8, 2), (700, 520, 2184, 28, 16, 2),
     (1281, 520, 2184, 28, 8, 2), (1300, 1024, 4096, 33, 8, 4), (1201, 1536, 5120, 5, 32, 2), (2560, 512, 2048, 28, 64, 2),
