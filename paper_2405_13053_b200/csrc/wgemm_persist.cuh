@@ -14,7 +14,8 @@
 //     it was 20 and 29, and the other pairs waited for it;
 //   - the LoRA expand is a few more k-steps of the same ring: the contraction goes on over the N r columns of us against
 //     the B rows of the tile, both by TMA.  A tile's expand is issued near the end of the NEXT tile's main loop, by
-//     which time the selection is ready: nothing waits for the routing;
+//     which time the selection is ready: nothing waits for the routing (its own
+//     main loop's where the routing kernels ran ahead);
 //   - where the kernels otherwise taken expand in fp32 (decode batches, few tiles of large ranks: persist_us_parts) us is
 //     three bf16 parts whose sum is w_j (A_e x_t)_q exactly: a k-step of the expand is then two stages, (B, part 0) and
 //     (part 1, part 2), so that B is read once; the routing kernels ahead write the parts.  Such a token's y depends on its
@@ -401,8 +402,10 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
     const bool leader = rank == 0;
     const int pair0 = (int)blockIdx.x >> 1, npairs = (int)gridDim.x >> 1;
     // where the tile before gets its expand: late, so that the selection is ready for the first tiles, and early enough for
-    // that tile's epilogue to end under the rest (12 k-steps: 4 us)
+    // that tile's epilogue to end under the rest (12 k-steps: 4 us).  With the routing ahead a tile gets its own there: at the end
+    // its loads and MMAs (3 - 3.5 us for three parts) had nothing to hide under
     const int mid = max(p.ksteps / 2, p.ksteps - 12);
+    const bool own = p.stacked_pairs == 0;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.stages; ++s) {
@@ -460,20 +463,20 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                     waited = true;
                 }
                 const int row0 = (t.row_pair * 2 + (int)rank) * kBM, tokh = t.tok_tile * p.BN + (int)rank * (p.BN / 2);
-                uint32_t own, full, dst;
+                uint32_t bar, full, dst;
                 for (int i = 0; i < p.esteps; ++i) {
-                    if (!slot(own, full, dst)) return false;
+                    if (!slot(bar, full, dst)) return false;
                     const int q0 = i * 8;                         // first of the 8 blocks
                     if (elect_one()) {
-                        if (leader) mbar_expect_tx(own, 2 * (uint32_t)p.stage_bytes);
+                        if (leader) mbar_expect_tx(bar, 2 * (uint32_t)p.stage_bytes);
                         tma_load_3d_grp(dst, &maps.B[t.mod], 0, p.cpa == 1 ? row0 / 8 : row0, q0 / p.cpa, full);
                         tma_load_2d_pair(dst + kWTileBytes, &maps.U[t.mod], q0 * 8, tokh, full);
                     }
                     __syncwarp();
                     if (p.parts == 1) continue;
-                    if (!slot(own, full, dst)) return false;
+                    if (!slot(bar, full, dst)) return false;
                     if (elect_one()) {                            // the other two parts: one where W0's rows would lie
-                        if (leader) mbar_expect_tx(own, 2 * (uint32_t)p.BN * 128u);
+                        if (leader) mbar_expect_tx(bar, 2 * (uint32_t)p.BN * 128u);
                         tma_load_2d_pair(dst, &maps.U[t.mod], (p.esteps + i) * kBK, tokh, full);
                         tma_load_2d_pair(dst + kWTileBytes, &maps.U[t.mod], (2 * p.esteps + i) * kBK, tokh, full);
                     }
@@ -492,19 +495,19 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                 const CUtensorMap* mW = !t.stacked ? &maps.W0[t.mod] : gate ? &maps.A0[t.mod] : &maps.A[t.mod];
                 const int w_row = !t.stacked ? row_tile * kBM : persist_first_row(p, t.row_pair, (int)rank) + (gate ? p.gate_rows : 0);
                 const uint32_t w_off = gate ? (uint32_t)p.gate_rows * 128u : 0u;
-                uint32_t own, full, dst;
+                uint32_t bar, full, dst;
                 for (int i = 0; i < p.ksteps && ok; ++i) {
-                    if (i == mid && pending) ok = expand(before);
-                    if (!ok || !(ok = slot(own, full, dst))) break;
+                    if (i == mid && (pending || own)) ok = expand(own ? t : before);
+                    if (!ok || !(ok = slot(bar, full, dst))) break;
                     if (elect_one()) {
-                        if (leader) mbar_expect_tx(own, 2 * (uint32_t)p.stage_bytes);
+                        if (leader) mbar_expect_tx(bar, 2 * (uint32_t)p.stage_bytes);
                         tma_load_2d_pair(dst + w_off, mW, i * kBK, w_row, full);
                         if (gate) tma_load_2d_pair(dst, &maps.G[t.mod], i * kBK, 0, full);
                         tma_load_2d_pair(dst + kWTileBytes, &maps.X, i * kBK, tokh, full);
                     }
                     __syncwarp();
                 }
-                pending = !t.stacked;
+                pending = !t.stacked && !own;
                 before = t;
             }
             if (ok && pending) ok = expand(before);
@@ -561,7 +564,7 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                     __syncwarp();
                     release();
                 }
-                if (elect_one()) umma_commit_pair(bar_accf + b * 8);
+                if (!own && elect_one()) umma_commit_pair(bar_accf + b * 8);
                 __syncwarp();
                 return true;
             };
@@ -575,7 +578,7 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                 }
                 uint32_t wa;
                 for (int i = 0; i < p.ksteps; ++i) {
-                    if (i == mid && pending && !(ok = expand(b ^ 1))) break;
+                    if (i == mid && (pending || own) && !(ok = expand(own ? b : b ^ 1))) break;
                     if (!(ok = next(wa))) break;
                     const uint64_t da = smem_desc_sw128(wa), db = smem_desc_sw128(wa + kWTileBytes);
                     if (elect_one()) {
@@ -588,7 +591,7 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                     release();
                 }
                 if (!ok) break;
-                pending = lin >= p.mod[0].tile0;
+                pending = lin >= p.mod[0].tile0 && !own;
                 if (!pending && elect_one()) umma_commit_pair(bar_accf + b * 8);
                 __syncwarp();
             }
