@@ -33,7 +33,7 @@
 // (4096 -> 4096 at 64 tokens 29.4 -> 18.7 us, 4096 -> 14336 at 2048 tokens 188 -> 178 us for the walk).
 //   warp 0 (both CTAs)  TMA producer; every copy signals the leader's full barrier, which expects both CTAs' bytes.
 //   warp 1 (leader)     MMA issue; stages are released and accumulators announced by commits that arrive in both CTAs.
-//   warps 2-9 (both)    epilogue: two groups of four warps take turns at chunks of CT tokens, each with a staging buffer of
+//   warps 2-9 (both)    epilogue: two groups of four warps take turns at chunks of 32 tokens, each with two staging buffers of
 //                       its own: TMEM -> bf16 -> shared memory -> TMA store.
 // Pairs wait for one another's selection, so with stacked tiles the launch is cooperative (all pairs resident).  Every wait
 // is bounded; the pair leaves together.
@@ -41,8 +41,10 @@
 
 namespace meteora {
 
-constexpr int kPersistStageBufs = 2;                              // one per epilogue group
-constexpr int kPersistStoreBytes = 64 * kBM * 2;                  // a staging buffer: up to 64 tokens x 128 rows of bf16
+constexpr int kPersistStageBufs = 2;                              // epilogue groups, each with staging buffers of its own
+constexpr int kPersistChunk = 32;                                 // tokens an epilogue group takes at a time
+constexpr int kPersistBufBytes = kPersistChunk * kBM * 2;         // as rows of bf16
+constexpr int kPersistStoreBytes = 2 * kPersistBufBytes;          // a group's staging buffers
 constexpr int kPersistMaxPairs = 74;
 constexpr int kPersistMaxN = 64;                                  // adapters the selection here takes
 constexpr int kPersistMaxStacked = 4;                             // pairs of stacked tiles per token tile
@@ -55,7 +57,7 @@ struct PersistMaps {                                              // per module,
 };
 struct PersistModule {
     int tile0;                    // its first tile
-    int row_tiles, row_pairs, group_pairs;   // group_pairs: row pairs per scheduling group
+    int row_pairs, group_pairs;   // group_pairs: row pairs per scheduling group
     const __nv_bfloat16* us;      // [T][parts][64 esteps]
     int32_t* topk_idx;
     float* topk_w;
@@ -63,10 +65,11 @@ struct PersistModule {
     int d_out;
 };
 struct PersistParams {
-    int T, BN, CT;                // tokens per tile, tokens per epilogue chunk (divides BN)
+    int T, BN;                    // tokens per tile
     int ksteps, esteps;           // main k-steps; expand k-steps (8 blocks of 8 columns each)
     int N, r, k, nblk, cpa;       // N r / 8 blocks, r / 8 blocks per adapter
     int stages, stage_bytes;
+    int tr;                       // kWalkNarrow: rows of W0 per CTA and tile, 128 or fewer (whole 8s from 64 up), which spreads a batch over the pairs
     int n_mod, tok_tiles, tiles;
     int stacked_pairs;            // pairs of 128-row tiles, [Wg; a share of A] each (0: us comes from the kernel ahead)
     int gate_rows, us_cols;       // Wg's rows padded to whole 32s; columns of a part of us that are read
@@ -241,7 +244,12 @@ __device__ __forceinline__ bool any_nonfinite(const uint4& v) {
     return any;
 }
 
-// A warp's 32 rows x `nt` tokens of a staged chunk of y ([token][128 rows]) in which some element is NaN: those of rows where some
+// Element (token, row) of a staged chunk of y: two blocks of [token][64 rows], 128-byte swizzle, or [token][tr rows].
+__device__ __forceinline__ int persist_y_at(int tr, int tok, int row) {
+    return tr < kBM ? tok * tr + row : ((row >> 6) * kPersistChunk + tok) * 64 + ((((row >> 3) & 7) ^ (tok & 7)) << 3) + (row & 7);
+}
+
+// A warp's 32 rows x `nt` tokens of a staged chunk of y in which some element is NaN: those of rows where some
 // adapter's B is not finite are computed again as W0 x + the picks' terms.  (A NaN of any other row is the row's own.)  Never
 // taken on finite weights; a row with such an entry costs a dot product per token.
 __device__ __noinline__ void persist_repair(const PersistParams& p, const PersistModule& mo, __nv_bfloat16* ystage, int tile_row0, int quad,
@@ -249,12 +257,12 @@ __device__ __noinline__ void persist_repair(const PersistParams& p, const Persis
     const int lane = threadIdx.x & 31, row0 = tile_row0 + quad * 32, row = row0 + lane;
     asm volatile("griddepcontrol.wait;" ::: "memory");               // (the producer has waited: this thread may read what it waited for)
     bool odd = false;
-    if (row < mo.d_out)
+    if (quad * 32 + lane < p.tr && row < mo.d_out)
         for (int e = 0; e < p.N; ++e)
             for (int c = 0; c < p.r; c += 8) odd |= any_nonfinite(*reinterpret_cast<const uint4*>(mo.B + ((size_t)e * mo.d_out + row) * p.r + c));
     const int cols = 64 * p.esteps;
     for (int i = 0; i < nt; ++i) {
-        unsigned todo = __ballot_sync(0xFFFFFFFFu, odd && __hisnan(ystage[i * kBM + quad * 32 + lane]));
+        unsigned todo = __ballot_sync(0xFFFFFFFFu, odd && __hisnan(ystage[persist_y_at(p.tr, i, quad * 32 + lane)]));
         const int t = tok0 + i;
         while (todo) {
             const int src = __ffs(todo) - 1;
@@ -269,7 +277,7 @@ __device__ __noinline__ void persist_repair(const PersistParams& p, const Persis
                 lora = fmaf(to_f32(mo.B[((size_t)e * mo.d_out + row0 + src) * p.r + q]), uw, lora);
             }
             lora = warp_sum(lora);
-            if (lane == src) ystage[i * kBM + quad * 32 + lane] = __float2bfloat16_rn(base + lora);
+            if (lane == src) ystage[persist_y_at(p.tr, i, quad * 32 + lane)] = __float2bfloat16_rn(base + lora);
         }
     }
 }
@@ -300,10 +308,10 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-// Tokens of an epilogue group (chunks grp, grp + 2, ... of CT tokens) are its slots 0, 1, ...: the tile's column of a slot.
+// Tokens of an epilogue group (chunks grp, grp + 2, ... of 32 tokens) are its slots 0, 1, ...: the tile's column of a slot.
 __device__ __forceinline__ int persist_column(const PersistParams& p, int grp, int slot) {
-    const int c = slot / p.CT;
-    return (grp + 2 * c) * p.CT + slot - c * p.CT;
+    const int c = slot / kPersistChunk;
+    return (grp + 2 * c) * kPersistChunk + slot - c * kPersistChunk;
 }
 
 // What a group knows about its 128 slots, in the upper half of its staging buffer (both CTAs of the pair hold the same)
@@ -385,8 +393,19 @@ __device__ __forceinline__ void persist_select(const PersistParams& p, float* s_
     asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
 }
 
+// What the issuing loops need to know at compile time: read from the parameters in the loops, the rows and k-steps of a stage cost
+// 0.4 - 0.8 us of 29 (4096 -> 4096 at 512 tokens).
+//   kWalkStacked  the routing in the walk, us rounded        k-steps one by one, 128 rows per CTA
+//   kWalkBase     base product behind routing kernels        the same, us in 1 or 3 parts
+//   kWalkNarrow   the same for up to 128 tokens              two k-steps per stage, tr rows per CTA, 3 parts
+enum { kWalkStacked = 0, kWalkBase = 1, kWalkNarrow = 2 };
+
+template <int kWalk>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads)
 k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant__ PersistParams p) {
+    constexpr bool own = kWalk != kWalkStacked;                   // a tile's expand is in its own main loop
+    constexpr int kc = kWalk == kWalkNarrow ? 2 : 1;              // k-steps per stage
+    const int tr = kWalk == kWalkNarrow ? p.tr : kBM, parts = kWalk == kWalkStacked ? 1 : kWalk == kWalkBase ? p.parts : 3;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t ring = (raw + 1023u) & ~1023u;
@@ -404,8 +423,7 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
     // where the tile before gets its expand: late, so that the selection is ready for the first tiles, and early enough for
     // that tile's epilogue to end under the rest (12 k-steps: 4 us).  With the routing ahead a tile gets its own there: at the end
     // its loads and MMAs (3 - 3.5 us for three parts) had nothing to hide under
-    const int mid = max(p.ksteps / 2, p.ksteps - 12);
-    const bool own = p.stacked_pairs == 0;
+    const int iters = (p.ksteps + kc - 1) / kc, mid = max(iters / 2, iters - 12 / kc);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.stages; ++s) {
@@ -436,16 +454,17 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
         // ------------------------------------------------------------------ TMA producer (both CTAs)
         {
             int s = 0, round = 0;                                 // ring slot, how often the ring has been filled
+            const uint32_t leader_bars = map_to_cta(bar_base, 0);
             bool waited = !p.pdl;
             // with stacked tiles x comes from the kernel ahead; else the kernel ahead is this call's routing, which read x
-            if (p.stacked_pairs > 0 && !waited) {
+            if (!own && !waited) {
                 asm volatile("griddepcontrol.wait;" ::: "memory");
                 waited = true;
             }
-            auto slot = [&](uint32_t& full, uint32_t& full_leader, uint32_t& dst) {   // the next free stage
+            auto slot = [&](uint32_t& bar, uint32_t& full, uint32_t& dst) {   // the next free stage; its barrier here and in the leader
                 if (round > 0 && !mbar_wait_warp(bar_base + (p.stages + s) * 8, (round & 1) ^ 1)) return false;
-                full = bar_base + s * 8;
-                full_leader = map_to_cta(full, 0);
+                bar = bar_base + s * 8;
+                full = leader_bars + s * 8;
                 dst = ring + s * p.stage_bytes;
                 if (++s == p.stages) {
                     s = 0;
@@ -453,8 +472,9 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                 }
                 return true;
             };
+            const uint32_t part = (uint32_t)p.BN / 2 * 128u;      // bytes of half a tile's tokens: of x, of a part of us
             auto expand = [&](const PersistTile& t) {
-                if (p.stacked_pairs > 0) {                        // the selection of these tokens
+                if (!own) {                                       // the selection of these tokens
                     const bool there = lane != 0 || wait_counter_slow(p.flags + t.mod * p.tok_tiles + t.tok_tile, 16 * p.stacked_pairs, 100);
                     if (!__all_sync(0xFFFFFFFFu, there)) return false;
                     asm volatile("fence.proxy.async;" ::: "memory");
@@ -462,21 +482,24 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                     asm volatile("griddepcontrol.wait;" ::: "memory");
                     waited = true;
                 }
-                const int row0 = (t.row_pair * 2 + (int)rank) * kBM, tokh = t.tok_tile * p.BN + (int)rank * (p.BN / 2);
+                const int row0 = (t.row_pair * 2 + (int)rank) * tr, tokh = t.tok_tile * p.BN + (int)rank * (p.BN / 2);
+                const int here = kc == 1 ? 1 : parts;             // a stage of two k-steps has room for all parts
                 uint32_t bar, full, dst;
                 for (int i = 0; i < p.esteps; ++i) {
                     if (!slot(bar, full, dst)) return false;
                     const int q0 = i * 8;                         // first of the 8 blocks
                     if (elect_one()) {
-                        if (leader) mbar_expect_tx(bar, 2 * (uint32_t)p.stage_bytes);
+                        if (leader) mbar_expect_tx(bar, 2 * ((uint32_t)tr * 128u + (uint32_t)here * part));
                         tma_load_3d_grp(dst, &maps.B[t.mod], 0, p.cpa == 1 ? row0 / 8 : row0, q0 / p.cpa, full);
                         tma_load_2d_pair(dst + kWTileBytes, &maps.U[t.mod], q0 * 8, tokh, full);
+                        for (int h = 1; h < here; ++h)
+                            tma_load_2d_pair(dst + 2 * kWTileBytes + (uint32_t)(h - 1) * part, &maps.U[t.mod], (h * p.esteps + i) * kBK, tokh, full);
                     }
                     __syncwarp();
-                    if (p.parts == 1) continue;
+                    if (here == parts) continue;
                     if (!slot(bar, full, dst)) return false;
                     if (elect_one()) {                            // the other two parts: one where W0's rows would lie
-                        if (leader) mbar_expect_tx(bar, 2 * (uint32_t)p.BN * 128u);
+                        if (leader) mbar_expect_tx(bar, 4 * part);
                         tma_load_2d_pair(dst, &maps.U[t.mod], (p.esteps + i) * kBK, tokh, full);
                         tma_load_2d_pair(dst + kWTileBytes, &maps.U[t.mod], (2 * p.esteps + i) * kBK, tokh, full);
                     }
@@ -490,22 +513,40 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
             for (int lin = pair0; lin < p.tiles && ok; lin += npairs) {
                 const PersistTile t(p, lin);
                 const int row_tile = t.row_pair * 2 + (int)rank, tokh = t.tok_tile * p.BN + (int)rank * (p.BN / 2);
-                // own 128 rows of the stacked matrix: Wg and rows of A behind it, or 128 rows of A (zeros past the end)
-                const bool gate = t.stacked && leader;
-                const CUtensorMap* mW = !t.stacked ? &maps.W0[t.mod] : gate ? &maps.A0[t.mod] : &maps.A[t.mod];
-                const int w_row = !t.stacked ? row_tile * kBM : persist_first_row(p, t.row_pair, (int)rank) + (gate ? p.gate_rows : 0);
-                const uint32_t w_off = gate ? (uint32_t)p.gate_rows * 128u : 0u;
+                const uint32_t tx = 2u * kc * ((uint32_t)(t.stacked ? kBM : tr) * 128u + part);
                 uint32_t bar, full, dst;
-                for (int i = 0; i < p.ksteps && ok; ++i) {
-                    if (i == mid && (pending || own)) ok = expand(own ? t : before);
-                    if (!ok || !(ok = slot(bar, full, dst))) break;
-                    if (elect_one()) {
-                        if (leader) mbar_expect_tx(bar, 2 * (uint32_t)p.stage_bytes);
-                        tma_load_2d_pair(dst + w_off, mW, i * kBK, w_row, full);
-                        if (gate) tma_load_2d_pair(dst, &maps.G[t.mod], i * kBK, 0, full);
-                        tma_load_2d_pair(dst + kWTileBytes, &maps.X, i * kBK, tokh, full);
+                if (kWalk == kWalkStacked && t.stacked) {
+                    // own 128 rows of the stacked matrix: Wg and rows of A behind it, or 128 rows of A (zeros past the end)
+                    const CUtensorMap* mW = leader ? &maps.A0[t.mod] : &maps.A[t.mod];
+                    const int w_row = persist_first_row(p, t.row_pair, (int)rank) + (leader ? p.gate_rows : 0);
+                    const uint32_t w_off = leader ? (uint32_t)p.gate_rows * 128u : 0u;
+                    for (int i = 0; i < iters && (ok = slot(bar, full, dst)); ++i) {   // (a pair's first tile: nothing is pending)
+                        if (elect_one()) {
+                            if (leader) mbar_expect_tx(bar, tx);
+                            tma_load_2d_pair(dst + w_off, mW, i * kBK, w_row, full);
+                            if (leader) tma_load_2d_pair(dst, &maps.G[t.mod], i * kBK, 0, full);
+                            tma_load_2d_pair(dst + kWTileBytes, &maps.X, i * kBK, tokh, full);
+                        }
+                        __syncwarp();
                     }
-                    __syncwarp();
+                } else {
+                    const CUtensorMap* mW = &maps.W0[t.mod];
+                    const int w_row = row_tile * tr;
+                    for (int i = 0; i < iters; ++i) {
+                        if (i == mid && (pending || own) && !(ok = expand(own ? t : before))) break;
+                        if (!(ok = slot(bar, full, dst))) break;
+                        if (elect_one()) {
+                            if (leader) mbar_expect_tx(bar, tx);
+                            if (kc == 1) {
+                                tma_load_2d_pair(dst, mW, i * kBK, w_row, full);
+                                tma_load_2d_pair(dst + kWTileBytes, &maps.X, i * kBK, tokh, full);
+                            } else {                              // two k-steps per copy (zeros past the end of the axis)
+                                tma_load_3d_grp(dst, mW, 0, w_row, 2 * i, full);
+                                tma_load_3d_grp(dst + 2 * kWTileBytes, &maps.X, 0, tokh, 2 * i, full);
+                            }
+                        }
+                        __syncwarp();
+                    }
                 }
                 pending = !t.stacked && !own;
                 before = t;
@@ -520,8 +561,9 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
         // ------------------------------------------------------------------ MMA issuer (leader only)
         if (leader) {
             const uint32_t idesc = instr_desc_bf16_pair_n(p.BN);
-            // B's rows in a stage: 16 columns (an MMA) of 128 rows every 4096 bytes, or 2 or 4 such side by side in rows of 64 or 128
-            const uint64_t b_desc = p.cpa == 1 ? smem_desc_plain(0, kBM * 16, 128) : smem_desc_rows(0, 16u * p.cpa);
+            // B's rows in a stage: 16 columns (an MMA) of the CTA's rows every 32 tr bytes, or 2 or 4 such side by side in rows of 64 or
+            // 128.  (The MMAs take 128 rows; with fewer the rest is whatever lies behind, in rows of the accumulator that nobody reads)
+            const uint64_t b_desc = p.cpa == 1 ? smem_desc_plain(0, tr * 16, 128) : smem_desc_rows(0, 16u * p.cpa);
             const int b_side = p.cpa <= 2 ? 0 : p.cpa == 4 ? 1 : 2;   // log2 of the MMAs side by side
             bool ok = true, pending = false;
             int s = 0, phase = 0, n = 0;
@@ -543,7 +585,10 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                     if (!next(wa)) return false;
                     const int first = s;                          // stage with the B rows: released with the parts behind it
                     uint64_t db[3] = {smem_desc_sw128(wa + kWTileBytes), 0, 0};
-                    if (p.parts > 1) {
+                    if (parts > 1 && kc == 2) {
+                        db[1] = smem_desc_sw128(wa + 2 * kWTileBytes);
+                        db[2] = smem_desc_sw128(wa + 2 * kWTileBytes + (uint32_t)p.BN / 2 * 128u);
+                    } else if (parts > 1) {
                         release();
                         if (!next(ua)) return false;
                         db[1] = smem_desc_sw128(ua);
@@ -553,13 +598,13 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                     if (elect_one()) {
 #pragma unroll
                         for (int h = 0; h < 3; ++h)
-                            if (h < p.parts)
+                            if (h < parts)
                                 for (int kk = 0; kk < nm; ++kk)
                                     umma_bf16_pair(tmem_base + b * kPairTokens,
-                                                   b_desc + ((wa + ((kk >> b_side) * (4096 << b_side)) + (kk & ((1 << b_side) - 1)) * 32) >> 4),
+                                                   b_desc + ((wa + ((kk >> b_side) * (tr * 32 << b_side)) + (kk & ((1 << b_side) - 1)) * 32) >> 4),
                                                    db[h] + (uint64_t)(kk * 2), idesc, 1);
                         umma_commit_pair(bar_base + (p.stages + first) * 8);
-                        if (p.parts > 1) umma_commit_pair(bar_base + (p.stages + s) * 8);
+                        if (parts > 1 && kc == 1) umma_commit_pair(bar_base + (p.stages + s) * 8);
                     }
                     __syncwarp();
                     release();
@@ -577,14 +622,20 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                     tc_fence_after();
                 }
                 uint32_t wa;
-                for (int i = 0; i < p.ksteps; ++i) {
+                for (int i = 0; i < iters; ++i) {
                     if (i == mid && (pending || own) && !(ok = expand(own ? b : b ^ 1))) break;
                     if (!(ok = next(wa))) break;
-                    const uint64_t da = smem_desc_sw128(wa), db = smem_desc_sw128(wa + kWTileBytes);
+                    const uint64_t da = smem_desc_sw128(wa), db = smem_desc_sw128(wa + kc * kWTileBytes);
                     if (elect_one()) {
 #pragma unroll
                         for (int kk = 0; kk < kBK / kUmmaK; ++kk)
                             umma_bf16_pair(acc, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc, (i | kk) != 0);
+                        if (kc == 2) {
+                            const uint64_t da2 = da + (uint64_t)(tr * 8), db2 = db + (uint64_t)(p.BN * 4);   // (descriptors count 16 bytes)
+#pragma unroll
+                            for (int kk = 0; kk < kBK / kUmmaK; ++kk)
+                                umma_bf16_pair(acc, da2 + (uint64_t)(kk * 2), db2 + (uint64_t)(kk * 2), idesc, 1);
+                        }
                         umma_commit_pair(bar_base + (p.stages + s) * 8);
                     }
                     __syncwarp();
@@ -606,28 +657,31 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
         const int quad = warp & 3, grp = warp < 6 ? 0 : 1;        // TMEM lanes 32 quad ..; group of four warps
         const int row_in_tile = quad * 32 + lane;
         const bool elected = (warp == 2 || warp == 6) && lane == 0;
-        const int chunks = p.BN / p.CT;
+        const int chunks = (p.BN + kPersistChunk - 1) / kPersistChunk;
         __nv_bfloat16* ystage = reinterpret_cast<__nv_bfloat16*>(store_ptr + grp * kPersistStoreBytes);
         const uint32_t ysmem = store + grp * kPersistStoreBytes;
         bool acc_ok = true;
+        // A first pass through the chunk code on whatever TMEM holds, results dropped: where a pair has a single tile its epilogue would
+        // otherwise fetch the code at the end of the launch, from L2 behind the other pairs' loads (KDRY)
+        bool dry = own;
         int n = 0;
-        for (int lin = pair0; lin < p.tiles; lin += npairs, ++n) {
-            const PersistTile t(p, lin);
+        for (int lin = dry ? pair0 - npairs : pair0; lin < p.tiles; lin += npairs, n += dry ? 0 : 1, dry = false) {
+            const PersistTile t(p, max(lin, 0));
             const int tile_m = t.row_pair * 2 + (int)rank, tok0 = t.tok_tile * p.BN, b = n & 1;
             const PersistModule& mo = p.mod[t.mod];
             // (after an expired wait the rest of the walk only keeps the barriers going)
-            acc_ok = __all_sync(0xFFFFFFFFu, acc_ok && mbar_wait(bar_accf + b * 8, (n >> 1) & 1));
+            if (!dry) acc_ok = __all_sync(0xFFFFFFFFu, acc_ok && mbar_wait(bar_accf + b * 8, (n >> 1) & 1));
             if (!acc_ok && lane == 0) {
                 atomicExch(p.status, 1);
                 atomicExch(p.status + 3, 5300);
             }
             tc_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(b * kPairTokens);
-            if (t.stacked) {
+            if (kWalk == kWalkStacked && t.stacked) {
                 int32_t* flag = p.flags + t.mod * p.tok_tiles + t.tok_tile;
                 // routing of the group's slots in the upper half of the staging buffer, us on its way out in the lower half
                 PersistRouting* rt = reinterpret_cast<PersistRouting*>(reinterpret_cast<uint8_t*>(ystage) + kPersistStoreBytes / 2);
-                const int nslots = grp < chunks ? (chunks - grp + 1) / 2 * p.CT : 0;
+                const int nslots = grp < chunks ? (chunks - grp + 1) / 2 * kPersistChunk : 0;
                 bool have = true;
                 if (rank == 0) {
                     const uint32_t peer_rt = map_to_cta(ysmem + kPersistStoreBytes / 2, 1);
@@ -727,48 +781,59 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                 }
                 continue;
             }
-            // a tile of one chunk (64 tokens at the most) is read by the first group alone: the other one owes its arrival all the same
-            if (grp >= chunks && elected) mbar_arrive_cluster(map_to_cta(bar_acce + b * 8, 0));
-            for (int c = grp; c < chunks; c += 2) {
-                uint32_t v[4][16];
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    if (16 * q < p.CT) tmem_ld16_issue(taddr + (uint32_t)(c * p.CT + 16 * q), v[q]);
+            // a tile of one chunk (32 tokens at the most) is read by the first group alone: the other one owes its arrival all the same
+            if (grp >= chunks && elected && !dry) mbar_arrive_cluster(map_to_cta(bar_acce + b * 8, 0));
+            // A chunk of y as fragments of 32 tokens x 16 rows, rounded, in two blocks of [token][64 rows] with 128-byte swizzle, or (fewer
+            // rows than 128) in rows of tr: four transposing stores per thread instead of 32 of 2 bytes.  Two buffers per group, so that
+            // a chunk is made while the one before is read out: KEP
+            const int y_row = quad * 32 + (lane >> 3) * 8;
+            const bool y_there = y_row < tr;                    // (rows past tr go to the end of the buffer, which no store reads)
+            const uint32_t y_lane = ysmem + (y_there ? (uint32_t)persist_y_at(tr, lane & 7, y_row) * 2u : (uint32_t)(kPersistBufBytes - 128 + (lane & 7) * 16));
+            const uint32_t y_step = !y_there ? 0u : tr == kBM ? 1024u : (uint32_t)tr * 16u;   // to the next 8 tokens
+            for (int c = grp, half = 0; c < (dry ? min(chunks, 2) : chunks); c += 2, half ^= 1) {
+                const int cols = min(kPersistChunk, p.BN - c * kPersistChunk);   // (the last one of a single token tile may be short)
+                const uint32_t buf = (uint32_t)half * kPersistBufBytes;
+                uint32_t v[2][16];                                // 32 tokens of 16 rows each
+                tmem_ld_frag_issue(taddr + (uint32_t)(c * kPersistChunk), v[0]);
+                tmem_ld_frag_issue(taddr + (16u << 16) + (uint32_t)(c * kPersistChunk), v[1]);
+                // this buffer's last store has been read out (of the one in between nobody knows)
+                if (elected) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
                 tmem_ld_wait();
                 const bool last = c + 2 >= chunks;
                 if (last) tc_fence_before();                      // this group's last read of the accumulator
-                // the staging buffer's last store has been read out
-                if (elected) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
                 asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
+                bool nan = false;
 #pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    if (16 * q < p.CT) {
+                for (int i = 0; i < 4; ++i)
+                    if (8 * i < cols) {
+                        float a[8];                               // [8 rows][2 tokens]
 #pragma unroll
-                        for (int i = 0; i < 16; ++i)
-                            ystage[(16 * q + i) * kBM + row_in_tile] = __float2bfloat16_rn(__uint_as_float(v[q][i]));
-                    }
-                if (p.parts > 1) {
-                    bool nan = false;
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        if (16 * q < p.CT) {
-#pragma unroll
-                            for (int i = 0; i < 16; ++i) nan |= __uint_as_float(v[q][i]) != __uint_as_float(v[q][i]);
+                        for (int g = 0; g < 8; ++g) {
+                            a[g] = __uint_as_float(v[g >> 2][4 * i + (g & 3)]);
+                            nan |= a[g] != a[g] && quad * 32 + (g >> 1) * 8 < tr;
                         }
-                    if (__any_sync(0xFFFFFFFFu, nan)) persist_repair(p, mo, ystage, tile_m * kBM, quad, tok0 + c * p.CT, min(p.CT, p.T - tok0 - c * p.CT));
+                        stmatrix_x4_trans(y_lane + buf + (uint32_t)i * y_step, pack_bf16(a[0], a[1]), pack_bf16(a[2], a[3]), pack_bf16(a[4], a[5]),
+                                          pack_bf16(a[6], a[7]));
+                    }
+                const int tok = tok0 + c * kPersistChunk;
+                if (parts > 1 && __any_sync(0xFFFFFFFFu, nan) && !dry) {
+                    __syncwarp();
+                    persist_repair(p, mo, ystage + buf / 2, tile_m * tr, quad, tok, min(cols, p.T - tok));
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> TMA read
                 asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
-                if (elected) {
+                if (elected && !dry) {
                     if (last) mbar_arrive_cluster(map_to_cta(bar_acce + b * 8, 0));
-                    if (tile_m < mo.row_tiles && tok0 + c * p.CT < p.T) {   // rows beyond d_out and tokens beyond T are clipped by the map
+                    // rows beyond d_out and tokens beyond T are clipped by the map; a group per chunk, also an empty one
+                    for (int h = 0; h < (tr == kBM ? 2 : 1) && tok < p.T && tile_m * tr + 64 * h < mo.d_out; ++h)
                         asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
-                                     ::"l"((uint64_t)&maps.Y[t.mod]), "r"(ysmem), "r"(tile_m * kBM), "r"(tok0 + c * p.CT)
+                                     ::"l"((uint64_t)&maps.Y[t.mod]), "r"(ysmem + buf + (uint32_t)(h * kPersistChunk * 128)), "r"(tile_m * tr + 64 * h), "r"(tok)
                                      : "memory");
-                        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-                    }
+                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                 }
             }
+            // (an odd number of chunks: the next tile begins with the same buffer again, so both stores have to be out)
+            if (((chunks - grp + 1) / 2) % 2 != 0 && elected) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
         }
         if (elected) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
@@ -776,7 +841,7 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
     __syncwarp();
     cluster_sync();                                               // nobody leaves while the peer may still signal it
     if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
-    if (p.stacked_pairs > 0 && threadIdx.x == 0) {                // the last CTA to leave readies the flags for the next call
+    if (kWalk == kWalkStacked && threadIdx.x == 0) {                // the last CTA to leave readies the flags for the next call
         if (atomicAdd(p.leave_ctr, 1) == (int)gridDim.x - 1) {
             for (int i = 0; i < p.n_mod * p.tok_tiles; ++i) p.flags[i] = 0;
             *p.leave_ctr = 0;

@@ -825,19 +825,19 @@ static int get_store_map(const void* y, int d_out, int T, int box_tokens, CUtens
     return r == CUDA_SUCCESS ? METEORA_OK : METEORA_ERR_CUDA;
 }
 
-// Tensor map of the adapters' B[N, d_out, r] (bf16) whose box holds, for 128 output rows, 64 rank entries as K-major MMA operands.
+// Tensor map of the adapters' B[N, d_out, r] (bf16) whose box holds, for `rows` outputs, 64 rank entries as K-major MMA operands.
 // Rank 8: 8 adapters as un-swizzled core matrices, [adapter][row][16 bytes]; 8 rows (128 bytes) are contiguous and the inner
 // axis.  Larger ranks: 64 / r adapters, [adapter][row][2 r bytes], swizzled over those 32, 64 or 128 bytes.  (As core matrices they
 // came in pieces of 16 bytes, 1450 cycles for a box: 5120 -> 5120 at 1531 tokens, rank 16, 87.7 us then and 81.9 now; 4096 -> 4096 at 2048 tokens, rank 32, 104 and 91.)
 // Needs d_out % 8 == 0, r / 8 in {1, 2, 4, 8}.
-static int get_adapter_map(const void* B, int N, int d_out, int r, CUtensorMap* out) {
+static int get_adapter_map(const void* B, int N, int d_out, int r, int rows, CUtensorMap* out) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return METEORA_ERR_CUDA;
     const bool core = r == 8;
     const cuuint32_t estride[3] = {1, 1, 1};
     const cuuint64_t gdim[3] = {core ? 64 : (cuuint64_t)r, core ? (cuuint64_t)d_out / 8 : (cuuint64_t)d_out, (cuuint64_t)N};
     const cuuint64_t gstride[2] = {core ? 128 : (cuuint64_t)r * 2, (cuuint64_t)d_out * r * 2};
-    const cuuint32_t box[3] = {core ? 64 : (cuuint32_t)r, core ? kBM / 8 : kBM, core ? 8 : 64 / (cuuint32_t)r};
+    const cuuint32_t box[3] = {core ? 64 : (cuuint32_t)r, (cuuint32_t)(core ? rows / 8 : rows), core ? 8 : 64 / (cuuint32_t)r};
     const CUtensorMapSwizzle swizzle = core      ? CU_TENSOR_MAP_SWIZZLE_NONE
                                        : r == 16 ? CU_TENSOR_MAP_SWIZZLE_32B
                                        : r == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
@@ -1427,7 +1427,7 @@ static int pair_tail_carve(const meteora_shape_t& s) {
 // ------------------------------------------------------------------------------------------------
 struct PersistPlan {
     bool ok;
-    int BN, CT, stages, stage_bytes, pairs, tok_tiles, tiles;
+    int walk, BN, tr, stages, stage_bytes, pairs, tok_tiles, tiles;
     int stacked_pairs, gate_rows, us_cols;                       // stacked_pairs 0: the routing comes from kernels of its own
     size_t smem;
 };
@@ -1449,6 +1449,11 @@ int persist_us_parts(const meteora_shape_t& s) {
     return pairs * 4 >= sm_count() || (s.r == 8 && s.N <= 80) ? 1 : 3;
 }
 
+typedef void (*PersistKernel)(const PersistMaps, const PersistParams);
+static PersistKernel persist_kernel(int walk) {
+    return walk == kWalkStacked ? k_wgemm_persist<kWalkStacked> : walk == kWalkBase ? k_wgemm_persist<kWalkBase> : k_wgemm_persist<kWalkNarrow>;
+}
+
 // Pairs the device holds at once (0: it cannot say).
 static int persist_pairs() {
     static std::atomic<int> cache[64];                           // 0: not asked yet, else pairs + 1
@@ -1461,11 +1466,12 @@ static int persist_pairs() {
         cfg.gridDim = dim3(2 * kPersistMaxPairs);
         cfg.blockDim = dim3(kThreads);
         cfg.dynamicSmemBytes = 227 * 1024;
-        if (cudaFuncSetAttribute(k_wgemm_persist, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
-            cudaOccupancyMaxActiveClusters(&n, k_wgemm_persist, &cfg) != cudaSuccess) {
-            cudaGetLastError();
-            return 0;
-        }
+        for (int walk : {kWalkBase, kWalkNarrow, kWalkStacked})
+            if (cudaFuncSetAttribute(persist_kernel(walk), cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
+                cudaOccupancyMaxActiveClusters(&n, persist_kernel(walk), &cfg) != cudaSuccess) {
+                cudaGetLastError();
+                return 0;
+            }
         have = std::min(n, kPersistMaxPairs) + 1;
         cache[dev].store(have, std::memory_order_relaxed);
     }
@@ -1480,10 +1486,12 @@ static PersistPlan make_persist_plan(const meteora_shape_t& s, const int* d_outs
     if (!tc_path_supported(s)) return pp;
     const int pairs = persist_pairs();
     if (pairs < 1) return pp;
-    // tokens per tile: 256-token tiles, narrower ones (whole 32s) where that spreads a ragged token count over as many tiles
+    // tokens per tile: 256-token tiles, narrower ones (whole 32s) where that spreads a ragged token count over as many tiles; a single
+    // tile is as narrow as its MMAs can be, its last epilogue chunk short (200 tokens: 208 columns, not 224; KBN)
     pp.tok_tiles = (s.T + kPairTokens - 1) / kPairTokens;
-    pp.BN = ((s.T + pp.tok_tiles - 1) / pp.tok_tiles + 31) / 32 * 32;
-    pp.CT = pp.BN % 64 == 0 ? 64 : 32;
+    const int width = pp.tok_tiles == 1 ? 16 : 32;
+    pp.BN = ((s.T + pp.tok_tiles - 1) / pp.tok_tiles + width - 1) / width * width;
+    pp.tr = kBM;
     for (int m = 0; m < G; ++m) {
         meteora_shape_t sm = s;
         sm.d_out = d_outs[m];
@@ -1525,8 +1533,23 @@ static PersistPlan make_persist_plan(const meteora_shape_t& s, const int* d_outs
         if (tn.persist != 2 && pp.tiles <= pairs && with > pairs) return pp;
         pp.tiles = with;
     }
+    // Up to 128 tokens the MMAs are short: two k-steps per stage, since waits, copies and commits cost the issuing warps about 400 cycles
+    // per stage whatever it holds (MMAs of 64 columns: 180 per k-step).  KKC
+    pp.walk = with_routing ? kWalkStacked : s.T <= kBM && s.d_in % kBK == 0 ? kWalkNarrow : kWalkBase;
+    // More than one round of them: tiles of fewer rows, so that the last round is not half empty.  KTR
+    if (pp.walk == kWalkNarrow && pp.tiles > pairs && pp.tiles <= 2 * pairs) {
+        const int late = std::min(8 * G, pairs / 2), slots = 2 * pairs - late;
+        auto tiles_of = [&](int rows) {
+            int n = 0;
+            for (int m = 0; m < G; ++m) n += (d_outs[m] + 2 * rows - 1) / (2 * rows);
+            return n;
+        };
+        while (pp.tr > 64 && tiles_of(pp.tr - 8) <= slots) pp.tr -= 8;
+        pp.tiles = tiles_of(pp.tr);
+    }
     pp.pairs = std::min(pairs, pp.tiles);
-    pp.stage_bytes = kWTileBytes + pp.BN / 2 * 128;
+    const int kc = pp.walk == kWalkNarrow ? 2 : 1;
+    pp.stage_bytes = kc * (kWTileBytes + pp.BN / 2 * 128);
     const size_t fixed = 1024 + (size_t)kPersistStageBufs * kPersistStoreBytes + 512;
     pp.stages = (int)std::min<size_t>((227 * 1024 - fixed) / pp.stage_bytes, 12);
     pp.smem = fixed + (size_t)pp.stages * pp.stage_bytes;
@@ -1566,17 +1589,20 @@ static int launch_persist(const PersistPlan& pp, const void* x, const GroupModul
     PersistMaps maps;
     PersistParams p = {};
     int rc;
-    if ((rc = get_tensor_map(x, s.d_in, s.T, pp.BN / 2, 0, &maps.X)) != METEORA_OK) return rc;
+    const int depth = pp.walk == kWalkNarrow ? 2 : 0;            // (3-D maps)
+    if ((rc = get_tensor_map(x, s.d_in, s.T, pp.BN / 2, depth, &maps.X)) != METEORA_OK) return rc;
     int tile0 = G * pp.stacked_pairs * pp.tok_tiles;
     p.parts = pp.stacked_pairs > 0 ? 1 : mods[0].ws.us_parts;     // (base products of several modules: decode batches, 3 for all)
     for (int m = 0; m < kMaxGroupModules; ++m) {
         const GroupModule& gm = mods[m < G ? m : 0];             // unused slots repeat module 0's (valid) maps
-        if ((rc = get_tensor_map(gm.W0, s.d_in, gm.d_out, kBM, 0, &maps.W0[m])) != METEORA_OK) return rc;
-        if ((rc = get_adapter_map(gm.B, s.N, gm.d_out, s.r, &maps.B[m])) != METEORA_OK) return rc;
+        if ((rc = get_tensor_map(gm.W0, s.d_in, gm.d_out, pp.tr, depth, &maps.W0[m])) != METEORA_OK) return rc;
+        if ((rc = get_adapter_map(gm.B, s.N, gm.d_out, s.r, pp.tr, &maps.B[m])) != METEORA_OK) return rc;
         if (gm.ws.us_parts != mods[0].ws.us_parts && pp.stacked_pairs == 0) return METEORA_ERR_UNSUPPORTED_SHAPE;   // (not planned)
         const int ld_us = gm.ws.us_cols * p.parts;
         if ((rc = get_tensor_map(gm.ws.us, ld_us, s.T, pp.BN / 2, 0, &maps.U[m])) != METEORA_OK) return rc;
-        if ((rc = get_store_map(gm.y, gm.d_out, s.T, pp.CT, &maps.Y[m])) != METEORA_OK) return rc;
+        if ((rc = get_store_map(gm.y, gm.d_out, s.T, kPersistChunk, &maps.Y[m], pp.tr == kBM ? 64 : pp.tr,
+                                pp.tr == kBM ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE)) != METEORA_OK)
+            return rc;
         if ((rc = get_store_map(gm.ws.us, ld_us, s.T, 32, &maps.S[m], 32, CU_TENSOR_MAP_SWIZZLE_64B)) != METEORA_OK) return rc;
         maps.A[m] = maps.A0[m] = maps.G[m] = maps.X;
         if (pp.stacked_pairs > 0) {
@@ -1585,8 +1611,7 @@ static int launch_persist(const PersistPlan& pp, const void* x, const GroupModul
             if ((rc = get_tensor_map(gm.Wg, s.d_in, s.N, pp.gate_rows, 0, &maps.G[m])) != METEORA_OK) return rc;
         }
         PersistModule& mo = p.mod[m];
-        mo.row_tiles = (gm.d_out + kBM - 1) / kBM;
-        mo.row_pairs = (mo.row_tiles + 1) / 2;
+        mo.row_pairs = (gm.d_out + 2 * pp.tr - 1) / (2 * pp.tr);
         mo.group_pairs = std::min(tuning().group_pairs > 0 ? tuning().group_pairs : std::max(1, (pp.pairs / pp.tok_tiles + 1) / 2), mo.row_pairs);
         mo.tile0 = m < G ? tile0 : 0x7FFFFFFF;
         mo.us = (const __nv_bfloat16*)gm.ws.us;
@@ -1599,7 +1624,6 @@ static int launch_persist(const PersistPlan& pp, const void* x, const GroupModul
     }
     p.T = s.T;
     p.BN = pp.BN;
-    p.CT = pp.CT;
     p.ksteps = (s.d_in + kBK - 1) / kBK;
     p.esteps = mods[0].ws.us_cols / kBK;
     p.N = s.N;
@@ -1609,6 +1633,7 @@ static int launch_persist(const PersistPlan& pp, const void* x, const GroupModul
     p.nblk = s.N * p.cpa;
     p.stages = pp.stages;
     p.stage_bytes = pp.stage_bytes;
+    p.tr = pp.tr;
     p.n_mod = G;
     p.tok_tiles = pp.tok_tiles;
     p.tiles = pp.tiles;
@@ -1643,14 +1668,14 @@ static int launch_persist(const PersistPlan& pp, const void* x, const GroupModul
     cfg.attrs = attr;
     cfg.numAttrs = na;
     p.pdl = want_pdl ? 1 : 0;
-    cudaError_t err = cudaLaunchKernelEx(&cfg, k_wgemm_persist, maps, p);
+    cudaError_t err = cudaLaunchKernelEx(&cfg, persist_kernel(pp.walk), maps, p);
     if (pp.stacked_pairs > 0 && launch_config_refused(err) && want_pdl) {   // the two attributes together: try without the second
         cudaGetLastError();
         pdl_accepted.store(false, std::memory_order_relaxed);
         tuning().pdl_decode_refused += 1;
         cfg.numAttrs = na - 1;
         p.pdl = 0;
-        err = cudaLaunchKernelEx(&cfg, k_wgemm_persist, maps, p);
+        err = cudaLaunchKernelEx(&cfg, persist_kernel(pp.walk), maps, p);
     }
     if (pp.stacked_pairs > 0 && launch_config_refused(err)) {    // the caller may take the routing kernels instead
         cudaGetLastError();

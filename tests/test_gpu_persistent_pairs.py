@@ -125,3 +125,42 @@ def test_selection_in_the_walk(T, d_in, d_out, N, r, k):
     ref = oracle.linear_forward_routed(w["x"][sel], w["W0"], w["A"], w["B"], w["Wg"], idx[sel])
     assert rel_l2(y[sel], ref) <= 5e-3
     assert bf16_bound_ok(y[sel], ref) <= 0.0
+
+
+# One token tile as wide as its tokens, in steps of 16: chunks of the epilogue that are whole, short and of one step; rows that end
+# inside a tile and inside one of its halves of 64.
+@pytest.mark.parametrize("T,d_out", [(49, 9216), (64, 9224), (72, 9288), (129, 9216), (200, 9408), (225, 9280), (240, 9352), (256, 9216)])
+def test_single_token_tile(T, d_out):
+    w = workloads.make_workload("one_tile", T=T, d_in=2048, d_out=d_out, dtype="bf16", seed=290 + T, b_std=0.3)
+    t = to_dev(w, "x", "W0", "A", "B", "Wg")
+    shape = mb.make_shape(T, 2048, d_out, 28, 8, 2, torch.bfloat16)
+    assert f"tile=256x{(T + 15) // 16 * 16}" in mb.meteora_describe_plan(shape), mb.meteora_describe_plan(shape)
+    ws = mb.alloc_workspace(shape)
+    guard = torch.full((T + 64, d_out), 7.0, device="cuda", dtype=torch.bfloat16)
+    y, idx, _ = mb.meteora_linear_forward(*t, 2, workspace=ws, return_routing=True, out=guard[:T])
+    assert mb.meteora_workspace_status(ws) == 0
+    assert (guard[T:] == 7.0).all()                      # nothing past the batch is written
+    y, idx = y.float().cpu().numpy(), idx.cpu().numpy()
+    o_idx, _, o_logits = oracle.gate_topk(w["x"], w["Wg"], 2)
+    check_selection(idx, o_idx, o_logits, 2)
+    sel = np.unique(np.concatenate([np.arange(0, T, 17), np.arange(15, T, 16), [T - 1]]))
+    ref = oracle.linear_forward_routed(w["x"][sel], w["W0"], w["A"], w["B"], w["Wg"], idx[sel])
+    assert rel_l2(y[sel], ref) <= 5e-3
+    assert bf16_bound_ok(y[sel], ref) <= 0.0
+
+
+# Decode batches of more than one round: tiles of fewer rows (8 to 56 less than 128 per CTA), ends inside and at the edge of a tile,
+# adapters of one block and of two.
+@pytest.mark.parametrize("T,d_in,d_outs,r", [(40, 2048, (14336, 14336), 8), (64, 2048, (11008, 11008), 8), (100, 2048, (13824, 13824), 8),
+                                             (128, 2048, (19000, 504), 8), (33, 2048, (20480,), 8), (64, 2048, (25608,), 16), (90, 2048, (14336, 14344), 8)])
+def test_tiles_of_fewer_rows(T, d_in, d_outs, r):
+    ws = [workloads.make_workload(f"rows/{m}", T=T, d_in=d_in, d_out=d, N=12, r=r, k=2, dtype="bf16", seed=9800 + T + m, b_std=0.3)
+          for m, d in enumerate(d_outs)]
+    for w in ws[1:]:
+        w.tensors["x"] = ws[0]["x"]
+    if len(d_outs) == 1:
+        t = to_dev(ws[0], "x", "W0", "A", "B", "Wg")
+        guard = torch.full((T + 64, d_outs[0]), 7.0, device="cuda", dtype=torch.bfloat16)
+        mb.meteora_linear_forward(*t, 2, out=guard[:T])
+        assert (guard[T:] == 7.0).all()
+    check_group(ws, 1e-2)
