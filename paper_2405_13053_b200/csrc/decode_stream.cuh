@@ -328,8 +328,7 @@ k_decode_stream(const __grid_constant__ DecodeMaps maps, const __grid_constant__
                     __syncwarp();
                 }
                 bool ok = true;
-                for (int i = pre; i < niter; ++i) {
-                    const int s = i % d.aux_stages, round = i / d.aux_stages;
+                for (int i = pre, s = 0, round = 1; i < niter; ++i) {   // (every stage is filled: pre is their number)
                     ok = mbar_wait_warp(bar_base + (d.bar_slots + s) * 8, (round & 1) ^ 1);
                     if (!ok) break;
                     const uint32_t full = bar_base + s * 8, dst = ring + s * aux_stage_bytes;
@@ -340,14 +339,14 @@ k_decode_stream(const __grid_constant__ DecodeMaps maps, const __grid_constant__
                         tma_load_3d(dst + kWTileBytes, &tmX1, 0, 0, ks0 + i, full);
                     }
                     __syncwarp();
+                    if (++s == d.aux_stages) s = 0, ++round;
                 }
                 if (!ok && lane == 0) stream_flag_error(d, 1, 400);
             }
         } else if (warp == 1) {
             if (active) {
                 bool ok = true;
-                for (int i = 0; i < niter; ++i) {
-                    const int s = i % d.aux_stages, round = i / d.aux_stages;
+                for (int i = 0, s = 0, round = 0; i < niter; ++i) {
                     ok = mbar_wait_warp(bar_base + s * 8, round & 1);
                     if (!ok) break;
                     tc_fence_after();
@@ -361,6 +360,7 @@ k_decode_stream(const __grid_constant__ DecodeMaps maps, const __grid_constant__
                         if (i == niter - 1) umma_commit(bar_acc);
                     }
                     __syncwarp();
+                    if (++s == d.aux_stages) s = 0, ++round;
                 }
                 if (niter == 0 || !ok) {                             // (a failed wait: whatever was issued)
                     if (elect_one()) umma_commit(bar_acc);
