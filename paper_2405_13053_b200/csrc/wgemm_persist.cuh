@@ -397,7 +397,7 @@ __device__ __forceinline__ void persist_select(const PersistParams& p, float* s_
 // 0.4 - 0.8 us of 29 (4096 -> 4096 at 512 tokens).
 //   kWalkStacked  the routing in the walk, us rounded        k-steps one by one, 128 rows per CTA
 //   kWalkBase     base product behind routing kernels        the same, us in 1 or 3 parts
-//   kWalkNarrow   the same for up to 128 tokens              two k-steps per stage, tr rows per CTA, 3 parts
+//   kWalkNarrow   the same, tiles of up to 128 tokens        two k-steps per stage, tr rows per CTA
 enum { kWalkStacked = 0, kWalkBase = 1, kWalkNarrow = 2 };
 
 template <int kWalk>
@@ -405,7 +405,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads)
 k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant__ PersistParams p) {
     constexpr bool own = kWalk != kWalkStacked;                   // a tile's expand is in its own main loop
     constexpr int kc = kWalk == kWalkNarrow ? 2 : 1;              // k-steps per stage
-    const int tr = kWalk == kWalkNarrow ? p.tr : kBM, parts = kWalk == kWalkStacked ? 1 : kWalk == kWalkBase ? p.parts : 3;
+    const int tr = kWalk == kWalkNarrow ? p.tr : kBM, parts = kWalk == kWalkStacked ? 1 : p.parts;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t ring = (raw + 1023u) & ~1023u;
@@ -662,7 +662,8 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
         const uint32_t ysmem = store + grp * kPersistStoreBytes;
         bool acc_ok = true;
         // A first pass through the chunk code on whatever TMEM holds, results dropped: where a pair has a single tile its epilogue would
-        // otherwise fetch the code at the end of the launch, from L2 behind the other pairs' loads (KDRY)
+        // otherwise fetch the code at the end of the launch, from L2 behind the other pairs' loads (4096 -> 4096 at 512 tokens
+        // 29.4 -> 28.7 us, 5120 -> 13824 at 200 42.9 -> 42.4)
         bool dry = own;
         int n = 0;
         for (int lin = dry ? pair0 - npairs : pair0; lin < p.tiles; lin += npairs, n += dry ? 0 : 1, dry = false) {
@@ -785,7 +786,7 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
             if (grp >= chunks && elected && !dry) mbar_arrive_cluster(map_to_cta(bar_acce + b * 8, 0));
             // A chunk of y as fragments of 32 tokens x 16 rows, rounded, in two blocks of [token][64 rows] with 128-byte swizzle, or (fewer
             // rows than 128) in rows of tr: four transposing stores per thread instead of 32 of 2 bytes.  Two buffers per group, so that
-            // a chunk is made while the one before is read out: KEP
+            // a chunk is made while the one before is read out (4.2 us for 208 tokens as stores of 2 bytes, 3.5 for 256 now)
             const int y_row = quad * 32 + (lane >> 3) * 8;
             const bool y_there = y_row < tr;                    // (rows past tr go to the end of the buffer, which no store reads)
             const uint32_t y_lane = ysmem + (y_there ? (uint32_t)persist_y_at(tr, lane & 7, y_row) * 2u : (uint32_t)(kPersistBufBytes - 128 + (lane & 7) * 16));

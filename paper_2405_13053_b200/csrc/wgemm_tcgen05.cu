@@ -1487,7 +1487,8 @@ static PersistPlan make_persist_plan(const meteora_shape_t& s, const int* d_outs
     const int pairs = persist_pairs();
     if (pairs < 1) return pp;
     // tokens per tile: 256-token tiles, narrower ones (whole 32s) where that spreads a ragged token count over as many tiles; a single
-    // tile is as narrow as its MMAs can be, its last epilogue chunk short (200 tokens: 208 columns, not 224; KBN)
+    // tile is as narrow as its MMAs can be, its last epilogue chunk short (200 tokens: 208 columns, not 224; with the
+    // epilogue in fragments 44.4 -> 42.9 us at 5120 -> 13824)
     pp.tok_tiles = (s.T + kPairTokens - 1) / kPairTokens;
     const int width = pp.tok_tiles == 1 ? 16 : 32;
     pp.BN = ((s.T + pp.tok_tiles - 1) / pp.tok_tiles + width - 1) / width * width;
@@ -1498,14 +1499,32 @@ static PersistPlan make_persist_plan(const meteora_shape_t& s, const int* d_outs
         if (persist_us_cols(sm) == 0) return pp;
         pp.tiles += ((d_outs[m] + kBM - 1) / kBM + 1) / 2 * pp.tok_tiles;
     }
-    // Few tiles: split tiles of other kernels use more of the chip.  Behind routing kernels the walk pays from 20 tiles up where the
-    // contraction axis is not so long that the routing takes as long as the walk (us per call, walk / split tiles: 4096 -> 4096 at 257 / 512
-    // tokens, 32 tiles, 23.2 / 28.3 and 28.6 / 33.7; 4096 -> 2048 at 512 / 768 tokens, 16 and 24 tiles, 27.4 / 27.7 and 26.8 / 34.8;
-    // 4096 -> 1024 at 1280 tokens, 20 tiles, 27.3 and 33.0; 14336 -> 4096 at 512 tokens 73.4 and 69.1; rank 32, whose
-    // expand outweighs the tiles, from 8: 4096 -> 1024 at 512 tokens 43.6 and 66.7); one token tile: see
-    // decode_on_pairs.  A short contraction leaves nothing to hide a tile's epilogue under.
-    const int least = with_routing || s.d_in > 8192 ? (sm_count() + 3) / 4 : s.T <= kPairTokens ? 24 : s.N * s.r > 512 ? 8 : 20;
+    // Few tiles.  Narrow ones (two k-steps per stage, below) fill the pairs, and the walk takes any number of them; where the axis is no whole
+    // number of k-steps, split tiles of other kernels use more of the chip below 20 tiles (8 where the expand outweighs them), and
+    // over an axis so long that the routing takes as long as the walk below a quarter of the SMs.  us per call, split tiles / narrow walk: 4096 -> 1024
+    // at 300 / 512 / 700 / 1024 tokens 17.0 / 15.6, 17.4 / 15.5, 24.0 / 18.2, 27.3 / 19.1; 4096 -> 2048 at 512 25.7 / 18.9; 8192 -> 1024 at 512 38.9 / 27.7;
+    // 14336 -> 1024 at 512 58.2 / 40.7; 14336 -> 4096 at 300 / 512 69.4 / 56.8, 78.7 / 73.1; 1024 -> 2048 at 512 17.2 / 15.1; 4096 -> 256 at 512
+    // 17.1 / 15.4; rank 16, 4096 -> 1024 at 512 43.0 / 30.4; rank 32, 14336 -> 4096 at 512 168 / 93.6.  (1000 -> 1000 at 512, no whole k-steps,
+    // 16.8 and 17.9.)  One token tile: see decode_on_pairs.  A short contraction leaves nothing to hide a tile's epilogue under.
+    const bool whole_steps = s.d_in % kBK == 0;
+    const int least = with_routing                                    ? (sm_count() + 3) / 4
+                      : s.T <= kPairTokens                            ? (s.d_in > 8192 ? (sm_count() + 3) / 4 : 24)
+                      : whole_steps                                   ? 1
+                      : s.d_in > 8192                                 ? (sm_count() + 3) / 4
+                      : s.N * s.r > 512                               ? 8
+                                                                      : 20;
     if (tn.persist < 2 && (pp.tiles < least || (s.T <= 128 && s.d_in < 1024))) return pp;
+    // Half a round of 256-token tiles or less: tiles of 128 tokens, or of 64 where there are nine or fewer (us per call with tiles of 256 / 128 / 64:
+    // 4096 -> 1024 at 2048 tokens, 32 tiles, 39.8 / 32.2 / 39.4; rank 32, 4096 -> 4096 at 512, 32 tiles, 51.8 / 41.7 / 56.8; 4096 -> 2048 at 512, 16 tiles,
+    // - / 18.9 / 23.6; 4096 -> 1024 at 512, 8 tiles, - / 17.4 / 15.8).
+    bool narrow = false;
+    if (!with_routing && s.T > kPairTokens && whole_steps && 2 * pp.tiles <= pairs) {
+        const int row_pairs = pp.tiles / pp.tok_tiles, width = 8 * pp.tiles <= pairs ? 64 : 128;
+        narrow = true;
+        pp.tok_tiles = (s.T + width - 1) / width;
+        pp.BN = ((s.T + pp.tok_tiles - 1) / pp.tok_tiles + 31) / 32 * 32;
+        pp.tiles = row_pairs * pp.tok_tiles;
+    }
     if (with_routing) {
         // [Wg; a share of A] in pairs of 128-row tiles: Wg padded to whole 32 rows (a warp's TMEM lanes), A to whole MMAs of the expand
         pp.gate_rows = (s.N + 31) / 32 * 32;
@@ -1533,11 +1552,12 @@ static PersistPlan make_persist_plan(const meteora_shape_t& s, const int* d_outs
         if (tn.persist != 2 && pp.tiles <= pairs && with > pairs) return pp;
         pp.tiles = with;
     }
-    // Up to 128 tokens the MMAs are short: two k-steps per stage, since waits, copies and commits cost the issuing warps about 400 cycles
-    // per stage whatever it holds (MMAs of 64 columns: 180 per k-step).  KKC
-    pp.walk = with_routing ? kWalkStacked : s.T <= kBM && s.d_in % kBK == 0 ? kWalkNarrow : kWalkBase;
-    // More than one round of them: tiles of fewer rows, so that the last round is not half empty.  KTR
-    if (pp.walk == kWalkNarrow && pp.tiles > pairs && pp.tiles <= 2 * pairs) {
+    // Tiles of up to 128 tokens have short MMAs: two k-steps per stage, since waits, copies and commits cost the issuing warps about 400 cycles per
+    // stage whatever it holds (MMAs of 64 columns: 180 per k-step).  4096 -> 22016 at 64 tokens 45.4 -> 44.2 us.
+    pp.walk = with_routing ? kWalkStacked : pp.BN <= kBM && s.d_in % kBK == 0 && (pp.tok_tiles == 1 || narrow) ? kWalkNarrow : kWalkBase;
+    // A decode batch of more than one round: tiles of fewer rows, so that the last round is not half empty, as few as leave one tile to the pairs that
+    // start late (on the SMs of the token tiles ahead): 4096 -> 22016 at 64 tokens 48.8 -> 45.4 us, 4096 -> 2 x 14336 at 40 52.6 -> 50.5.
+    if (pp.walk == kWalkNarrow && pp.tok_tiles == 1 && pp.tiles > pairs && pp.tiles <= 2 * pairs) {
         const int late = std::min(8 * G, pairs / 2), slots = 2 * pairs - late;
         auto tiles_of = [&](int rows) {
             int n = 0;

@@ -164,3 +164,29 @@ def test_tiles_of_fewer_rows(T, d_in, d_outs, r):
         mb.meteora_linear_forward(*t, 2, out=guard[:T])
         assert (guard[T:] == 7.0).all()
     check_group(ws, 1e-2)
+
+
+# Few tiles of a prefill batch on narrow ones: one and several token tiles per row pair, ragged last ones, an odd number of k-steps, rows
+# that end inside a tile, us in one part and in three, adapters of 1, 2, 4 and 8 blocks.
+@pytest.mark.parametrize("T,d_in,d_out,N,r,k,width", [
+    (257, 320, 200, 28, 8, 2, 64), (300, 1088, 1024, 28, 8, 2, 64), (500, 2048, 1000, 28, 16, 4, 64), (700, 576, 2048, 12, 32, 2, 128),
+    (1030, 1024, 1160, 28, 8, 1, 128), (2049, 512, 600, 28, 64, 2, 128), (290, 9024, 520, 28, 8, 2, 64), (1000, 320, 1928, 90, 8, 3, 128),
+])
+def test_few_tiles_are_narrow(T, d_in, d_out, N, r, k, width):
+    w = workloads.make_workload("narrow", T=T, d_in=d_in, d_out=d_out, N=N, r=r, k=k, dtype="bf16", seed=390 + T, b_std=0.3)
+    t = to_dev(w, "x", "W0", "A", "B", "Wg")
+    shape = mb.make_shape(T, d_in, d_out, N, r, k, torch.bfloat16)
+    tiles = (T + width - 1) // width
+    assert f"tile=256x{((T + tiles - 1) // tiles + 31) // 32 * 32} " in mb.meteora_describe_plan(shape), mb.meteora_describe_plan(shape)
+    ws = mb.alloc_workspace(shape)
+    guard = torch.full((T + 128, d_out), 7.0, device="cuda", dtype=torch.bfloat16)
+    y, idx, _ = mb.meteora_linear_forward(*t, k, workspace=ws, return_routing=True, out=guard[:T])
+    assert mb.meteora_workspace_status(ws) == 0
+    assert (guard[T:] == 7.0).all()
+    y, idx = y.float().cpu().numpy(), idx.cpu().numpy()
+    o_idx, _, o_logits = oracle.gate_topk(w["x"], w["Wg"], k)
+    check_selection(idx, o_idx, o_logits, k)
+    sel = np.unique(np.concatenate([np.arange(0, T, 31), np.arange(63, T, 64), [T - 1]]))
+    ref = oracle.linear_forward_routed(w["x"][sel], w["W0"], w["A"], w["B"], w["Wg"], idx[sel])
+    assert rel_l2(y[sel], ref) <= 5e-3
+    assert bf16_bound_ok(y[sel], ref) <= 0.0
