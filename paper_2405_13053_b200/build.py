@@ -13,7 +13,7 @@ CSRC = os.path.join(_PKG, "csrc")
 LIB_PATH = os.path.join(_PKG, "libmeteora.so")
 NATIVE_PATH = os.path.join(_PKG, "_native.so")
 NATIVE_SOURCE = "native.cpp"
-SOURCES = ["api.cu", "gate_topk.cu", "route.cu", "lora.cu", "gemm_simt.cu", "wgemm_tcgen05.cu", "lora_static.cu",
+SOURCES = ["api.cu", "host_copy.cu", "gate_topk.cu", "route.cu", "lora.cu", "gemm_simt.cu", "wgemm_tcgen05.cu", "lora_static.cu",
            "gate_backward.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xptxas", "-v"]

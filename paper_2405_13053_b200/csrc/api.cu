@@ -447,14 +447,9 @@ int meteora_linear_forward_host(const void* x_host, const void* W0, const void* 
     if (workspace_bytes < ws.bytes) return METEORA_ERR_WORKSPACE_TOO_SMALL;
     cudaStream_t st = (cudaStream_t)stream;
     const size_t es = elem_size(shape->dtype);
-    if (cudaMemcpyAsync(ws.x_dev, x_host, (size_t)shape->T * shape->d_in * es, cudaMemcpyHostToDevice, st) !=
-        cudaSuccess)
-        return METEORA_ERR_CUDA;
+    if ((rc = launch_host_copy(ws.x_dev, x_host, (size_t)shape->T * shape->d_in * es, true, st)) != METEORA_OK) return rc;
     if ((rc = forward_device(ws.x_dev, W0, A, B, Wg, *shape, ws.y_dev, ws, st)) != METEORA_OK) return rc;
-    if (cudaMemcpyAsync(y_host, ws.y_dev, (size_t)shape->T * shape->d_out * es, cudaMemcpyDeviceToHost, st) !=
-        cudaSuccess)
-        return METEORA_ERR_CUDA;
-    return METEORA_OK;
+    return launch_host_copy(y_host, ws.y_dev, (size_t)shape->T * shape->d_out * es, false, st);
 }
 
 size_t meteora_workspace_bytes(const meteora_shape_t* shape) {

@@ -79,6 +79,8 @@ int launch_shrink_segments(const void* x, const void* A, const int32_t* offsets,
                            const meteora_shape_t& s, float* u, cudaStream_t st);
 int launch_expand(const void* B, const int32_t* topk_idx, const float* topk_w, const float* u,
                   const meteora_shape_t& s, float* delta, cudaStream_t st);
+// host_copy.cu: x_host to the workspace, y back
+int launch_host_copy(void* dst, const void* src, size_t bytes, bool to_device, cudaStream_t st);
 // gemm_simt.cu
 size_t simt_part_floats(const meteora_shape_t& s);   // scratch of the plain path: sizes Workspace::simt_part
 int launch_forward_simt(const void* x, const void* W0, const void* A, const void* B, const void* Wg, const meteora_shape_t& s,
