@@ -78,7 +78,7 @@ int launch_shrink(const void* x, const void* A, const int32_t* topk_idx, const i
 int launch_shrink_segments(const void* x, const void* A, const int32_t* offsets, const int32_t* perm,
                            const meteora_shape_t& s, float* u, cudaStream_t st);
 int launch_expand(const void* B, const int32_t* topk_idx, const float* topk_w, const float* u,
-                  const meteora_shape_t& s, float* delta, cudaStream_t st);
+                  const meteora_shape_t& s, float* delta, int32_t* status, cudaStream_t st);
 // host_copy.cu: x_host to the workspace, y back
 int launch_host_copy(void* dst, const void* src, size_t bytes, bool to_device, cudaStream_t st);
 // gemm_simt.cu
@@ -112,6 +112,10 @@ int launch_token_forward(const void* x, const void* A, const void* Wg, const met
 bool token_shrink_supported(const meteora_shape_t& s);
 int launch_token_shrink(const void* x, const void* A, const int32_t* topk_idx, const meteora_shape_t& s, float* u, int32_t* status,
                         bool beside, cudaStream_t st);
+// the LoRA term's expand as a tensor-core product (wgemm_tcgen05.cu + expand_tile.cuh)
+bool expand_tile_supported(const meteora_shape_t& s);
+int launch_expand_tile(const void* B, const int32_t* topk_idx, const float* topk_w, const float* u, const meteora_shape_t& s, float* delta,
+                       int32_t* status, cudaStream_t st);
 // dWg as a tensor-core product (wgemm_tcgen05.cu + gate_dwg.cuh)
 bool gate_dwg_tc_supported(const meteora_shape_t& s);
 int gate_dwg_shares(const meteora_shape_t& s);

@@ -310,8 +310,9 @@ int launch_shrink_segments(const void* x, const void* A, const int32_t* offsets,
 }
 
 int launch_expand(const void* B, const int32_t* topk_idx, const float* topk_w, const float* u,
-                  const meteora_shape_t& s, float* delta, cudaStream_t st) {
+                  const meteora_shape_t& s, float* delta, int32_t* status, cudaStream_t st) {
     if (s.T == 0) return METEORA_OK;
+    if (expand_tile_supported(s)) return launch_expand_tile(B, topk_idx, topk_w, u, s, delta, status, st);
     // the staged rows of all adapters for 128 outputs have to fit, next to 8 warps' values of 4 tokens
     const size_t slab_smem = (size_t)s.N * s.r * 256 + (size_t)8 * kSlabTokens * s.k * (s.r + 1) * 4;
     const int r8 = s.r / 8;

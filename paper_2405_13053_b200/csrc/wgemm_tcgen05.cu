@@ -757,6 +757,7 @@ k_wgemm(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__ CUtens
 #include "token_tile.cuh"
 #include "wgemm_persist.cuh"
 #include "gate_dwg.cuh"
+#include "expand_tile.cuh"
 
 namespace meteora {
 
@@ -2861,6 +2862,50 @@ int launch_gate_dwg_tc(const void* x, const int32_t* topk_idx, const float* topk
     return cuda_status(cudaLaunchKernelEx(&cfg, k_gate_dwg_sum, (const float*)part, shares, n, dWg));
 }
 
+// The LoRA term's expand on the tensor cores (expand_tile.cuh): B's rows and the tiles' token operands have to fit, and the batch
+// has to be worth the start.
+bool expand_tile_supported(const meteora_shape_t& s) {
+    return s.dtype == METEORA_BF16 && s.r % 8 == 0 && (long long)s.T * s.k * s.d_out >= kExtMinWork && (s.N * (s.r / 8) + 1) / 2 * 2 <= kExtMaxBlocks && !tuning().force_simt;
+}
+
+int launch_expand_tile(const void* B, const int32_t* topk_idx, const float* topk_w, const float* u, const meteora_shape_t& s, float* delta,
+                       int32_t* status, cudaStream_t st) {
+    static std::atomic<bool> attr_set[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return METEORA_ERR_CUDA;
+    if (dev < 0 || dev >= 64) return METEORA_ERR_UNSUPPORTED_SHAPE;
+    if (!attr_set[dev].load(std::memory_order_relaxed)) {
+        if (cudaFuncSetAttribute(k_expand_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kExtMaxSmem) != cudaSuccess) return METEORA_ERR_CUDA;
+        attr_set[dev].store(true, std::memory_order_relaxed);
+    }
+    ExpandTileParams p = {};
+    p.T = s.T;
+    p.d_out = s.d_out;
+    p.N = s.N;
+    p.r = s.r;
+    p.k = s.k;
+    p.nblk = (s.N * (s.r / 8) + 1) / 2 * 2;
+    p.B = (const __nv_bfloat16*)B;
+    p.topk_idx = topk_idx;
+    p.topk_w = topk_w;
+    p.u = u;
+    p.delta = delta;
+    p.status = status;
+    // one wave: as many shares of the tokens as there are SMs for
+    const int row_blocks = (s.d_out + kBM - 1) / kBM, blocks = (s.T + kExtTok - 1) / kExtTok;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(row_blocks, std::max(1, std::min(148 / row_blocks, blocks)));
+    cfg.blockDim = dim3(kExtThreads);
+    cfg.dynamicSmemBytes = 1024 + kExtHead + (size_t)p.nblk * (kExtABlock + kExtStages * kExtBBlock);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = tuning().pdl ? 1 : 0;
+    return cuda_status(cudaLaunchKernelEx(&cfg, k_expand_tile, p));
+}
+
 // Human-readable launch plan of meteora_linear_forward for this shape (for logs and benchmark records).
 int describe_plan(const meteora_shape_t& s, char* buf, size_t n) {
     if (!tc_path_supported(s)) return snprintf(buf, n, "path=simt");
@@ -2932,3 +2977,4 @@ extern "C" int meteora_trace_read(unsigned long long* host, size_t count) {
     return cudaMemcpyFromSymbol(host, meteora::g_fused_trace, count * sizeof(unsigned long long)) == cudaSuccess ? 0 : -5;
 }
 #endif
+
