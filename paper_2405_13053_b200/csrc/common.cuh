@@ -111,7 +111,7 @@ int launch_token_forward(const void* x, const void* A, const void* Wg, const met
                          bool beside, cudaStream_t st);
 bool token_shrink_supported(const meteora_shape_t& s);
 int launch_token_shrink(const void* x, const void* A, const int32_t* topk_idx, const meteora_shape_t& s, float* u, int32_t* status,
-                        bool beside, cudaStream_t st);
+                        bool beside, bool pair, bool dual, cudaStream_t st);
 // the LoRA term's expand as a tensor-core product (wgemm_tcgen05.cu + expand_tile.cuh)
 bool expand_tile_supported(const meteora_shape_t& s);
 int launch_expand_tile(const void* B, const int32_t* topk_idx, const float* topk_w, const float* u, const meteora_shape_t& s, float* delta,

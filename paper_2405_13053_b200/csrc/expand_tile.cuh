@@ -11,9 +11,9 @@
 // and by the loop of an operand: its product (850 cycles), then clearing and scattering (2000 - 2600 beside the others); hence four of
 // 32 tokens (two of 64, in the same memory: 4096 -> 14336 at 4096 tokens 186 us for the LoRA term, now 123).  k_expand_slab on
 // CUDA cores, bound by unpacking B and by shared-memory reads, has the shorter start: us for the LoRA term with that kernel / with
-// this one, by T k d_out: 0.8 M (200 tokens, 4096, k 1) 24.1 / 27.5; 1.6 M (200, 4096, k 2) 19.8 / 22.5; 2.0 M (2000, 1024, k 1)
-// 29.7 / 29.7; 2.5 M (300, 4096, k 2) 24.3 / 23.6; 14.7 M (512, 14336, k 2) 41.2 / 34.3; 16.8 M (2048, 4096, k 2) 48.5 / 42.4; 60 M
-// (3000, 5000, k 4) 89.2 / 65.0; 117 M (4096, 14336, k 2) 173 / 123: this one from 2 M on (kExtMinWork).
+// this one, by T k d_out: 0.8 M (200 tokens, 4096, k 1) 24.1 / 27.5; 1.6 M (200, 4096, k 2) 19.8 / 22.5; 2.5 M (300, 4096, k 2)
+// 24.3 / 24.6; 4.2 M (512, 4096, k 2) 26.5 / 25.2; 14.7 M (512, 14336, k 2) 41.4 / 34.7; 16.8 M (2048, 4096, k 2) 48.6 / 43.0; 60 M
+// (3000, 5000, k 4) 89.5 / 64.7; 117 M (4096, 14336, k 2) 174 / 123: this one from 3 M on (kExtMinWork).
 // The product multiplies the zeros of adapters that a token did not pick, and 0 times an infinity or a NaN is NaN: an element
 // that is NaN is computed again from the picks alone.
 #pragma once
@@ -24,7 +24,7 @@ constexpr int kExtStages = 4;                       // token operands and accumu
 constexpr int kExtTok = 32;                         // tokens per tile
 constexpr int kExtCols = 3 * kExtTok;               // accumulator columns: three parts
 constexpr int kExtABlock = kBM * 16, kExtBBlock = kExtCols * 16;   // bytes per 8 columns of K
-constexpr long long kExtMinWork = 1 << 21;          // T k d_out
+constexpr long long kExtMinWork = 3 << 20;          // T k d_out
 constexpr int kExtMaxBlocks = 28;                   // what fits beside B's rows
 constexpr int kExtBuilders = 64;                    // threads per token operand
 constexpr int kExtEpilogue = 128;                   // threads per tile; two such groups take turns

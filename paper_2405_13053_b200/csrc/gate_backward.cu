@@ -243,8 +243,8 @@ int launch_gate_backward(const void* x, const void* A, const void* B, const void
         // u and z per slot from token tiles, side by side (the second launch does not read the first one's results), then
         // the Jacobian with dWg as a tensor-core product: 3 - 4 launches, each resident under the one ahead
         if (B && (rc = launch_transpose_b(B, s, Bt, st)) != METEORA_OK) return rc;
-        if ((rc = launch_token_shrink(x, A, topk_idx, s, u, status, false, st)) != METEORA_OK) return rc;
-        if ((rc = launch_token_shrink(dy, Bt, topk_idx, sb, z, status, true, st)) != METEORA_OK) return rc;
+        if ((rc = launch_token_shrink(x, A, topk_idx, s, u, status, false, true, false, st)) != METEORA_OK) return rc;
+        if ((rc = launch_token_shrink(dy, Bt, topk_idx, sb, z, status, true, true, false, st)) != METEORA_OK) return rc;
         return launch_gate_dwg_tc(x, topk_idx, topk_w, u, z, s, status, part, dlogit_out, dWg, st);
     }
     // the header's first words take the error flags of the tensor-core kernels

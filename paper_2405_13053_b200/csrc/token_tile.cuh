@@ -132,8 +132,10 @@ __device__ __forceinline__ void token_round(const TokenTileParams& p, uint32_t p
     }
 }
 
-// S: CTAs of the cluster that shares a tile.
-template <int S>
+// S: CTAs of the cluster that shares a tile.  DUAL (one round of columns): the MMAs go to two accumulators in turn, added in fp32.
+// The tensor cores cut what they add to an accumulator off instead of rounding it, so an error grows with the steps into one: LoRA
+// term over 4096 products 7.0e-7 with one, 4.3e-7 with two.  (A kernel of its own: as a branch it took 0.3 us where it was not used)
+template <int S, bool DUAL>
 __global__ void __launch_bounds__(kThreads)
 k_token_tile(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmG, const __grid_constant__ CUtensorMap tmA,
              const TokenTileParams p) {
@@ -211,7 +213,8 @@ k_token_tile(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CU
                         const uint32_t idesc = instr_desc_bf16(p.cols[tile]);
 #pragma unroll
                         for (int kk = 0; kk < kBK / kUmmaK; ++kk)
-                            umma_bf16(tmem_base + tile * kTokCols, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc, (i | kk) != 0);
+                            umma_bf16(tmem_base + (tile + (DUAL ? kk & 1 : 0)) * kTokCols, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc,
+                                      DUAL ? i > 0 || kk > 1 : (i | kk) != 0);
                     }
                     umma_commit(bar_base + (p.stages + s) * 8);
                 }
@@ -247,7 +250,19 @@ k_token_tile(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CU
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
                     if (c0 + 16 * q < c_end) tmem_ld16_issue(src + (uint32_t)(c0 + 16 * q), v[q]);
-                tmem_ld_wait();
+                if (DUAL) {                                          // (both accumulators behind one wait)
+                    uint32_t v2[4][16];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (c0 + 16 * q < c_end) tmem_ld16_issue(src + (uint32_t)(kTokCols + c0 + 16 * q), v2[q]);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) v[q][i] = __float_as_uint(__uint_as_float(v[q][i]) + __uint_as_float(v2[q][i]));
+                } else {
+                    tmem_ld_wait();
+                }
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
                     if (c0 + 16 * q < c_end) {

@@ -32,13 +32,13 @@ def _delta(x, A, B, idx, w):
     return mb.meteora_lora_delta(x, A, B, idx, w, offsets, perm)
 
 
-# either side of the smallest work it takes (2^21 picks x outputs); one token beyond a tile of 32, a tile and a row block that are
+# either side of the smallest work it takes (3 * 2^20 picks x outputs); one token beyond a tile of 32, a tile and a row block that are
 # nearly empty; several rounds of the four operands; an odd number of columns of 8, ranks of several; most picks (several values
 # per thread); the most columns that fit, and two more than that
 @pytest.mark.parametrize("T,d_in,d_out,N,r,k", [
-    (1, 64, 262144, 28, 8, 8), (33, 64, 32001, 28, 8, 2), (64, 64, 16383, 28, 8, 2), (64, 64, 16384, 28, 8, 2), (97, 72, 8193, 3, 8, 3),
-    (410, 64, 1030, 7, 24, 5), (1573, 64, 4096, 28, 8, 2), (4099, 64, 520, 28, 8, 1), (300, 64, 20000, 28, 8, 8), (1000, 128, 264, 14, 16, 8),
-    (3600, 64, 200, 3, 64, 3), (6000, 64, 200, 30, 8, 2),
+    (1, 64, 400000, 28, 8, 8), (50, 64, 32001, 28, 8, 2), (64, 64, 24575, 28, 8, 2), (64, 64, 24576, 28, 8, 2), (130, 72, 8193, 3, 8, 3),
+    (620, 64, 1030, 7, 24, 5), (1573, 64, 4096, 28, 8, 2), (6100, 64, 520, 28, 8, 1), (300, 64, 20000, 28, 8, 8), (1500, 128, 264, 14, 16, 8),
+    (5300, 64, 200, 3, 64, 3), (6000, 64, 200, 30, 8, 2),
 ])
 @pytest.mark.parametrize("twice", [False, True])
 def test_expand_tile(T, d_in, d_out, N, r, k, twice):
@@ -53,7 +53,7 @@ def test_expand_tile(T, d_in, d_out, N, r, k, twice):
 
 
 def test_only_the_picks_count():
-    x, A, B, idx, w = _problem(4000, 64, 300, 28, 8, 2)
+    x, A, B, idx, w = _problem(5300, 64, 300, 28, 8, 2)
     ref = _delta(x, A, B, idx, w)
     B2, x2 = B.clone(), x.clone()
     B2[5, 17, 3], B2[9, 140, 0], B2[11, 299, 7] = float("inf"), float("nan"), float("-inf")
@@ -66,5 +66,5 @@ def test_only_the_picks_count():
     assert torch.equal(~torch.isfinite(got), odd)
     # what was NaN in the product is computed again in another order: fp32 sums of 16 terms
     torch.testing.assert_close(got[~odd], ref[~odd], rtol=0, atol=float(2.0 ** -20 * ref.abs().max()))
-    infinite = (idx == 5).any(dim=1) & (torch.arange(4000, device="cuda") != 70)
+    infinite = (idx == 5).any(dim=1) & (torch.arange(5300, device="cuda") != 70)
     assert torch.isinf(got[infinite, 17]).all()
