@@ -422,8 +422,9 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
     const int pair0 = (int)blockIdx.x >> 1, npairs = (int)gridDim.x >> 1;
     // where the tile before gets its expand: late, so that the selection is ready for the first tiles, and early enough for
     // that tile's epilogue to end under the rest (12 k-steps: 4 us).  With the routing ahead a tile gets its own there: at the end
-    // its loads and MMAs (3 - 3.5 us for three parts) had nothing to hide under
-    const int iters = (p.ksteps + kc - 1) / kc, mid = max(iters / 2, iters - 12 / kc);
+    // its loads and MMAs (3 - 3.5 us for three parts) had nothing to hide under; but not ahead of its main product's first step, which
+    // clears the accumulator: behind the loop (mid == iters) where that has one iteration
+    const int iters = (p.ksteps + kc - 1) / kc, mid = max(max(iters / 2, iters - 12 / kc), own ? 1 : 0);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.stages; ++s) {
@@ -532,9 +533,9 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                 } else {
                     const CUtensorMap* mW = &maps.W0[t.mod];
                     const int w_row = row_tile * tr;
-                    for (int i = 0; i < iters; ++i) {
+                    for (int i = 0; i <= iters; ++i) {
                         if (i == mid && (pending || own) && !(ok = expand(own ? t : before))) break;
-                        if (!(ok = slot(bar, full, dst))) break;
+                        if (i == iters || !(ok = slot(bar, full, dst))) break;
                         if (elect_one()) {
                             if (leader) mbar_expect_tx(bar, tx);
                             if (kc == 1) {
@@ -622,9 +623,9 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                     tc_fence_after();
                 }
                 uint32_t wa;
-                for (int i = 0; i < iters; ++i) {
+                for (int i = 0; i <= iters; ++i) {
                     if (i == mid && (pending || own) && !(ok = expand(own ? b : b ^ 1))) break;
-                    if (!(ok = next(wa))) break;
+                    if (i == iters || !(ok = next(wa))) break;
                     const uint64_t da = smem_desc_sw128(wa), db = smem_desc_sw128(wa + kc * kWTileBytes);
                     if (elect_one()) {
 #pragma unroll

@@ -190,3 +190,37 @@ def test_few_tiles_are_narrow(T, d_in, d_out, N, r, k, width):
     ref = oracle.linear_forward_routed(w["x"][sel], w["W0"], w["A"], w["B"], w["Wg"], idx[sel])
     assert rel_l2(y[sel], ref) <= 5e-3
     assert bf16_bound_ok(y[sel], ref) <= 0.0
+
+
+# Contraction axes of one iteration of the main loop (64 elements a step, two steps in the narrow walk), of a part of one, and of two
+# and three: the expand may not come ahead of the step that clears the accumulator.  Narrow tiles of 64 and 128 tokens, 256-token tiles
+# behind the routing kernels (us in one part and in three) and with the routing inside (knob 2).  W0 = 0 leaves the LoRA term alone, whose
+# absence no tolerance can hide.
+@pytest.mark.parametrize("T,d_in,d_out,N,r,k,persist", [
+    (257, 64, 200, 28, 8, 2, 1), (300, 64, 256, 28, 8, 2, 1), (300, 128, 256, 28, 16, 2, 1), (300, 192, 256, 28, 8, 2, 1), (512, 128, 1024, 28, 8, 2, 1),
+    (512, 64, 2048, 12, 64, 2, 1), (2048, 64, 1024, 28, 8, 2, 1), (600, 64, 256, 90, 8, 2, 1), (2048, 128, 520, 28, 64, 4, 1),
+    (4096, 8, 1024, 28, 8, 2, 1), (4096, 56, 1024, 28, 16, 2, 1), (4096, 64, 1024, 28, 8, 2, 3), (4096, 72, 1024, 28, 8, 2, 1), (2048, 56, 768, 12, 64, 2, 1),
+    (4096, 136, 1024, 28, 8, 2, 3), (512, 8, 2560, 100, 8, 2, 1), (4096, 64, 2048, 28, 8, 2, 2), (4096, 8, 2048, 28, 16, 2, 2), (4096, 72, 4096, 28, 8, 2, 2),
+])
+def test_short_contraction_axes_keep_the_lora_term(T, d_in, d_out, N, r, k, persist):
+    w = workloads.make_workload("short_axis", T=T, d_in=d_in, d_out=d_out, N=N, r=r, k=k, dtype="bf16", seed=490 + T + d_in, b_std=0.3)
+    x, W0, A, B, Wg = to_dev(w, "x", "W0", "A", "B", "Wg")
+    mb.meteora_set_tuning("persist", persist)
+    try:
+        shape = mb.make_shape(T, d_in, d_out, N, r, k, torch.bfloat16)
+        plan = mb.meteora_describe_plan(shape)
+        assert "persistent_pairs=" in plan and ("path=persistent_prefill" in plan) == (persist == 2), plan
+        ws = mb.alloc_workspace(shape)
+        y, idx, _ = mb.meteora_linear_forward(x, W0, A, B, Wg, k, workspace=ws, return_routing=True)
+        lora = mb.meteora_linear_forward(x, torch.zeros_like(W0), A, B, Wg, k, workspace=ws)
+        assert mb.meteora_workspace_status(ws) == 0
+    finally:
+        mb.meteora_set_tuning("persist", 1)
+    y, lora, idx = y.float().cpu().numpy(), lora.float().cpu().numpy(), idx.cpu().numpy()
+    o_idx, _, o_logits = oracle.gate_topk(w["x"], w["Wg"], k)
+    check_selection(idx, o_idx, o_logits, k)
+    sel = np.unique(np.concatenate([np.arange(0, T, 61), np.arange(255, T, 256), [T - 1]]))
+    ref = oracle.linear_forward_routed(w["x"][sel], w["W0"], w["A"], w["B"], w["Wg"], idx[sel])
+    assert rel_l2(y[sel], ref) <= 5e-3
+    ref = oracle.linear_forward_routed(w["x"][sel], 0 * w["W0"], w["A"], w["B"], w["Wg"], idx[sel])
+    assert rel_l2(lora[sel], ref) <= 5e-3                # (us and y rounded to bf16 once each: 2 x 1.7e-3)
