@@ -66,6 +66,7 @@ __global__ void __launch_bounds__(kExtThreads, 1) k_expand_tile(const ExpandTile
     // per stage: full (the builders' threads), done (the MMAs' commit), free (the epilogue's threads)
     const uint32_t bar_full = head, bar_done = bar_full + kExtStages * 8, bar_free = bar_done + kExtStages * 8;
     uint32_t* const tmem_slot = reinterpret_cast<uint32_t*>(head_ptr + 120);
+    volatile int* const s_late = reinterpret_cast<volatile int*>(head_ptr + 124);   // a builder's wait ran out: no tile from there on is a result
     uint8_t* const s_pick = head_ptr + 128;                          // [stage][token][pick]: the adapter that holds the pick's values; 0xFF: none
     const uint32_t rows_at = head + kExtHead, toks_at = rows_at + (uint32_t)p.nblk * kExtABlock;
     const uint32_t tok_bytes = (uint32_t)p.nblk * kExtBBlock;
@@ -91,6 +92,7 @@ __global__ void __launch_bounds__(kExtThreads, 1) k_expand_tile(const ExpandTile
     for (int v = p.N * r8 * kBM + threadIdx.x; v < p.nblk * kBM; v += kExtThreads) reinterpret_cast<uint4*>(rows_ptr)[v] = make_uint4(0u, 0u, 0u, 0u);
     for (int v = threadIdx.x; v < min(nb, kExtStages) * (int)tok_bytes / 16; v += kExtThreads) reinterpret_cast<uint4*>(toks_ptr)[v] = make_uint4(0u, 0u, 0u, 0u);
     if (threadIdx.x == 0) {
+        *s_late = 0;
         for (int s = 0; s < kExtStages; ++s) {
             mbar_init(bar_full + s * 8, kExtBuilders);
             mbar_init(bar_done + s * 8, 1);
@@ -216,8 +218,9 @@ __global__ void __launch_bounds__(kExtThreads, 1) k_expand_tile(const ExpandTile
         for (int i = group; i < nb; i += kExtStages) {
             const int s = group, round = i / kExtStages;
             if (round > 0) {
-                ok = mbar_wait(bar_done + s * 8, (round & 1) ^ 1);
-                if (!ok) break;
+                // (each thread by itself; one whose wait ran out goes on all the same: the others count on it at the barriers below)
+                ok = ok && mbar_wait(bar_done + s * 8, (round & 1) ^ 1);
+                if (!ok) *s_late = 1;
                 clear(s, mine[0]);
                 clear(s, mine[1]);
                 for (int it = tid + 2 * kExtBuilders; it < items; it += kExtBuilders) clear(s, place(it));
@@ -253,7 +256,7 @@ __global__ void __launch_bounds__(kExtThreads, 1) k_expand_tile(const ExpandTile
         for (int i = (warp - kExtFirstEpi) / 4; i < nb; i += 2) {
             const int s = i % kExtStages, t0 = (b0 + i) * kExtTok;
             ok = ok && mbar_wait(bar_done + s * 8, (i / kExtStages) & 1);
-            ok = __all_sync(0xFFFFFFFFu, ok);
+            ok = __all_sync(0xFFFFFFFFu, ok && *s_late == 0);         // (written ahead of the arrivals that this tile's product waited for)
             tc_fence_after();
             const uint32_t src = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(s * 128);
             uint32_t v[3][kExtTok];
@@ -292,7 +295,7 @@ __global__ void __launch_bounds__(kExtThreads, 1) k_expand_tile(const ExpandTile
         }
         where = 3;
     }
-    if (!ok && lane == 0 && p.status) {
+    if (__any_sync(0xFFFFFFFFu, !ok) && lane == 0 && p.status) {
         atomicExch(p.status, 1);
         atomicExch(p.status + where, 5000 + where);
     }
