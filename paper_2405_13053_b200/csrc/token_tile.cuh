@@ -33,6 +33,7 @@ struct TokenTileParams {
     int a_group;               // adapters per grid row (SHRINK: the adapters may be dealt to several clusters per tile)
     int stages, stage_bytes, tmem_cols, pitch;   // pitch: floats per token of the shared-memory copy of a round
     int rounds, cols[2];       // accumulators of up to 256 columns
+    int acc2;                  // DUAL: first column of the second one
     float inv_tau;
     int32_t* topk_idx;         // out (GATE, FORWARD) or in
     float* topk_w;             // (not read by SHRINK)
@@ -213,7 +214,7 @@ k_token_tile(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CU
                         const uint32_t idesc = instr_desc_bf16(p.cols[tile]);
 #pragma unroll
                         for (int kk = 0; kk < kBK / kUmmaK; ++kk)
-                            umma_bf16(tmem_base + (tile + (DUAL ? kk & 1 : 0)) * kTokCols, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc,
+                            umma_bf16(tmem_base + (DUAL ? (kk & 1) * p.acc2 : tile * kTokCols), da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc,
                                       DUAL ? i > 0 || kk > 1 : (i | kk) != 0);
                     }
                     umma_commit(bar_base + (p.stages + s) * 8);
@@ -254,7 +255,7 @@ k_token_tile(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CU
                     uint32_t v2[4][16];
 #pragma unroll
                     for (int q = 0; q < 4; ++q)
-                        if (c0 + 16 * q < c_end) tmem_ld16_issue(src + (uint32_t)(kTokCols + c0 + 16 * q), v2[q]);
+                        if (c0 + 16 * q < c_end) tmem_ld16_issue(src + (uint32_t)(p.acc2 + c0 + 16 * q), v2[q]);
                     tmem_ld_wait();
 #pragma unroll
                     for (int q = 0; q < 4; ++q)

@@ -868,6 +868,15 @@ int tc_stacked_pitch(const meteora_shape_t& s, int* col_logits) {
     return a_tiles * kBM + (int)align_up((size_t)s.N, 32);
 }
 
+// Shared memory that a launch asks for at least with `cols` TMEM columns per CTA.  tcgen05.alloc waits without a limit for columns that
+// another CTA of the SM holds, and that CTA may wait for one of the first one's cluster or launch elsewhere.  A CTA takes 1 KB of the
+// SM's 228 beside what it asks for; with 13.5 KB for every 32 columns those that an SM takes in, of whatever launches and streams,
+// need no more than its 512 columns together (17 x 13.5 > 228).
+constexpr size_t kTmemShare = 13 * 1024 + 512;
+static_assert((512 / 32 + 1) * kTmemShare > 228 * 1024, "CTAs with 17 x 32 columns may not fit an SM");
+static_assert(512 / 32 * kTmemShare <= 227 * 1024, "a CTA with all columns must fit");
+static constexpr size_t smem_with_tmem(size_t smem, int cols) { return std::max(smem, (size_t)cols / 32 * kTmemShare - 1024); }
+
 struct Plan;
 static Plan make_plan(int row_tiles, int T, int K, bool lora, int N, int r, int k, bool fused_epi = false,
                       int bn_force = 0, bool no_mma_expand = false, int K2 = 0, int splits_force = 0, int zcap_force = 0);
@@ -1035,7 +1044,7 @@ static Plan make_plan(int row_tiles, int T, int K, bool lora, int N, int r, int 
     while (cols < bn) cols *= 2;
     pl.tmem_cols = cols;
     pl.epi_off = (int)align_up((size_t)(2 * std::max(stages, 16) + 3) * 8 + 16, 128);
-    pl.smem = 1024 + (size_t)stages * stage_bytes + pl.epi_off + epi_bytes;
+    pl.smem = smem_with_tmem(1024 + (size_t)stages * stage_bytes + pl.epi_off + epi_bytes, cols);
     // Large ranks with the expand on CUDA cores stage k * r floats per token: if that does not leave room for two
     // ring stages, take fewer tokens per tile.
     if (pl.smem > 227 * 1024 && bn_force == 0 && tn.tile_tokens == 0) {
@@ -1113,7 +1122,7 @@ static StackedPairPlan make_stacked_pair_plan(const meteora_shape_t& s) {
     const int fill = std::max(1, sm_count() / (2 * pairs));
     sp.zsplits = std::min(std::min(zcap, std::min(fill, stacked_zsplits_bound(s.T))), std::max(1, ksteps / 4));
     sp.stages = std::min(6, std::max(2, (ksteps + sp.zsplits - 1) / sp.zsplits));
-    sp.smem = 1024 + (size_t)sp.stages * (kWTileBytes + kPairHalf * 128) + 256;
+    sp.smem = smem_with_tmem(1024 + (size_t)sp.stages * (kWTileBytes + kPairHalf * 128) + 256, kPairTokens);
     sp.ok = true;
     return sp;
 }
@@ -1291,7 +1300,7 @@ static PairPlan make_pair_plan(const meteora_shape_t& s) {
         if (smem <= 226 * 1024 && stages * stage >= std::max(us, ystage)) {
             pp.stages = tuning().stages > 1 && tuning().stages < stages ? tuning().stages : stages;
             pp.epi_off = (int)align_up((size_t)(2 * pp.stages + 3) * 8 + 16, 128);
-            pp.smem = 1024 + pp.stages * stage + pp.epi_off + slab;
+            pp.smem = smem_with_tmem(1024 + pp.stages * stage + pp.epi_off + slab, kPairTokens);
             pp.ok = pp.stages * stage >= std::max(us, ystage);
             return pp;
         }
@@ -1573,7 +1582,7 @@ static PersistPlan make_persist_plan(const meteora_shape_t& s, const int* d_outs
     pp.stage_bytes = kc * (kWTileBytes + pp.BN / 2 * 128);
     const size_t fixed = 1024 + (size_t)kPersistStageBufs * kPersistStoreBytes + 512;
     pp.stages = (int)std::min<size_t>((227 * 1024 - fixed) / pp.stage_bytes, 12);
-    pp.smem = fixed + (size_t)pp.stages * pp.stage_bytes;
+    pp.smem = smem_with_tmem(fixed + (size_t)pp.stages * pp.stage_bytes, 512);
     pp.ok = pp.stages >= 2;
     return pp;
 }
@@ -1914,7 +1923,7 @@ static FusedPlan make_fused_plan(const meteora_shape_t& s, const int* d_outs, in
     int cols = 32;
     while (cols < std::max(2, segs) * pl.BN) cols *= 2;           // one accumulator per row tile a unit range can touch
     pl.tmem_cols = cols;
-    pl.smem = 1024 + ring_bytes + pl.epi_off + epi_bytes;
+    pl.smem = smem_with_tmem(1024 + ring_bytes + pl.epi_off + epi_bytes, cols);
     const int nks_aux = (ksteps + fp.aux_slices - 1) / fp.aux_slices;
     fp.aux_stages = (int)std::min<size_t>(std::min<size_t>(ring_bytes / chunk, 16), (size_t)std::max(nks_aux, 1));
     fp.why = 4;
@@ -2229,7 +2238,7 @@ static StreamPlan make_stream_plan_with(const meteora_shape_t& s, const int* d_o
         sp.aux_stages = (int)std::min<size_t>(std::min<size_t>(ring_bytes / aux_stage_bytes, kStreamBarSlots),
                                               (size_t)std::max(nks_aux, 1));
         sp.ring_bytes = (int)ring_bytes;
-        sp.smem = fixed + ring_bytes;
+        sp.smem = smem_with_tmem(fixed + ring_bytes, cols);
         sp.ctas_per_sm = per_sm;
         break;
     }
@@ -2498,7 +2507,7 @@ static ClusterPlan make_cluster_plan(const meteora_shape_t& s) {
     if (stages < 2) return cp;
     cp.stages = stages;
     cp.ring_bytes = (int)(stages * stage_bytes);
-    cp.smem = 1024 + cp.ring_bytes + tail_bytes;
+    cp.smem = smem_with_tmem(1024 + cp.ring_bytes + tail_bytes, cp.tmem_cols);
     cp.why = 0;
     cp.ok = true;
     return cp;
@@ -2604,6 +2613,7 @@ struct TokenPlan {
     bool ok;
     int S, stages, stage_bytes, tmem_cols, pitch, rounds, cols[2], gate_box, a_box, a_copies;
     bool dual;
+    int acc2;              // its second accumulator's first column
     int groups, a_group;   // clusters per tile, each with its own adapters (SHRINK), and adapters per cluster
     size_t smem;
     long long cost;
@@ -2701,7 +2711,7 @@ static TokenPlan make_token_plan_with(const meteora_shape_t& s, int mode, int gr
     tp.stages = (int)std::min<size_t>((kTokenSmem - 2048) / tp.stage_bytes, (size_t)std::min(16, std::max(iters, 2)));
     // the accumulators' copy and, behind it, the owned tokens' summed logits
     const size_t own = (size_t)((kTokTile + tp.S - 1) / tp.S) * 4 * (s.N | 1);
-    tp.smem = 2048 + std::max((size_t)tp.stages * tp.stage_bytes, (size_t)kTokTile * tp.pitch * 4 + own);
+    tp.smem = smem_with_tmem(2048 + std::max((size_t)tp.stages * tp.stage_bytes, (size_t)kTokTile * tp.pitch * 4 + own), tp.tmem_cols);
     tp.ok = tp.stages >= 2 && tp.smem <= kTokenSmem;
     return tp;
 }
@@ -2767,6 +2777,7 @@ static int launch_token_tile(const TokenPlan& tp, int mode, const meteora_shape_
     p.stages = tp.stages;
     p.stage_bytes = tp.stage_bytes;
     p.tmem_cols = tp.tmem_cols;
+    p.acc2 = tp.acc2;
     p.pitch = tp.pitch;
     p.rounds = tp.rounds;
     p.cols[0] = tp.cols[0];
@@ -2823,7 +2834,9 @@ int launch_token_shrink(const void* x, const void* A, const int32_t* topk_idx, c
     TokenPlan tp = pair ? make_shrink_pair_plan(s) : make_token_plan(s, TOKEN_SHRINK);
     if (dual && tp.rounds == 1) {
         tp.dual = true;
-        tp.tmem_cols = 2 * kTokCols;
+        tp.acc2 = (tp.cols[0] + 31) / 32 * 32;
+        while (tp.tmem_cols < tp.acc2 + tp.cols[0]) tp.tmem_cols *= 2;
+        tp.smem = smem_with_tmem(tp.smem, tp.tmem_cols);
     }
     return launch_token_tile(tp, TOKEN_SHRINK, s, x, nullptr, A, p, st);
 }
@@ -2845,7 +2858,7 @@ int launch_gate_dwg_tc(const void* x, const int32_t* topk_idx, const float* topk
     CUtensorMap mX;
     int rc;
     if ((rc = get_tensor_map(x, s.d_in, s.T, kDwgTok, 0, &mX)) != METEORA_OK) return rc;
-    constexpr size_t smem = 1024 + (size_t)kDwgStages * (kDwgXBytes + kDwgLBytes) + 256 + 2 * kDwgSlots * 4;
+    constexpr size_t smem = smem_with_tmem(1024 + (size_t)kDwgStages * (kDwgXBytes + kDwgLBytes) + 256 + 2 * kDwgSlots * 4, kDwgCols);
     static std::atomic<bool> attr_set[64];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return METEORA_ERR_CUDA;
@@ -2922,7 +2935,7 @@ int launch_expand_tile(const void* B, const int32_t* topk_idx, const float* topk
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(row_blocks, std::max(1, std::min(148 / row_blocks, blocks)));
     cfg.blockDim = dim3(kExtThreads);
-    cfg.dynamicSmemBytes = 1024 + kExtHead + (size_t)p.nblk * (kExtABlock + kExtStages * kExtBBlock);
+    cfg.dynamicSmemBytes = smem_with_tmem(1024 + kExtHead + (size_t)p.nblk * (kExtABlock + kExtStages * kExtBBlock), 512);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
