@@ -45,6 +45,7 @@ constexpr int kPersistStageBufs = 2;                              // epilogue gr
 constexpr int kPersistChunk = 32;                                 // tokens an epilogue group takes at a time
 constexpr int kPersistBufBytes = kPersistChunk * kBM * 2;         // as rows of bf16
 constexpr int kPersistStoreBytes = 2 * kPersistBufBytes;          // a group's staging buffers
+constexpr int kPersistAcc2 = 128;                                 // kWalkNarrow: column of a tile's second accumulator
 constexpr int kPersistMaxPairs = 74;
 constexpr int kPersistMaxN = 64;                                  // adapters the selection here takes
 constexpr int kPersistMaxStacked = 4;                             // pairs of stacked tiles per token tile
@@ -401,7 +402,8 @@ __device__ __forceinline__ void persist_select(const PersistParams& p, float* s_
 enum { kWalkStacked = 0, kWalkBase = 1, kWalkNarrow = 2 };
 
 template <int kWalk>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads)
+// (one CTA per SM: for more the compiler keeps to 48 or 64 registers, and with the second accumulator the issuing loops spill: + 3 us)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant__ PersistParams p) {
     constexpr bool own = kWalk != kWalkStacked;                   // a tile's expand is in its own main loop
     constexpr int kc = kWalk == kWalkNarrow ? 2 : 1;              // k-steps per stage
@@ -425,6 +427,16 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
     // its loads and MMAs (3 - 3.5 us for three parts) had nothing to hide under; but not ahead of its main product's first step, which
     // clears the accumulator: behind the loop (mid == iters) where that has one iteration
     const int iters = (p.ksteps + kc - 1) / kc, mid = max(max(iters / 2, iters - 12 / kc), own ? 1 : 0);
+
+    // kWalkNarrow sums the two k-steps of a stage, and every other MMA of the expand, into an accumulator of their own each, 128 columns
+    // apart: the tensor cores cut off what they add instead of rounding it, so the error grows with the MMAs into one.  An expand in three
+    // parts of a prefill batch, which other kernels did in fp32, has the other two accumulators of the pair, whose only tile this is, to
+    // itself.  Error of the fp32 sums against 64 bits (rms over the size of y, which a last few columns make cancel), with the split tiles
+    // that short prompts took before / one accumulator / now: 4096 -> 1024 at 512 tokens 2.06e-6 / 4.42e-6 / 2.10e-6, with an expand of rank 16
+    // 2.05e-6 / 4.57e-6 / 2.09e-6; 14336 -> 1024 7.85e-6 / 16.2e-6 / 7.84e-6; 1024 -> 1024 4.46e-7 / 9.60e-7 / 4.44e-7.  4096 -> 1024 at 512 tokens
+    // takes 14.5 / 14.4 us with one accumulator / two, rank 32 with the expand apart 29.5 / 29.9.
+    const bool apart = kc == 2 && parts > 1 && p.tok_tiles > 1 && p.tiles <= npairs;
+    const uint32_t expand_odd = kc == 2 && p.nblk > 2 ? kPersistAcc2 : 0;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.stages; ++s) {
@@ -601,9 +613,9 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                         for (int h = 0; h < 3; ++h)
                             if (h < parts)
                                 for (int kk = 0; kk < nm; ++kk)
-                                    umma_bf16_pair(tmem_base + b * kPairTokens,
+                                    umma_bf16_pair(tmem_base + (apart ? kPairTokens : b * kPairTokens) + (kk & 1) * expand_odd,
                                                    b_desc + ((wa + ((kk >> b_side) * (tr * 32 << b_side)) + (kk & ((1 << b_side) - 1)) * 32) >> 4),
-                                                   db[h] + (uint64_t)(kk * 2), idesc, 1);
+                                                   db[h] + (uint64_t)(kk * 2), idesc, !apart || (i | h | (expand_odd ? kk >> 1 : kk)) != 0);
                         umma_commit_pair(bar_base + (p.stages + first) * 8);
                         if (parts > 1 && kc == 1) umma_commit_pair(bar_base + (p.stages + s) * 8);
                     }
@@ -635,7 +647,7 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                             const uint64_t da2 = da + (uint64_t)(tr * 8), db2 = db + (uint64_t)(p.BN * 4);   // (descriptors count 16 bytes)
 #pragma unroll
                             for (int kk = 0; kk < kBK / kUmmaK; ++kk)
-                                umma_bf16_pair(acc, da2 + (uint64_t)(kk * 2), db2 + (uint64_t)(kk * 2), idesc, 1);
+                                umma_bf16_pair(acc + kPersistAcc2, da2 + (uint64_t)(kk * 2), db2 + (uint64_t)(kk * 2), idesc, (i | kk) != 0);
                         }
                         umma_commit_pair(bar_base + (p.stages + s) * 8);
                     }
@@ -798,9 +810,35 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                 uint32_t v[2][16];                                // 32 tokens of 16 rows each
                 tmem_ld_frag_issue(taddr + (uint32_t)(c * kPersistChunk), v[0]);
                 tmem_ld_frag_issue(taddr + (16u << 16) + (uint32_t)(c * kPersistChunk), v[1]);
+                uint32_t v2[2][16];                               // the second accumulator's
+                if (kc == 2) {
+                    tmem_ld_frag_issue(taddr + (uint32_t)(kPersistAcc2 + c * kPersistChunk), v2[0]);
+                    tmem_ld_frag_issue(taddr + (16u << 16) + (uint32_t)(kPersistAcc2 + c * kPersistChunk), v2[1]);
+                }
                 // this buffer's last store has been read out (of the one in between nobody knows)
                 if (elected) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
                 tmem_ld_wait();
+                if (kc == 2) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) v[h][i] = __float_as_uint(__uint_as_float(v[h][i]) + __uint_as_float(v2[h][i]));
+                    if (apart) {
+                        uint32_t e[2][2][16];
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) {
+                            tmem_ld_frag_issue(taddr + (uint32_t)(kPairTokens + q * (int)expand_odd + c * kPersistChunk), e[q][0]);
+                            tmem_ld_frag_issue(taddr + (16u << 16) + (uint32_t)(kPairTokens + q * (int)expand_odd + c * kPersistChunk), e[q][1]);
+                        }
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int h = 0; h < 2; ++h)
+#pragma unroll
+                            for (int i = 0; i < 16; ++i)
+                                v[h][i] = __float_as_uint(__uint_as_float(v[h][i]) +
+                                                          (__uint_as_float(e[0][h][i]) + (expand_odd ? __uint_as_float(e[1][h][i]) : 0.f)));
+                    }
+                }
                 const bool last = c + 2 >= chunks;
                 if (last) tc_fence_before();                      // this group's last read of the accumulator
                 asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");

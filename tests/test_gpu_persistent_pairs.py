@@ -224,3 +224,27 @@ def test_short_contraction_axes_keep_the_lora_term(T, d_in, d_out, N, r, k, pers
     assert rel_l2(y[sel], ref) <= 5e-3
     ref = oracle.linear_forward_routed(w["x"][sel], 0 * w["W0"], w["A"], w["B"], w["Wg"], idx[sel])
     assert rel_l2(lora[sel], ref) <= 5e-3                # (us and y rounded to bf16 once each: 2 x 1.7e-3)
+
+
+# The fp32 sums behind a bf16 y, made visible: equal tokens whose last four columns cancel the sum of the others (each weight the bf16 part
+# that the ones before leave), so that y is the error.  The tensor cores cut off what they add: 2.1e-6 of the sum's size (rms) over 4096
+# products in two accumulators, 4.4e-6 in one, with the expand of rank 16 in three parts as without one; in two over 14336 7.8e-6.
+@pytest.mark.parametrize("T,d_in,d_out,r,b_std,limit", [(512, 4096, 1024, 8, 0.0, 3e-6), (700, 4096, 1024, 8, 0.0, 3e-6), (512, 4096, 1024, 16, 0.05, 3e-6),
+                                                        (300, 4096, 1024, 64, 0.05, 3e-6), (512, 14336, 1024, 8, 0.0, 1.1e-5), (64, 4096, 14336, 8, 0.0, 3e-6)])
+def test_narrow_tiles_sum_into_two_accumulators(T, d_in, d_out, r, b_std, limit):
+    N, k = 28, 2
+    g = torch.Generator(device="cuda").manual_seed(d_in + r)
+    rand = lambda *s: torch.randn(*s, device="cuda", generator=g)  # noqa: E731
+    x, W0 = rand(d_in).bfloat16(), (0.02 * rand(d_out, d_in)).bfloat16()
+    A, B, Wg = (rand(N, r, d_in) / d_in ** 0.5).bfloat16(), (b_std * rand(N, d_out, r)).bfloat16(), (rand(N, d_in) / d_in ** 0.5).bfloat16()
+    x[-4:], W0[:, -4:] = 1, 0
+    logits, idx = (Wg.double() @ x.double()).topk(k)
+    w = torch.softmax(logits, 0)
+    y = W0.double() @ x.double() + sum(w[j] * (B[idx[j]].double() @ (A[idx[j]].double() @ x.double())) for j in range(k))
+    rest = -y
+    for c in range(d_in - 4, d_in):
+        W0[:, c] = rest.bfloat16()
+        rest = rest - W0[:, c].double()
+    got = mb.meteora_linear_forward(x.repeat(T, 1), W0, A, B, Wg, k)
+    assert torch.equal(got, got[:1].expand(T, d_out))
+    assert float((got[0].double() + rest).pow(2).mean().sqrt() / y.pow(2).mean().sqrt()) <= limit
