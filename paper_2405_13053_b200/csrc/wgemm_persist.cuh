@@ -427,6 +427,10 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
     // its loads and MMAs (3 - 3.5 us for three parts) had nothing to hide under; but not ahead of its main product's first step, which
     // clears the accumulator: behind the loop (mid == iters) where that has one iteration
     const int iters = (p.ksteps + kc - 1) / kc, mid = max(max(iters / 2, iters - 12 / kc), own ? 1 : 0);
+    // A short axis reaches that point before the routing is ready, and the loads behind it would wait with it: a pair's first tile then
+    // gets its own behind the loop (us, in the loop / behind it: 1024 -> 4096 at 300 tokens 13.9 / 12.6, 2048 -> 2560 at 2048 32.0 / 28.9, 2048 -> 9216 at
+    // 64 14.3 / 12.9, 2560 -> 14336 at 128 17.1 / 16.2; from 48 k-steps on it hides less than it waits: 3072 -> 14336 at 64 16.9 / 17.1, 4096 27.0 / 27.8)
+    const int mid0 = own && p.ksteps <= 40 ? iters : mid;
 
     // kWalkNarrow sums the two k-steps of a stage, and every other MMA of the expand, into an accumulator of their own each, 128 columns
     // apart: the tensor cores cut off what they add instead of rounding it, so the error grows with the MMAs into one.  An expand in three
@@ -546,7 +550,7 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                     const CUtensorMap* mW = &maps.W0[t.mod];
                     const int w_row = row_tile * tr;
                     for (int i = 0; i <= iters; ++i) {
-                        if (i == mid && (pending || own) && !(ok = expand(own ? t : before))) break;
+                        if (i == (lin == pair0 ? mid0 : mid) && (pending || own) && !(ok = expand(own ? t : before))) break;
                         if (i == iters || !(ok = slot(bar, full, dst))) break;
                         if (elect_one()) {
                             if (leader) mbar_expect_tx(bar, tx);
@@ -636,7 +640,7 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                 }
                 uint32_t wa;
                 for (int i = 0; i <= iters; ++i) {
-                    if (i == mid && (pending || own) && !(ok = expand(own ? b : b ^ 1))) break;
+                    if (i == (n == 0 ? mid0 : mid) && (pending || own) && !(ok = expand(own ? b : b ^ 1))) break;
                     if (i == iters || !(ok = next(wa))) break;
                     const uint64_t da = smem_desc_sw128(wa), db = smem_desc_sw128(wa + kc * kWTileBytes);
                     if (elect_one()) {
