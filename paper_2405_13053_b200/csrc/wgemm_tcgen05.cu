@@ -2731,13 +2731,17 @@ static TokenPlan make_token_plan(const meteora_shape_t& s, int mode) {
 
 // The plan of two shrinks that run side by side (gate's gradient): where clusters of four CTAs or more hold both launches at once
 // they share the SMs (2048 tokens: 64 CTAs each and one wave, 86.6 us for the training step; 96 each and two waves 91.9), else
-// each is planned as if alone (smaller clusters: 3000 tokens, 2000 -> 5000, 111.6 alone, 113.0 shared).
+// each is planned as if alone (smaller clusters: 3000 tokens, 2000 -> 5000, 111.6 alone, 113.0 shared).  A smaller cluster's CTAs add more
+// products into one accumulator each, so they take two (error of dlogit at 2048 tokens, 4096 -> 4096: alone 1.20e-6, shared with one 1.85e-6,
+// with two 0.87e-6); where the columns leave no room for those (rank 16 and 28 adapters), each is planned as if alone.
 static TokenPlan make_shrink_pair_plan(const meteora_shape_t& s) {
     const TokenPlan alone = make_token_plan(s, TOKEN_SHRINK);
     if (!alone.ok || alone.groups > 1) return alone;
-    const TokenPlan shared = make_token_plan_with(s, TOKEN_SHRINK, 1, 2);
+    TokenPlan shared = make_token_plan_with(s, TOKEN_SHRINK, 1, 2);
     const int tiles = (s.T + kTokTile - 1) / kTokTile;
-    return shared.ok && shared.S >= 4 && 2 * tiles <= token_cluster_capacity(shared.S) ? shared : alone;
+    if (!shared.ok || shared.S < 4 || 2 * tiles > token_cluster_capacity(shared.S) || (shared.S < alone.S && shared.rounds > 1)) return alone;
+    shared.dual = shared.S < alone.S;
+    return shared;
 }
 
 // Clusters of S CTAs of kThreads, launched programmatically dependent.
@@ -2832,8 +2836,8 @@ int launch_token_shrink(const void* x, const void* A, const int32_t* topk_idx, c
     p.clear_status = status && !beside ? 1 : 0;
     p.late_wait = beside && tuning().pdl ? 1 : 0;
     TokenPlan tp = pair ? make_shrink_pair_plan(s) : make_token_plan(s, TOKEN_SHRINK);
-    if (dual && tp.rounds == 1) {
-        tp.dual = true;
+    tp.dual = (tp.dual || dual) && tp.rounds == 1;
+    if (tp.dual) {
         tp.acc2 = (tp.cols[0] + 31) / 32 * 32;
         while (tp.tmem_cols < tp.acc2 + tp.cols[0]) tp.tmem_cols *= 2;
         tp.smem = smem_with_tmem(tp.smem, tp.tmem_cols);

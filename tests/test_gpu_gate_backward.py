@@ -132,3 +132,20 @@ def test_gate_backward_keeps_a_non_finite_token_to_its_own_picks(T):
     assert torch.isnan(dWg[own]).all()                    # its dlogit is NaN
     # the others: the same fp32 sums, in another order where a column was summed again
     assert rel_l2(dWg[~own].cpu().numpy(), clean[~own].cpu().numpy()) <= 1e-6
+
+
+# The tensor cores cut off what they add to an accumulator: measured 2^-25 of the sum per MMA (16 products) into it.  The bounds are those of
+# clusters that have the SMs to themselves: 6 CTAs per tile at 2048 tokens, 16 at 700, 8 at 1500 and rank 16.
+@pytest.mark.parametrize("T,d,N,r,ctas", [(2048, 4096, 28, 8, 6), (700, 4096, 8, 8, 16), (1500, 2048, 28, 16, 8)])
+def test_shrinks_side_by_side_are_as_exact_as_alone(T, d, N, r, ctas):
+    g = torch.Generator(device="cuda").manual_seed(T)
+    rand = lambda *s: torch.randn(*s, device="cuda", generator=g)  # noqa: E731
+    x, dy = rand(T, d).bfloat16(), rand(T, d).bfloat16()
+    A, B = (rand(N, r, d) / d ** 0.5).bfloat16(), (0.3 * rand(N, d, r)).bfloat16()
+    idx = torch.rand(T, N, device="cuda", generator=g).topk(2, dim=1).indices.int().contiguous()
+    wts = torch.softmax(rand(T, 2), dim=1)
+    dWg, dlogit = mb.meteora_gate_backward(x, A, B, dy, idx, wts)
+    o_dlogit, o_dWg = _slot_sums(x, A, B, dy, idx, wts, 1.0)
+    bound = 2.0 ** -25 * (d / 16 / ctas + 1)
+    assert rel_l2(dlogit.cpu().numpy(), o_dlogit.cpu().numpy()) <= bound
+    assert rel_l2(dWg.cpu().numpy(), o_dWg.cpu().numpy()) <= bound
