@@ -95,7 +95,8 @@ int meteora_route(const int32_t* topk_idx, int T, int k, int N, int32_t* counts,
  *   delta[t,:] = sum_j topk_w[t,j] * B[topk_idx[t,j]] (A[topk_idx[t,j]] x[t]).
  * The shrink (x A_i) runs adapter by adapter over the grouped slots (offsets, perm from
  * meteora_route), the expand and weighted sum run token by token.
- *   delta[T,d_out] fp32.  workspace: device scratch of at least meteora_workspace_bytes(shape).
+ *   delta[T,d_out] fp32.  workspace: device scratch of at least meteora_workspace_bytes(shape); bounded waits
+ *   of this call that expired are reported by meteora_workspace_status.
  */
 int meteora_lora_delta(const void* x, const void* A, const void* B, const int32_t* topk_idx,
                        const float* topk_w, const int32_t* offsets, const int32_t* perm,

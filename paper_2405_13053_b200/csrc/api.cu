@@ -248,7 +248,7 @@ int meteora_lora_delta(const void* x, const void* A, const void* B, const int32_
     const Workspace ws = carve_workspace(*shape, workspace);
     if (workspace_bytes < ws.bytes) return METEORA_ERR_WORKSPACE_TOO_SMALL;
     cudaStream_t st = (cudaStream_t)stream;
-    if ((rc = launch_shrink(x, A, topk_idx, offsets, perm, *shape, ws.uw, st)) != METEORA_OK) return rc;
+    if ((rc = launch_shrink(x, A, topk_idx, offsets, perm, *shape, ws.uw, ws.status, st)) != METEORA_OK) return rc;
     return launch_expand(B, topk_idx, topk_w, ws.uw, *shape, delta, ws.status, st);
 }
 

@@ -74,7 +74,7 @@ int launch_route(const int32_t* topk_idx, int T, int k, int N, int32_t* counts, 
                  cudaStream_t st);
 // lora.cu
 int launch_shrink(const void* x, const void* A, const int32_t* topk_idx, const int32_t* offsets, const int32_t* perm,
-                  const meteora_shape_t& s, float* u, cudaStream_t st);
+                  const meteora_shape_t& s, float* u, int32_t* status, cudaStream_t st);
 int launch_shrink_segments(const void* x, const void* A, const int32_t* offsets, const int32_t* perm,
                            const meteora_shape_t& s, float* u, cudaStream_t st);
 int launch_expand(const void* B, const int32_t* topk_idx, const float* topk_w, const float* u,

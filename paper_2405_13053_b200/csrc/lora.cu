@@ -290,8 +290,8 @@ k_expand_slab(const __nv_bfloat16* __restrict__ B, const int32_t* __restrict__ t
 // Where the tensor cores take the layer, the picks' shrink comes from token tiles (all adapters as one dense product, the
 // picks gathered on the chip); else adapter by adapter over the bucketed slots.
 int launch_shrink(const void* x, const void* A, const int32_t* topk_idx, const int32_t* offsets, const int32_t* perm,
-                  const meteora_shape_t& s, float* u, cudaStream_t st) {
-    if (token_shrink_supported(s)) return launch_token_shrink(x, A, topk_idx, s, u, nullptr, false, false, expand_tile_supported(s), st);
+                  const meteora_shape_t& s, float* u, int32_t* status, cudaStream_t st) {
+    if (token_shrink_supported(s)) return launch_token_shrink(x, A, topk_idx, s, u, status, false, false, expand_tile_supported(s), st);
     return launch_shrink_segments(x, A, offsets, perm, s, u, st);
 }
 

@@ -60,6 +60,6 @@ extern "C" int meteora_lora_delta_static(const void* x, const void* A, const voi
     cudaStream_t st = (cudaStream_t)stream;
     // Nothing in the scratch has to start at zero: the shrink writes u[slot, :] for every slot of the
     // permutation before the expand reads it, so what an earlier call left there is never seen.
-    if ((rc = launch_shrink(x, A, topk_idx, offsets, perm, *s, u, st)) != METEORA_OK) return rc;
+    if ((rc = launch_shrink(x, A, topk_idx, offsets, perm, *s, u, nullptr, st)) != METEORA_OK) return rc;
     return launch_expand(B, topk_idx, topk_w, u, *s, delta, nullptr, st);
 }

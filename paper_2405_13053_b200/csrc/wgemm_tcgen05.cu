@@ -2823,7 +2823,7 @@ int launch_token_forward(const void* x, const void* A, const void* Wg, const met
 
 bool token_shrink_supported(const meteora_shape_t& s) { return make_token_plan(s, TOKEN_SHRINK).ok; }
 
-// status (optional) is cleared first; `beside`: launched right behind another shrink whose results it does not read; pair: one of
+// status (optional) is cleared first for the gate's gradient, which has a workspace of its own; `beside`: launched right behind another shrink whose results it does not read; pair: one of
 // two such; dual: two accumulators where they fit (the expand behind it is on the tensor cores too, whose cut-off sums would
 // otherwise add to the error: 1 - 3 % more; with both it is 8 - 50 % smaller than with CUDA cores behind one accumulator.  0.4 us
 // that a small batch would feel)
@@ -2833,7 +2833,7 @@ int launch_token_shrink(const void* x, const void* A, const int32_t* topk_idx, c
     p.topk_idx = const_cast<int32_t*>(topk_idx);
     p.u = u;
     p.status = status;
-    p.clear_status = status && !beside ? 1 : 0;
+    p.clear_status = status && pair && !beside ? 1 : 0;
     p.late_wait = beside && tuning().pdl ? 1 : 0;
     TokenPlan tp = pair ? make_shrink_pair_plan(s) : make_token_plan(s, TOKEN_SHRINK);
     tp.dual = (tp.dual || dual) && tp.rounds == 1;
