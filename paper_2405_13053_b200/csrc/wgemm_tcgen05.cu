@@ -1488,6 +1488,8 @@ static int persist_pairs() {
     return have - 1;
 }
 
+static int token_forward_ctas(const meteora_shape_t& s);
+
 // One module, or a group of modules that share x; with_routing: gate, selection and shrink as the walk's first tiles.
 static PersistPlan make_persist_plan(const meteora_shape_t& s, const int* d_outs, int G, bool with_routing) {
     PersistPlan pp = {};
@@ -1527,13 +1529,20 @@ static PersistPlan make_persist_plan(const meteora_shape_t& s, const int* d_outs
     // Half a round of 256-token tiles or less: tiles of 128 tokens, or of 64 where there are nine or fewer (us per call with tiles of 256 / 128 / 64:
     // 4096 -> 1024 at 2048 tokens, 32 tiles, 39.8 / 32.2 / 39.4; rank 32, 4096 -> 4096 at 512, 32 tiles, 51.8 / 41.7 / 56.8; 4096 -> 2048 at 512, 16 tiles,
     // - / 18.9 / 23.6; 4096 -> 1024 at 512, 8 tiles, - / 17.4 / 15.8).
+    // But 20 tiles and more of a short axis and up to 1024 tokens stay as they are where all their pairs find SMs beside the routing's CTAs, of which
+    // narrow ones would wait for some: half as long a main loop is then worth less than the wait (us, narrow / 256: 1024 -> 2048 at 700 / 1024 tokens 17.3 / 15.2, 18.4 / 15.9, at 800, where
+    // neither fits, 17.6 / 19.1; 2048 -> 2048 at 700 / 1024 20.1 / 18.1, 21.5 / 18.0; 3072 -> 2048 at 1024 24.7 / 22.4; 4096 -> 2048 at 700 / 1024 25.4 / 27.1,
+    // 27.6 / 26.8).  (Beyond 1024 tokens only layers of up to 7 row pairs have so few tiles: 1024 -> 1024 at 1280 17.9 / 15.9.)  Below 20 the alternative were split tiles, which sum into two accumulators as narrow ones do and 256-token ones do not.
     bool narrow = false;
     if (!with_routing && s.T > kPairTokens && whole_steps && 2 * pp.tiles <= pairs) {
-        const int row_pairs = pp.tiles / pp.tok_tiles, width = 8 * pp.tiles <= pairs ? 64 : 128;
-        narrow = true;
-        pp.tok_tiles = (s.T + width - 1) / width;
-        pp.BN = ((s.T + pp.tok_tiles - 1) / pp.tok_tiles + 31) / 32 * 32;
-        pp.tiles = row_pairs * pp.tok_tiles;
+        const int row_pairs = pp.tiles / pp.tok_tiles, width = 8 * pp.tiles <= pairs ? 64 : 128, tok_tiles = (s.T + width - 1) / width;
+        const int beside = pp.tiles >= 20 && s.T <= 1024 && s.d_in <= 48 * kBK ? token_forward_ctas(s) : 0, sms = 2 * pairs;
+        narrow = !(beside > 0 && beside + 2 * pp.tiles <= sms && beside + 2 * row_pairs * tok_tiles > sms);
+        if (narrow) {
+            pp.tok_tiles = tok_tiles;
+            pp.BN = ((s.T + pp.tok_tiles - 1) / pp.tok_tiles + 31) / 32 * 32;
+            pp.tiles = row_pairs * pp.tok_tiles;
+        }
     }
     if (with_routing) {
         // [Wg; a share of A] in pairs of 128-row tiles: Wg padded to whole 32 rows (a warp's TMEM lanes), A to whole MMAs of the expand
@@ -2806,6 +2815,12 @@ int launch_token_gate(const void* x, const void* Wg, const meteora_shape_t& s, i
 }
 
 bool token_forward_supported(const meteora_shape_t& s) { return make_token_plan(s, TOKEN_FORWARD).ok; }
+
+// CTAs of that launch (0: the routing comes from other kernels).
+static int token_forward_ctas(const meteora_shape_t& s) {
+    const TokenPlan tp = make_token_plan(s, TOKEN_FORWARD);
+    return tp.ok ? (s.T + kTokTile - 1) / kTokTile * tp.S : 0;
+}
 
 int launch_token_forward(const void* x, const void* A, const void* Wg, const meteora_shape_t& s, const Workspace& ws, void* us,
                          bool beside, cudaStream_t st) {
