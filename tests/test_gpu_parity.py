@@ -214,8 +214,8 @@ FORWARD_CASES = [
     dict(T=20, d_in=256, d_out=128, N=8, r=8, k=1, dtype="bf16"),                 # top-1
     dict(T=40, d_in=512, d_out=256, N=28, r=32, k=4, dtype="bf16"),               # rank 32, top-4, decode batch
     dict(T=30, d_in=512, d_out=384, N=28, r=4, k=2, dtype="bf16"),                # rank 4: adapters zero-padded to 8
-    dict(T=300, d_in=1024, d_out=256, N=28, r=8, k=2, dtype="bf16"),              # short prefill grid: two CTAs per 128-token tile
-    dict(T=700, d_in=8192, d_out=512, N=28, r=8, k=2, dtype="bf16"),              # long axis: two CTAs per 256-token tile
+    dict(T=300, d_in=1024, d_out=256, N=28, r=8, k=2, dtype="bf16"),              # few tiles, whole k-steps: the walk's narrow tiles
+    dict(T=700, d_in=8192, d_out=512, N=28, r=8, k=2, dtype="bf16"),              # the same over a long axis
     dict(T=300, d_in=256, d_out=256, N=12, r=12, k=3, dtype="bf16"),              # rank 12 -> 16, prefill batch
     dict(T=600, d_in=512, d_out=200, N=28, r=64, k=2, dtype="bf16"),              # rank 64 prefill, d_out % 8 == 0 only
     dict(T=24, d_in=256, d_out=136, N=4, r=8, k=4, dtype="bf16", temperature=20.0),  # k = N with temperature
@@ -232,6 +232,18 @@ def test_forward_small_shapes(case):
         check_forward(w, y_tol=1e-4)
     else:
         check_forward(w, y_tol=1e-2)
+
+
+# what short prefill batches take: the walk's narrow tiles over whole k-steps; else split tiles of 128 tokens, of 256 over a long axis, with
+# the expand on the tensor cores or (rank 24) in fp32
+@pytest.mark.parametrize("T,d_in,d_out,r,plan", [
+    (512, 4096, 1024, 8, " tile=256x64 "), (300, 1024, 256, 8, " tile=256x64 "), (700, 8192, 512, 8, " tile=256x64 "),
+    (300, 1000, 256, 8, " cluster=2 tile_tokens=128 "), (700, 8200, 512, 8, " cluster=2 tile_tokens=256 "),
+    (300, 520, 256, 24, " cluster=2 tile_tokens=128 "), (700, 8200, 512, 24, " cluster=2 tile_tokens=256 "),
+])
+def test_short_prefill_tiles(T, d_in, d_out, r, plan):
+    assert plan in mb.meteora_describe_plan(mb.make_shape(T, d_in, d_out, 28, r, 2, torch.bfloat16))
+    check_forward(wl(T=T, d_in=d_in, d_out=d_out, N=28, r=r, k=2, dtype="bf16"), y_tol=1e-2)
 
 
 @pytest.mark.parametrize("T", workloads.CONFIG1_T)

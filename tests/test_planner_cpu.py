@@ -50,6 +50,8 @@ def test_prefill_on_pairs_and_the_carved_last_wave():
 
 
 def test_short_prefill_grids_put_two_ctas_on_a_tile():
+    # (without a device there are no pairs of SMs to ask for: on one these shapes, of whole k-steps, take the persistent walk, and the
+    # split tiles serve axes that are no multiple of 64 and ranks that do not pad to 8, 16, 32 or 64)
     p = plan(512, 14336, 4096)                  # long contraction axis: 256-token tiles, two CTAs each
     assert "base_ctas=128 cluster=2 tile_tokens=256 " in p, p
     p = plan(512, 4096, 1024)                   # 32 tiles of 128 tokens: two CTAs each
