@@ -221,7 +221,7 @@ int meteora_gate_topk(const void* x, const void* Wg, const meteora_shape_t* shap
     if (shape->T == 0) return METEORA_OK;
     if (!x || !Wg || !topk_idx || !topk_w) return METEORA_ERR_INVALID_ARG;
     if (!aligned16(x) || !aligned16(Wg)) return METEORA_ERR_MISALIGNED;
-    if (token_gate_supported(*shape)) return launch_token_gate(x, Wg, *shape, topk_idx, topk_w, logits, (cudaStream_t)stream);
+    if (token_gate_supported(*shape)) return launch_token_gate(x, Wg, *shape, topk_idx, topk_w, logits, nullptr, false, (cudaStream_t)stream);
     return launch_gate_topk(x, Wg, *shape, topk_idx, topk_w, logits, (cudaStream_t)stream);
 }
 

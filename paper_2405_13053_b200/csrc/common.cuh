@@ -105,7 +105,7 @@ int launch_base_lora_tc(const void* x, const void* W0, const void* B, const mete
 // token tiles (wgemm_tcgen05.cu + token_tile.cuh): gate, selection, shrink of the picks, gate gradient
 bool token_gate_supported(const meteora_shape_t& s);
 int launch_token_gate(const void* x, const void* Wg, const meteora_shape_t& s, int32_t* topk_idx, float* topk_w, float* logits,
-                      cudaStream_t st);
+                      int32_t* status, bool beside, cudaStream_t st);
 bool token_forward_supported(const meteora_shape_t& s);
 int launch_token_forward(const void* x, const void* A, const void* Wg, const meteora_shape_t& s, const Workspace& ws, void* us,
                          bool beside, cudaStream_t st);

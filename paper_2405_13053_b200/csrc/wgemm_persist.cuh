@@ -18,12 +18,13 @@
 //     main loop's where the routing kernels ran ahead);
 //   - where the kernels otherwise taken expand in fp32 (decode batches, few tiles of large ranks: persist_us_parts) us is
 //     three bf16 parts whose sum is w_j (A_e x_t)_q exactly: a k-step of the expand is then two stages, (B, part 0) and
-//     (part 1, part 2), so that B is read once; the routing kernels ahead write the parts.  Such a token's y depends on its
+//     (part 1, part 2), or on narrow tiles one with all of them, so that B is read once; the routing kernels ahead write the parts.  Such a token's y depends on its
 //     own picks alone, also where an adapter that it did not pick holds an infinity or a NaN: 0 times those is NaN, and a
-//     NaN of such a row is computed again from the picks.  Measured against rounded parts: 4096 -> 2 x 14336 at 64 tokens
-//     49.9 -> 52.2 us, 5120 -> 13824 at 200 tokens 37.3 -> 39.4 (four stages more per tile);
+//     NaN of such a row is computed again from the picks.  Against a rounded operand this cost, when a
+//     tile's four k-steps took two stages each, 2.1 - 2.3 us (5120 -> 13824 at 200 tokens, where they still do, 37.3 -> 39.4);
 //   - modules that share x (q/k/v, gate/up) are one walk: their tiles fill rounds of pairs together.
-// Where A has more rows than four pairs of stacked tiles take, the batch more stacked tiles than pairs, one round of tiles would become two, or
+// Where [Wg; A] has more than 512 rows, or where it saves a round, a launch of gate tiles ahead selects, and the stacked tiles are A's rows alone.
+// Where A has more than four pairs take, the batch more stacked tiles than pairs, one round of tiles would become two, or
 // us is three parts, the routing kernels ahead write us and only the base product runs here (stacked_pairs = 0).
 // What bounds it: the tensor cores under the board's power limit (514 cycles per 64-element k-step and 256 x 256 tile, of
 // the 512 that its four MMAs take).  All pairs walk the contraction axis in step, so a line of W0 or x is fetched once for the pairs
@@ -73,7 +74,7 @@ struct PersistParams {
     int tr;                       // kWalkNarrow: rows of W0 per CTA and tile, 128 or fewer (whole 8s from 64 up), which spreads a batch over the pairs
     int n_mod, tok_tiles, tiles;
     int stacked_pairs;            // pairs of 128-row tiles, [Wg; a share of A] each (0: us comes from the kernel ahead)
-    int gate_rows, us_cols;       // Wg's rows padded to whole 32s; columns of a part of us that are read
+    int gate_rows, us_cols;       // Wg's rows padded to whole 32s (0: the kernel ahead selects); columns of a part of us that are read
     int parts;                    // of us: 1 or 3
     float inv_tau;
     int32_t* flags;               // [module][token tile]: warps whose part of us is written; zero between calls
@@ -394,6 +395,26 @@ __device__ __forceinline__ void persist_select(const PersistParams& p, float* s_
     asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
 }
 
+// The same from what the kernel ahead selected, by a group of four warps for itself.
+__device__ __forceinline__ void persist_load_routing(const PersistParams& p, const PersistModule& mo, PersistRouting* rt, int grp, int quad,
+                                                     int nslots, int tok0) {
+    const int slot = quad * 32 + (threadIdx.x & 31);
+    if (slot < nslots) {
+        const int t = tok0 + persist_column(p, grp, slot);
+        unsigned long long picks = ~0ull;
+        if (t < p.T) {
+            picks = p.k < 8 ? ~0ull << (8 * p.k) : 0ull;
+#pragma unroll 1
+            for (int j = 0; j < p.k; ++j) {
+                picks |= (unsigned long long)(__ldcg(mo.topk_idx + (size_t)t * p.k + j) & 0xFF) << (8 * j);
+                rt->w[j][slot] = __ldcg(mo.topk_w + (size_t)t * p.k + j);
+            }
+        }
+        rt->picks[slot] = picks;
+    }
+    asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
+}
+
 // What the issuing loops need to know at compile time: read from the parameters in the loops, the rows and k-steps of a stage cost
 // 0.4 - 0.8 us of 29 (4096 -> 4096 at 512 tokens).
 //   kWalkStacked  the routing in the walk, us rounded        k-steps one by one, 128 rows per CTA
@@ -473,8 +494,8 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
             int s = 0, round = 0;                                 // ring slot, how often the ring has been filled
             const uint32_t leader_bars = map_to_cta(bar_base, 0);
             bool waited = !p.pdl;
-            // with stacked tiles x comes from the kernel ahead; else the kernel ahead is this call's routing, which read x
-            if (!own && !waited) {
+            // with the selection in the walk x comes from the kernel ahead; else the kernel ahead is this call's routing, which read x
+            if (!own && p.gate_rows > 0 && !waited) {
                 asm volatile("griddepcontrol.wait;" ::: "memory");
                 waited = true;
             }
@@ -541,7 +562,7 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                         if (elect_one()) {
                             if (leader) mbar_expect_tx(bar, tx);
                             tma_load_2d_pair(dst + w_off, mW, i * kBK, w_row, full);
-                            if (leader) tma_load_2d_pair(dst, &maps.G[t.mod], i * kBK, 0, full);
+                            if (leader && p.gate_rows > 0) tma_load_2d_pair(dst, &maps.G[t.mod], i * kBK, 0, full);
                             tma_load_2d_pair(dst + kWTileBytes, &maps.X, i * kBK, tokh, full);
                         }
                         __syncwarp();
@@ -701,7 +722,10 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                 PersistRouting* rt = reinterpret_cast<PersistRouting*>(reinterpret_cast<uint8_t*>(ystage) + kPersistStoreBytes / 2);
                 const int nslots = grp < chunks ? (chunks - grp + 1) / 2 * kPersistChunk : 0;
                 bool have = true;
-                if (rank == 0) {
+                if (p.gate_rows == 0) {
+                    asm volatile("griddepcontrol.wait;" ::: "memory");
+                    persist_load_routing(p, mo, rt, grp, quad, nslots, tok0);
+                } else if (rank == 0) {
                     const uint32_t peer_rt = map_to_cta(ysmem + kPersistStoreBytes / 2, 1);
                     if (p.gate_rows <= 32)
                         persist_select<1>(p, reinterpret_cast<float*>(ystage), rt, peer_rt, taddr, grp, quad, nslots, tok0);
@@ -786,7 +810,7 @@ k_wgemm_persist(const __grid_constant__ PersistMaps maps, const __grid_constant_
                 __syncwarp();
                 asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
                 if (elected) mbar_arrive_cluster(map_to_cta(bar_acce + b * 8, 0));
-                if (rank == 0 && t.row_pair == 0) {               // the routing for the caller
+                if (rank == 0 && t.row_pair == 0 && p.gate_rows > 0) {   // the routing for the caller
 #pragma unroll 1
                     for (int i = quad * 32 + lane; i < nslots * p.k; i += 128) {
                         const int j = i / nslots, slot = i - j * nslots, e = (int)(rt->picks[slot] >> (8 * j)) & 0xFF;

@@ -1552,6 +1552,22 @@ static PersistPlan make_persist_plan(const meteora_shape_t& s, const int* d_outs
         if (pp.stacked_pairs > kPersistMaxStacked || s.N > kPersistMaxN || G * pp.tok_tiles > kMaxFusedRowTiles ||
             G * pp.stacked_pairs * pp.tok_tiles > pairs)             // (a stacked tile is a pair's first)
             return pp;
+        // Logits of a stacked tile are sums over the whole axis in one accumulator, of which the tensor cores cut off as they add: the error of the routing
+        // weights grows with the axis, where other kernels split it over CTAs (1531 tokens, 4096 -> 4096, 64 adapters: inside 1.9e-6, with the stacked
+        // shrink 4.1e-7, from gate tiles 2.1e-7).  With more than 512 rows of [Wg; A], which those others took before, a launch of gate tiles
+        // selects ahead and the stacked tiles are A's rows alone, rounded to bf16 anyway.  us with the stacked shrink / routing inside / gate ahead: 4096 ->
+        // 4096, 64 adapters, at 1531 / 2048 / 4096 tokens 71.8 / 53.4 / 63.6, 74.2 / 73.8 / 65.7, 139 / 131 / 123; 14336 -> 4096 at 2048 211 / 250 / 202; rank
+        // 32, 4096 -> 4096 at 2048 92.7 / 77.7 / 87.9.  With fewer rows where that is a round of tiles less (50 adapters, 14336 -> 4096 at 2048, inside /
+        // ahead 247 / 210; 5120 -> 5120, three rounds either way, 100 / 105).
+        if (pp.stacked_pairs > 2) {
+            const int alone = (pp.us_cols + 2 * kBM - 1) / (2 * kBM);
+            auto rounds = [&](int n) { return (pp.tiles + G * n * pp.tok_tiles + pairs - 1) / pairs; };
+            if (pp.gate_rows + pp.us_cols > 4 * kBM || rounds(alone) < rounds(pp.stacked_pairs)) {
+                if (!token_gate_supported(s)) return pp;
+                pp.gate_rows = 0;
+                pp.stacked_pairs = alone;
+            }
+        }
         if (tn.persist == 3) return pp;
         // the stacked tiles write us rounded to bf16: not where it is three parts (knob 2, a measurement: all the same).  The
         // routing ahead costs such a batch nothing: 4096 -> 2 x 14336 at 64 / 128 tokens 54.4 / 56.3 us, with parts written from
@@ -1647,7 +1663,7 @@ static int launch_persist(const PersistPlan& pp, const void* x, const GroupModul
         if (pp.stacked_pairs > 0) {
             if ((rc = get_tensor_map(gm.A, s.d_in, s.N * s.r, kBM, 0, &maps.A[m])) != METEORA_OK) return rc;
             if ((rc = get_tensor_map(gm.A, s.d_in, s.N * s.r, kBM - pp.gate_rows, 0, &maps.A0[m])) != METEORA_OK) return rc;
-            if ((rc = get_tensor_map(gm.Wg, s.d_in, s.N, pp.gate_rows, 0, &maps.G[m])) != METEORA_OK) return rc;
+            if (pp.gate_rows > 0 && (rc = get_tensor_map(gm.Wg, s.d_in, s.N, pp.gate_rows, 0, &maps.G[m])) != METEORA_OK) return rc;
         }
         PersistModule& mo = p.mod[m];
         mo.row_pairs = (gm.d_out + 2 * pp.tr - 1) / (2 * pp.tr);
@@ -1723,12 +1739,17 @@ static int launch_persist(const PersistPlan& pp, const void* x, const GroupModul
     return cuda_status(err);
 }
 
-// The whole layer of one module or of a group of modules that share x, one launch.
+// The whole layer of one module or of a group of modules that share x, one launch (and one of gate tiles per module).
 int launch_persist_forward(const void* x, const GroupModule* mods, int G, const meteora_shape_t& s, int32_t* status, int32_t* flags,
                            cudaStream_t st) {
     int d_outs[kMaxGroupModules] = {};
     for (int m = 0; m < G; ++m) d_outs[m] = mods[m].d_out;
-    return launch_persist(make_persist_plan(s, d_outs, G, true), x, mods, G, s, status, flags, tuning().pdl != 0, st);
+    const PersistPlan pp = make_persist_plan(s, d_outs, G, true);
+    for (int m = 0; m < G && pp.gate_rows == 0; ++m) {
+        const int rc = launch_token_gate(x, mods[m].Wg, s, mods[m].ws.topk_idx, mods[m].ws.topk_w, nullptr, status, m > 0, st);
+        if (rc != METEORA_OK) return rc;
+    }
+    return launch_persist(pp, x, mods, G, s, status, flags, tuning().pdl != 0, st);
 }
 
 // The base products of modules whose routing and us are there: one launch.
@@ -2805,9 +2826,12 @@ static int launch_token_tile(const TokenPlan& tp, int mode, const meteora_shape_
 
 bool token_gate_supported(const meteora_shape_t& s) { return make_token_plan(s, TOKEN_GATE).ok; }
 
+// (status may be null; `beside`: launched right behind another gate whose results it does not read)
 int launch_token_gate(const void* x, const void* Wg, const meteora_shape_t& s, int32_t* topk_idx, float* topk_w, float* logits,
-                      cudaStream_t st) {
+                      int32_t* status, bool beside, cudaStream_t st) {
     TokenTileParams p = {};
+    p.status = status;
+    p.late_wait = beside && tuning().pdl ? 1 : 0;
     p.topk_idx = topk_idx;
     p.topk_w = topk_w;
     p.logits = logits;
@@ -2994,9 +3018,9 @@ int describe_plan(const meteora_shape_t& s, char* buf, size_t n) {
     const PersistPlan whole = make_persist_plan(s, &s.d_out, 1, true);
     if (whole.ok && !on_pairs)
         return snprintf(buf, n,
-                        "path=persistent_prefill launches=1 base=pairs_of_ctas persistent_pairs=%d tiles=%d stacked_tiles=%d tile=256x%d "
+                        "path=persistent_prefill launches=%d base=pairs_of_ctas persistent_pairs=%d tiles=%d stacked_tiles=%d tile=256x%d "
                         "stages=%d smem=%zu expand=mma",
-                        whole.pairs, whole.tiles, whole.stacked_pairs * whole.tok_tiles, whole.BN, whole.stages, whole.smem);
+                        whole.gate_rows > 0 ? 1 : 2, whole.pairs, whole.tiles, whole.stacked_pairs * whole.tok_tiles, whole.BN, whole.stages, whole.smem);
     const PersistPlan ps = make_persist_plan(s, &s.d_out, 1, false);
     if (ps.ok)
         return snprintf(buf, n,

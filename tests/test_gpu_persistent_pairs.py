@@ -248,3 +248,42 @@ def test_narrow_tiles_sum_into_two_accumulators(T, d_in, d_out, r, b_std, limit)
     got = mb.meteora_linear_forward(x.repeat(T, 1), W0, A, B, Wg, k)
     assert torch.equal(got, got[:1].expand(T, d_out))
     assert float((got[0].double() + rest).pow(2).mean().sqrt() / y.pow(2).mean().sqrt()) <= limit
+
+
+# More than 512 rows of [Wg; A], or a round of tiles less with it: gate tiles select ahead, the walk's stacked tiles are A alone.  Error of the routing weights over
+# 4096 products: 1.9e-6 from a stacked tile's one accumulator, 2^-25 per MMA (16 products) of a CTA from gate tiles.
+@pytest.mark.parametrize("T,d_in,d_out,N,r,k,persist", [(1100, 512, 4352, 64, 8, 2, 1), (300, 200, 264, 64, 8, 8, 2), (513, 328, 520, 28, 32, 2, 2),
+                                                        (257, 64, 256, 60, 8, 1, 2), (2048, 320, 4096, 50, 8, 2, 1), (700, 640, 1000, 48, 16, 3, 2), (700, 4096, 1024, 64, 8, 2, 2)])
+def test_gate_tiles_ahead_of_the_walk(T, d_in, d_out, N, r, k, persist):
+    g = torch.Generator(device="cuda").manual_seed(T + N)
+    rand = lambda *s: torch.randn(*s, device="cuda", generator=g)  # noqa: E731
+    x, W0 = rand(T, d_in).bfloat16(), (rand(d_out, d_in) / d_in ** 0.5).bfloat16()
+    A, B, Wg = (rand(N, r, d_in) / d_in ** 0.5).bfloat16(), (0.3 * rand(N, d_out, r)).bfloat16(), (rand(N, d_in) / d_in ** 0.5).bfloat16()
+    shape = mb.make_shape(T, d_in, d_out, N, r, k, torch.bfloat16)
+    ws = mb.alloc_workspace(shape)
+    mb.meteora_set_tuning("persist", persist)
+    try:
+        assert "path=persistent_prefill launches=2 " in mb.meteora_describe_plan(shape)
+        outs = []
+        for W in (W0, 0 * W0, W0):
+            y, idx, w = mb.meteora_linear_forward(x, W, A, B, Wg, k, workspace=ws, return_routing=True)
+            outs.append((y, idx.clone(), w.clone()))
+        assert mb.meteora_workspace_status(ws) == 0
+        two = mb.meteora_linear_forward_group(x, [W0, W0], [A, A], [B, B], [Wg, Wg], k)
+    finally:
+        mb.meteora_set_tuning("persist", 1)
+    y, idx, w = outs[0]
+    assert torch.equal(y, outs[2][0]) and torch.equal(idx, outs[1][1])
+    logits = x.double() @ Wg.double().T
+    picked = logits.gather(1, idx.long())
+    assert float((logits.topk(k, dim=1).values - picked).abs().max()) <= 1e-5      # (ties of fp32 sums apart)
+    ref_w = torch.softmax(picked, dim=1)
+    assert rel_l2(w.cpu().numpy(), ref_w.cpu().numpy()) <= 2.0 ** -25 * 32 + 2e-7
+    mask = torch.zeros(T, N, dtype=torch.double, device="cuda").scatter_(1, idx.long(), w.double())
+    u = (x.double() @ A.double().reshape(N * r, -1).T).view(T, N, r) * mask[:, :, None]
+    lora = u.view(T, N * r) @ B.double().permute(0, 2, 1).reshape(N * r, -1)
+    base = x.double() @ W0.double().T
+    assert rel_l2(outs[1][0].float().cpu().numpy(), lora.cpu().numpy()) <= 5e-3    # (us and y rounded to bf16 once each: 2 x 1.7e-3)
+    assert rel_l2(y.float().cpu().numpy(), (base + lora).cpu().numpy()) <= 5e-3
+    for z in two:
+        assert torch.equal(z, y)
