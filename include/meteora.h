@@ -233,6 +233,10 @@ int meteora_gate_backward_bt(const void* x, const void* A, const void* Bt, const
  * the device, the layer runs, y_host[T,d_out] is copied back, all on `stream` (pinned host memory
  * makes the copies asynchronous).  Weights and workspace stay device pointers.  The call does not
  * synchronise: y_host is valid once `stream` has been synchronised by the caller.
+ * A copy of up to 512 KB from or to 16-byte aligned pinned memory is a kernel that addresses that memory
+ * over the link: shorter for the call, but it needs SMs, so that beside a launch of another stream that fills
+ * the device it waits for SMs where a copy engine would not.  Larger copies, pageable and unaligned memory
+ * go to the copy engine.  In a captured call the copies are kernel and memcpy nodes alike.
  */
 int meteora_linear_forward_host(const void* x_host, const void* W0, const void* A, const void* B,
                                 const void* Wg, const meteora_shape_t* shape, void* y_host, void* workspace,

@@ -3,11 +3,12 @@
 //
 // The link bounds a large copy and the hand-overs around it a small one: between a copy engine's copy and a kernel lie about
 // 5 us each way, between two kernels of a stream 1 - 3, and a kernel that is launched dependent has the layer's first
-// weights on their way while x still arrives.  us per call with the engine / with this kernel, one stream: 4096 -> 4096 at 1
-// token 26.9 / 19.1, at 32 39.4 / 30.6; 4096 -> 14336 at 8 50.3 / 37.1.  16 such calls over four streams, where copies of both
+// weights on their way while x still arrives.  us per call with the engine / with this kernel, one stream, calls in a row:
+// 4096 -> 4096 at 1 token 24.6 / 16.4, at 32 36.1 / 34.6; 4096 -> 14336 at 8 48.6 / 39.6.  16 calls over four streams, where copies of both
 // directions share the link: 188 / 135 at 1 token, 257 / 204 at 32, 379 / 332 at 64 (512 KB each way), but 569 / 628 at 128: there
 // the engine's larger packets count, so copies of more than 512 KB stay with it, and so does memory that the device cannot
-// address.  148 CTAs, four 16-byte loads of a thread in flight: at 64 KB all SMs are ahead of 16 (5.3 against 7.2 us).
+// address.  The price: beside another stream's launch that fills the device a copy waits for SMs, where the engine would not.
+// 148 CTAs, four 16-byte loads of a thread in flight: at 64 KB all SMs are ahead of 16 (5.3 against 7.2 us).
 #include <cuda.h>
 
 #include <algorithm>
